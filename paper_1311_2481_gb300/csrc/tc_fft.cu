@@ -181,40 +181,6 @@ __global__ void __launch_bounds__(256) k_theta(const V* __restrict__ H1, V* __re
     }
 }
 
-// ---------------------------------------------------------------- forward z-pass
-__global__ void __launch_bounds__(256) k_zfwd(const double2* __restrict__ H2, double2* __restrict__ N,
-                                              int N_r, int M, int K, double scale,
-                                              const double2* __restrict__ tw, Radices rad, int Lf,
-                                              int m0, int mcnt, int r0, int nh) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int Pz = rad.n;
-    double2* a = reinterpret_cast<double2*>(smem_raw);
-    double2* b = a + (size_t)Lf * Pz;
-    const int cg = blockIdx.x % (3 / Lf);     // component group (Lf = 3: all three)
-    const int m = m0 + (blockIdx.x / (3 / Lf)) % mcnt;
-    const int rl = (blockIdx.x / (3 / Lf)) / mcnt;
-    const int r = r0 + rl;
-    const size_t fstride = (size_t)nh * (M + 1) * Pz;
-    const double2* h = H2 + ((size_t)rl * (M + 1) + m) * Pz;
-    const int nk = 2 * K + 1;
-    const size_t S = (size_t)N_r * (M + 1) * nk;
-    for (int idx = threadIdx.x; idx < Lf * Pz; idx += blockDim.x) {
-        const int l = idx / Pz;
-        const int z = idx - l * Pz;
-        a[idx] = h[(cg * Lf + l) * fstride + z];
-    }
-    __syncthreads();
-    double2* res = smem_fft(a, b, Lf, tw, false, rad);
-    for (int idx = threadIdx.x; idx < Lf * nk; idx += blockDim.x) {
-        const int l = idx / nk;
-        const int c = cg * Lf + l;
-        const int kk = idx - l * nk;
-        const int k = kk - K;
-        const double2 v = res[(size_t)l * Pz + (k < 0 ? k + Pz : k)];
-        N[(size_t)c * S + ((size_t)r * (M + 1) + m) * nk + kk] = make_double2(v.x * scale, v.y * scale);
-    }
-}
-
 // ---------------------------------------------------------------- length-specialised z passes
 // Same work as k_zinv / k_zfwd with compile-time radix plans (radices <= 8) and padded lines.
 __device__ __forceinline__ double2 zinv_value(const double2* __restrict__ u, const double* __restrict__ w1,
@@ -276,86 +242,37 @@ __global__ void __launch_bounds__(NT, 2) k_zinv_s64(const double2* __restrict__ 
     }
 }
 
-template <int PZ, int LF, int NT>
-__global__ void __launch_bounds__(NT, 2) k_zfwd_s64(const double2* __restrict__ H2, double2* __restrict__ N,
-                                                    int N_r, int M, int K, double scale,
-                                                    const double2* __restrict__ tw, int m0, int mcnt, int r0, int nh) {
-    constexpr int LP = cft::padded<PZ>();
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    double2* a = reinterpret_cast<double2*>(smem_raw);
-    double2* b = a + LF * LP;
-    constexpr int groups = 3 / LF;
-    const int cg = blockIdx.x % groups;
-    const int m = m0 + (blockIdx.x / groups) % mcnt;
-    const int rl = (blockIdx.x / groups) / mcnt;
-    const int r = r0 + rl;
-    const size_t fstride = (size_t)nh * (M + 1) * PZ;
-    const double2* h = H2 + ((size_t)rl * (M + 1) + m) * PZ;
-    const int nk = 2 * K + 1;
-    const size_t S = (size_t)N_r * (M + 1) * nk;
-#pragma unroll
-    for (int l = 0; l < LF; ++l)
-        for (int z = threadIdx.x; z < PZ; z += NT) a[l * LP + cft::pd(z)] = h[(cg * LF + l) * fstride + z];
-    __syncthreads();
-    const double2* X = cft::passes<PZ, 0, 1, LF, NT, false, double2, true>(a, b, tw);
-    const size_t e0 = ((size_t)r * (M + 1) + m) * nk;
-    for (int kk = threadIdx.x; kk < nk; kk += NT) {
-        const int k = kk - K;
-        const int z = k < 0 ? k + PZ : k;
-#pragma unroll
-        for (int l = 0; l < LF; ++l) {
-            const double2 v = X[l * LP + cft::pd(z)];
-            N[(size_t)(cg * LF + l) * S + e0 + kk] = make_double2(v.x * scale, v.y * scale);
-        }
-    }
-}
-
 namespace {
 
 // The FP64 staging kernels below process the radial rows r0 .. r0 + nh - 1 and address their
 // staging lines (H1, H2) as nh rows; the spectral arrays keep all N_r rows.
 
-template <int PZ, int L, int LF, int NT>
-tc_status zpass64(tc_plan* p, const double2* u, double2* H1, const double2* H2, double2* N, cudaStream_t s,
-                  bool inverse, int ma, int mb, int r0, int nh) {
+template <int PZ, int L, int NT>
+tc_status zpass64(tc_plan* p, const double2* u, double2* H1, cudaStream_t s, int r0, int nh) {
     constexpr int LP = cft::padded<PZ>();
-    const int mc = mb - ma;
-    if (inverse) {
-        const size_t sm = (size_t)2 * L * LP * sizeof(double2);
-        TC_CUDA(p, cudaFuncSetAttribute(k_zinv_s64<PZ, L, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-        const int slot = prof_begin(p, kKZinv, s);
-        k_zinv_s64<PZ, L, NT><<<nh * mc * (9 / L), NT, sm, s>>>(u, H1, p->d_w1, p->d_col0, p->N_r, p->M,
-                                                               p->K, p->k_z, p->d_tw_z, ma, r0, nh);
-        prof_end(p, slot, s);
-        TC_LAUNCHED(p, "k_zinv_s64");
-    } else {
-        const size_t sm = (size_t)2 * LF * LP * sizeof(double2);
-        TC_CUDA(p, cudaFuncSetAttribute(k_zfwd_s64<PZ, LF, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-        const double scale = 1.0 / ((double)p->P_t * (double)p->P_z);
-        const int slot = prof_begin(p, kKZfwd, s);
-        k_zfwd_s64<PZ, LF, NT><<<nh * mc * (3 / LF), NT, sm, s>>>(H2, N, p->N_r, p->M, p->K, scale,
-                                                                 p->d_tw_z, ma, mc, r0, nh);
-        prof_end(p, slot, s);
-        TC_LAUNCHED(p, "k_zfwd_s64");
-    }
+    const size_t sm = (size_t)2 * L * LP * sizeof(double2);
+    TC_CUDA(p, cudaFuncSetAttribute(k_zinv_s64<PZ, L, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    const int slot = prof_begin(p, kKZinv, s);
+    k_zinv_s64<PZ, L, NT><<<nh * (p->M + 1) * (9 / L), NT, sm, s>>>(u, H1, p->d_w1, p->d_col0, p->N_r, p->M,
+                                                                   p->K, p->k_z, p->d_tw_z, 0, r0, nh);
+    prof_end(p, slot, s);
+    TC_LAUNCHED(p, "k_zinv_s64");
     return TC_OK;
 }
 
-// length-specialised FP64 z passes over m in [ma, mb); TC_ERR_ARG if P_z has no compile-time plan
-tc_status zpass64_s(tc_plan* p, const double2* u, double2* H1, const double2* H2, double2* N, cudaStream_t s,
-                    bool inverse, int ma, int mb, int r0, int nh) {
+// length-specialised FP64 inverse z pass; TC_ERR_ARG if P_z has no compile-time plan
+tc_status zpass64_s(tc_plan* p, const double2* u, double2* H1, cudaStream_t s, int r0, int nh) {
     switch (p->P_z) {
-        case 12: return zpass64<12, 9, 3, 64>(p, u, H1, H2, N, s, inverse, ma, mb, r0, nh);
-        case 24: return zpass64<24, 9, 3, 64>(p, u, H1, H2, N, s, inverse, ma, mb, r0, nh);
-        case 48: return zpass64<48, 9, 3, 128>(p, u, H1, H2, N, s, inverse, ma, mb, r0, nh);
-        case 96: return zpass64<96, 9, 3, 128>(p, u, H1, H2, N, s, inverse, ma, mb, r0, nh);
-        case 192: return zpass64<192, 9, 3, 256>(p, u, H1, H2, N, s, inverse, ma, mb, r0, nh);
-        case 384: return zpass64<384, 3, 3, 128>(p, u, H1, H2, N, s, inverse, ma, mb, r0, nh);
-        // one line per block from 768 on: three FP64 lines would take 76 KB and more
-        case 768: return zpass64<768, 3, 1, 256>(p, u, H1, H2, N, s, inverse, ma, mb, r0, nh);
-        case 1152: return zpass64<1152, 1, 1, 128>(p, u, H1, H2, N, s, inverse, ma, mb, r0, nh);
-        case 1536: return zpass64<1536, 1, 1, 256>(p, u, H1, H2, N, s, inverse, ma, mb, r0, nh);
-        case 2304: return zpass64<2304, 1, 1, 256>(p, u, H1, H2, N, s, inverse, ma, mb, r0, nh);
+        case 12: return zpass64<12, 9, 64>(p, u, H1, s, r0, nh);
+        case 24: return zpass64<24, 9, 64>(p, u, H1, s, r0, nh);
+        case 48: return zpass64<48, 9, 128>(p, u, H1, s, r0, nh);
+        case 96: return zpass64<96, 9, 128>(p, u, H1, s, r0, nh);
+        case 192: return zpass64<192, 9, 256>(p, u, H1, s, r0, nh);
+        case 384: return zpass64<384, 3, 128>(p, u, H1, s, r0, nh);
+        case 768: return zpass64<768, 3, 256>(p, u, H1, s, r0, nh);
+        case 1152: return zpass64<1152, 1, 128>(p, u, H1, s, r0, nh);
+        case 1536: return zpass64<1536, 1, 256>(p, u, H1, s, r0, nh);
+        case 2304: return zpass64<2304, 1, 256>(p, u, H1, s, r0, nh);
     }
     return TC_ERR_ARG;
 }
@@ -370,51 +287,18 @@ bool zpass64_ok(const tc_plan* p) {
 
 }  // namespace
 
-// inverse z pass (with the radial stencil) of the lines of m in [ma, mb), rows r0 .. r0 + nh - 1
-static tc_status zinv64(tc_plan* p, const double2* u, double2* H1, cudaStream_t s, int ma, int mb, int r0, int nh) {
-    if (zpass64_ok(p)) return zpass64_s(p, u, H1, nullptr, nullptr, s, true, ma, mb, r0, nh);
+// FP64 inverse z pass with the radial stencil, rows r0 .. r0 + nh - 1 (forward lines of the adjoint)
+tc_status launch_zinv_fp64(tc_plan* p, const double2* u, double2* H1, cudaStream_t s, int r0, int nh) {
+    if (zpass64_ok(p)) return zpass64_s(p, u, H1, s, r0, nh);
     const int L = p->zinv_lines;
     const size_t sm1 = (size_t)2 * L * p->P_z * sizeof(double2);
     TC_CUDA(p, cudaFuncSetAttribute(k_zinv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1));
     const int slot = prof_begin(p, kKZinv, s);
-    k_zinv<<<nh * (mb - ma) * (9 / L), p->thr_zinv, sm1, s>>>(u, H1, p->d_w1, p->d_col0, p->N_r, p->M, p->K,
-                                                             p->k_z, L, p->d_tw_z, p->rad_z, ma, r0, nh);
+    k_zinv<<<nh * (p->M + 1) * (9 / L), p->thr_zinv, sm1, s>>>(u, H1, p->d_w1, p->d_col0, p->N_r, p->M, p->K,
+                                                              p->k_z, L, p->d_tw_z, p->rad_z, 0, r0, nh);
     prof_end(p, slot, s);
     TC_LAUNCHED(p, "k_zinv");
     return TC_OK;
-}
-
-// forward z pass of the lines of m in [ma, mb), rows r0 .. r0 + nh - 1, into N
-static tc_status zfwd64(tc_plan* p, const double2* H2, double2* N, cudaStream_t s, int ma, int mb, int r0, int nh) {
-    if (zpass64_ok(p)) return zpass64_s(p, nullptr, nullptr, H2, N, s, false, ma, mb, r0, nh);
-    const int Lf = p->zfwd_lines;
-    const size_t sm3 = (size_t)2 * Lf * p->P_z * sizeof(double2);
-    TC_CUDA(p, cudaFuncSetAttribute(k_zfwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm3));
-    const double scale = 1.0 / ((double)p->P_t * (double)p->P_z);
-    const int slot = prof_begin(p, kKZfwd, s);
-    k_zfwd<<<nh * (mb - ma) * (3 / Lf), p->thr_zfwd, sm3, s>>>(H2, N, p->N_r, p->M, p->K, scale, p->d_tw_z,
-                                                              p->rad_z, Lf, ma, mb - ma, r0, nh);
-    prof_end(p, slot, s);
-    TC_LAUNCHED(p, "k_zfwd");
-    return TC_OK;
-}
-
-static tc_status theta64(tc_plan* p, const double2* H1, double2* H2, cudaStream_t s, int r0, int nh) {
-    if (p->theta_zt_forced == 0 && theta_s_zt(p, true) > 0) return launch_theta_s64(p, H1, H2, s, r0, nh);
-    const int zt = p->zt;
-    const size_t sm2 = (size_t)2 * 6 * zt * p->P_t * sizeof(double2);
-    TC_CUDA(p, cudaFuncSetAttribute(k_theta<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2));
-    const int slot = prof_begin(p, kKTheta, s);
-    k_theta<double2><<<nh * (p->P_z / zt), p->thr_theta, sm2, s>>>(H1, H2, p->d_ir, r0, nh, p->M, p->P_z,
-                                                                  (double)p->m_p, zt, p->d_tw_t, p->rad_t,
-                                                                  nullptr);
-    prof_end(p, slot, s);
-    TC_LAUNCHED(p, "k_theta");
-    return TC_OK;
-}
-
-tc_status launch_zinv_fp64(tc_plan* p, const double2* u, double2* H1, cudaStream_t s, int r0, int nh) {
-    return zinv64(p, u, H1, s, 0, p->M + 1, r0, nh);
 }
 
 // theta pass of the mixed form with the generic kernel: FP32 lines (H1, H2 in float2), all rows
@@ -430,9 +314,8 @@ tc_status launch_theta32(tc_plan* p, const float2* H1, float2* H2, cudaStream_t 
     return TC_OK;
 }
 
-// The nonlinear term.  FP64 lines: the three transforms slab by slab of p->stage_rows radial
-// rows (a row's transforms read no other row's staging), so the staging holds 12 line sets of
-// stage_rows rows.  Mixed form: FP32 lines of all rows (tc_mixed.cu).
+// The nonlinear term.  FP64: fixed-point lines of p->stage_rows radial rows at a time (tc_fx_z.cu).
+// Mixed form: FP32 lines of all rows (tc_mixed.cu).
 tc_status launch_nonlinear(tc_plan* p, const double2* u, double2* N, char* ws, cudaStream_t s) {
     if (p->precision == TC_MIXED && p->opt.mean_fp32) {
         TC_TRY_STATUS(launch_nl_pre32(p, u, ws, s, 0, p->M + 1));
@@ -452,15 +335,7 @@ tc_status launch_nonlinear(tc_plan* p, const double2* u, double2* N, char* ws, c
         TC_CUDA(p, cudaStreamWaitEvent(s, p->mean_ev[1], 0));
         return launch_mean00_fin(p, N, ws, s);
     }
-    double2* H1 = reinterpret_cast<double2*>(ws + p->ws.H1);
-    double2* H2 = reinterpret_cast<double2*>(ws + p->ws.H2);
-    for (int r0 = 0; r0 < p->N_r; r0 += p->stage_rows) {
-        const int nh = p->N_r - r0 < p->stage_rows ? p->N_r - r0 : p->stage_rows;
-        TC_TRY_STATUS(zinv64(p, u, H1, s, 0, p->M + 1, r0, nh));
-        TC_TRY_STATUS(theta64(p, H1, H2, s, r0, nh));
-        TC_TRY_STATUS(zfwd64(p, H2, N, s, 0, p->M + 1, r0, nh));
-    }
-    return TC_OK;
+    return launch_nonlinear_fx(p, u, N, ws, s);
 }
 
 }  // namespace tc

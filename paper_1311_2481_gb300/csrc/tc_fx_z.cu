@@ -1,0 +1,416 @@
+// FP64 form of the nonlinear term N(u) = u . grad u (Sec. 3.2 step 1, Eq. NS_cyl) on the
+// P_theta x P_z dealiased grid (Sec. 3.1), in 64-bit fixed point (tc_fx.cuh).  Four kernels, the
+// staging lines H1 and H2 in the workspace between them (the single-GPU counterpart of the
+// paper's global transposes, Sec. 4):
+//
+//   k_fx_dr     per (c, mode, 8 rows): d_r u by the FD stencil (Sec. 3.1), to FP64, into the H2
+//               region, which is free until the theta pass
+//   k_fx_zinv   per (r, m, c): the lines of u, d_r u and d_z u = i k k_z u, zero-padded inverse
+//               transforms along z                                     -> H1[9][r][m][z]
+//   k_fx_theta  per (r, z tile): the 12 real fields as 6 complex inverse transforms along theta
+//               (two real fields per line; d_theta = i m m_p applied here), the products with
+//               the curvature terms, and the forward transforms of N_r + i N_theta (giving N_+
+//               and N_- directly) and of N_z (two z per line)           -> H2[3][r][m][z]
+//   k_fx_zfwd   per (r, m): forward transforms along z, truncation, 1/(P_theta P_z), to FP64.
+//
+// Exponents.  Every H1 line has its own (chosen from the sum of the moduli of its input, so
+// that no partial sum overflows), with a bound of its largest value; from these each theta
+// block takes the exponents of its six line kinds.  Products are taken from lines shifted up
+// to their true maximum, and N's line to the sum of its moduli before the forward transform.
+// A NaN or Inf anywhere in a row of u makes N of that row NaN, as the FP64 transforms did.
+#include <algorithm>
+
+#include "tc_fx_nl.cuh"
+
+namespace tc {
+
+using namespace fx;
+
+namespace {
+
+constexpr int kDrRows = 8;      // rows per thread of k_fx_dr (its exponents assume 8)
+constexpr int kZThreads = 512;  // most threads of a transform block (128 registers each)
+
+// exponent arrays of nh staged rows, in the fxe region: e1[9][nh][M+1] (exponent, largest
+// |re| + |im| in units of 2^32), e2[nh][tiles][2], e2max[nh][2]
+struct Exps {
+    int2* e1;
+    int* e2;
+    int* e2max;
+};
+
+// ---------------------------------------------------------------- radial derivative
+// Rows j0 .. j0 + 7 of the real or imaginary part of one column per thread: 16 rows are
+// converted once to the exponent of the largest, each output is 27 32-bit multiply-adds
+// instead of 9 FP64 FMAs of 64 issue cycles each.  The products' low limbs that are left out
+// amount to 2^-57 of max |u| sum |w|.  Where a row's own stencil reaches only values 2^4 or
+// more below that maximum, and in the four rows next to each wall, whose stencils are shorter
+// (u falls off towards the wall), the row is taken in FP64.  Tiles start at multiples of kDrRows whatever r0, so that
+// a row's result does not depend on the slab it is staged in.
+__global__ void __launch_bounds__(128) k_fx_dr(const double* __restrict__ u, double* __restrict__ du,
+                                               const int2* __restrict__ w, const int* __restrict__ ew,
+                                               const double* __restrict__ w1, const int* __restrict__ col0, int N,
+                                               int ncol, int r0, int nh) {
+    const int c = blockIdx.z, tile = (r0 / kDrRows + blockIdx.y) * kDrRows - r0, j0 = r0 + tile;
+    const int col = blockIdx.x * blockDim.x + threadIdx.x;
+    if (col >= ncol) return;
+    const double* src = u + (size_t)c * N * ncol + col;
+    double d[kDrRows + 8];
+#pragma unroll
+    for (int i = 0; i < kDrRows + 8; ++i) {
+        const int j = j0 - 4 + i;
+        d[i] = j >= 0 && j < N ? __ldg(&src[(size_t)j * ncol]) : 0.0;
+    }
+    // lo[i], hi[i]: largest exponents of entries i .. 6 and 9 .. i + 8; every stencil holds 7 and 8
+    int lo[kDrRows], hi[kDrRows];
+    lo[7] = hi[0] = max(bexp(d[7]), bexp(d[8]));
+#pragma unroll
+    for (int i = 6; i >= 0; --i) lo[i] = max(lo[i + 1], bexp(d[i]));
+#pragma unroll
+    for (int i = 1; i < kDrRows; ++i) hi[i] = max(hi[i - 1], bexp(d[i + 8]));
+    const int e = max(lo[0], hi[kDrRows - 1]);
+    lim x[kDrRows + 8];
+#pragma unroll
+    for (int i = 0; i < kDrRows + 8; ++i) x[i] = split(fix(d[i], e + 5));   // |x| < 2^57: nine products fit 64 bits
+#pragma unroll
+    for (int i = 0; i < kDrRows; ++i) {
+        const int j = j0 + i;
+        if (tile + i >= nh) break;
+        if (tile + i < 0) continue;
+        double o = 0.0;
+        if (j < 4 || j > N - 5 || e - max(lo[i], hi[i]) > 3) {
+            const int c0 = __ldg(&col0[j]);
+            double v[kStencil];   // rows outside [0, N) (N < 9) have weight 0
+#pragma unroll
+            for (int t = 0; t < kStencil; ++t) v[t] = (unsigned)(c0 + t) < (unsigned)N ? __ldg(&src[(ptrdiff_t)(c0 + t) * ncol]) : 0.0;
+#pragma unroll
+            for (int t = 0; t < kStencil; ++t) o = fma(__ldg(&w1[j * kStencil + t]), v[t], o);
+        } else {
+            long long m = 0, s = 0;
+#pragma unroll
+            for (int t = 0; t < kStencil; ++t) {
+                const int2 v = __ldg(&w[j * kStencil + t]);
+                m = mad(x[i + t].h, v.y, mad(x[i + t].l, v.x, m));
+                s = mad(x[i + t].h, v.x, s);
+            }
+            o = e == 2047 ? nan64() : to_double(take(s + (m >> 32), m, 25), e + __ldg(&ew[j]) - 1084);
+        }
+        du[((size_t)c * nh + tile + i) * ncol + col] = o;
+    }
+}
+
+// s[line] = max / sum over the threads of a line, tl consecutive threads per line (line < 0 or
+// >= NL: none).  From 32 threads per line on, a warp holds at most two lines and reduces each
+// in registers; 32 atomics on one address would take turns.
+template <int NL, bool MAX> __device__ __forceinline__ void line_reduce(unsigned* s, int line, unsigned v, int tl) {
+    if (tl < 32) {
+        if (line < NL) {
+            if (MAX) atomicMax(&s[line], v);
+            else atomicAdd(&s[line], v);
+        }
+        return;
+    }
+    const int first = __shfl_sync(0xffffffffu, line, 0), last = __shfl_sync(0xffffffffu, line, 31);
+    const unsigned a = line == first ? v : 0u, b = line == first ? 0u : v;
+    const unsigned ra = MAX ? __reduce_max_sync(0xffffffffu, a) : __reduce_add_sync(0xffffffffu, a);
+    const unsigned rb = first == last ? 0u : MAX ? __reduce_max_sync(0xffffffffu, b) : __reduce_add_sync(0xffffffffu, b);
+    if ((threadIdx.x & 31) == 0) {
+        if (first < NL) {
+            if (MAX) atomicMax(&s[first], ra);
+            else atomicAdd(&s[first], ra);
+        }
+        if (last != first && last < NL) {
+            if (MAX) atomicMax(&s[last], rb);
+            else atomicAdd(&s[last], rb);
+        }
+    }
+}
+
+// ---------------------------------------------------------------- inverse z pass
+// NL lines per block, out of the nine (d, c) of an (r, m), d = 0, 1, 2 for u, d_r u, d_z u.  tl
+// threads per line hold its entries (at most 8 each) from the load to the fixed-point line.
+template <class PL, int NL>
+__global__ void __launch_bounds__(kZThreads) k_fx_zinv(const double2* __restrict__ u, const double2* __restrict__ du,
+                                                       cx* __restrict__ H1, int2* __restrict__ e1, int N, int M, int K,
+                                                       double kz, int r0, int nh, FxPlan f, const int4* __restrict__ tw,
+                                                       int tl, unsigned mtl, int* __restrict__ e2max,
+                                                       const double* __restrict__ w1, const int* __restrict__ col0) {
+    extern __shared__ cx buf[];
+    __shared__ unsigned s_e[NL], s_l1[NL], s_mx[NL];
+    const PL pl(f);
+    const int P = pl.size(), lp = line_pitch(P), nk = 2 * K + 1, nmode = (M + 1) * nk;
+    int t = blockIdx.x;
+    const int f0 = t % (9 / NL) * NL;   // lines in the order 3 c + d: a block reads few lines of u
+    t /= 9 / NL;
+    const int rl = t % nh, m = t / nh;   // rows fastest: neighbouring blocks share cache lines of u
+    if (m == 0 && f0 == 0 && threadIdx.x < 2) e2max[rl * 2 + threadIdx.x] = 4 * kExpZero;   // the theta pass takes maxima here
+    if (threadIdx.x < NL) {
+        s_e[threadIdx.x] = 0;
+        s_l1[threadIdx.x] = 0;
+        s_mx[threadIdx.x] = 0;
+    }
+    __syncthreads();
+    const int line = NL == 1 ? 0 : udiv(threadIdx.x, mtl), i0 = threadIdx.x - line * tl;
+    const bool on = line < NL;
+    const int c = (f0 + line) / 3, d = f0 + line - 3 * c;
+    double2 x[8];
+    int e = 0;
+    if (on) {
+        const double2* src = d == 1 && du ? du + ((size_t)c * nh + rl) * nmode + (size_t)m * nk
+                                          : u + ((size_t)c * N + r0 + rl) * nmode + (size_t)m * nk;
+        if (NL == 9 && d == 1 && !du) {   // d_r u here, in FP64
+            const int j0 = __ldg(&col0[r0 + rl]);
+            const double2* a = u + ((ptrdiff_t)c * N + j0) * nmode + (ptrdiff_t)m * nk;
+            double w[kStencil];   // rows outside [0, N) (N < 9) have weight 0
+#pragma unroll
+            for (int q = 0; q < kStencil; ++q) w[q] = __ldg(&w1[(r0 + rl) * kStencil + q]);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                x[i] = make_double2(0.0, 0.0);
+                if (i0 + i * tl < nk) {
+                    double2 y = make_double2(0.0, 0.0);   // two sums: half the chain of dependent FMAs
+#pragma unroll
+                    for (int q = 0; q < kStencil; ++q) {
+                        const double2 v = (unsigned)(j0 + q) < (unsigned)N ? __ldg(&a[(ptrdiff_t)q * nmode + i0 + i * tl]) : make_double2(0.0, 0.0);
+                        double2& o = q & 1 ? y : x[i];
+                        o.x = fma(w[q], v.x, o.x);
+                        o.y = fma(w[q], v.y, o.y);
+                    }
+                    x[i].x += y.x;
+                    x[i].y += y.y;
+                }
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) x[i] = i0 + i * tl < nk ? __ldg(&src[i0 + i * tl]) : make_double2(0.0, 0.0);
+        }
+        if (d == 2) {   // the FP64 pipe is otherwise idle here
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const double kk = kz * (i0 + i * tl - K);
+                x[i] = make_double2(-kk * x[i].y, kk * x[i].x);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) e = max(e, max(bexp(x[i].x), bexp(x[i].y)));
+    }
+    line_reduce<NL, true>(s_e, line, (unsigned)e, tl);
+    zero_band(pl, buf, lp, NL, K + 1, P - K);
+    __syncthreads();
+    cx v[8];
+    unsigned l1 = 0;
+    if (on) {
+        e = (int)s_e[line];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            v[i] = mk(fix(x[i].x, e), fix(x[i].y, e));
+            l1 += ((mag_hi(v[i].x) + mag_hi(v[i].y)) >> 11) + 1;
+        }
+    }
+    line_reduce<NL, false>(s_l1, line, l1, tl);
+    __syncthreads();
+    if (on) {
+        // sum of moduli < s_l1 2^43: shifted to below 2^62
+        const int s = max(0, bits(s_l1[line]) - 19);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int k = i0 + i * tl - K;
+            if (k <= K) buf[line * lp + (k >= 0 ? k : k + P)] = mk(v[i].x >> s, v[i].y >> s);
+        }
+    }
+    __syncthreads();
+    transform(pl, buf, lp, NL, tw, true);
+    unsigned mx = 0;
+    if (on) {
+        cx* dst = H1 + (((size_t)(3 * d + c) * nh + rl) * (M + 1) + m) * P;
+        for (int p = i0; p < P; p += tl) {
+            const cx o = buf[line * lp + pd(p)];
+            dst[p] = o;
+            mx = max(mx, mag_hi(o.x) + mag_hi(o.y) + 2);
+        }
+    }
+    line_reduce<NL, true>(s_mx, line, mx, tl);
+    __syncthreads();
+    if (on && i0 == 0) {
+        const int s = max(0, bits(s_l1[line]) - 19);
+        e1[((size_t)(3 * d + c) * nh + rl) * (M + 1) + m] =
+            e == 0 ? make_int2(kExpZero, 0) : e == 2047 ? make_int2(kExpNaN, 0) : make_int2(e - 1022 + s, (int)s_mx[line]);
+    }
+}
+
+// ---------------------------------------------------------------- forward z pass
+template <class PL, int NL>
+__global__ void __launch_bounds__(kZThreads) k_fx_zfwd(const cx* __restrict__ H2, double2* __restrict__ Nh,
+                                                       const int* __restrict__ e2, const int* __restrict__ e2max, int N,
+                                                       int M, int K, double scale, int r0, int nh, int zt, unsigned mzt,
+                                                       FxPlan f, const int4* __restrict__ tw, int tl, unsigned mtl) {
+    extern __shared__ cx buf[];
+    __shared__ unsigned s_l1[NL];
+    const PL pl(f);
+    const int P = pl.size(), lp = line_pitch(P), nk = 2 * K + 1, nmode = (M + 1) * nk;
+    int t = blockIdx.x;
+    const int c0 = t % (3 / NL) * NL;
+    t /= 3 / NL;
+    const int m = t % (M + 1), rl = t / (M + 1);
+    if (threadIdx.x < NL) s_l1[threadIdx.x] = 0;
+    __syncthreads();
+    const int line = NL == 1 ? 0 : udiv(threadIdx.x, mtl), i0 = threadIdx.x - line * tl, c = c0 + line;
+    const bool on = line < NL;
+    const int E = e2max[rl * 2 + (c == 2)];
+    cx v[8];
+    unsigned l1 = 0;
+    if (on) {
+        const cx* h = H2 + (((size_t)c * nh + rl) * (M + 1) + m) * P;
+        const int* er = e2 + (size_t)rl * (P / zt) * 2 + (c == 2);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = i0 + i * tl < P ? h[i0 + i * tl] : mk(0, 0);
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (i0 + i * tl < P) {
+                const int te = E - __ldg(&er[udiv(i0 + i * tl, mzt) * 2]);
+                v[i] = mk(shr(v[i].x, te), shr(v[i].y, te));
+                l1 += ((mag_hi(v[i].x) + mag_hi(v[i].y)) >> 11) + 1;
+            }
+    }
+    line_reduce<NL, false>(s_l1, line, l1, tl);
+    __syncthreads();
+    const int s = on ? max(0, bits(s_l1[line]) - 19) : 0;
+    if (on) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (i0 + i * tl < P) buf[line * lp + i0 + i * tl] = mk(v[i].y >> s, v[i].x >> s);   // exchanged
+    }
+    __syncthreads();
+    transform(pl, buf, lp, NL, tw, false);
+    if (on) {
+        const bool bad = E > kExpNaN / 2;
+        double2* dst = Nh + ((size_t)c * N + r0 + rl) * nmode + (size_t)m * nk;
+        for (int kk = i0; kk < nk; kk += tl) {
+            const cx o = buf[line * lp + pd(kk >= K ? kk - K : kk - K + P)];
+            dst[kk] = bad ? make_double2(nan64(), nan64())
+                          : make_double2(to_double(o.y, E + s - 62) * scale, to_double(o.x, E + s - 62) * scale);
+        }
+    }
+}
+
+Exps exps(tc_plan* p, char* ws) {
+    Exps e;
+    e.e1 = reinterpret_cast<int2*>(ws + p->ws.fxe);
+    e.e2max = reinterpret_cast<int*>(e.e1 + (size_t)9 * p->N_r * (p->M + 1));
+    e.e2 = e.e2max + 2 * p->N_r;
+    return e;
+}
+
+}  // namespace
+
+size_t fx_exp_bytes(const tc_plan* p) {
+    return (size_t)9 * p->N_r * (p->M + 1) * sizeof(int2) + (size_t)2 * p->N_r * sizeof(int) +
+           (size_t)2 * p->N_r * p->P_z * sizeof(int);
+}
+
+namespace {
+
+// Launch shapes.  z passes: as many of the lines of an (r, m) per block as give it about 128
+// threads at n / 8 each.
+int lines_zinv(int P) { return P <= 96 ? 9 : P <= 768 ? 3 : 1; }
+int lines_zfwd(int P) { return P <= 768 ? 3 : 1; }
+
+template <class PL, int L9, int L3>
+tc_status z_pass(tc_plan* p, const double2* u, const double2* du, cx* H1, const cx* H2, double2* Nh, const Exps& e, const int4* tw,
+                 cudaStream_t s, bool inverse, int r0, int nh) {
+    // at least a thread for 8 entries of a line; 4 in the short ones, where latency counts
+    const int P = p->P_z, nl = inverse ? L9 : L3, thr = round32(nl * (P <= 48 ? (P + 3) / 4 : (P + 7) / 8)), tl = thr / nl;
+    const size_t sm = (size_t)nl * line_pitch(P) * sizeof(cx);
+    if (inverse) {
+        auto k = k_fx_zinv<PL, L9>;
+        TC_CUDA(p, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        k<<<nh * (p->M + 1) * (9 / L9), thr, sm, s>>>(u, du, H1, e.e1, p->N_r, p->M, p->K, p->k_z, r0, nh, p->fx_z, tw, tl, magic(tl),
+                                               e.e2max, p->d_w1, p->d_col0);
+        TC_LAUNCHED(p, "k_fx_zinv");
+    } else {
+        auto k = k_fx_zfwd<PL, L3>;
+        TC_CUDA(p, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        k<<<nh * (p->M + 1) * (3 / L3), thr, sm, s>>>(H2, Nh, e.e2, e.e2max, p->N_r, p->M, p->K, 1.0 / ((double)p->P_t * (double)P), r0,
+                                                     nh, p->fx_zt, magic(p->fx_zt), p->fx_z, tw, tl, magic(tl));
+        TC_LAUNCHED(p, "k_fx_zfwd");
+    }
+    return TC_OK;
+}
+
+// lengths with a compile-time plan, and the z values of their theta blocks (0: none)
+bool static_z(int P) {
+    switch (P) {
+        case 12: case 24: case 36: case 48: case 72: case 96: case 144: case 192: case 288: case 384: case 576: case 768: case 1152:
+        case 1536: case 2304: return true;
+    }
+    return false;
+}
+}  // namespace
+
+const int* fx_static_radices(int n) {
+    switch (n) {
+#define TC_FX_R(P) case P: return Radix<P>::r;
+        TC_FX_R(12) TC_FX_R(24) TC_FX_R(36) TC_FX_R(48) TC_FX_R(72) TC_FX_R(96) TC_FX_R(144) TC_FX_R(192) TC_FX_R(288) TC_FX_R(384) TC_FX_R(576)
+        TC_FX_R(768) TC_FX_R(1152) TC_FX_R(1536) TC_FX_R(2304)
+#undef TC_FX_R
+    }
+    return nullptr;
+}
+
+namespace {
+
+// The transforms of rows r0 .. r0 + nh - 1.
+tc_status fx_rows(tc_plan* p, const double2* u, double2* Nh, char* ws, cudaStream_t s, int r0, int nh) {
+    cx* H1 = reinterpret_cast<cx*>(ws + p->ws.H1);
+    cx* H2 = reinterpret_cast<cx*>(ws + p->ws.H2);
+    double2* du = reinterpret_cast<double2*>(H2);
+    const Exps e = exps(p, ws);
+    int slot = prof_begin(p, kKZinv, s);
+    if (p->P_z <= 96 && p->S <= 65536) {
+        // small problems: the inverse z pass takes d_r u itself, in FP64.  Its 18 FMAs per value
+        // then cost less than a launch (S = 5000: 0.4 us of the FP64 pipe against 7 us).
+        du = nullptr;
+    } else {
+        k_fx_dr<<<dim3((2 * p->nmode + 127) / 128, (r0 + nh + kDrRows - 1) / kDrRows - r0 / kDrRows, 3), 128, 0, s>>>(
+            reinterpret_cast<const double*>(u), reinterpret_cast<double*>(du), p->d_fx_w1, p->d_fx_ew, p->d_w1, p->d_col0, p->N_r,
+            2 * p->nmode, r0, nh);
+        TC_LAUNCHED(p, "k_fx_dr");
+    }
+    const bool sz = p->theta_zt_forced == 0 && static_z(p->P_z) && 3 * p->K <= p->P_z;
+    const int4* twz = p->d_fx_tw_z + (sz ? p->fx_z.table : 0);
+    auto z = [&](bool inverse) -> tc_status {
+        switch (sz ? p->P_z : 0) {
+#define TC_FX_Z(P, A, B) case P: return z_pass<Ct<P>, A, B>(p, u, du, H1, H2, Nh, e, twz, s, inverse, r0, nh);
+            TC_FX_Z(12, 9, 3) TC_FX_Z(24, 9, 3) TC_FX_Z(36, 9, 3) TC_FX_Z(48, 9, 3) TC_FX_Z(72, 9, 3) TC_FX_Z(96, 9, 3) TC_FX_Z(144, 3, 3)
+            TC_FX_Z(192, 3, 3) TC_FX_Z(288, 3, 3) TC_FX_Z(384, 3, 3) TC_FX_Z(576, 3, 3) TC_FX_Z(768, 3, 3) TC_FX_Z(1152, 1, 1) TC_FX_Z(1536, 1, 1)
+            TC_FX_Z(2304, 1, 1)
+#undef TC_FX_Z
+        }
+        if (p->P_z <= 96) return z_pass<Rt, 9, 3>(p, u, du, H1, H2, Nh, e, twz, s, inverse, r0, nh);
+        if (p->P_z <= 768) return z_pass<Rt, 3, 3>(p, u, du, H1, H2, Nh, e, twz, s, inverse, r0, nh);
+        return z_pass<Rt, 1, 1>(p, u, du, H1, H2, Nh, e, twz, s, inverse, r0, nh);
+    };
+    TC_TRY_STATUS(z(true));
+    prof_end(p, slot, s);
+    slot = prof_begin(p, kKTheta, s);
+    ThetaArgs a{H1, H2, e.e1, e.e2, e.e2max, p->d_fx_ir, p->d_fx_mm, p->d_fx_tw_t, r0, nh, p->M, p->P_z, p->fx_zt, p->fx_emm,
+                magic(p->fx_zt), magic(p->P_t), (long long)p->m_p};
+    TC_TRY_STATUS(launch_fx_theta(p, a, s));
+    prof_end(p, slot, s);
+    slot = prof_begin(p, kKZfwd, s);
+    TC_TRY_STATUS(z(false));
+    prof_end(p, slot, s);
+    return TC_OK;
+}
+
+}  // namespace
+
+// N(u) in FP64, slab by slab of p->stage_rows radial rows (a row's transforms read no other
+// row's staging)
+tc_status launch_nonlinear_fx(tc_plan* p, const double2* u, double2* Nh, char* ws, cudaStream_t s) {
+    for (int r0 = 0; r0 < p->N_r; r0 += p->stage_rows)
+        TC_TRY_STATUS(fx_rows(p, u, Nh, ws, s, r0, std::min(p->stage_rows, p->N_r - r0)));
+    return TC_OK;
+}
+
+}  // namespace tc

@@ -5,6 +5,7 @@
 #include <cstdint>
 #include <cstdio>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/tc.h"
@@ -26,6 +27,18 @@ struct Radices {
     int r[kMaxRadix];
 };
 
+// Passes of a fixed-point transform (tc_fx.cuh): radices up to 16, each pass with its own
+// twiddle table (R - 1) x ns, and multiplicative inverses for the index divisions.
+constexpr int kFxPasses = 6;
+struct FxPass {
+    int r, ns, nb, tw;     // radix, product of the earlier radices, n / r, offset in the table
+    unsigned mnb, mns;     // ceil(2^32 / nb), ceil(2^32 / ns)
+};
+struct FxPlan {
+    int n, np, table;      // length, passes, entries of the twiddle table
+    FxPass p[kFxPasses];
+};
+
 // Byte offsets of the workspace regions (all 256-byte aligned).
 // Every region is scratch of one library call; regions that no call uses at the same time
 // share memory (see tc_plan.cu).
@@ -35,6 +48,7 @@ struct Workspace {
     size_t H2;      // theta-pass output: 3 line sets, rows and precision as H1
     size_t P32;     // mixed form: u', d_r u' in FP32, 6 x S float2
     size_t mean;    // mixed form: segment sums of the mean mode of N (mean00_part_doubles)
+    size_t fxe;     // FP64 plans: exponents of the fixed-point lines of all rows (tc_fx_nl.cu)
     size_t Ncur;    // N^i: vector field (everything before it is the forward staging)
     size_t uE;      // start-up Euler result: vector field
     size_t pstar;   // split path only: p* (scalar), u* (vector), phi (scalar)
@@ -68,6 +82,7 @@ struct tc_plan {
     int nmode;       // (M+1)(2K+1)
     int nmode_half;  // (M+1)(K+1)
     tc::Radices rad_z, rad_t;
+    int fx_zt;                     // z values per fixed-point theta block
     int zt, zt32;                  // z values per theta-pass block (FP64 / FP32 lines)
     int theta_zt_forced;           // tc_options.theta_zt (> 0: generic transform kernels)
     int theta_variant;             // tc_options.theta_variant (launch shape of the FP32 streamed theta pass)
@@ -93,6 +108,7 @@ struct tc_plan {
     std::vector<double> fac2, spk, rinv;
     std::vector<uint8_t> piv2;
     std::vector<double> tw_z, tw_t;  // interleaved complex exp(+2 pi i j / n)
+    tc::FxPlan fx_z{}, fx_t{};       // fixed-point transforms along z and theta
     // device plan
     double* d_r = nullptr;
     double* d_ir = nullptr;          // 1 / r_j
@@ -113,6 +129,15 @@ struct tc_plan {
     double2* d_tw_t = nullptr;
     float2* d_tw_z32 = nullptr;
     float2* d_tw_t32 = nullptr;
+    // fixed-point constants: twiddles (two limbs of cos, two of sin), m m_p and 1/r_j (limbs and
+    // exponent), D1 weights centred on their row (limbs, one exponent per row)
+    int4* d_fx_tw_z = nullptr;
+    int4* d_fx_tw_t = nullptr;
+    int2* d_fx_mm = nullptr;
+    int fx_emm = 0;
+    int4* d_fx_ir = nullptr;
+    int2* d_fx_w1 = nullptr;
+    int* d_fx_ew = nullptr;
     // non-finite flag: mapped pinned host memory that the update kernels set when they write
     // a NaN/Inf into the state; tc_step reports and clears it
     int* h_nonfinite = nullptr;
@@ -186,12 +211,15 @@ int prof_begin(tc_plan* p, int kid, cudaStream_t s);
 void prof_end(tc_plan* p, int slot, cudaStream_t s);
 
 // ------------------------------------------------------------------ launchers
+tc_status launch_nonlinear_fx(tc_plan* p, const double2* u, double2* Nh, char* ws, cudaStream_t s);
+size_t fx_exp_bytes(const tc_plan* p);
+int fx_zt(const tc_plan* p, int forced);
+const int* fx_static_radices(int n);   // radices of the compile-time plan of length n, nullptr if none
 tc_status launch_nonlinear(tc_plan* p, const double2* u, double2* N, char* ws, cudaStream_t s);
 tc_status launch_zinv_fp64(tc_plan* p, const double2* u, double2* H1, cudaStream_t s, int r0, int nh);
 tc_status launch_theta32(tc_plan* p, const float2* H1, float2* H2, cudaStream_t s);
 int theta_s_zt(const tc_plan* p, bool fp64);
 tc_status launch_theta_s(tc_plan* p, const float2* H1, float2* H2, cudaStream_t s);
-tc_status launch_theta_s64(tc_plan* p, const double2* H1, double2* H2, cudaStream_t s, int r0, int nh);
 tc_status launch_nl_pre32(tc_plan* p, const double2* u, char* ws, cudaStream_t s, int ma, int mb);
 tc_status launch_nl_theta32(tc_plan* p, char* ws, cudaStream_t s);
 tc_status launch_nl_post32(tc_plan* p, const double2* u, double2* N, char* ws, cudaStream_t s, int ma, int mb);

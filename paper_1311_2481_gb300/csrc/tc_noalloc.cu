@@ -32,9 +32,12 @@
 namespace {
 
 constexpr size_t kStaticScratchBytes = (size_t)80 << 20;
+// behind the lines, the exponents of the FP64 form's fixed-point lines: at most 3/8 of a byte
+// per 8 bytes of lines (fx_exp_bytes against 12 line sets, P_z >= 3), and rounding
+constexpr size_t kStaticExpBytes = (size_t)12 << 20;
 constexpr int kMaxDevices = 64;
 
-static __device__ __align__(256) unsigned char g_scratch[kStaticScratchBytes];
+static __device__ __align__(256) unsigned char g_scratch[kStaticScratchBytes + kStaticExpBytes];
 
 std::mutex g_mu;
 void* g_scratch_ptr[kMaxDevices] = {nullptr};
@@ -68,11 +71,15 @@ extern "C" tc_status tc_nonlinear_noalloc(tc_plan* plan, const void* u_hat, void
     }
     // staging used by the transform kernels: H1 (9 line sets), H2 (3 line sets) and, for the
     // mixed form, the FP32 split of u and d_r u -- every workspace region before N^i
-    const size_t need = plan->ws.Ncur;
+    const size_t need = plan->ws.fxe;
     if (need > kStaticScratchBytes) {
         snprintf(plan->err, sizeof(plan->err),
                  "tc_nonlinear_noalloc: this plan needs %zu bytes of staging but the static scratch "
                  "holds %zu bytes (80 MiB); use tc_nonlinear with a workspace", need, kStaticScratchBytes);
+        return TC_ERR_ARG;
+    }
+    if (plan->ws.Ncur > kStaticScratchBytes + kStaticExpBytes) {
+        snprintf(plan->err, sizeof(plan->err), "tc_nonlinear_noalloc: the exponents of this plan do not fit the static scratch");
         return TC_ERR_ARG;
     }
     int dev = -1;

@@ -135,6 +135,84 @@ static void twiddles(int n, std::vector<double>& tw) {
     }
 }
 
+// Radices of a fixed-point transform of length n = 2^a 3^b: the sequence of least cost per
+// point, in issue slots (butterfly, twiddle multiplications after the first pass, and about
+// 20 for a pass through shared memory), smallest radix first.
+static void fx_search(int n, std::vector<int>& cur, double cost, std::vector<int>& best, double& best_cost) {
+    static const int kR[7] = {2, 3, 4, 6, 8, 9, 12};
+    static const double kB[7] = {4, 13, 8, 17, 17, 38, 21};
+    if (n == 1) {
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = cur;
+        }
+        return;
+    }
+    if ((int)cur.size() == kFxPasses) return;
+    for (int i = 0; i < 7; ++i)
+        if (n % kR[i] == 0 && (cur.empty() || kR[i] >= cur.back())) {
+            cur.push_back(kR[i]);
+            fx_search(n / kR[i], cur, cost + kB[i] + 20 + (cur.size() > 1 ? 26.0 * (kR[i] - 1) / kR[i] : 0.0), best, best_cost);
+            cur.pop_back();
+        }
+}
+
+static FxPlan fx_plan(int n, const int* radices = nullptr) {
+    std::vector<int> cur, best;
+    double c = 1e30;
+    if (radices) {
+        while (n > 1) {
+            best.push_back(*radices);
+            n /= *radices++;
+        }
+        for (int r : best) n *= r;
+    } else {
+        fx_search(n, cur, 0.0, best, c);
+    }
+    FxPlan f{};
+    f.n = n;
+    f.np = (int)best.size();
+    auto magic = [](int d) { return d <= 1 ? 0u : (unsigned)((((unsigned long long)1 << 32) + d - 1) / d); };
+    int ns = 1, off = 0;
+    for (int p = 0; p < f.np; ++p) {
+        FxPass& q = f.p[p];
+        q.r = best[p];
+        q.ns = ns;
+        q.nb = n / q.r;
+        q.tw = off;
+        q.mnb = magic(q.nb);
+        q.mns = magic(ns);
+        if (p > 0) off += (q.r - 1) * ns;
+        ns *= q.r;
+    }
+    f.table = off;
+    return f;
+}
+
+// x 2^62 in two signed limbs, for |x| <= 1
+static void fx_limbs(long double x, int& h, int& l) {
+    const long long v = (long long)std::floor(x * 4611686018427387904.0L + 0.5L);
+    l = (int)(unsigned)(unsigned long long)v;
+    h = (int)((v - l) >> 32);
+}
+
+// pass tables exp(+2 pi i q k / (ns R)), entry (q - 1) ns + k of pass p >= 1
+static std::vector<int4> fx_twiddles(const FxPlan& f) {
+    std::vector<int4> t(std::max(1, f.table));
+    for (int p = 1; p < f.np; ++p) {
+        const FxPass& s = f.p[p];
+        for (int q = 1; q < s.r; ++q)
+            for (int k = 0; k < s.ns; ++k) {
+                const long double a = 2.0L * kPiL * (long double)(q * k) / (long double)(s.ns * s.r);
+                int4 v;
+                fx_limbs(cosl(a), v.x, v.y);
+                fx_limbs(sinl(a), v.z, v.w);
+                t[s.tw + (q - 1) * s.ns + k] = v;
+            }
+    }
+    return t;
+}
+
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Block size for a kernel whose FP64 work is Stockham passes over `lines` transforms of
@@ -443,6 +521,49 @@ static tc_status upload(tc_plan* p) {
     }
     TC_CUDA(p, put((void**)&p->d_tw_z, p->tw_z.data(), p->tw_z.size() * sizeof(double)));
     TC_CUDA(p, put((void**)&p->d_tw_t, p->tw_t.data(), p->tw_t.size() * sizeof(double)));
+    if (p->precision != TC_MIXED || p->adjoint) {   // constants of the fixed-point transforms
+        // tables of the run-time plans, followed by those of the compile-time plans
+        std::vector<int4> tz = fx_twiddles(p->fx_z), tt = fx_twiddles(p->fx_t);
+        for (int z = 0; z < 2; ++z) {
+            std::vector<int4>& t = z ? tz : tt;
+            t.resize(z ? p->fx_z.table : p->fx_t.table);
+            if (const int* r = fx_static_radices(z ? p->P_z : p->P_t)) {
+                const std::vector<int4> more = fx_twiddles(fx_plan(z ? p->P_z : p->P_t, r));
+                t.insert(t.end(), more.begin(), more.end());
+            }
+            if (t.empty()) t.push_back(make_int4(0, 0, 0, 0));
+        }
+        TC_CUDA(p, put((void**)&p->d_fx_tw_z, tz.data(), tz.size() * sizeof(int4)));
+        TC_CUDA(p, put((void**)&p->d_fx_tw_t, tt.data(), tt.size() * sizeof(int4)));
+        std::vector<int2> mm(p->M + 1);
+        const long double top = (long double)p->M * p->m_p;
+        p->fx_emm = (int)std::ceil(std::log2(top));
+        for (int m = 0; m <= p->M; ++m) fx_limbs(std::ldexp((long double)m * p->m_p, -p->fx_emm), mm[m].x, mm[m].y);
+        TC_CUDA(p, put((void**)&p->d_fx_mm, mm.data(), mm.size() * sizeof(int2)));
+        std::vector<int4> fir(p->N_r);
+        std::vector<int2> w(p->w1.size(), make_int2(0, 0));
+        std::vector<int> ew(p->N_r);
+        for (int j = 0; j < p->N_r; ++j) {
+            int e;
+            const double x = std::frexp(1.0 / p->r[j], &e);
+            fx_limbs(x, fir[j].x, fir[j].y);
+            fir[j].z = e;
+            fir[j].w = 0;
+            long double sum = 0;
+            for (int t = 0; t < kStencil; ++t) sum += std::fabs((long double)p->w1[(size_t)j * kStencil + t]);
+            std::frexp((double)sum * (1 + 1e-9), &ew[j]);
+            // the stencil of row j reaches rows j - 4 .. j + 4: entry t is row j - 4 + t
+            for (int t = 0; t < kStencil; ++t) {
+                const int c = p->col0[j] + t - (j - 4);
+                const double v = p->w1[(size_t)j * kStencil + t];
+                if (v != 0.0 && c >= 0 && c < kStencil)
+                    fx_limbs(std::ldexp((long double)v, -ew[j]), w[(size_t)j * kStencil + c].x, w[(size_t)j * kStencil + c].y);
+            }
+        }
+        TC_CUDA(p, put((void**)&p->d_fx_ir, fir.data(), fir.size() * sizeof(int4)));
+        TC_CUDA(p, put((void**)&p->d_fx_w1, w.data(), w.size() * sizeof(int2)));
+        TC_CUDA(p, put((void**)&p->d_fx_ew, ew.data(), ew.size() * sizeof(int)));
+    }
     std::vector<float> f(p->tw_z.begin(), p->tw_z.end());
     TC_CUDA(p, put((void**)&p->d_tw_z32, f.data(), f.size() * sizeof(float)));
     f.assign(p->tw_t.begin(), p->tw_t.end());
@@ -500,7 +621,8 @@ static void free_device(tc_plan* p) {
         p->mean_stream = nullptr;
     }
     void* ptrs[] = {p->d_r, p->d_ir, p->d_w1, p->d_w1f, p->d_dsc, p->d_w2, p->d_col0, p->d_d1t_row, p->d_d1t_w, p->d_fac, p->d_piv,
-                    p->d_fac2, p->d_piv2, p->d_spk, p->d_rinv, p->d_tw_z, p->d_tw_t, p->d_tw_z32, p->d_tw_t32};
+                    p->d_fac2, p->d_piv2, p->d_spk, p->d_rinv, p->d_tw_z, p->d_tw_t, p->d_tw_z32, p->d_tw_t32,
+                    p->d_fx_tw_z, p->d_fx_tw_t, p->d_fx_mm, p->d_fx_ir, p->d_fx_w1, p->d_fx_ew};
     for (void* q : ptrs)
         if (q) cudaFree(q);
     if (p->h_nonfinite) cudaFreeHost(p->h_nonfinite);
@@ -647,6 +769,9 @@ tc_status tc_plan_create_ex(tc_plan** out, int N_r, int M, int K, int m_p, doubl
     p->zfwd_lines32 = lines_for(sizeof(float2), 3);
     p->zt = zt_for(sizeof(double2), o.theta_zt > 0 ? o.theta_zt : 4, 200 * 1024);
     p->zt32 = zt_for(sizeof(float2), o.theta_zt > 0 ? o.theta_zt : 8, o.theta_zt > 0 ? 200 * 1024 : 76 * 1024);
+    p->fx_z = fx_plan(Pz);
+    p->fx_t = fx_plan(Pt);
+    p->fx_zt = fx_zt(p, o.theta_zt);
     p->pc_modes = o.pc_modes;
     p->theta_zt_forced = o.theta_zt;
     p->theta_variant = o.theta_variant;
@@ -697,6 +822,7 @@ tc_status tc_plan_create_ex(tc_plan** out, int N_r, int M, int K, int m_p, doubl
         p->ws.mean = take(0);
     }
     const size_t fwd_staging = off;
+    p->ws.fxe = take(p->precision == TC_MIXED && !p->adjoint ? 0 : fx_exp_bytes(p));
     p->ws.Ncur = take(3 * p->S * cplx);
     p->ws.uE = take(3 * p->S * cplx);
     // steps 2-5: fused kernel while 8 modes' four columns fit in 96 KB of shared memory,

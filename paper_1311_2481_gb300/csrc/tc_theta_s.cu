@@ -336,19 +336,4 @@ tc_status launch_theta_s(tc_plan* p, const float2* H1, float2* H2, cudaStream_t 
     return TC_ERR_ARG;
 }
 
-tc_status launch_theta_s64(tc_plan* p, const double2* H1, double2* H2, cudaStream_t s, int r0, int nh) {
-    if (theta_s_zt(p, true) == 0) return TC_ERR_ARG;
-    const double2* tw = p->d_tw_t;
-    // the FUSE form measured no faster with FP64 lines (0.4425 vs 0.4445 ms at the bench size):
-    // the FP64 pipe, not shared memory, bounds this kernel
-    switch (p->P_t) {
-        case 96: return run_theta_s<double2, 96, 4, 128, 3, true>(p, H1, H2, tw, s, r0, nh);
-        case 192: return run_theta_s<double2, 192, 2, 128, 3, true>(p, H1, H2, tw, s, r0, nh);
-        case 384: return run_theta_s<double2, 384, 2, 256, 2, true>(p, H1, H2, tw, s, r0, nh);
-        case 768: return run_theta_s<double2, 768, 1, 256, 2, true>(p, H1, H2, tw, s, r0, nh);
-        case 1152: return run_theta_s<double2, 1152, 1, 384, 1, true>(p, H1, H2, tw, s, r0, nh);
-    }
-    return TC_ERR_ARG;
-}
-
 }  // namespace tc
