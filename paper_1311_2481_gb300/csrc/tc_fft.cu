@@ -21,64 +21,6 @@
 
 namespace tc {
 
-// ---------------------------------------------------------------- inverse z-pass
-// Field f of H1: f = 3 d + c, c in {+, -, z}, d in {u, d_r u, d_z u}.
-__global__ void __launch_bounds__(256) k_zinv(const double2* __restrict__ u, double2* __restrict__ H1,
-                                              const double* __restrict__ w1, const int* __restrict__ col0,
-                                              int N_r, int M, int K, double kz, int L,
-                                              const double2* __restrict__ tw, Radices rad, int m0,
-                                              int r0, int nh) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int Pz = rad.n;
-    double2* a = reinterpret_cast<double2*>(smem_raw);
-    double2* b = a + (size_t)L * Pz;
-    const int groups = 9 / L;
-    const int g = blockIdx.x % groups;
-    const int rm = blockIdx.x / groups;
-    const int rl = rm % nh;        // r fastest: blocks sharing stencil rows run together
-    const int r = r0 + rl;
-    const int m = m0 + rm / nh;
-    const int nk = 2 * K + 1;
-    const size_t S = (size_t)N_r * (M + 1) * nk;
-    const size_t colstride = (size_t)(M + 1) * nk;
-    const int c0 = col0[r];
-    for (int idx = threadIdx.x; idx < L * Pz; idx += blockDim.x) {
-        const int l = idx / Pz;
-        const int q = idx - l * Pz;
-        const int k = q <= K ? q : q - Pz;
-        double2 x = make_double2(0.0, 0.0);
-        if (k >= -K && k <= K) {
-            const int f = g * L + l;
-            const int c = f % 3, d = f / 3;
-            const double2* base = u + (size_t)c * S + (size_t)m * nk + (k + K);
-            if (d == 1) {
-#pragma unroll
-                for (int t = 0; t < kStencil; ++t) {
-                    const double w = __ldg(&w1[r * kStencil + t]);
-                    const double2 y = __ldg(&base[(size_t)(c0 + t) * colstride]);
-                    x.x += w * y.x;
-                    x.y += w * y.y;
-                }
-            } else {
-                x = __ldg(&base[(size_t)r * colstride]);
-                if (d == 2) {
-                    const double kk = kz * k;
-                    x = make_double2(-kk * x.y, kk * x.x);
-                }
-            }
-        }
-        a[idx] = x;
-    }
-    __syncthreads();
-    double2* res = smem_fft(a, b, L, tw, true, rad);
-    for (int idx = threadIdx.x; idx < L * Pz; idx += blockDim.x) {
-        const int l = idx / Pz;
-        const int z = idx - l * Pz;
-        const int f = g * L + l;
-        H1[(((size_t)f * nh + rl) * (M + 1) + m) * Pz + z] = res[idx];
-    }
-}
-
 // ---------------------------------------------------------------- theta pass + products
 // Line p of a z value (6 per z):  0 (u_r, u_t)  1 (d_r u_r, d_r u_t)  2 (d_t u_r, d_t u_t)
 //                                 3 (d_z u_r, d_z u_t)  4 (u_z, d_r u_z)  5 (d_t u_z, d_z u_z)
@@ -179,126 +121,6 @@ __global__ void __launch_bounds__(256) k_theta(const V* __restrict__ H1, V* __re
         H2[fstride + o] = cconj(Qm);
         H2[2 * fstride + o] = nz;
     }
-}
-
-// ---------------------------------------------------------------- length-specialised z passes
-// Same work as k_zinv / k_zfwd with compile-time radix plans (radices <= 8) and padded lines.
-__device__ __forceinline__ double2 zinv_value(const double2* __restrict__ u, const double* __restrict__ w1,
-                                              int c0, size_t S, size_t colstride, int r, int m, int nk,
-                                              int K, int f, int k, double kz) {
-    const int c = f % 3, d = f / 3;
-    const double2* base = u + (size_t)c * S + (size_t)m * nk + (k + K);
-    double2 x = make_double2(0.0, 0.0);
-    if (d == 1) {
-#pragma unroll
-        for (int t = 0; t < kStencil; ++t) {
-            const double w = __ldg(&w1[r * kStencil + t]);
-            const double2 y = __ldg(&base[(size_t)(c0 + t) * colstride]);
-            x.x += w * y.x;
-            x.y += w * y.y;
-        }
-    } else {
-        x = __ldg(&base[(size_t)r * colstride]);
-        if (d == 2) {
-            const double kk = kz * k;
-            x = make_double2(-kk * x.y, kk * x.x);
-        }
-    }
-    return x;
-}
-
-template <int PZ, int L, int NT>
-__global__ void __launch_bounds__(NT, 2) k_zinv_s64(const double2* __restrict__ u, double2* __restrict__ H1,
-                                                    const double* __restrict__ w1, const int* __restrict__ col0,
-                                                    int N_r, int M, int K, double kz, const double2* __restrict__ tw,
-                                                    int m0, int r0, int nh) {
-    constexpr int LP = cft::padded<PZ>();
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    double2* a = reinterpret_cast<double2*>(smem_raw);
-    double2* b = a + L * LP;
-    constexpr int groups = 9 / L;
-    const int g = blockIdx.x % groups;
-    const int rm = blockIdx.x / groups;
-    const int rl = rm % nh;
-    const int r = r0 + rl;
-    const int m = m0 + rm / nh;
-    const int nk = 2 * K + 1;
-    const size_t S = (size_t)N_r * (M + 1) * nk;
-    const size_t colstride = (size_t)(M + 1) * nk;
-    const int c0 = col0[r];
-#pragma unroll
-    for (int l = 0; l < L; ++l)
-        for (int q = threadIdx.x; q < PZ; q += NT) {
-            const int k = q <= K ? q : q - PZ;
-            if (k >= -K) a[l * LP + cft::pd(q)] = zinv_value(u, w1, c0, S, colstride, r, m, nk, K, g * L + l, k, kz);
-        }
-    __syncthreads();
-    // the band K < q < PZ - K is zero: the first pass does not read it
-    const double2* X = cft::passes<PZ, 0, 1, L, NT, true, double2, true>(a, b, tw, K + 1, PZ - K);
-#pragma unroll
-    for (int l = 0; l < L; ++l) {
-        double2* dst = H1 + (((size_t)(g * L + l) * nh + rl) * (M + 1) + m) * PZ;
-        for (int z = threadIdx.x; z < PZ; z += NT) dst[z] = X[l * LP + cft::pd(z)];
-    }
-}
-
-namespace {
-
-// The FP64 staging kernels below process the radial rows r0 .. r0 + nh - 1 and address their
-// staging lines (H1, H2) as nh rows; the spectral arrays keep all N_r rows.
-
-template <int PZ, int L, int NT>
-tc_status zpass64(tc_plan* p, const double2* u, double2* H1, cudaStream_t s, int r0, int nh) {
-    constexpr int LP = cft::padded<PZ>();
-    const size_t sm = (size_t)2 * L * LP * sizeof(double2);
-    TC_CUDA(p, cudaFuncSetAttribute(k_zinv_s64<PZ, L, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    const int slot = prof_begin(p, kKZinv, s);
-    k_zinv_s64<PZ, L, NT><<<nh * (p->M + 1) * (9 / L), NT, sm, s>>>(u, H1, p->d_w1, p->d_col0, p->N_r, p->M,
-                                                                   p->K, p->k_z, p->d_tw_z, 0, r0, nh);
-    prof_end(p, slot, s);
-    TC_LAUNCHED(p, "k_zinv_s64");
-    return TC_OK;
-}
-
-// length-specialised FP64 inverse z pass; TC_ERR_ARG if P_z has no compile-time plan
-tc_status zpass64_s(tc_plan* p, const double2* u, double2* H1, cudaStream_t s, int r0, int nh) {
-    switch (p->P_z) {
-        case 12: return zpass64<12, 9, 64>(p, u, H1, s, r0, nh);
-        case 24: return zpass64<24, 9, 64>(p, u, H1, s, r0, nh);
-        case 48: return zpass64<48, 9, 128>(p, u, H1, s, r0, nh);
-        case 96: return zpass64<96, 9, 128>(p, u, H1, s, r0, nh);
-        case 192: return zpass64<192, 9, 256>(p, u, H1, s, r0, nh);
-        case 384: return zpass64<384, 3, 128>(p, u, H1, s, r0, nh);
-        case 768: return zpass64<768, 3, 256>(p, u, H1, s, r0, nh);
-        case 1152: return zpass64<1152, 1, 128>(p, u, H1, s, r0, nh);
-        case 1536: return zpass64<1536, 1, 256>(p, u, H1, s, r0, nh);
-        case 2304: return zpass64<2304, 1, 256>(p, u, H1, s, r0, nh);
-    }
-    return TC_ERR_ARG;
-}
-
-bool zpass64_ok(const tc_plan* p) {
-    switch (p->P_z) {
-        case 12: case 24: case 48: case 96: case 192: case 384: case 768: case 1152: case 1536: case 2304:
-            return p->theta_zt_forced == 0;
-    }
-    return false;
-}
-
-}  // namespace
-
-// FP64 inverse z pass with the radial stencil, rows r0 .. r0 + nh - 1 (forward lines of the adjoint)
-tc_status launch_zinv_fp64(tc_plan* p, const double2* u, double2* H1, cudaStream_t s, int r0, int nh) {
-    if (zpass64_ok(p)) return zpass64_s(p, u, H1, s, r0, nh);
-    const int L = p->zinv_lines;
-    const size_t sm1 = (size_t)2 * L * p->P_z * sizeof(double2);
-    TC_CUDA(p, cudaFuncSetAttribute(k_zinv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1));
-    const int slot = prof_begin(p, kKZinv, s);
-    k_zinv<<<nh * (p->M + 1) * (9 / L), p->thr_zinv, sm1, s>>>(u, H1, p->d_w1, p->d_col0, p->N_r, p->M, p->K,
-                                                              p->k_z, L, p->d_tw_z, p->rad_z, 0, r0, nh);
-    prof_end(p, slot, s);
-    TC_LAUNCHED(p, "k_zinv");
-    return TC_OK;
 }
 
 // theta pass of the mixed form with the generic kernel: FP32 lines (H1, H2 in float2), all rows

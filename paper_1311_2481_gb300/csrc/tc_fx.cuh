@@ -74,6 +74,7 @@ __device__ __forceinline__ long long mulhi(lim x, lim c, int sh, long long rnd) 
     const long long mid = mad(x.h, c.l, mad(x.l, c.h, rnd));
     return shr(mad(x.h, c.h, mid >> 32), sh);
 }
+constexpr long long kHalf32 = 1ll << 31;   // half_of(32)
 __device__ __forceinline__ long long half_of(int sh) { return sh > 0 && sh < 62 ? 1ll << (sh - 1) : 0ll; }
 
 // v (c + i s) or its conjugate
@@ -294,10 +295,16 @@ __device__ __forceinline__ void butterfly(cx (&v)[R], int ns, int k, const int4*
     dft<R, true>(v);
 }
 
+// right shifts of the input, taken in the first pass: lines < nl0 by (x0, y0), others by (x1, y1)
+struct InShift {
+    bool on = false;
+    int x0 = 0, y0 = 0, x1 = 0, y1 = 0;
+};
+
 // [qlo, qhi): inputs known to be zero
 template <int R, int QLO, int QHI>
 __device__ __forceinline__ void pass(cx* buf, int lp, int nl, bool first, int ns, int nb, unsigned mnb, unsigned mns,
-                                     const int4* __restrict__ tw, bool want_max, int nl0, uint4& mx, bool fold) {
+                                     const int4* __restrict__ tw, bool want_max, int nl0, uint4& mx, bool fold, const InShift& in) {
     constexpr int B = per_thread_of(R);
     cx v[B][R];
     int ln[B], jj[B];
@@ -315,6 +322,11 @@ __device__ __forceinline__ void pass(cx* buf, int lp, int nl, bool first, int ns
                 else if (first) v[b][q] = src[j + q * nb];
                 else if (fold && nb % 8 == 0) v[b][q] = src[pd(j) + q * pd(nb)];
                 else v[b][q] = src[pd(j + q * nb)];
+            }
+            if (first && in.on) {
+                const int sx = line < nl0 ? in.x0 : in.x1, sy = line < nl0 ? in.y0 : in.y1;
+#pragma unroll
+                for (int q = 0; q < R; ++q) v[b][q] = mk(shr(v[b][q].x, sx), shr(v[b][q].y, sy));
             }
             const int k = first ? 0 : fold ? j % ns : j - udiv(j, mns) * ns;
             butterfly<R>(v[b], first ? 1 : ns, k, tw);
@@ -350,25 +362,26 @@ __device__ __forceinline__ void pass(cx* buf, int lp, int nl, bool first, int ns
 }
 
 template <int N, int P, bool BAND>
-__device__ __forceinline__ void pass_of(cx* buf, int lp, int nl, const int4* __restrict__ tw, bool want_max, int nl0, uint4& mx) {
+__device__ __forceinline__ void pass_of(cx* buf, int lp, int nl, const int4* __restrict__ tw, bool want_max, int nl0, uint4& mx,
+                                        const InShift& in) {
     using C = Ct<N>;
     constexpr bool z = P == 0 && BAND;
     pass<C::r(P), z ? C::qlo() : 0, z ? C::qhi() : 0>(buf, lp, nl, P == 0, C::ns(P), C::nb(P), 0u, 0u, tw + C::tw(P),
-                                                      want_max && P == C::np - 1, nl0, mx, true);
+                                                      want_max && P == C::np - 1, nl0, mx, true, in);
 }
 // band: the input is zero in [n/3 + 1, 2n/3), and entries the first pass skips are not read
 template <int N>
 __device__ __forceinline__ uint4 transform(const Ct<N>&, cx* buf, int lp, int nl, const int4* __restrict__ tw, bool band,
-                                           bool want_max = false, int nl0 = 0) {
+                                           bool want_max = false, int nl0 = 0, const InShift& in = InShift{}) {
     uint4 mx = make_uint4(0, 0, 0, 0);
-    if (band) pass_of<N, 0, true>(buf, lp, nl, tw, false, 0, mx);
-    else pass_of<N, 0, false>(buf, lp, nl, tw, false, 0, mx);
-    pass_of<N, 1, false>(buf, lp, nl, tw, want_max, nl0, mx);
-    if constexpr (Ct<N>::np > 2) pass_of<N, 2, false>(buf, lp, nl, tw, want_max, nl0, mx);
+    if (band) pass_of<N, 0, true>(buf, lp, nl, tw, false, nl0, mx, in);
+    else pass_of<N, 0, false>(buf, lp, nl, tw, false, nl0, mx, in);
+    pass_of<N, 1, false>(buf, lp, nl, tw, want_max, nl0, mx, in);
+    if constexpr (Ct<N>::np > 2) pass_of<N, 2, false>(buf, lp, nl, tw, want_max, nl0, mx, in);
     return mx;
 }
 __device__ __forceinline__ uint4 transform(const Rt& pl, cx* buf, int lp, int nl, const int4* __restrict__ tw, bool,
-                                           bool want_max = false, int nl0 = 0) {
+                                           bool want_max = false, int nl0 = 0, const InShift& in = InShift{}) {
     uint4 mx = make_uint4(0, 0, 0, 0);
 #pragma unroll 1
     for (int p = 0; p < pl.f.np; ++p) {
@@ -376,7 +389,7 @@ __device__ __forceinline__ uint4 transform(const Rt& pl, cx* buf, int lp, int nl
         const bool wm = want_max && p == pl.f.np - 1;
         const int4* t = tw + s.tw;
 #define TC_FX_PASS(R) \
-    case R: pass<R, 0, 0>(buf, lp, nl, p == 0, s.ns, s.nb, s.mnb, s.mns, t, wm, nl0, mx, false); break;
+    case R: pass<R, 0, 0>(buf, lp, nl, p == 0, s.ns, s.nb, s.mnb, s.mns, t, wm, nl0, mx, false, in); break;
         switch (s.r) {
             TC_FX_PASS(2) TC_FX_PASS(3) TC_FX_PASS(4) TC_FX_PASS(6) TC_FX_PASS(8) TC_FX_PASS(9) TC_FX_PASS(12)
         }

@@ -16,26 +16,6 @@ namespace {
 // memory.  The last pass of a phase keeps its outputs in registers; the threads of L0 and
 // then those of L1 add their products.
 
-// Exponents of a sum that takes one or two products: shifts of the old sum and of the
-// products, with their rounding constants.
-struct Sum {
-    int so, s1, s2;
-    long long ro, r1, r2;
-    __device__ __forceinline__ void set(int& E, int e1, int e2) {
-        const int En = max(E, max(e1, e2)) + 2;
-        so = min(En - E, 63);
-        s1 = En - e1 - 2;
-        s2 = En - e2 - 2;
-        ro = half_of(so);
-        r1 = half_of(s1 + 32);
-        r2 = half_of(s2 + 32);
-        E = En;
-    }
-    __device__ __forceinline__ long long old(long long x) const { return (x + ro) >> so; }
-    __device__ __forceinline__ long long first(lim a, lim b) const { return mulhi(a, b, s1, r1); }
-    __device__ __forceinline__ long long second(lim a, lim b) const { return mulhi(a, b, s2, r2); }
-};
-
 template <class PL, int ZT, int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB) k_fx_theta(ThetaArgs a, FxPlan f) {
     extern __shared__ cx buf[];
@@ -64,69 +44,11 @@ __global__ void __launch_bounds__(NT, MINB) k_fx_theta(ThetaArgs a, FxPlan f) {
         f(0, 0, false); f(0, 1, false); f(1, 2, false); f(2, 5, false); f(3, 3, false); f(3, 4, false);
         f(4, 0, true); f(4, 1, true); f(5, 6, false); f(5, 7, false); f(6, 2, true); f(7, 8, false);
     };
-    int er[8];      // largest exponent of a kind
-    float sum[8];   // sum of the values, in units of 2^32 at that exponent
-    {
-        int2 v[9];
-#pragma unroll
-        for (int s = 0; s < 8; ++s) er[s] = 4 * kExpZero;
-        for (int m = threadIdx.x; m <= M; m += nt) {
-#pragma unroll
-            for (int q = 0; q < 9; ++q) v[q] = __ldg(&eh[q * es + m]);
-            bound([&](int s, int q, bool mul) {
-                if (!mul || m > 0) er[s] = max(er[s], v[q].x);
-            });
-        }
-        if (threadIdx.x < 8) s_E[threadIdx.x] = 4 * kExpZero;
-        if (threadIdx.x < 12) s_mx[threadIdx.x >> 2][threadIdx.x & 3] = 0;
-        __syncthreads();
-        int mine = 0;
-#pragma unroll
-        for (int s = 0; s < 8; ++s) {
-            const int x = __reduce_max_sync(0xffffffffu, er[s]);
-            if (lane == s) mine = x;
-        }
-        if (lane < 8) atomicMax(&s_E[lane], mine);
-        __syncthreads();
-#pragma unroll
-        for (int s = 0; s < 8; ++s) {
-            er[s] = s_E[s];
-            sum[s] = 0.f;
-        }
-        for (int m = threadIdx.x; m <= M; m += nt) {
-            const float mm = (float)(m * a.mp);
-#pragma unroll
-            for (int q = 0; q < 9; ++q) v[q] = __ldg(&eh[q * es + m]);
-            bound([&](int s, int q, bool mul) {
-                // 2^(e - er), 0 below 2^-100; both signs of m count for the real pairs
-                const int d = min(er[s] - v[q].x, 127);
-                const float x = (float)(unsigned)v[q].y * __int_as_float(max(127 - d, 0) << 23) * (s == 1 || s == 2 || s >= 6 ? 2.f : 1.f);
-                sum[s] += mul ? x * mm : x;
-            });
-        }
-#pragma unroll
-        for (int s = 0; s < 8; ++s)
-#pragma unroll
-            for (int o = 16; o; o >>= 1) sum[s] += __shfl_xor_sync(0xffffffffu, sum[s], o);
-        if (lane == 0) {
-#pragma unroll
-            for (int s = 0; s < 8; ++s) s_bound[wid][s] = sum[s];
-        }
-        __syncthreads();
-#pragma unroll
-        for (int s = 0; s < 8; ++s) {
-            sum[s] = 0.f;
-            for (int w = 0; w < nw; ++w) sum[s] += s_bound[w][s];   // in a fixed order
-        }
-    }
-    // sums brought below 2^62, the parts of a real pair below 2^61 each
-    auto kind = [&](int s) {
-        const int b = ((__float_as_int(sum[s] * 1.001f) >> 23) & 0xff) - 126;   // sum < 2^b
-        const bool mul = s == 4 || s == 6, half = s == 1 || s == 2 || s >= 6;
-        int E = er[s] + max(0, b - (half ? 29 : 30));
-        if (mul) E = max(E, er[s] + a.emm - 30);   // keeps the shift of the products with m m_p positive
-        return E;
-    };
+    int er[8];
+    float sum[8];
+    line_bounds<9, 8, NT>([&](int q, int m) { return __ldg(&eh[q * es + m]); }, bound, 0xc6u, M, a.mp, nt, s_E, s_bound, er, sum);
+    if (threadIdx.x < 12) s_mx[threadIdx.x >> 2][threadIdx.x & 3] = 0;   // barriers follow before its use
+    auto kind = [&](int s) { return kind_exponent(er[s], sum[s], s == 4 || s == 6, (0xc6u >> s) & 1, a.emm); };
     const int E0 = kind(0), E1x = kind(1), E1y = kind(2), E2 = kind(3), E3 = kind(4), E4 = kind(5), E5x = kind(6), E5y = kind(7);
     if (max(max(max(E0, E1x), max(E1y, E2)), max(max(E3, E4), max(E5x, E5y))) > kExpNaN / 2) {
         if (threadIdx.x < 2) {
@@ -148,45 +70,14 @@ __global__ void __launch_bounds__(NT, MINB) k_fx_theta(ThetaArgs a, FxPlan f) {
         for (int i = threadIdx.x; i < zt * (M + 1); i += nt) {
             const int m = divz(i), z = i - m * zt;
             const size_t o = (size_t)m * Pz + z;
-            cx A = h[fa * fs + o], C = h[(fa + 1) * fs + o];
-            cx X = h[(PH == 1 ? 0 : 2) * fs + o], Y = h[(PH == 0 ? 5 : PH == 1 ? 1 : 8) * fs + o];
-            const int ta = Ea - eh[fa * es + m].x, tc = Ea - eh[(fa + 1) * es + m].x;
-            const int ex = eh[(PH == 1 ? 0 : 2) * es + m].x, ey = eh[(PH == 0 ? 5 : PH == 1 ? 1 : 8) * es + m].x;
-            A = mk(shr(A.x, ta), shr(A.y, ta));
-            C = mk(shr(C.x, tc), shr(C.y, tc));
-            cx* l0 = buf + z * lp;
+            constexpr int fx_ = PH == 1 ? 0 : 2, fy_ = PH == 0 ? 5 : PH == 1 ? 1 : 8;
+            const cx A = h[fa * fs + o], C = h[(fa + 1) * fs + o], X = h[fx_ * fs + o], Y = h[fy_ * fs + o];
+            const int ea = eh[fa * es + m].x, ec = eh[(fa + 1) * es + m].x, ex = eh[fx_ * es + m].x, ey = eh[fy_ * es + m].x;
+            put_pair(buf + z * lp, P, m, shr2(A, Ea - ea), shr2(C, Ea - ec));
             cx* l1 = buf + (zt + z) * lp;
-            const int mn = P - m;
-            if (m == 0) {
-                l0[0] = mk((A.x + C.x) >> 1, (A.y - C.y) >> 1);
-            } else {
-                l0[m] = A;
-                l0[mn] = conj(C);
-            }
-            if (PH > 0) {   // i m m_p X
-                const lim F = {a.mm[m].x, a.mm[m].y};
-                const int sh = 30 - a.emm + (PH == 1 ? E3 : E5x) - ex;
-                X = mk(-mulsh(split(X.y), F, sh), mulsh(split(X.x), F, sh));
-                if (PH == 1) {
-                    const int sy = 30 - a.emm + E3 - ey;
-                    Y = mk(-mulsh(split(Y.y), F, sy), mulsh(split(Y.x), F, sy));
-                }
-            } else {
-                X = mk(shr(X.x, E1x - ex), shr(X.y, E1x - ex));
-            }
-            if (PH != 1) {
-                const int ty = (PH == 0 ? E1y : E5y) - ey;
-                Y = mk(shr(Y.x, ty), shr(Y.y, ty));
-            }
-            if (m == 0) {
-                l1[0] = PH == 1 ? mk(0, 0) : mk(X.x, Y.x);
-            } else if (PH == 1) {
-                l1[m] = X;
-                l1[mn] = conj(Y);
-            } else {
-                l1[m] = mk(X.x - Y.y, X.y + Y.x);
-                l1[mn] = mk(X.x + Y.y, Y.x - X.y);
-            }
+            if (PH == 0) put_real2(l1, P, m, shr2(X, E1x - ex), shr2(Y, E1y - ey));
+            else if (PH == 1) put_pair(l1, P, m, imul(X, a.mm[m], a.emm, E3, ex), imul(Y, a.mm[m], a.emm, E3, ey));
+            else put_real2(l1, P, m, imul(X, a.mm[m], a.emm, E5x, ex), shr2(Y, E5y - ey));
         }
     };
     auto products = [&](auto ph) {

@@ -129,7 +129,9 @@ template <int NL, bool MAX> __device__ __forceinline__ void line_reduce(unsigned
 // ---------------------------------------------------------------- inverse z pass
 // NL lines per block, out of the nine (d, c) of an (r, m), d = 0, 1, 2 for u, d_r u, d_z u.  tl
 // threads per line hold its entries (at most 8 each) from the load to the fixed-point line.
-template <class PL, int NL>
+// ADJ: the three lines of the adjoint field Nbar = u instead, (s_r, s_t, s_z) = c_m scale (Nbar_+ +
+// Nbar_-, -i (Nbar_+ - Nbar_-), Nbar_z) with c_m = 1 for m = 0 and 1/2 beyond (kz: the scale).
+template <class PL, int NL, bool ADJ>
 __global__ void __launch_bounds__(kZThreads) k_fx_zinv(const double2* __restrict__ u, const double2* __restrict__ du,
                                                        cx* __restrict__ H1, int2* __restrict__ e1, int N, int M, int K,
                                                        double kz, int r0, int nh, FxPlan f, const int4* __restrict__ tw,
@@ -140,10 +142,12 @@ __global__ void __launch_bounds__(kZThreads) k_fx_zinv(const double2* __restrict
     const PL pl(f);
     const int P = pl.size(), lp = line_pitch(P), nk = 2 * K + 1, nmode = (M + 1) * nk;
     int t = blockIdx.x;
-    const int f0 = t % (9 / NL) * NL;   // lines in the order 3 c + d: a block reads few lines of u
-    t /= 9 / NL;
+    constexpr int NF = ADJ ? 3 : 9;
+    const int f0 = t % (NF / NL) * NL;   // lines in the order 3 c + d: a block reads few lines of u
+    t /= NF / NL;
     const int rl = t % nh, m = t / nh;   // rows fastest: neighbouring blocks share cache lines of u
-    if (m == 0 && f0 == 0 && threadIdx.x < 2) e2max[rl * 2 + threadIdx.x] = 4 * kExpZero;   // the theta pass takes maxima here
+    constexpr int NE = ADJ ? 6 : 2;      // the theta pass takes maxima here
+    if (m == 0 && f0 == 0 && threadIdx.x < NE) e2max[rl * NE + threadIdx.x] = 4 * kExpZero;
     if (threadIdx.x < NL) {
         s_e[threadIdx.x] = 0;
         s_l1[threadIdx.x] = 0;
@@ -152,10 +156,31 @@ __global__ void __launch_bounds__(kZThreads) k_fx_zinv(const double2* __restrict
     __syncthreads();
     const int line = NL == 1 ? 0 : udiv(threadIdx.x, mtl), i0 = threadIdx.x - line * tl;
     const bool on = line < NL;
-    const int c = (f0 + line) / 3, d = f0 + line - 3 * c;
+    const int c = ADJ ? f0 + line : (f0 + line) / 3, d = ADJ ? 0 : f0 + line - 3 * c;
     double2 x[8];
     int e = 0;
-    if (on) {
+    if (ADJ && on) {
+        const double2* a = u + (size_t)(r0 + rl) * nmode + (size_t)m * nk;
+        const size_t S = (size_t)N * nmode;
+        const double cm = (m == 0 ? 1.0 : 0.5) * kz;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int k = i0 + i * tl;
+            x[i] = make_double2(0.0, 0.0);
+            if (k < nk) {
+                if (c == 2) {
+                    const double2 v = __ldg(&a[2 * S + k]);
+                    x[i] = make_double2(cm * v.x, cm * v.y);
+                } else {
+                    const double2 p = __ldg(&a[k]), n = __ldg(&a[S + k]);
+                    x[i] = c == 0 ? make_double2(cm * (p.x + n.x), cm * (p.y + n.y)) : make_double2(cm * (p.y - n.y), -cm * (p.x - n.x));
+                }
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) e = max(e, max(bexp(x[i].x), bexp(x[i].y)));
+    }
+    if (!ADJ && on) {
         const double2* src = d == 1 && du ? du + ((size_t)c * nh + rl) * nmode + (size_t)m * nk
                                           : u + ((size_t)c * N + r0 + rl) * nmode + (size_t)m * nk;
         if (NL == 9 && d == 1 && !du) {   // d_r u here, in FP64
@@ -239,57 +264,97 @@ __global__ void __launch_bounds__(kZThreads) k_fx_zinv(const double2* __restrict
 }
 
 // ---------------------------------------------------------------- forward z pass
-template <class PL, int NL>
-__global__ void __launch_bounds__(kZThreads) k_fx_zfwd(const cx* __restrict__ H2, double2* __restrict__ Nh,
-                                                       const int* __restrict__ e2, const int* __restrict__ e2max, int N,
-                                                       int M, int K, double scale, int r0, int nh, int zt, unsigned mzt,
-                                                       FxPlan f, const int4* __restrict__ tw, int tl, unsigned mtl) {
+// Lines of H2 (the three components of N), or (ADJ) of H3: A, R, Z of one component, of which
+// ubar += A - i k k_z Z and Rhat = R.  NL = 3 lines per block, or one: then line l0 of each
+// component (ADJ), or each component in its own block.
+struct ZfwdOut {
+    double2* out;    // N, or ubar
+    double2* Rh;     // Rhat of the staged rows
+    double scale;    // of N
+    double kz;
+    int l0;
+};
+
+template <class PL, int NL, bool ADJ>
+__global__ void __launch_bounds__(kZThreads) k_fx_zfwd(const cx* __restrict__ H2, ZfwdOut w, const int* __restrict__ e2,
+                                                       const int* __restrict__ e2max, int N, int M, int K, int r0, int nh, int zt,
+                                                       unsigned mzt, FxPlan f, const int4* __restrict__ tw, int tl, unsigned mtl) {
     extern __shared__ cx buf[];
     __shared__ unsigned s_l1[NL];
     const PL pl(f);
+    constexpr int NE = ADJ ? 6 : 2;
     const int P = pl.size(), lp = line_pitch(P), nk = 2 * K + 1, nmode = (M + 1) * nk;
     int t = blockIdx.x;
-    const int c0 = t % (3 / NL) * NL;
-    t /= 3 / NL;
+    constexpr int NB = ADJ ? 3 : 3 / NL;   // blocks per (r, m)
+    const int b = t % NB;
+    t /= NB;
     const int m = t % (M + 1), rl = t / (M + 1);
     if (threadIdx.x < NL) s_l1[threadIdx.x] = 0;
     __syncthreads();
-    const int line = NL == 1 ? 0 : udiv(threadIdx.x, mtl), i0 = threadIdx.x - line * tl, c = c0 + line;
+    const int line = NL == 1 ? 0 : udiv(threadIdx.x, mtl), i0 = threadIdx.x - line * tl;
     const bool on = line < NL;
-    const int E = e2max[rl * 2 + (c == 2)];
+    // component and kind (A, R, Z) of this thread's line, its field and exponent
+    const int c = ADJ ? b : b * NL + line, l = ADJ ? (NL == 1 ? w.l0 : line) : 0;
+    const int field = 3 * l + c, ie = 2 * l + (c == 2);
+    const int E = on ? e2max[rl * NE + ie] : 0;
     cx v[8];
     unsigned l1 = 0;
     if (on) {
-        const cx* h = H2 + (((size_t)c * nh + rl) * (M + 1) + m) * P;
-        const int* er = e2 + (size_t)rl * (P / zt) * 2 + (c == 2);
+        const cx* h = H2 + (((size_t)field * nh + rl) * (M + 1) + m) * P;
+        const int* er = e2 + (size_t)rl * (P / zt) * NE + ie;
 #pragma unroll
         for (int i = 0; i < 8; ++i) v[i] = i0 + i * tl < P ? h[i0 + i * tl] : mk(0, 0);
 #pragma unroll
         for (int i = 0; i < 8; ++i)
             if (i0 + i * tl < P) {
-                const int te = E - __ldg(&er[udiv(i0 + i * tl, mzt) * 2]);
+                const int te = E - __ldg(&er[udiv(i0 + i * tl, mzt) * NE]);
                 v[i] = mk(shr(v[i].x, te), shr(v[i].y, te));
                 l1 += ((mag_hi(v[i].x) + mag_hi(v[i].y)) >> 11) + 1;
             }
     }
     line_reduce<NL, false>(s_l1, line, l1, tl);
     __syncthreads();
-    const int s = on ? max(0, bits(s_l1[line]) - 19) : 0;
     if (on) {
+        const int s = max(0, bits(s_l1[line]) - 19);
 #pragma unroll
         for (int i = 0; i < 8; ++i)
             if (i0 + i * tl < P) buf[line * lp + i0 + i * tl] = mk(v[i].y >> s, v[i].x >> s);   // exchanged
     }
     __syncthreads();
     transform(pl, buf, lp, NL, tw, false);
-    if (on) {
-        const bool bad = E > kExpNaN / 2;
-        double2* dst = Nh + ((size_t)c * N + r0 + rl) * nmode + (size_t)m * nk;
-        for (int kk = i0; kk < nk; kk += tl) {
-            const cx o = buf[line * lp + pd(kk >= K ? kk - K : kk - K + P)];
-            dst[kk] = bad ? make_double2(nan64(), nan64())
-                          : make_double2(to_double(o.y, E + s - 62) * scale, to_double(o.x, E + s - 62) * scale);
+    // line q's value of mode k (index kk = k + K), from its own exponent
+    auto value = [&](int q, int kk, int Eq) {
+        const cx o = buf[q * lp + pd(kk >= K ? kk - K : kk - K + P)];
+        const int s = Eq + max(0, bits(s_l1[q]) - 19) - 62;
+        return Eq > kExpNaN / 2 ? make_double2(nan64(), nan64()) : make_double2(to_double(o.y, s), to_double(o.x, s));
+    };
+    const size_t e0 = ((size_t)c * N + r0 + rl) * nmode + (size_t)m * nk, h0 = ((size_t)c * nh + rl) * nmode + (size_t)m * nk;
+    if (!ADJ) {
+        if (on)
+            for (int kk = i0; kk < nk; kk += tl) {
+                const double2 o = value(line, kk, E);
+                w.out[e0 + kk] = make_double2(o.x * w.scale, o.y * w.scale);
+            }
+        return;
+    }
+    const int* em = e2max + rl * NE + (c == 2);
+    for (int kk = threadIdx.x; kk < nk; kk += blockDim.x) {
+        const double kzk = w.kz * (kk - K);
+        if (NL == 3 || w.l0 != 1) {
+            double2 u = w.out[e0 + kk];
+            if (NL == 3 || w.l0 == 0) {
+                const double2 A = value(0, kk, em[0]);
+                u.x += A.x;
+                u.y += A.y;
+            }
+            if (NL == 3 || w.l0 == 2) {
+                const double2 Z = value(NL == 3 ? 2 : 0, kk, em[4]);
+                u.x += kzk * Z.y;
+                u.y -= kzk * Z.x;
+            }
+            w.out[e0 + kk] = u;
         }
+        if (NL == 3 || w.l0 == 1) w.Rh[h0 + kk] = value(NL == 3 ? 1 : 0, kk, em[2]);
     }
 }
 
@@ -310,32 +375,54 @@ size_t fx_exp_bytes(const tc_plan* p) {
 
 namespace {
 
-// Launch shapes.  z passes: as many of the lines of an (r, m) per block as give it about 128
-// threads at n / 8 each.
-int lines_zinv(int P) { return P <= 96 ? 9 : P <= 768 ? 3 : 1; }
-int lines_zfwd(int P) { return P <= 768 ? 3 : 1; }
+// What a z pass does: the inverse one of u (or of Nbar), the forward one into N (or into ubar
+// and Rhat).
+struct ZPass {
+    bool inverse, adj;
+    const double2* in;    // u or Nbar
+    const double2* du;    // d_r u (nullptr: taken by the pass)
+    cx* H;                // lines written or read
+    int2* e1;             // exponents of the lines of an inverse pass
+    int* e2max;
+    const int* e2;
+    ZfwdOut out;
+    int r0, nh, zt;
+};
 
+// Launch shapes: as many of the lines of an (r, m) per block as give it about 128 threads at
+// n / 8 each (L9 of nine, L3 of three).
 template <class PL, int L9, int L3>
-tc_status z_pass(tc_plan* p, const double2* u, const double2* du, cx* H1, const cx* H2, double2* Nh, const Exps& e, const int4* tw,
-                 cudaStream_t s, bool inverse, int r0, int nh) {
+tc_status z_pass(tc_plan* p, const ZPass& a, const int4* tw, cudaStream_t s) {
     // at least a thread for 8 entries of a line; 4 in the short ones, where latency counts
-    const int P = p->P_z, nl = inverse ? L9 : L3, thr = round32(nl * (P <= 48 ? (P + 3) / 4 : (P + 7) / 8)), tl = thr / nl;
+    const int P = p->P_z, nl = a.inverse && !a.adj ? L9 : L3, thr = round32(nl * (P <= 48 ? (P + 3) / 4 : (P + 7) / 8)), tl = thr / nl;
     const size_t sm = (size_t)nl * line_pitch(P) * sizeof(cx);
-    if (inverse) {
-        auto k = k_fx_zinv<PL, L9>;
+    const int rm = a.nh * (p->M + 1);
+    const double scale = 1.0 / ((double)p->P_t * (double)P);
+    auto inv = [&](auto k, int lines) -> tc_status {
         TC_CUDA(p, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-        k<<<nh * (p->M + 1) * (9 / L9), thr, sm, s>>>(u, du, H1, e.e1, p->N_r, p->M, p->K, p->k_z, r0, nh, p->fx_z, tw, tl, magic(tl),
-                                               e.e2max, p->d_w1, p->d_col0);
+        k<<<rm * (lines / nl), thr, sm, s>>>(a.in, a.du, a.H, a.e1, p->N_r, p->M, p->K, a.adj ? scale : p->k_z, a.r0, a.nh, p->fx_z, tw, tl,
+                                             magic(tl), a.e2max, p->d_w1, p->d_col0);
         TC_LAUNCHED(p, "k_fx_zinv");
-    } else {
-        auto k = k_fx_zfwd<PL, L3>;
+        return TC_OK;
+    };
+    auto fwd = [&](auto k, int blocks, int l0) -> tc_status {
+        ZfwdOut o = a.out;
+        o.scale = scale;
+        o.kz = p->k_z;
+        o.l0 = l0;
         TC_CUDA(p, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-        k<<<nh * (p->M + 1) * (3 / L3), thr, sm, s>>>(H2, Nh, e.e2, e.e2max, p->N_r, p->M, p->K, 1.0 / ((double)p->P_t * (double)P), r0,
-                                                     nh, p->fx_zt, magic(p->fx_zt), p->fx_z, tw, tl, magic(tl));
+        k<<<rm * blocks, thr, sm, s>>>(a.H, o, a.e2, a.e2max, p->N_r, p->M, p->K, a.r0, a.nh, a.zt, magic(a.zt), p->fx_z, tw, tl, magic(tl));
         TC_LAUNCHED(p, "k_fx_zfwd");
-    }
+        return TC_OK;
+    };
+    if (a.inverse) return a.adj ? inv(k_fx_zinv<PL, L3, true>, 3) : inv(k_fx_zinv<PL, L9, false>, 9);
+    if (!a.adj) return fwd(k_fx_zfwd<PL, L3, false>, 3 / L3, 0);
+    if (L3 == 3) return fwd(k_fx_zfwd<PL, L3, true>, 3, 0);
+    for (int l = 0; l < 3; ++l) TC_TRY_STATUS(fwd(k_fx_zfwd<PL, L3, true>, 3, l));
     return TC_OK;
 }
+
+tc_status run_z(tc_plan* p, const ZPass& a, cudaStream_t s);
 
 // lengths with a compile-time plan, and the z values of their theta blocks (0: none)
 bool static_z(int P) {
@@ -359,13 +446,24 @@ const int* fx_static_radices(int n) {
 
 namespace {
 
-// The transforms of rows r0 .. r0 + nh - 1.
-tc_status fx_rows(tc_plan* p, const double2* u, double2* Nh, char* ws, cudaStream_t s, int r0, int nh) {
-    cx* H1 = reinterpret_cast<cx*>(ws + p->ws.H1);
-    cx* H2 = reinterpret_cast<cx*>(ws + p->ws.H2);
-    double2* du = reinterpret_cast<double2*>(H2);
-    const Exps e = exps(p, ws);
-    int slot = prof_begin(p, kKZinv, s);
+tc_status run_z(tc_plan* p, const ZPass& a, cudaStream_t s) {
+    const bool st = p->theta_zt_forced == 0 && static_z(p->P_z) && 3 * p->K <= p->P_z;
+    const int4* tw = p->d_fx_tw_z + (st ? p->fx_z.table : 0);
+    switch (st ? p->P_z : 0) {
+#define TC_FX_Z(P, A, B) case P: return z_pass<Ct<P>, A, B>(p, a, tw, s);
+        TC_FX_Z(12, 9, 3) TC_FX_Z(24, 9, 3) TC_FX_Z(36, 9, 3) TC_FX_Z(48, 9, 3) TC_FX_Z(72, 9, 3) TC_FX_Z(96, 9, 3) TC_FX_Z(144, 3, 3)
+        TC_FX_Z(192, 3, 3) TC_FX_Z(288, 3, 3) TC_FX_Z(384, 3, 3) TC_FX_Z(576, 3, 3) TC_FX_Z(768, 3, 3) TC_FX_Z(1152, 1, 1)
+        TC_FX_Z(1536, 1, 1) TC_FX_Z(2304, 1, 1)
+#undef TC_FX_Z
+    }
+    if (p->P_z <= 96) return z_pass<Rt, 9, 3>(p, a, tw, s);
+    if (p->P_z <= 768) return z_pass<Rt, 3, 3>(p, a, tw, s);
+    return z_pass<Rt, 1, 1>(p, a, tw, s);
+}
+
+// inverse z pass of u with its derivatives, rows r0 .. r0 + nh - 1; du: scratch of 3 nh (M+1)(2K+1)
+tc_status zinv_u(tc_plan* p, const double2* u, double2* du, cx* H1, const Exps& e, cudaStream_t s, int r0, int nh) {
+    const int slot = prof_begin(p, kKZinv, s);
     if (p->P_z <= 96 && p->S <= 65536) {
         // small problems: the inverse z pass takes d_r u itself, in FP64.  Its 18 FMAs per value
         // then cost less than a launch (S = 5000: 0.4 us of the FP64 pipe against 7 us).
@@ -376,34 +474,61 @@ tc_status fx_rows(tc_plan* p, const double2* u, double2* Nh, char* ws, cudaStrea
             2 * p->nmode, r0, nh);
         TC_LAUNCHED(p, "k_fx_dr");
     }
-    const bool sz = p->theta_zt_forced == 0 && static_z(p->P_z) && 3 * p->K <= p->P_z;
-    const int4* twz = p->d_fx_tw_z + (sz ? p->fx_z.table : 0);
-    auto z = [&](bool inverse) -> tc_status {
-        switch (sz ? p->P_z : 0) {
-#define TC_FX_Z(P, A, B) case P: return z_pass<Ct<P>, A, B>(p, u, du, H1, H2, Nh, e, twz, s, inverse, r0, nh);
-            TC_FX_Z(12, 9, 3) TC_FX_Z(24, 9, 3) TC_FX_Z(36, 9, 3) TC_FX_Z(48, 9, 3) TC_FX_Z(72, 9, 3) TC_FX_Z(96, 9, 3) TC_FX_Z(144, 3, 3)
-            TC_FX_Z(192, 3, 3) TC_FX_Z(288, 3, 3) TC_FX_Z(384, 3, 3) TC_FX_Z(576, 3, 3) TC_FX_Z(768, 3, 3) TC_FX_Z(1152, 1, 1) TC_FX_Z(1536, 1, 1)
-            TC_FX_Z(2304, 1, 1)
-#undef TC_FX_Z
-        }
-        if (p->P_z <= 96) return z_pass<Rt, 9, 3>(p, u, du, H1, H2, Nh, e, twz, s, inverse, r0, nh);
-        if (p->P_z <= 768) return z_pass<Rt, 3, 3>(p, u, du, H1, H2, Nh, e, twz, s, inverse, r0, nh);
-        return z_pass<Rt, 1, 1>(p, u, du, H1, H2, Nh, e, twz, s, inverse, r0, nh);
-    };
-    TC_TRY_STATUS(z(true));
+    TC_TRY_STATUS(run_z(p, ZPass{true, false, u, du, H1, e.e1, e.e2max, nullptr, {}, r0, nh, 1}, s));
     prof_end(p, slot, s);
-    slot = prof_begin(p, kKTheta, s);
+    return TC_OK;
+}
+
+// The transforms of rows r0 .. r0 + nh - 1.
+tc_status fx_rows(tc_plan* p, const double2* u, double2* Nh, char* ws, cudaStream_t s, int r0, int nh) {
+    cx* H1 = reinterpret_cast<cx*>(ws + p->ws.H1);
+    cx* H2 = reinterpret_cast<cx*>(ws + p->ws.H2);
+    const Exps e = exps(p, ws);
+    TC_TRY_STATUS(zinv_u(p, u, reinterpret_cast<double2*>(H2), H1, e, s, r0, nh));
+    int slot = prof_begin(p, kKTheta, s);
     ThetaArgs a{H1, H2, e.e1, e.e2, e.e2max, p->d_fx_ir, p->d_fx_mm, p->d_fx_tw_t, r0, nh, p->M, p->P_z, p->fx_zt, p->fx_emm,
                 magic(p->fx_zt), magic(p->P_t), (long long)p->m_p};
     TC_TRY_STATUS(launch_fx_theta(p, a, s));
     prof_end(p, slot, s);
     slot = prof_begin(p, kKZfwd, s);
-    TC_TRY_STATUS(z(false));
+    TC_TRY_STATUS(run_z(p, ZPass{false, false, nullptr, nullptr, H2, nullptr, e.e2max, e.e2, {Nh, nullptr, 0, 0, 0}, r0, nh, p->fx_zt}, s));
     prof_end(p, slot, s);
     return TC_OK;
 }
 
 }  // namespace
+
+// exponents of the transposed term's lines: e1a[3][stage_rows][M+1], e2max[stage_rows][6], e2[stage_rows][P_z][6]
+size_t fx_adj_exp_bytes(const tc_plan* p) {
+    return (size_t)p->stage_rows * ((size_t)3 * (p->M + 1) * sizeof(int2) + 6 * sizeof(int) + (size_t)6 * p->P_z * sizeof(int));
+}
+
+// ubar += (the transposed transforms and products of Nbar about u), rows r0 .. r0 + nh - 1, but
+// for the radial stencil: Rhat takes the part that k_drT brings in
+tc_status launch_adjoint_rows_fx(tc_plan* p, const double2* u, const double2* Nbar, double2* ubar, double2* Rh, char* ws, cudaStream_t s,
+                                 int r0, int nh) {
+    cx* H1 = reinterpret_cast<cx*>(ws + p->ws.H1a);
+    cx* Ha = reinterpret_cast<cx*>(ws + p->ws.Ha);
+    cx* H3 = reinterpret_cast<cx*>(ws + p->ws.H3);
+    const Exps e = exps(p, ws);
+    int2* e1a = reinterpret_cast<int2*>(ws + p->ws.fxa);
+    int* e2max = reinterpret_cast<int*>(e1a + (size_t)3 * p->stage_rows * (p->M + 1));
+    int* e2 = e2max + (size_t)6 * p->stage_rows;
+    TC_TRY_STATUS(zinv_u(p, u, Rh, H1, e, s, r0, nh));   // Rhat is free until the forward z pass
+    int slot = prof_begin(p, kKZinvAdj, s);
+    TC_TRY_STATUS(run_z(p, ZPass{true, true, Nbar, nullptr, Ha, e1a, e2max, nullptr, {}, r0, nh, 1}, s));
+    prof_end(p, slot, s);
+    slot = prof_begin(p, kKThetaAdj, s);
+    const int zt = fx_zt_adj(p, p->theta_zt_forced);
+    ThetaAdjArgs a{H1, Ha, H3, e.e1, e1a, e2, e2max, p->d_fx_ir, p->d_fx_mm, p->d_fx_tw_t, r0, nh, p->M, p->P_z, zt, p->fx_emm,
+                   magic(zt), magic(p->P_t), (long long)p->m_p};
+    TC_TRY_STATUS(launch_fx_theta_adj(p, a, s));
+    prof_end(p, slot, s);
+    slot = prof_begin(p, kKZfwdAdj, s);
+    TC_TRY_STATUS(run_z(p, ZPass{false, true, nullptr, nullptr, H3, nullptr, e2max, e2, {ubar, Rh, 0, 0, 0}, r0, nh, zt}, s));
+    prof_end(p, slot, s);
+    return TC_OK;
+}
 
 // N(u) in FP64, slab by slab of p->stage_rows radial rows (a row's transforms read no other
 // row's staging)

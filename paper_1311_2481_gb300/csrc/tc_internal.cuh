@@ -59,6 +59,7 @@ struct Workspace {
     size_t H1a;     // recomputed forward lines of u: 9 line sets
     size_t Ha;      // adjoint lines of Nbar: 3 line sets
     size_t H3;      // adjoint theta-pass output: 9 line sets
+    size_t fxa;     // exponents of the adjoint's fixed-point lines (tc_fx_z.cu)
     size_t Rhat;    // adjoint d_r lines before the transposed stencil: 3 x stage_rows rows of modes
     size_t Nbar;    // adjoint of N: vector field
     size_t abar;    // start-up adjoint temporaries: 3 vector fields
@@ -213,10 +214,13 @@ void prof_end(tc_plan* p, int slot, cudaStream_t s);
 // ------------------------------------------------------------------ launchers
 tc_status launch_nonlinear_fx(tc_plan* p, const double2* u, double2* Nh, char* ws, cudaStream_t s);
 size_t fx_exp_bytes(const tc_plan* p);
+size_t fx_adj_exp_bytes(const tc_plan* p);
+int fx_zt_adj(const tc_plan* p, int forced);
+tc_status launch_adjoint_rows_fx(tc_plan* p, const double2* u, const double2* Nbar, double2* ubar, double2* Rh, char* ws,
+                                 cudaStream_t s, int r0, int nh);
 int fx_zt(const tc_plan* p, int forced);
 const int* fx_static_radices(int n);   // radices of the compile-time plan of length n, nullptr if none
 tc_status launch_nonlinear(tc_plan* p, const double2* u, double2* N, char* ws, cudaStream_t s);
-tc_status launch_zinv_fp64(tc_plan* p, const double2* u, double2* H1, cudaStream_t s, int r0, int nh);
 tc_status launch_theta32(tc_plan* p, const float2* H1, float2* H2, cudaStream_t s);
 int theta_s_zt(const tc_plan* p, bool fp64);
 tc_status launch_theta_s(tc_plan* p, const float2* H1, float2* H2, cudaStream_t s);

@@ -855,6 +855,7 @@ tc_status tc_plan_create_ex(tc_plan** out, int N_r, int M, int K, int m_p, doubl
         p->ws.H1a = take(9 * hst * cplx);
         p->ws.Ha = take(3 * hst * cplx);
         p->ws.H3 = take(9 * hst * cplx);
+        p->ws.fxa = take(fx_adj_exp_bytes(p));
         p->ws.Rhat = take(3 * (size_t)p->stage_rows * p->nmode * cplx);
         off = std::max(off, split_end);
         p->ws.Nbar = take(3 * p->S * cplx);   // written by the adjoint advance

@@ -111,3 +111,25 @@ def test_zero_and_mean_flow_only(tc):
     u = I.base_state(ops.r, 4, 6, 0.5, 100.0, 0.0)
     N, ref, _, _ = both(tc, 12, 4, 6, u=u)
     assert np.linalg.norm(N - ref) <= 1e-14 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("N_r,M,P_t,K,P_z,rows", [(11, 12, 36, 27, 81, 0), (10, 5, 16, 40, 243, 0), (10, 2, 6, 320, 972, 0),
+                                                  (10, 2, 6, 384, 1152, 4), (12, 40, 81, 4, 12, 5), (10, 4, 12, 2, 6, 0),
+                                                  (10, 24, 72, 6, 18, 3), (10, 96, 288, 4, 12, 0)])
+def test_adjoint_lengths(tc, N_r, M, P_t, K, P_z, rows):
+    """The transposed transforms at lengths with one z per block, odd tiles, one line per block
+    (P_z > 768) and run-time plans, against the oracle's adjoint step.  1e-11 as the other
+    adjoint tests ask: the oracle's own solves round at that level."""
+    cfg = dict(N_r=N_r, M=M, K=K, m_p=1, eta=0.5, Re_i=50.0, Re_o=0.0, L_z=LZ, dt=1e-3)
+    ops = O.Operators(O.Params(**cfg, P_theta=P_t, P_z=P_z))
+    u0 = I.initial_state(ops.r, M, K, 1, LZ, 0.5, 50.0, 0.0, kind="box", amp=1e-2)
+    st = O.State(u0, u0, u0, None, True)
+    y = [I.random_spectral((3,) + ops.prm.shape(), seed=s) for s in (1, 2, 3)]
+    ref = O.adjoint_step(ops, st, *y)
+    plan = tc.Plan(**cfg, P_theta=P_t, P_z=P_z, stage_rows=rows)
+    fwd = tc.State(plan, torch.from_numpy(u0))
+    fwd.started = True
+    bar = tc.StateBar(*[torch.from_numpy(v).cuda() for v in y])
+    plan.adjoint_step(fwd, bar)
+    for got, want in zip((bar.u, bar.u_prev, bar.N_prev), ref):
+        assert np.linalg.norm(got.cpu().numpy() - want) <= 1e-11 * np.linalg.norm(want)
