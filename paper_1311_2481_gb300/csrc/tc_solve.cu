@@ -827,6 +827,93 @@ __global__ void __launch_bounds__(256) k_update_mx(double2* u, double2* up, cons
 
 // x <- A^{-1} x for every mode of nfields consecutive fields (system sets set0, set0+1, ...):
 // thread (field, mode, part) runs the register-window substitution down its global column.
+// smem_band_solve on a column in global memory, in the same arithmetic: the right-hand side's
+// rows come in through the ring with the factors, D rows ahead.  Used while a launch has few
+// warps (launch_split_solve): there each row waited one memory latency.
+constexpr int kGD = 6;   // ring depth (2, 3, 4, 5, 6, 8: 325, 325, 290, 275, 267, 267 us for a Poisson solve, N_r = 256, M = 64, K = 128)
+template <int D>
+__device__ __forceinline__ void gmem_band_solve(double* __restrict__ x, size_t st, int N, const double* __restrict__ F,
+                                                const uint8_t* __restrict__ P, int M1K1) {
+    const size_t rs = (size_t)kBands * M1K1;
+    double w0 = x[0], w1 = N > 1 ? x[st] : 0.0, w2 = N > 2 ? x[2 * st] : 0.0, w3 = N > 3 ? x[3 * st] : 0.0,
+           w4 = N > 4 ? x[4 * st] : 0.0;
+    double lr[D][4], br[D];
+    int pr[D];
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+        pr[d] = d < N ? P[(size_t)d * M1K1] : 0;
+        br[d] = d + 5 < N ? x[(size_t)(d + 5) * st] : 0.0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) lr[d][q] = d < N ? __ldg(&F[(size_t)d * rs + (size_t)q * M1K1]) : 0.0;
+    }
+    for (int j0 = 0; j0 < N; j0 += D) {
+#pragma unroll
+        for (int d = 0; d < D; ++d) {
+            const int j = j0 + d;
+            if (j < N) {
+                const int pj = pr[d];
+                const double l1 = lr[d][0], l2 = lr[d][1], l3 = lr[d][2], l4 = lr[d][3], b = br[d];
+                if (j + D < N) {
+                    const double* Fr = F + (size_t)(j + D) * rs;
+                    pr[d] = P[(size_t)(j + D) * M1K1];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) lr[d][q] = __ldg(&Fr[(size_t)q * M1K1]);
+                }
+                br[d] = j + D + 5 < N ? x[(size_t)(j + D + 5) * st] : 0.0;
+                if (pj == 1) { double q = w0; w0 = w1; w1 = q; }
+                else if (pj == 2) { double q = w0; w0 = w2; w2 = q; }
+                else if (pj == 3) { double q = w0; w0 = w3; w3 = q; }
+                else if (pj == 4) { double q = w0; w0 = w4; w4 = q; }
+                x[(size_t)j * st] = w0;
+                w1 = fma(-l1, w0, w1);
+                w2 = fma(-l2, w0, w2);
+                w3 = fma(-l3, w0, w3);
+                w4 = fma(-l4, w0, w4);
+                w0 = w1; w1 = w2; w2 = w3; w3 = w4;
+                w4 = b;
+            }
+        }
+    }
+    double v1 = 0.0, v2 = 0.0, v3 = 0.0, v4 = 0.0, v5 = 0.0, v6 = 0.0, v7 = 0.0, v8 = 0.0;
+    double ur[D][9];
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+        const int j = N - 1 - d;
+        br[d] = j >= 0 ? x[(size_t)j * st] : 0.0;
+#pragma unroll
+        for (int q = 0; q < 9; ++q) ur[d][q] = j >= 0 ? __ldg(&F[(size_t)j * rs + (size_t)(4 + q) * M1K1]) : 0.0;
+    }
+    for (int j0 = N - 1; j0 >= 0; j0 -= D) {
+#pragma unroll
+        for (int d = 0; d < D; ++d) {
+            const int j = j0 - d;
+            if (j >= 0) {
+                double uc[9];
+#pragma unroll
+                for (int q = 0; q < 9; ++q) uc[q] = ur[d][q];
+                double s = br[d];
+                if (j - D >= 0) {
+                    br[d] = x[(size_t)(j - D) * st];
+#pragma unroll
+                    for (int q = 0; q < 9; ++q) ur[d][q] = __ldg(&F[(size_t)(j - D) * rs + (size_t)(4 + q) * M1K1]);
+                }
+                s = fma(-uc[8], v8, s);
+                s = fma(-uc[7], v7, s);
+                s = fma(-uc[6], v6, s);
+                s = fma(-uc[5], v5, s);
+                s = fma(-uc[4], v4, s);
+                s = fma(-uc[3], v3, s);
+                s = fma(-uc[2], v2, s);
+                s = fma(-uc[1], v1, s);
+                const double xj = s * uc[0];
+                x[(size_t)j * st] = xj;
+                v8 = v7; v7 = v6; v6 = v5; v5 = v4; v4 = v3; v3 = v2; v2 = v1; v1 = xj;
+            }
+        }
+    }
+}
+
+template <int D>
 __global__ void k_band_solve_g(double2* __restrict__ x, const double* __restrict__ fac,
                                const uint8_t* __restrict__ piv, int set0, int nfields, Geo g) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;   // (mode, part); y = field
@@ -839,12 +926,28 @@ __global__ void k_band_solve_g(double2* __restrict__ x, const double* __restrict
     const size_t mk = (size_t)m * g.K1 + (k < 0 ? -k : k);
     const size_t per_set = (size_t)g.N * kBands * g.M1K1;
     const int set = set0 + fld;
-    smem_band_solve(x + (size_t)fld * g.S, g.nmode, mode, part, g.N, fac + (size_t)set * per_set + mk,
-                    piv + (size_t)set * g.N * g.M1K1 + mk, g.M1K1);
+    const double* F = fac + (size_t)set * per_set + mk;
+    const uint8_t* P = piv + (size_t)set * g.N * g.M1K1 + mk;
+    if (D > 1) gmem_band_solve<D>(reinterpret_cast<double*>(x + (size_t)fld * g.S + mode) + part, (size_t)2 * g.nmode, g.N, F, P, g.M1K1);
+    else smem_band_solve(x + (size_t)fld * g.S, g.nmode, mode, part, g.N, F, P, g.M1K1);
 }
 
 // Stand-alone solve of one system set for all modes (tc_helmholtz_solve): columns staged in
 // shared memory, real and imaginary parts by separate threads.
+// One system for every mode in two partitions, T modes per block (as in k_pc's solve phases).
+__global__ void __launch_bounds__(128) k_band_solve_s2(double2* __restrict__ x, PCArgs a, int set, Geo g, int T) {
+    extern __shared__ double2 sm[];
+    const int N = g.N, mode0 = blockIdx.x * T, nT = min(T, g.nmode - mode0), t = threadIdx.x % T;
+    for (int j = threadIdx.x / T; j < N; j += blockDim.x / T)
+        sm[j * T + t] = t < nT ? x[(size_t)j * g.nmode + mode0 + t] : make_double2(0.0, 0.0);
+    __syncthreads();
+    if (threadIdx.x < 4 * nT) half_solve(a, g, sm, set, T, nT, mode0, threadIdx.x);
+    __syncthreads();
+    spike_combine(a, g, sm, 1, set, T, nT, mode0, reinterpret_cast<double*>(sm + (size_t)N * T));
+    if (t < nT)
+        for (int j = threadIdx.x / T; j < N; j += blockDim.x / T) x[(size_t)j * g.nmode + mode0 + t] = sm[j * T + t];
+}
+
 __global__ void __launch_bounds__(256) k_band_solve_s(double2* __restrict__ x, const double* __restrict__ fac,
                                                       const uint8_t* __restrict__ piv, int set, Geo g, int T) {
     extern __shared__ double2 sm[];
@@ -985,6 +1088,22 @@ static int pc_modes(const tc_plan* p, int nmode) {
 
 tc_status launch_solve(tc_plan* p, int set, double2* x, int nfields, cudaStream_t s) {
     Geo g = geo(p);
+    if (p->part_h > 0) {
+        // two partitions: half the chain of substitutions, which bounds this launch
+        g.sh = p->part_h;
+        PCArgs a{};
+        a.fac2 = p->d_fac2; a.piv2 = p->d_piv2; a.spk = p->d_spk; a.rinv = p->d_rinv;
+        const int T = 16;
+        const size_t sm = (size_t)p->N_r * T * sizeof(double2) + (size_t)T * 16 * sizeof(double);
+        TC_CUDA(p, cudaFuncSetAttribute(k_band_solve_s2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        for (int f = 0; f < nfields; ++f) {
+            const int slot = prof_begin(p, set == kSetP ? kKSolveP : kKSolveH, s);
+            k_band_solve_s2<<<blocks_for(g.nmode, T), 128, sm, s>>>(x + (size_t)f * g.S, a, set + f, g, T);
+            prof_end(p, slot, s);
+            TC_LAUNCHED(p, "k_band_solve_s2");
+        }
+        return TC_OK;
+    }
     int T = 32;
     while (T > 1 && (size_t)p->N_r * T * sizeof(double2) > 96 * 1024) T /= 2;
     const size_t sm = (size_t)p->N_r * T * sizeof(double2);
@@ -1009,7 +1128,14 @@ static tc_status launch_advance_split(tc_plan* p, const double2* u, double2* u_p
     double2* us = reinterpret_cast<double2*>(ws + p->ws.ustar);
     double2* phi = reinterpret_cast<double2*>(ws + p->ws.phi);   // also holds X before phi
     const dim3 g1(g.N, blocks_for(nm, 128));
-    auto sgrid = [&](int nf) { return dim3(blocks_for((size_t)2 * nm, 128), nf); };
+    // nf substitutions with the factor sets set ..: the ring while a launch has fewer than 24 warps
+    // per SM (20.6 warps: 680 against 706 us), the plain one beyond, where other warps cover the
+    // latency and 40 registers more per thread do not pay (27 warps: 793 against 1008 us)
+    auto split_solve = [&](double2* x, int set, int nf) {
+        const dim3 grid(blocks_for((size_t)2 * nm, 128), nf);
+        const bool ring = (size_t)2 * nm * nf < (size_t)24 * 32 * p->num_sms;
+        (ring ? k_band_solve_g<kGD> : k_band_solve_g<1>)<<<grid, 128, 0, s>>>(x, p->d_fac, p->d_piv, set, nf, g);
+    };
     // mixed form: the radial stencils in double-FP32 (the *_mx kernels), tiles of 32 x 32
     const bool mx = p->precision == TC_MIXED;
     const dim3 gx(blocks_for(nm, kXsM), blocks_for(g.N, kXsR)), bx(kXsM, 8);
@@ -1026,7 +1152,7 @@ static tc_status launch_advance_split(tc_plan* p, const double2* u, double2* u_p
     prof_end(p, slot, s);
     TC_LAUNCHED(p, "k_rhs_pressure");
     slot = prof_begin(p, kKSolveP, s);
-    k_band_solve_g<<<sgrid(1), 128, 0, s>>>(ps, p->d_fac, p->d_piv, kSetP, 1, g);
+    split_solve(ps, kSetP, 1);
     prof_end(p, slot, s);
     TC_LAUNCHED(p, "k_band_solve_g");
     slot = prof_begin(p, kKRhsVelocity, s);
@@ -1039,7 +1165,7 @@ static tc_status launch_advance_split(tc_plan* p, const double2* u, double2* u_p
     prof_end(p, slot, s);
     TC_LAUNCHED(p, "k_rhs_velocity");
     slot = prof_begin(p, kKSolveH, s);
-    k_band_solve_g<<<sgrid(3), 128, 0, s>>>(us, p->d_fac, p->d_piv, kSetHp, 3, g);
+    split_solve(us, kSetHp, 3);
     prof_end(p, slot, s);
     TC_LAUNCHED(p, "k_band_solve_g");
     slot = prof_begin(p, kKRhsDiv, s);
@@ -1050,7 +1176,7 @@ static tc_status launch_advance_split(tc_plan* p, const double2* u, double2* u_p
     prof_end(p, slot, s);
     TC_LAUNCHED(p, "k_rhs_div");
     slot = prof_begin(p, kKSolveP, s);
-    k_band_solve_g<<<sgrid(1), 128, 0, s>>>(phi, p->d_fac, p->d_piv, kSetP, 1, g);
+    split_solve(phi, kSetP, 1);
     prof_end(p, slot, s);
     TC_LAUNCHED(p, "k_band_solve_g");
     slot = prof_begin(p, kKUpdate, s);
