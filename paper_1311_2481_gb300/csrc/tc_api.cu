@@ -72,12 +72,10 @@ tc_status tc_helmholtz_solve(tc_plan* plan, int which, const void* rhs, void* x,
     TC_TRY(check_device_ptr(plan, rhs, "rhs", plan->S * sizeof(double2)));
     TC_TRY(check_device_ptr(plan, x, "x", plan->S * sizeof(double2)));
     TC_TRY(check_ws(plan, ws));
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (rhs != x)
-        TC_CUDA(plan, cudaMemcpyAsync(x, rhs, plan->S * sizeof(double2), cudaMemcpyDeviceToDevice, s));
     const int set = (which == TC_P_STAR || which == TC_PHI) ? kSetP
                   : which == TC_U_PLUS ? kSetHp : which == TC_U_MINUS ? kSetHm : kSetHz;
-    return launch_solve(plan, set, static_cast<double2*>(x), 1, s);
+    return launch_solve(plan, set, static_cast<const double2*>(rhs), static_cast<double2*>(x),
+                        static_cast<cudaStream_t>(stream));
 }
 
 tc_status tc_step(tc_plan* plan, tc_state* st, int nsteps, void* ws, void* stream) {

@@ -230,7 +230,7 @@ tc_status launch_nl_post32(tc_plan* p, const double2* u, double2* N, char* ws, c
 size_t mean00_part_doubles(const tc_plan* p);
 tc_status launch_mean00_part(tc_plan* p, const double2* u, char* ws, cudaStream_t s);
 tc_status launch_mean00_fin(tc_plan* p, double2* N, char* ws, cudaStream_t s);
-tc_status launch_solve(tc_plan* p, int set, double2* x, int nfields, cudaStream_t s);
+tc_status launch_solve(tc_plan* p, int set, const double2* rhs, double2* x, cudaStream_t s);
 tc_status launch_advance(tc_plan* p, const double2* u, double2* u_prev, const double2* Ncur,
                          double2* N_prev, double2* p_out, double2* u_out, char* ws,
                          bool commit, cudaStream_t s, int ma = 0, int mb = -1);

@@ -935,11 +935,12 @@ __global__ void k_band_solve_g(double2* __restrict__ x, const double* __restrict
 // Stand-alone solve of one system set for all modes (tc_helmholtz_solve): columns staged in
 // shared memory, real and imaginary parts by separate threads.
 // One system for every mode in two partitions, T modes per block (as in k_pc's solve phases).
-__global__ void __launch_bounds__(128) k_band_solve_s2(double2* __restrict__ x, PCArgs a, int set, Geo g, int T) {
+// rhs may be x: a block reads its columns before it writes them.
+__global__ void __launch_bounds__(128) k_band_solve_s2(const double2* rhs, double2* x, PCArgs a, int set, Geo g, int T) {
     extern __shared__ double2 sm[];
     const int N = g.N, mode0 = blockIdx.x * T, nT = min(T, g.nmode - mode0), t = threadIdx.x % T;
     for (int j = threadIdx.x / T; j < N; j += blockDim.x / T)
-        sm[j * T + t] = t < nT ? x[(size_t)j * g.nmode + mode0 + t] : make_double2(0.0, 0.0);
+        sm[j * T + t] = t < nT ? rhs[(size_t)j * g.nmode + mode0 + t] : make_double2(0.0, 0.0);
     __syncthreads();
     if (threadIdx.x < 4 * nT) half_solve(a, g, sm, set, T, nT, mode0, threadIdx.x);
     __syncthreads();
@@ -948,7 +949,7 @@ __global__ void __launch_bounds__(128) k_band_solve_s2(double2* __restrict__ x, 
         for (int j = threadIdx.x / T; j < N; j += blockDim.x / T) x[(size_t)j * g.nmode + mode0 + t] = sm[j * T + t];
 }
 
-__global__ void __launch_bounds__(256) k_band_solve_s(double2* __restrict__ x, const double* __restrict__ fac,
+__global__ void __launch_bounds__(256) k_band_solve_s(const double2* rhs, double2* x, const double* __restrict__ fac,
                                                       const uint8_t* __restrict__ piv, int set, Geo g, int T) {
     extern __shared__ double2 sm[];
     const int N = g.N;
@@ -956,7 +957,7 @@ __global__ void __launch_bounds__(256) k_band_solve_s(double2* __restrict__ x, c
     const int nT = min(T, g.mhi - mode0);
     for (int idx = threadIdx.x; idx < N * T; idx += blockDim.x) {
         const int j = idx / T, t = idx - (idx / T) * T;
-        sm[idx] = t < nT ? x[(size_t)j * g.nmode + mode0 + t] : make_double2(0.0, 0.0);
+        sm[idx] = t < nT ? rhs[(size_t)j * g.nmode + mode0 + t] : make_double2(0.0, 0.0);
     }
     __syncthreads();
     if (threadIdx.x < 2 * nT) {
@@ -1086,8 +1087,10 @@ static int pc_modes(const tc_plan* p, int nmode) {
     return T;
 }
 
-tc_status launch_solve(tc_plan* p, int set, double2* x, int nfields, cudaStream_t s) {
+// x = A^{-1} rhs of the factor set for every mode (rhs may be x)
+tc_status launch_solve(tc_plan* p, int set, const double2* rhs, double2* x, cudaStream_t s) {
     Geo g = geo(p);
+    const int prof = set == kSetP ? kKSolveP : kKSolveH;
     if (p->part_h > 0) {
         // two partitions: half the chain of substitutions, which bounds this launch
         g.sh = p->part_h;
@@ -1096,24 +1099,20 @@ tc_status launch_solve(tc_plan* p, int set, double2* x, int nfields, cudaStream_
         const int T = 16;
         const size_t sm = (size_t)p->N_r * T * sizeof(double2) + (size_t)T * 16 * sizeof(double);
         TC_CUDA(p, cudaFuncSetAttribute(k_band_solve_s2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-        for (int f = 0; f < nfields; ++f) {
-            const int slot = prof_begin(p, set == kSetP ? kKSolveP : kKSolveH, s);
-            k_band_solve_s2<<<blocks_for(g.nmode, T), 128, sm, s>>>(x + (size_t)f * g.S, a, set + f, g, T);
-            prof_end(p, slot, s);
-            TC_LAUNCHED(p, "k_band_solve_s2");
-        }
+        const int slot = prof_begin(p, prof, s);
+        k_band_solve_s2<<<blocks_for(g.nmode, T), 128, sm, s>>>(rhs, x, a, set, g, T);
+        prof_end(p, slot, s);
+        TC_LAUNCHED(p, "k_band_solve_s2");
         return TC_OK;
     }
     int T = 32;
     while (T > 1 && (size_t)p->N_r * T * sizeof(double2) > 96 * 1024) T /= 2;
     const size_t sm = (size_t)p->N_r * T * sizeof(double2);
     TC_CUDA(p, cudaFuncSetAttribute(k_band_solve_s, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    for (int f = 0; f < nfields; ++f) {
-        const int slot = prof_begin(p, set == kSetP ? kKSolveP : kKSolveH, s);
-        k_band_solve_s<<<blocks_for(g.nmode, T), 64, sm, s>>>(x + (size_t)f * g.S, p->d_fac, p->d_piv, set + f, g, T);
-        prof_end(p, slot, s);
-        TC_LAUNCHED(p, "k_band_solve_s");
-    }
+    const int slot = prof_begin(p, prof, s);
+    k_band_solve_s<<<blocks_for(g.nmode, T), 64, sm, s>>>(rhs, x, p->d_fac, p->d_piv, set, g, T);
+    prof_end(p, slot, s);
+    TC_LAUNCHED(p, "k_band_solve_s");
     return TC_OK;
 }
 
