@@ -439,5 +439,73 @@ __device__ __forceinline__ double to_double(long long X, int s) {
     return __longlong_as_double((long long)(b | (X < 0 ? 0x8000000000000000ull : 0ull)));
 }
 __device__ __forceinline__ double nan64() { return __longlong_as_double(0x7ff8000000000000ll); }
+
+// ---------------------------------------------------------------- radial stencils
+// The window of R consecutive rows j0 .. j0 + R - 1 of a real column: rows j0 - 4 .. j0 + R + 3,
+// converted once to the exponent of the largest, |x| < 2^57 so that nine products fit 64 bits.
+// An output then costs 27 32-bit multiply-adds instead of 9 FP64 FMAs of 64 issue cycles per
+// warp, plus (R + 8) / R conversions.  The low limbs' products that are left out amount to
+// 2^-57 of max |f| sum |w|: where a row's own stencil reaches only values 2^4 or more below the
+// window's largest (far), and in the four rows next to each wall, whose stencils are shorter and
+// whose values fall off towards the wall, the row is left to the FP64 sum (stencil_fp64), as it
+// is next to a NaN or an Inf and near the smallest numbers.
+constexpr int kFar = 3, kLowExp = 70;
+// fix() for emax > kLowExp, where zeros and subnormals are shifted out like all that is small
+__device__ __forceinline__ long long fix_tile(double d, int emax) {
+    const int h = __double2hiint(d);
+    const unsigned mh = ((unsigned)h & 0xfffffu) | 0x100000u, ml = (unsigned)__double2loint(d);
+    unsigned long long m = ((unsigned long long)((mh << 9) | (ml >> 23)) << 32) | (ml << 9);
+    asm("shr.u64 %0, %0, %1;" : "+l"(m) : "r"(emax - ((h >> 20) & 0x7ff)));
+    return h < 0 ? -(long long)m : (long long)m;
+}
+template <int R> struct Tile {
+    lim x[R + 8];
+    int e, own[R];   // exponents of the window and of each row's stencil
+    __device__ __forceinline__ bool far(int i) const { return e >= 2047 || e <= kLowExp || e - own[i] > kFar; }
+    // weights w[9] and their exponent ew of the row j0 + i
+    __device__ __forceinline__ double row(int i, const int2* __restrict__ w, int ew) const {
+        long long m = 0, s = 0;
+#pragma unroll
+        for (int t = 0; t < kStencil; ++t) {
+            const int2 v = __ldg(&w[t]);
+            m = mad(x[i + t].h, v.y, mad(x[i + t].l, v.x, m));
+            s = mad(x[i + t].h, v.x, s);
+        }
+        return to_double(take(s + (m >> 32), m, 25), e + ew - 1084);
+    }
+    // exponents of the entries 0 .. R + 7: every row's stencil holds the entries R - 1 .. 8
+    __device__ __forceinline__ void exponents(const int (&b)[R + 8]) {
+        static_assert(R <= 9, "the rows' stencils share an entry");
+        int lo[R], hi[R];
+        int c = 0;
+#pragma unroll
+        for (int i = R - 1; i <= 8; ++i) c = max(c, b[i]);
+        lo[R - 1] = hi[0] = c;
+#pragma unroll
+        for (int i = R - 2; i >= 0; --i) lo[i] = max(lo[i + 1], b[i]);
+#pragma unroll
+        for (int i = 1; i < R; ++i) hi[i] = max(hi[i - 1], b[i + 8]);
+        e = max(lo[0], hi[R - 1]);
+#pragma unroll
+        for (int i = 0; i < R; ++i) own[i] = max(lo[i], hi[i]);
+    }
+    __device__ __forceinline__ void load(const double (&d)[R + 8]) {
+        int b[R + 8];
+#pragma unroll
+        for (int i = 0; i < R + 8; ++i) b[i] = bexp(d[i]);
+        exponents(b);
+#pragma unroll
+        for (int i = 0; i < R + 8; ++i) x[i] = split(fix_tile(d[i], e + 5));
+    }
+    // the window of a + d, added after the conversion (one exponent more)
+    __device__ __forceinline__ void load(const double (&a)[R + 8], const double (&d)[R + 8]) {
+        int b[R + 8];
+#pragma unroll
+        for (int i = 0; i < R + 8; ++i) b[i] = max(bexp(a[i]), bexp(d[i])) + 1;
+        exponents(b);
+#pragma unroll
+        for (int i = 0; i < R + 8; ++i) x[i] = split(fix_tile(a[i], e + 5) + fix_tile(d[i], e + 5));
+    }
+};
 }  // namespace fx
 }  // namespace tc

@@ -28,7 +28,7 @@ using namespace fx;
 
 namespace {
 
-constexpr int kDrRows = 8;      // rows per thread of k_fx_dr (its exponents assume 8)
+constexpr int kDrRows = 8;      // rows per thread of k_fx_dr
 constexpr int kZThreads = 512;  // most threads of a transform block (128 registers each)
 
 // exponent arrays of nh staged rows, in the fxe region: e1[9][nh][M+1] (exponent, largest
@@ -40,13 +40,9 @@ struct Exps {
 };
 
 // ---------------------------------------------------------------- radial derivative
-// Rows j0 .. j0 + 7 of the real or imaginary part of one column per thread: 16 rows are
-// converted once to the exponent of the largest, each output is 27 32-bit multiply-adds
-// instead of 9 FP64 FMAs of 64 issue cycles each.  The products' low limbs that are left out
-// amount to 2^-57 of max |u| sum |w|.  Where a row's own stencil reaches only values 2^4 or
-// more below that maximum, and in the four rows next to each wall, whose stencils are shorter
-// (u falls off towards the wall), the row is taken in FP64.  Tiles start at multiples of kDrRows whatever r0, so that
-// a row's result does not depend on the slab it is staged in.
+// Rows j0 .. j0 + 7 of the real or imaginary part of one column per thread (fx::Tile).  Tiles
+// start at multiples of kDrRows whatever r0, so that a row's result does not depend on the slab
+// it is staged in.
 __global__ void __launch_bounds__(128) k_fx_dr(const double* __restrict__ u, double* __restrict__ du,
                                                const int2* __restrict__ w, const int* __restrict__ ew,
                                                const double* __restrict__ w1, const int* __restrict__ col0, int N,
@@ -61,24 +57,15 @@ __global__ void __launch_bounds__(128) k_fx_dr(const double* __restrict__ u, dou
         const int j = j0 - 4 + i;
         d[i] = j >= 0 && j < N ? __ldg(&src[(size_t)j * ncol]) : 0.0;
     }
-    // lo[i], hi[i]: largest exponents of entries i .. 6 and 9 .. i + 8; every stencil holds 7 and 8
-    int lo[kDrRows], hi[kDrRows];
-    lo[7] = hi[0] = max(bexp(d[7]), bexp(d[8]));
-#pragma unroll
-    for (int i = 6; i >= 0; --i) lo[i] = max(lo[i + 1], bexp(d[i]));
-#pragma unroll
-    for (int i = 1; i < kDrRows; ++i) hi[i] = max(hi[i - 1], bexp(d[i + 8]));
-    const int e = max(lo[0], hi[kDrRows - 1]);
-    lim x[kDrRows + 8];
-#pragma unroll
-    for (int i = 0; i < kDrRows + 8; ++i) x[i] = split(fix(d[i], e + 5));   // |x| < 2^57: nine products fit 64 bits
+    Tile<kDrRows> x;
+    x.load(d);
 #pragma unroll
     for (int i = 0; i < kDrRows; ++i) {
         const int j = j0 + i;
         if (tile + i >= nh) break;
         if (tile + i < 0) continue;
         double o = 0.0;
-        if (j < 4 || j > N - 5 || e - max(lo[i], hi[i]) > 3) {
+        if (j < 4 || j > N - 5 || x.far(i)) {
             const int c0 = __ldg(&col0[j]);
             double v[kStencil];   // rows outside [0, N) (N < 9) have weight 0
 #pragma unroll
@@ -86,14 +73,7 @@ __global__ void __launch_bounds__(128) k_fx_dr(const double* __restrict__ u, dou
 #pragma unroll
             for (int t = 0; t < kStencil; ++t) o = fma(__ldg(&w1[j * kStencil + t]), v[t], o);
         } else {
-            long long m = 0, s = 0;
-#pragma unroll
-            for (int t = 0; t < kStencil; ++t) {
-                const int2 v = __ldg(&w[j * kStencil + t]);
-                m = mad(x[i + t].h, v.y, mad(x[i + t].l, v.x, m));
-                s = mad(x[i + t].h, v.x, s);
-            }
-            o = e == 2047 ? nan64() : to_double(take(s + (m >> 32), m, 25), e + __ldg(&ew[j]) - 1084);
+            o = x.row(i, w + j * kStencil, __ldg(&ew[j]));
         }
         du[((size_t)c * nh + tile + i) * ncol + col] = o;
     }

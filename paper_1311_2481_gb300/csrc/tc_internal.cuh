@@ -174,8 +174,9 @@ template <typename V> __host__ __device__ __forceinline__ V cmuli(V a) { V c; c.
 
 // true if either part of v is a NaN or an Inf: exponent bits all set (integer test, no FP64
 // instruction)
+__device__ __forceinline__ bool nonfinite1(double v) { return (__double2hiint(v) & 0x7ff00000) == 0x7ff00000; }
 __device__ __forceinline__ bool nonfinite2(double2 v) {
-    return ((__double2hiint(v.x) & 0x7ff00000) == 0x7ff00000) | ((__double2hiint(v.y) & 0x7ff00000) == 0x7ff00000);
+    return nonfinite1(v.x) | nonfinite1(v.y);
 }
 
 // ------------------------------------------------------------------ error helpers

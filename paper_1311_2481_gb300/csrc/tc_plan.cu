@@ -541,14 +541,19 @@ static tc_status upload(tc_plan* p) {
         for (int m = 0; m <= p->M; ++m) fx_limbs(std::ldexp((long double)m * p->m_p, -p->fx_emm), mm[m].x, mm[m].y);
         TC_CUDA(p, put((void**)&p->d_fx_mm, mm.data(), mm.size() * sizeof(int2)));
         std::vector<int4> fir(p->N_r);
-        std::vector<int2> w(p->w1.size(), make_int2(0, 0));
-        std::vector<int> ew(p->N_r);
         for (int j = 0; j < p->N_r; ++j) {
             int e;
             const double x = std::frexp(1.0 / p->r[j], &e);
             fx_limbs(x, fir[j].x, fir[j].y);
             fir[j].z = e;
             fir[j].w = 0;
+        }
+        TC_CUDA(p, put((void**)&p->d_fx_ir, fir.data(), fir.size() * sizeof(int4)));
+    }
+    {   // fixed-point weights of the radial stencils
+        std::vector<int2> w(p->w1.size(), make_int2(0, 0));
+        std::vector<int> ew(p->N_r);
+        for (int j = 0; j < p->N_r; ++j) {
             long double sum = 0;
             for (int t = 0; t < kStencil; ++t) sum += std::fabs((long double)p->w1[(size_t)j * kStencil + t]);
             std::frexp((double)sum * (1 + 1e-9), &ew[j]);
@@ -560,7 +565,6 @@ static tc_status upload(tc_plan* p) {
                     fx_limbs(std::ldexp((long double)v, -ew[j]), w[(size_t)j * kStencil + c].x, w[(size_t)j * kStencil + c].y);
             }
         }
-        TC_CUDA(p, put((void**)&p->d_fx_ir, fir.data(), fir.size() * sizeof(int4)));
         TC_CUDA(p, put((void**)&p->d_fx_w1, w.data(), w.size() * sizeof(int2)));
         TC_CUDA(p, put((void**)&p->d_fx_ew, ew.data(), ew.size() * sizeof(int)));
     }

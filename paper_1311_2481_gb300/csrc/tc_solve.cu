@@ -16,7 +16,7 @@
 
 #include "tc_internal.cuh"
 #include "tc_solve_core.cuh"
-#include "tc_split.cuh"
+#include "tc_fx.cuh"
 
 namespace tc {
 
@@ -29,11 +29,12 @@ struct PCArgs {
     double2* up_out;    // commit: u_prev <- u^i
     double2* Np_out;    // commit: N_prev <- N^i
     double2* p;         // commit: p <- p^{i+1}
-    const double* rn;
     const double* ir;   // 1 / r_j
     const double* w1;
     const double* w2;
     const int* col0;
+    const int2* fw;       // fixed-point stencil weights and their exponents
+    const int* few;
     const double* fac;
     const uint8_t* piv;
     const double* fac2;   // two-partition form (g.sh > 0): factors of the diagonal blocks,
@@ -44,6 +45,8 @@ struct PCArgs {
     double Re_i, Re_o;
     int commit;
 };
+
+constexpr int kChunkF = 4, kChunkB = 2;   // rows of factors per register chunk (3, 2: 2 % and 4, 3: 9 % slower k_pc)
 
 // Thread lt of the 4 nT threads of one system solves one half of it for one (mode, part):
 // threads [0, 2nT) rows [0, sh), threads [2nT, 4nT) rows [sh, N), each with the pivoted LU
@@ -57,7 +60,7 @@ __device__ __forceinline__ void half_solve(const PCArgs& a, const Geo& g, double
     const size_t mk = (size_t)m * g.K1 + (k < 0 ? -k : k);
     const size_t per_set = (size_t)g.N * kBands * g.M1K1;
     const int r0 = half ? g.sh : 0, n = half ? g.N - g.sh : g.sh;
-    smem_band_solve<kPCDepth>(X + (size_t)r0 * T, T, t, part, n,
+    smem_band_solve_c<kChunkF, kChunkB>(X + (size_t)r0 * T, T, t, part, n,
                               a.fac2 + (size_t)set * per_set + (size_t)r0 * kBands * g.M1K1 + mk,
                               a.piv2 + ((size_t)set * g.N + r0) * g.M1K1 + mk, g.M1K1);
 }
@@ -111,32 +114,83 @@ __device__ __forceinline__ void spike_combine(const PCArgs& a, const Geo& g, dou
     __syncthreads();
 }
 
-// Mixed form: the radial stencil sum_q w_q f_q over the 9 values v[q] of one complex column,
-// stored as exact FP32 pairs (hi re, hi im, lo re, lo im), with split weights w: a compensated
-// dot product (Ogita-Rump-Oishi), assembled in FP64.  The pairs carry 47 bits of each value,
-// so the error is about 2^-46 of sum |w_q f_q|.
-__device__ __forceinline__ double2 xs_stencil(const float4* v, int vstride, const float2* w) {
-    float sx = 0.f, cx = 0.f, sy = 0.f, cy = 0.f;
+// L_pm v (c = 0, 1 for +, -) at row j of component c of u: one half of lap_r
+__device__ __forceinline__ double2 lap_pm(const double2* __restrict__ u, const PCArgs& a, int c, int j, int mode, double mm,
+                                          double kk, const Geo& g) {
+    const double2* f = u + (size_t)c * g.S;
+    const double ir = a.ir[j], ir2 = ir * ir;
+    const double2 d1 = drow(f, a.w1, a.col0, j, g.nmode, mode);
+    const double2 d2 = drow(f, a.w2, a.col0, j, g.nmode, mode);
+    const double2 v = f[(size_t)j * g.nmode + mode];
+    const double diag = -mm * mm * ir2 - kk * kk - ir2 + (c == 0 ? -2.0 : 2.0) * mm * ir2;
+    return make_double2(d2.x + ir * d1.x + diag * v.x, d2.y + ir * d1.y + diag * v.y);
+}
+
+// The element loops of k_pc with a radial stencil: body(j, i, d, pre(j)) for the real and imaginary
+// parts of all rows of the block's modes, i the index of the part's double in the [N][T] arrays
+// in shared memory, d the radial derivative at row j of F (of F + F2).  pre: the body's load from
+// device memory, issued ahead of the stencil.
+// FX: rows 4 .. N - 5 in tiles of kTileRows rows per thread in fixed point, the four next to each
+// wall in FP64 one per thread, by the other half of the block first.  Otherwise all in FP64.
+// The FP64 pipe takes 16 cycles of its SM per warp instruction, and k_pc issues 5900 of them per
+// 16 modes of 64 rows with FP64 stencils, 4400 without: 252 -> 219 us at N_r = 64, M = 32, K = 64
+// (8 rows per tile: 230 us, fewer threads with work and more rows left to FP64).
+constexpr int kTileRows = 4;   // rows per thread, here and in the split path
+template <bool FX, bool PAIR, class Pre, class Body>
+__device__ __forceinline__ void stencil_rows(const PCArgs& a, const double2* F, const double2* F2, int N, int T, Pre pre,
+                                             Body body) {
+    using namespace fx;
+    const int c = threadIdx.x % (2 * T), step = blockDim.x / (2 * T), st = 2 * T;
+    const double* f = reinterpret_cast<const double*>(F) + c;
+    const double* f2 = reinterpret_cast<const double*>(F2) + c;
+    auto fp64 = [&](int j, int c0) {
+        double o = 0.0;
 #pragma unroll
-    for (int q = 0; q < kStencil; ++q) {
-        const float4 f = v[q * vstride];
-        xs::dot_acc(sx, cx, w[q].x, w[q].y, f.x, f.z);
-        xs::dot_acc(sy, cy, w[q].x, w[q].y, f.y, f.w);
+        for (int q = 0; q < kStencil; ++q) {
+            const int n = (c0 + q) * st;
+            o = fma(__ldg(&a.w1[j * kStencil + q]), PAIR ? f[n] + f2[n] : f[n], o);
+        }
+        return o;
+    };
+    if (FX) {
+        for (int j0 = 4 + kTileRows * (threadIdx.x / st); j0 < N - 4; j0 += kTileRows * step) {
+            double d[kTileRows], g[kTileRows];
+#pragma unroll
+            for (int i = 0; i < kTileRows; ++i) g[i] = pre(min(j0 + i, N - 1));
+            {
+                Tile<kTileRows> X;
+                double v[kTileRows + 8], v2[kTileRows + 8];
+#pragma unroll
+                for (int i = 0; i < kTileRows + 8; ++i) {
+                    const int j = j0 - 4 + i;
+                    v[i] = j < N ? f[j * st] : 0.0;
+                    if (PAIR) v2[i] = j < N ? f2[j * st] : 0.0;
+                }
+                if (PAIR) X.load(v, v2);
+                else X.load(v);
+#pragma unroll
+                for (int i = 0; i < kTileRows; ++i) {
+                    const int j = min(j0 + i, N - 5);
+                    d[i] = X.far(i) ? fp64(j, j - 4) : X.row(i, a.fw + j * kStencil, __ldg(&a.few[j]));
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < kTileRows; ++i)
+                if (j0 + i < N - 4) body(j0 + i, (j0 + i) * st + c, d[i], g[i]);
+        }
     }
-    return make_double2(xs::f2d_bits(sx) + xs::f2d_bits(cx), xs::f2d_bits(sy) + xs::f2d_bits(cy));
+    const int nw = FX ? min(N, 8) : N;   // FX: rows 0 .. 3 and N - 4 .. N - 1
+    for (int i = (threadIdx.x ^ (blockDim.x >> 1)) / st; i < nw; i += step) {
+        const int j = !FX || N < 8 || i < 4 ? i : N - 8 + i;
+        const double g = pre(j);
+        body(j, j * st + c, fp64(j, __ldg(&a.col0[j])), g);
+    }
 }
 
 // Steps 2-5 of Sec. 3.2 for the T modes of this block: pressure prediction (Eq. pressure
 // with the Neumann rows of Eq. ppBC), velocity prediction (Eq. vel), correction potential
 // (Eq. correction) and update (Eq. update).
-// MX (mixed form): the four radial stencils -- of X, p*, u*_+ + u*_- and phi -- in
-// double-FP32: the column is split once into exact FP32 pairs in shared memory (XS, with the
-// split weights SW), the stencil is a compensated dot product of the pairs (xs_stencil), the
-// result is assembled in FP64; the solves and everything else stay FP64.
-// The (0, 0) mode's stencils stay FP64 too (the mean flow, see the per-stage kernels): the
-// block that holds it computes that column's stencils in one pass, a row per thread, before
-// each phase (D00), so its warps do not diverge into FP64 stencils in the phase itself.
-template <int NTH, bool MX>
+template <int NTH, bool FX>
 __global__ void __launch_bounds__(NTH, 512 / NTH) k_pc(PCArgs a, Geo g, int T) {
     extern __shared__ double2 sm[];
     const int N = g.N;
@@ -145,45 +199,8 @@ __global__ void __launch_bounds__(NTH, 512 / NTH) k_pc(PCArgs a, Geo g, int T) {
     double2* C1 = sm + items;
     double2* C2 = C1 + items;
     double2* C3 = C2 + items;
-    float4* XS = reinterpret_cast<float4*>(C3 + items) + 3 * T * 16 / 2;   // after the spike scratch
-    float2* SW = reinterpret_cast<float2*>(XS + items);
-    double2* D00 = reinterpret_cast<double2*>(SW + ((N * kStencil + 1) & ~1));   // 16-byte aligned
     const int mode0 = g.mlo + blockIdx.x * T;
     const int nT = min(T, g.mhi - mode0);
-    // column of the (0, 0) mode in this block, or -1
-    const int t00 = (g.K >= mode0 && g.K < mode0 + nT) ? g.K - mode0 : -1;
-    if (MX) {
-        for (int i = threadIdx.x; i < N * kStencil; i += blockDim.x) SW[i] = xs::split_hl(a.w1[i]);
-    }
-    // XS <- split of the column(s) (F + F2), D00 <- the FP64 stencil of column t00, a barrier
-    auto split_cols = [&](const double2* F, const double2* F2) {
-        if (t00 >= 0) {
-            for (int j = threadIdx.x; j < N; j += blockDim.x) {
-                double2 d = sdrow(F, a.w1, a.col0, j, T, t00);
-                if (F2) {
-                    const double2 d2 = sdrow(F2, a.w1, a.col0, j, T, t00);
-                    d.x += d2.x;
-                    d.y += d2.y;
-                }
-                D00[j] = d;
-            }
-        }
-        for (int i = threadIdx.x; i < items; i += blockDim.x) {
-            double2 x = F[i];
-            if (F2) {
-                x.x += F2[i].x;
-                x.y += F2[i].y;
-            }
-            const float2 p = xs::split_hl(x.x), q = xs::split_hl(x.y);
-            XS[i] = make_float4(p.x, q.x, p.y, q.y);
-        }
-        __syncthreads();
-    };
-    // D1 of the split column at row j, mode t; the (0, 0) column's from D00
-    auto xsrow = [&](int j, int t) {
-        if (t == t00) return D00[j];
-        return xs_stencil(XS + a.col0[j] * T + t, T, SW + j * kStencil);
-    };
     const size_t per_set = (size_t)N * kBands * g.M1K1;
     const double c1 = g.c1;   // 1 / (2 dt)
     // T divides the block size, so every element a thread visits in the element loops below
@@ -197,62 +214,57 @@ __global__ void __launch_bounds__(NTH, 512 / NTH) k_pc(PCArgs a, Geo g, int T) {
     const int kq = modeq - mq * g.nk - g.K;
     const double mmq = g.mp * mq, kkq = g.kz * kq;
 
-    // A1: X = (2N - N_prev)_r into C1
+    const bool in = tq < nT;
+    double2* Lw = C3 + items;   // scratch of the spikes, free until then: L_pm u at the walls
+
+    // A1: (2N - N_prev)_+, _-, _z into C1, C2, C3; the halves of the wall Laplacians of u and
+    // u_prev, one (field, component, wall, mode) per thread
+#pragma unroll 2
     for (int j = threadIdx.x / T; j < N; j += jstep) {
-        const int idx = j * T + tq, t = tq;
-        double2 x = make_double2(0.0, 0.0);
-        if (t < nT) {
-            const size_t e = (size_t)j * g.nmode + mode0 + t;
-            const double2 n1 = a.Nc[e], n0 = a.Np[e], m1 = a.Nc[g.S + e], m0 = a.Np[g.S + e];
-            x.x = 0.5 * ((2.0 * n1.x - n0.x) + (2.0 * m1.x - m0.x));
-            x.y = 0.5 * ((2.0 * n1.y - n0.y) + (2.0 * m1.y - m0.y));
-        }
-        C1[idx] = x;
-        if (MX) {
-            const float2 p = xs::split_hl(x.x), q = xs::split_hl(x.y);
-            XS[idx] = make_float4(p.x, q.x, p.y, q.y);
-        }
-    }
-    __syncthreads();
-    if (MX && t00 >= 0) {   // the (0, 0) column's stencil of X in FP64
-        for (int j = threadIdx.x; j < N; j += blockDim.x) D00[j] = sdrow(C1, a.w1, a.col0, j, T, t00);
-        __syncthreads();
-    }
-    // A2: pressure right-hand side into C0
-    for (int j = threadIdx.x / T; j < N; j += jstep) {
-        const int idx = j * T + tq, t = tq;
-        double2 out = make_double2(0.0, 0.0);
-        if (t < nT) {
-            const int mode = modeq, m = mq, k = kq;
-            const double mm = mmq, kk = kkq;
-            const double r = a.rn[j], ir = a.ir[j];
-            const size_t e = (size_t)j * g.nmode + mode;
-            if (j == 0 || j == N - 1) {
-                if (!(j == N - 1 && m == 0 && k == 0)) {
-                    const double2 l0 = lap_r(a.u, a.w1, a.w2, a.col0, r, j, mode, mm, kk, g);
-                    const double2 l1 = lap_r(a.up, a.w1, a.w2, a.col0, r, j, mode, mm, kk, g);
-                    const double2 X = C1[idx];
-                    out.x = -X.x + 2.0 * l0.x - l1.x;
-                    out.y = -X.y + 2.0 * l0.y - l1.y;
-                }
-            } else {
-                const double2 d = MX ? xsrow(j, t) : sdrow(C1, a.w1, a.col0, j, T, t);
-                const double2 X = C1[idx];
-                const double2 n1 = a.Nc[e], n0 = a.Np[e], m1 = a.Nc[g.S + e], m0 = a.Np[g.S + e];
-                const double2 z1 = a.Nc[2 * g.S + e], z0 = a.Np[2 * g.S + e];
-                const double dpx = (2.0 * n1.x - n0.x) - (2.0 * m1.x - m0.x);
-                const double dpy = (2.0 * n1.y - n0.y) - (2.0 * m1.y - m0.y);
-                const double nzx = 2.0 * z1.x - z0.x, nzy = 2.0 * z1.y - z0.y;
-                out.x = -(d.x + X.x * ir + 0.5 * mm * ir * dpx - kk * nzy);
-                out.y = -(d.y + X.y * ir + 0.5 * mm * ir * dpy + kk * nzx);
+        const int idx = j * T + tq;
+        double2 n[3] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0), make_double2(0.0, 0.0)};
+        if (in) {
+            const size_t e = (size_t)j * g.nmode + modeq;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const double2 n1 = __ldg(&a.Nc[c * g.S + e]), n0 = __ldg(&a.Np[c * g.S + e]);
+                n[c] = make_double2(2.0 * n1.x - n0.x, 2.0 * n1.y - n0.y);
             }
         }
-        C0[idx] = out;
+        C1[idx] = n[0];
+        C2[idx] = n[1];
+        C3[idx] = n[2];
     }
+    for (int i = threadIdx.x / T; i < 8; i += jstep)
+        if (in) Lw[i * T + tq] = lap_pm(i & 4 ? a.up : a.u, a, i & 1, i & 2 ? N - 1 : 0, modeq, mmq, kkq, g);
+    __syncthreads();
+    // the columns as doubles; the mode and part of this thread in the stencil loops
+    double *D0 = reinterpret_cast<double*>(C0), *D1 = D0 + 2 * items, *D2 = D1 + 2 * items, *D3 = D2 + 2 * items;
+    const int ts = threadIdx.x % (2 * T) >> 1, part = threadIdx.x & 1, modes = mode0 + ts, ms = modes / g.nk;
+    const int ks = modes - ms * g.nk - g.K;
+    const bool ins = ts < nT;
+    const double mms = g.mp * ms, kks = (part ? 1 : -1) * (g.kz * ks);   // i k of the other part: kks times it
+    // A2: pressure right-hand side into C0
+    auto ir = [&](int j) { return __ldg(&a.ir[j]); };
+    stencil_rows<FX, true>(a, C1, C2, N, T, ir, [&](int j, int i, double d, double irj) {
+        double out = 0.0;
+        const double n = D1[i], m = D2[i];
+        if (j == 0 || j == N - 1) {
+            if (ins && !(j == N - 1 && ms == 0 && ks == 0)) {
+                const double* L = reinterpret_cast<const double*>(Lw + (j == 0 ? 0 : 2 * T) + ts) + part;
+                out = -0.5 * (n + m) + (L[0] + L[2 * T]) - 0.5 * (L[8 * T] + L[10 * T]);
+            }
+        } else {
+            const double hr = 0.5 * irj;
+            out = -(fma(mms * hr, n - m, fma(n + m, hr, 0.5 * d)) + kks * D3[i ^ 1]);
+        }
+        D0[i] = out;
+    });
     __syncthreads();
     // B: p* = P^{-1} b_p (real and imaginary parts by separate threads).  Meanwhile the
     // warps without a substitution precompute the part of the velocity right-hand sides that
-    // does not depend on p*: (4u - u_prev)/(2dt) - (2N - N_prev), and the Dirichlet rows.
+    // does not depend on p*, (4u - u_prev)/(2dt) - (2N - N_prev), in place of the latter, and the
+    // Dirichlet rows.
     // With two partitions (g.sh > 0) 4 nT threads solve, two per (mode, part).
     const bool sp = g.sh > 0;
     double* Xr = reinterpret_cast<double*>(C3 + items);
@@ -265,7 +277,7 @@ __global__ void __launch_bounds__(NTH, 512 / NTH) k_pc(PCArgs a, Geo g, int T) {
             const int t = threadIdx.x >> 1, part = threadIdx.x & 1;
             const int mode = mode0 + t, m = mode / g.nk, k = mode - m * g.nk - g.K;
             const size_t mk = (size_t)m * g.K1 + (k < 0 ? -k : k);
-            smem_band_solve<kPCDepth>(C0, T, t, part, N, a.fac + (size_t)kSetP * per_set + mk,
+            smem_band_solve_c<kChunkF, kChunkB>(C0, T, t, part, N, a.fac + (size_t)kSetP * per_set + mk,
                             a.piv + (size_t)kSetP * N * g.M1K1 + mk, g.M1K1);
         }
     }
@@ -275,24 +287,26 @@ __global__ void __launch_bounds__(NTH, 512 / NTH) k_pc(PCArgs a, Geo g, int T) {
     if (spare0 ? threadIdx.x >= helper0 : true) {
         const int first = spare0 ? helper0 : 0;   // a multiple of 32: (threadIdx.x - first) % T == tq
         for (int j = (threadIdx.x - first) / T; j < N; j += ((int)blockDim.x - first) / T) {
-            const int idx = j * T + tq, t = tq;
+            const int idx = j * T + tq;
             double2 o[3] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0), make_double2(0.0, 0.0)};
-            if (t < nT) {
-                const int mode = modeq, m = mq, k = kq;
+            if (in) {
                 if (j == 0 || j == N - 1) {
-                    if (m == 0 && k == 0) {
+                    if (mq == 0 && kq == 0) {
                         const double Re = j == 0 ? a.Re_i : a.Re_o;
                         o[0].y = Re;
                         o[1].y = -Re;
                     }
                 } else {
-                    const size_t e = (size_t)j * g.nmode + mode;
+                    const size_t e = (size_t)j * g.nmode + modeq;
+                    o[0] = C1[idx];
+                    o[1] = C2[idx];
+                    o[2] = C3[idx];
 #pragma unroll
                     for (int c = 0; c < 3; ++c) {
                         const size_t ec = (size_t)c * g.S + e;
-                        const double2 uu = a.u[ec], q = a.up[ec], n1 = a.Nc[ec], n0 = a.Np[ec];
-                        o[c].x = (4.0 * uu.x - q.x) * c1 - (2.0 * n1.x - n0.x);
-                        o[c].y = (4.0 * uu.y - q.y) * c1 - (2.0 * n1.y - n0.y);
+                        const double2 uu = a.u[ec], q = a.up[ec];
+                        o[c].x = (4.0 * uu.x - q.x) * c1 - o[c].x;
+                        o[c].y = (4.0 * uu.y - q.y) * c1 - o[c].y;
                     }
                 }
             }
@@ -303,22 +317,17 @@ __global__ void __launch_bounds__(NTH, 512 / NTH) k_pc(PCArgs a, Geo g, int T) {
     }
     __syncthreads();
     if (sp) spike_combine(a, g, C0, 1, kSetP, T, nT, mode0, Xr);
-    if (MX) split_cols(C0, nullptr);
     // C: velocity right-hand sides: subtract grad_h p* on interior rows; p <- p* (commit)
-    for (int j = threadIdx.x / T; j < N && tq < nT; j += jstep) {
-        const int idx = j * T + tq, t = tq;
-        const int mode = modeq;
-        const double2 pv = C0[idx];
-        if (a.commit) a.p[(size_t)j * g.nmode + mode] = pv;
-        if (j == 0 || j == N - 1) continue;
-        const double2 d = MX ? xsrow(j, t) : sdrow(C0, a.w1, a.col0, j, T, t);
-        const double tt = mmq * a.ir[j];
-        const double kk = kkq;
-        double2 v;
-        v = C1[idx]; v.x -= d.x - tt * pv.x; v.y -= d.y - tt * pv.y; C1[idx] = v;
-        v = C2[idx]; v.x -= d.x + tt * pv.x; v.y -= d.y + tt * pv.y; C2[idx] = v;
-        v = C3[idx]; v.x += kk * pv.y; v.y -= kk * pv.x; C3[idx] = v;
-    }
+    stencil_rows<FX, false>(a, C0, nullptr, N, T, ir, [&](int j, int i, double d, double irj) {
+        if (!ins) return;
+        const double pv = D0[i];
+        if (a.commit) reinterpret_cast<double*>(a.p)[2 * ((size_t)j * g.nmode + modes) + part] = pv;
+        if (j == 0 || j == N - 1) return;
+        const double tp = mms * irj * pv;
+        D1[i] -= d - tp;
+        D2[i] -= d + tp;
+        D3[i] -= kks * D0[i ^ 1];
+    });
     __syncthreads();
     // D: the three Helmholtz solves.  Meanwhile the other warps rotate the history (nothing
     // reads u_prev or N_prev after C): u_prev <- u^i, N_prev <- N^i (commit).
@@ -334,7 +343,7 @@ __global__ void __launch_bounds__(NTH, 512 / NTH) k_pc(PCArgs a, Geo g, int T) {
             const int mode = mode0 + t, m = mode / g.nk, k = mode - m * g.nk - g.K;
             const size_t mk = (size_t)m * g.K1 + (k < 0 ? -k : k);
             const int set = kSetHp + c;
-            smem_band_solve<kPCDepth>(C1 + (size_t)c * items, T, t, part, N, a.fac + (size_t)set * per_set + mk,
+            smem_band_solve_c<kChunkF, kChunkB>(C1 + (size_t)c * items, T, t, part, N, a.fac + (size_t)set * per_set + mk,
                             a.piv + (size_t)set * N * g.M1K1 + mk, g.M1K1);
         }
     } else if (a.commit && threadIdx.x >= helper1) {
@@ -360,25 +369,14 @@ __global__ void __launch_bounds__(NTH, 512 / NTH) k_pc(PCArgs a, Geo g, int T) {
         }
     }
     // E: div_h u* into C0 (homogeneous Neumann / Dirichlet rows)
-    if (MX) split_cols(C1, C2);   // the stencil of u*_+ + u*_-
-    for (int j = threadIdx.x / T; j < N; j += jstep) {
-        const int idx = j * T + tq, t = tq;
-        double2 out = make_double2(0.0, 0.0);
-        if (t < nT && j > 0 && j < N - 1) {
-            const double mm = mmq, kk = kkq, ir = a.ir[j];
-            double2 ds;
-            if (MX) {
-                ds = xsrow(j, t);
-            } else {
-                const double2 dp = sdrow(C1, a.w1, a.col0, j, T, t), dm = sdrow(C2, a.w1, a.col0, j, T, t);
-                ds = make_double2(dp.x + dm.x, dp.y + dm.y);
-            }
-            const double2 vp = C1[idx], vm = C2[idx], vz = C3[idx];
-            out.x = 0.5 * ds.x + 0.5 * (vp.x + vm.x) * ir + 0.5 * mm * ir * (vp.x - vm.x) - kk * vz.y;
-            out.y = 0.5 * ds.y + 0.5 * (vp.y + vm.y) * ir + 0.5 * mm * ir * (vp.y - vm.y) + kk * vz.x;
+    stencil_rows<FX, true>(a, C1, C2, N, T, ir, [&](int j, int i, double d, double irj) {
+        double out = 0.0;
+        if (ins && j > 0 && j < N - 1) {
+            const double hr = 0.5 * irj, vp = D1[i], vm = D2[i];
+            out = 0.5 * d + (vp + vm) * hr + mms * hr * (vp - vm) + kks * D3[i ^ 1];
         }
-        C0[idx] = out;
-    }
+        D0[i] = out;
+    });
     __syncthreads();
     // F: phi = P^{-1} div_h u*
     if (threadIdx.x < nsolve) {
@@ -388,39 +386,28 @@ __global__ void __launch_bounds__(NTH, 512 / NTH) k_pc(PCArgs a, Geo g, int T) {
             const int t = threadIdx.x >> 1, part = threadIdx.x & 1;
             const int mode = mode0 + t, m = mode / g.nk, k = mode - m * g.nk - g.K;
             const size_t mk = (size_t)m * g.K1 + (k < 0 ? -k : k);
-            smem_band_solve<kPCDepth>(C0, T, t, part, N, a.fac + (size_t)kSetP * per_set + mk,
+            smem_band_solve_c<kChunkF, kChunkB>(C0, T, t, part, N, a.fac + (size_t)kSetP * per_set + mk,
                             a.piv + (size_t)kSetP * N * g.M1K1 + mk, g.M1K1);
         }
     }
     __syncthreads();
     if (sp) spike_combine(a, g, C0, 1, kSetP, T, nT, mode0, Xr);
-    if (MX) split_cols(C0, nullptr);
     // G: u^{i+1} = u* - grad_h phi, p^{i+1} = p* + 3 phi / (2 dt), history rotation
     bool bad = false;
-    for (int j = threadIdx.x / T; j < N && tq < nT; j += jstep) {
-        const int idx = j * T + tq, t = tq;
-        const size_t e = (size_t)j * g.nmode + modeq;
-        const double2 f = C0[idx];
-        const double2 d = MX ? xsrow(j, t) : sdrow(C0, a.w1, a.col0, j, T, t);
-        const double tt = mmq * a.ir[j];
-        const double kk = kkq;
-        const double2 gph[3] = {make_double2(d.x - tt * f.x, d.y - tt * f.y),
-                                make_double2(d.x + tt * f.x, d.y + tt * f.y),
-                                make_double2(-kk * f.y, kk * f.x)};
-        const double2 us[3] = {C1[idx], C2[idx], C3[idx]};
+    double* pw = a.commit && ins ? reinterpret_cast<double*>(a.p) + 2 * (size_t)modes + part : nullptr;
+    auto p0 = [&](int j) { return pw ? pw[2 * (size_t)j * g.nmode] : 0.0; };
+    stencil_rows<FX, false>(a, C0, nullptr, N, T, p0, [&](int j, int i, double d, double p) {
+        if (!ins) return;
+        const size_t e = 2 * ((size_t)j * g.nmode + modes) + part;
+        const double f = D0[i], tf = mms * __ldg(&a.ir[j]) * f;
+        const double un[3] = {D1[i] - (d - tf), D2[i] - (d + tf), D3[i] - kks * D0[i ^ 1]};
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            const size_t ec = (size_t)c * g.S + e;
-            const double2 un = make_double2(us[c].x - gph[c].x, us[c].y - gph[c].y);
-            a.u_out[ec] = un;
-            bad |= nonfinite2(un);
+            reinterpret_cast<double*>(a.u_out)[2 * c * g.S + e] = un[c];
+            bad |= nonfinite1(un[c]);
         }
-        if (a.commit) {
-            const double q = 3.0 * c1;   // 3 / (2 dt)
-            const double2 ps = a.p[e];
-            a.p[e] = make_double2(ps.x + q * f.x, ps.y + q * f.y);
-        }
-    }
+        if (pw) pw[2 * (size_t)j * g.nmode] = p + 3.0 * c1 * f;   // 3 / (2 dt)
+    });
     if (bad && a.nonfinite) *a.nonfinite = 1;
 }
 
@@ -437,41 +424,112 @@ __global__ void k_nn_r(const double2* __restrict__ Nc, const double2* __restrict
     if (mode >= g.mhi) return;
     const size_t e = (size_t)blockIdx.x * g.nmode + mode;
     const double2 n1 = Nc[e], n0 = Np[e], m1 = Nc[g.S + e], m0 = Np[g.S + e];
-    X[e] = make_double2(0.5 * ((2.0 * n1.x - n0.x) + (2.0 * m1.x - m0.x)),
-                        0.5 * ((2.0 * n1.y - n0.y) + (2.0 * m1.y - m0.y)));
+    X[e] = make_double2((n1.x - 0.5 * n0.x) + (m1.x - 0.5 * m0.x), (n1.y - 0.5 * n0.y) + (m1.y - 0.5 * m0.y));
+}
+
+// The stages below take the radial stencil of kTileRows consecutive rows of the real or imaginary
+// part of one mode per thread in fixed point (fx::Tile; FP64 next to the walls); the two threads of
+// a mode then trade halves, and each has both parts of half the rows for the rest, in FP64.  With
+// FP64 stencils the FP64 pipe bounded these kernels; now memory and what FP64 is left do.  N_r = 256,
+// M = 64, K = 128, before and after: right-hand sides of step 2 478 -> 257 us, of step 3 443 -> 309,
+// of step 4 438 -> 168, update 301 -> 277 (8 rows per tile: 263, 313, 185, 328).
+struct Stencil {
+    const double* w1;
+    const int* col0;
+    const int2* fw;
+    const int* few;
+};
+struct Cols {
+    int mode, part, m, k, j0;
+    bool in;
+};
+
+// grid: x over the parts of the modes, y = row tile
+__device__ __forceinline__ Cols cols(const Geo& g) {
+    Cols c;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    c.mode = g.mlo + (t >> 1);
+    c.part = t & 1;
+    c.in = c.mode < g.mhi;
+    c.m = c.mode / g.nk;
+    c.k = c.mode - c.m * g.nk - g.K;
+    c.j0 = blockIdx.y * kTileRows;
+    return c;
+}
+
+// body(j, e, d) for half of the tile's rows: d the radial derivative of F (of F + F2) at row j of
+// the thread's mode, e the index of the element
+template <bool PAIR, class Body>
+__device__ __forceinline__ void tile_rows(const Cols& c, const Stencil& s, const Geo& g, const double2* __restrict__ F,
+                                          const double2* __restrict__ F2, Body body) {
+    using namespace fx;
+    constexpr int H = kTileRows / 2;
+    const int N = g.N;
+    const size_t st = 2 * (size_t)g.nmode;
+    const double* f = reinterpret_cast<const double*>(F) + 2 * (size_t)c.mode + c.part;
+    const double* f2 = reinterpret_cast<const double*>(F2) + 2 * (size_t)c.mode + c.part;
+    double d[kTileRows];
+    {
+        double v[kTileRows + 8], v2[kTileRows + 8];
+#pragma unroll
+        for (int i = 0; i < kTileRows + 8; ++i) {
+            const int j = c.j0 - 4 + i;
+            const bool on = c.in && j >= 0 && j < N;
+            v[i] = on ? __ldg(&f[(size_t)j * st]) : 0.0;
+            if (PAIR) v2[i] = on ? __ldg(&f2[(size_t)j * st]) : 0.0;
+        }
+        Tile<kTileRows> X;
+        if (PAIR) X.load(v, v2);
+        else X.load(v);
+#pragma unroll
+        for (int i = 0; i < kTileRows; ++i) {
+            const int j = c.j0 + i;
+            d[i] = 0.0;
+            if (!c.in || j >= N) continue;
+            if (j < 4 || j > N - 5 || X.far(i)) {
+                const int c0 = __ldg(&s.col0[j]);
+#pragma unroll
+                for (int t = 0; t < kStencil; ++t) {
+                    const size_t o = (size_t)(c0 + t) * st;
+                    const double w = __ldg(&s.w1[j * kStencil + t]), x = __ldg(&f[o]);
+                    d[i] = fma(w, PAIR ? x + __ldg(&f2[o]) : x, d[i]);
+                }
+            } else {
+                d[i] = X.row(i, s.fw + j * kStencil, __ldg(&s.few[j]));
+            }
+        }
+    }
+    double2 q[H];   // rows j0 + H part .. + H - 1
+#pragma unroll
+    for (int i = 0; i < H; ++i) {
+        const double give = c.part ? d[i] : d[i + H], keep = c.part ? d[i + H] : d[i];
+        const double got = __shfl_xor_sync(0xffffffffu, give, 1);
+        q[i] = c.part ? make_double2(got, keep) : make_double2(keep, got);
+    }
+    if (!c.in) return;
+#pragma unroll
+    for (int i = 0; i < H; ++i) {
+        const int j = c.j0 + H * c.part + i;
+        if (j < N) body(j, (size_t)j * g.nmode + c.mode, q[i]);
+    }
 }
 
 // Step 2 right-hand side on the interior rows: div_h(-(2N - N_prev)) (the wall rows:
 // k_rhs_pressure_walls).
-__global__ void k_rhs_pressure(const double2* __restrict__ u, const double2* __restrict__ up,
-                               const double2* __restrict__ Nc, const double2* __restrict__ Np,
-                               const double2* __restrict__ X, double2* __restrict__ b,
-                               const double* __restrict__ rn, const double* __restrict__ irn,
-                               const double* __restrict__ w1, const double* __restrict__ w2,
-                               const int* __restrict__ col0, Geo g) {
-    // grid: x = radial row (fastest, so neighbouring rows of a mode range run together and
-    // the stencil's rows stay in cache), y over modes
-    const int mode = g.mlo + blockIdx.y * blockDim.x + threadIdx.x;
-    if (mode >= g.mhi) return;
-    const int j = blockIdx.x + 1;   // interior rows (k_rhs_pressure_walls takes the walls)
-    const size_t e = (size_t)j * g.nmode + mode;
-    const int m = mode / g.nk;
-    const int k = mode - m * g.nk - g.K;
-    const double mm = g.mp * m, kk = g.kz * k;
-    const double ir = irn[j];
-    double2 out = make_double2(0.0, 0.0);
-    {
-        const double2 d = drow(X, w1, col0, j, g.nmode, mode);
-        const double2 x = X[e];
-        const double2 n1 = Nc[e], n0 = Np[e], m1 = Nc[g.S + e], m0 = Np[g.S + e];
-        const double2 z1 = Nc[2 * g.S + e], z0 = Np[2 * g.S + e];
-        const double dpx = (2.0 * n1.x - n0.x) - (2.0 * m1.x - m0.x);
-        const double dpy = (2.0 * n1.y - n0.y) - (2.0 * m1.y - m0.y);
-        const double nzx = 2.0 * z1.x - z0.x, nzy = 2.0 * z1.y - z0.y;
-        out.x = -(d.x + x.x * ir + 0.5 * mm * ir * dpx - kk * nzy);
-        out.y = -(d.y + x.y * ir + 0.5 * mm * ir * dpy + kk * nzx);
-    }
-    b[e] = out;
+__global__ void __launch_bounds__(128) k_rhs_pressure(const double2* __restrict__ Nc, const double2* __restrict__ Np,
+                                                      const double2* __restrict__ X, double2* __restrict__ b,
+                                                      const double* __restrict__ irn, Stencil s, Geo g) {
+    const Cols c = cols(g);
+    const double mm = g.mp * c.m, kk = g.kz * c.k;
+    tile_rows<false>(c, s, g, X, nullptr, [&](int j, size_t e, double2 d) {
+        if (j == 0 || j == g.N - 1) return;
+        const double2 x = __ldg(&X[e]), n1 = __ldg(&Nc[e]), n0 = __ldg(&Np[e]);
+        const double2 z1 = __ldg(&Nc[2 * g.S + e]), z0 = __ldg(&Np[2 * g.S + e]);
+        const double ir = __ldg(&irn[j]), mr = mm * ir;
+        // (2N - N_prev)_+ - x = ((2N - N_prev)_+ - (2N - N_prev)_-) / 2
+        b[e] = make_double2(-(d.x + x.x * ir + mr * ((2.0 * n1.x - n0.x) - x.x) - kk * (2.0 * z1.y - z0.y)),
+                            -(d.y + x.y * ir + mr * ((2.0 * n1.y - n0.y) - x.y) + kk * (2.0 * z1.x - z0.x)));
+    });
 }
 
 // Step 2 right-hand side on the two wall rows: the consistent Neumann value of Eq. ppBC
@@ -500,328 +558,93 @@ __global__ void k_rhs_pressure_walls(const double2* __restrict__ u, const double
     b[e] = out;
 }
 
-// Step 3 right-hand sides, all three components per (row, mode) so that the radial
-// stencil of p* is applied once: (4u - u_prev)/(2dt) - (2N - N_prev) - grad_h p*;
-// Dirichlet rows.  commit: p <- p* (p^{i+1} is completed in the update).
-__global__ void k_rhs_velocity(const double2* __restrict__ u, const double2* __restrict__ up,
-                               const double2* __restrict__ Nc, const double2* __restrict__ Np,
-                               const double2* __restrict__ ps, double2* __restrict__ rhs,
-                               double2* __restrict__ p_out, const double* __restrict__ irn,
-                               const double* __restrict__ w1, const int* __restrict__ col0,
-                               double Re_i, double Re_o, Geo g) {
-    const int mode = g.mlo + blockIdx.y * blockDim.x + threadIdx.x;   // x = radial row
-    if (mode >= g.mhi) return;
-    const int j = blockIdx.x;
-    const size_t e = (size_t)j * g.nmode + mode;
-    const int m = mode / g.nk;
-    const int k = mode - m * g.nk - g.K;
-    const double2 pv = ps[e];
-    if (p_out) p_out[e] = pv;
-    if (j == 0 || j == g.N - 1) {
-        const double Re = (m == 0 && k == 0) ? (j == 0 ? Re_i : Re_o) : 0.0;
-        rhs[e] = make_double2(0.0, Re);
-        rhs[g.S + e] = make_double2(0.0, -Re);
-        rhs[2 * g.S + e] = make_double2(0.0, 0.0);
-        return;
-    }
-    const double2 d = drow(ps, w1, col0, j, g.nmode, mode);
-    const double tt = g.mp * m * irn[j], kk = g.kz * k;
-    const double2 gp[3] = {make_double2(d.x - tt * pv.x, d.y - tt * pv.y),
-                           make_double2(d.x + tt * pv.x, d.y + tt * pv.y),
-                           make_double2(-kk * pv.y, kk * pv.x)};
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const size_t ec = (size_t)c * g.S + e;
-        const double2 a = u[ec], q = up[ec], n1 = Nc[ec], n0 = Np[ec];
-        rhs[ec] = make_double2((4.0 * a.x - q.x) * g.c1 - (2.0 * n1.x - n0.x) - gp[c].x,
-                               (4.0 * a.y - q.y) * g.c1 - (2.0 * n1.y - n0.y) - gp[c].y);
-    }
-}
-
-// Step 4 right-hand side: div_h u* on interior rows, homogeneous Neumann / Dirichlet rows.
-__global__ void k_rhs_div(const double2* __restrict__ us, double2* __restrict__ b,
-                          const double* __restrict__ irn, const double* __restrict__ w1,
-                          const int* __restrict__ col0, Geo g) {
-    const int mode = g.mlo + blockIdx.y * blockDim.x + threadIdx.x;   // x = radial row
-    if (mode >= g.mhi) return;
-    const int j = blockIdx.x;
-    const size_t e = (size_t)j * g.nmode + mode;
-    if (j == 0 || j == g.N - 1) { b[e] = make_double2(0.0, 0.0); return; }
-    const int m = mode / g.nk;
-    const int k = mode - m * g.nk - g.K;
-    const double mm = g.mp * m, kk = g.kz * k, ir = irn[j];
-    const int c0 = col0[j];
-    double2 d = make_double2(0.0, 0.0);
-#pragma unroll
-    for (int t = 0; t < kStencil; ++t) {
-        const double wt = __ldg(&w1[j * kStencil + t]);
-        const size_t o = (size_t)(c0 + t) * g.nmode + mode;
-        const double2 a = us[o], q = us[g.S + o];
-        d.x += wt * (a.x + q.x);
-        d.y += wt * (a.y + q.y);
-    }
-    const double2 vp = us[e], vm = us[g.S + e], vz = us[2 * g.S + e];
-    b[e] = make_double2(0.5 * d.x + 0.5 * (vp.x + vm.x) * ir + 0.5 * mm * ir * (vp.x - vm.x) - kk * vz.y,
-                        0.5 * d.y + 0.5 * (vp.y + vm.y) * ir + 0.5 * mm * ir * (vp.y - vm.y) + kk * vz.x);
-}
-
-// Step 5, all components per (row, mode): u^{i+1} = u* - grad_h phi; p^{i+1} = p* + 3 phi/(2dt).
-// commit: rotate the history in place (u_prev <- u^i, u <- u^{i+1}, N_prev <- N^i, p += 3 phi/(2dt));
-// otherwise write u^{i+1} to u_out only.
-__global__ void k_update(double2* u, double2* up, const double2* Nc, double2* Np, double2* p,
-                         const double2* __restrict__ us, const double2* __restrict__ phi,
-                         double2* __restrict__ u_out, const double* __restrict__ irn,
-                         const double* __restrict__ w1, const int* __restrict__ col0, int commit,
-                         int* __restrict__ nonfinite, Geo g) {
-    const int mode = g.mlo + blockIdx.y * blockDim.x + threadIdx.x;   // x = radial row
-    if (mode >= g.mhi) return;
-    const int j = blockIdx.x;
-    const size_t e = (size_t)j * g.nmode + mode;
-    const int m = mode / g.nk;
-    const int k = mode - m * g.nk - g.K;
-    const double2 f = phi[e];
-    const double2 d = drow(phi, w1, col0, j, g.nmode, mode);
-    const double tt = g.mp * m * irn[j], kk = g.kz * k;
-    const double2 gph[3] = {make_double2(d.x - tt * f.x, d.y - tt * f.y),
-                            make_double2(d.x + tt * f.x, d.y + tt * f.y),
-                            make_double2(-kk * f.y, kk * f.x)};
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const size_t ec = (size_t)c * g.S + e;
-        const double2 s = us[ec];
-        const double2 un = make_double2(s.x - gph[c].x, s.y - gph[c].y);
-        if (nonfinite2(un) && nonfinite) *nonfinite = 1;
-        if (commit) {
-            up[ec] = u[ec];
-            u[ec] = un;
-            Np[ec] = Nc[ec];
-        } else {
-            u_out[ec] = un;
-        }
-    }
-    if (commit) {
-        const double q = 3.0 * g.c1;
-        const double2 a = p[e];
-        p[e] = make_double2(a.x + q * f.x, a.y + q * f.y);
-    }
-}
-
-// ---------------------------------------------------------------- split path, mixed form
-// The same four per-stage kernels for TC_MIXED plans, with each radial stencil (of X, p*,
-// u*_+ + u*_- and phi) in double-FP32 instead of FP64: the FP64 pipe, which bounds these
-// kernels, then carries only the rest.  The (0, 0) mode keeps the FP64 stencil: it carries
-// the mean flow, a smooth profile some 1e5 times larger near the clustered walls than the
-// differences of neighbouring rows its derivative rests on, so the 47 bits of the split
-// would cost it 1e-9 of the wall shear (and the torque follows it).  A block takes a tile of 32 modes x 32 rows; the
-// tile's window of rows is read once and each value split once into an exact FP32 pair
-// (hi, lo) in shared memory, the stencil is a compensated dot product of the pairs (about 44
-// significant bits, against FP32 transforms elsewhere in the form), and the result is
-// assembled in FP64.  Everything else keeps the FP64 arithmetic of the FP64 kernels.
-constexpr int kXsM = 32;                     // modes per tile (one warp row)
-constexpr int kXsR = 32;                     // rows per tile
-constexpr int kXsWin = kXsR + kStencil - 1;  // window rows
-
-struct XsTile {
-    int mode;   // this thread's mode
-    bool in;    // mode < g.mhi
-    int r0, r1, jlo;
-};
-
-__device__ __forceinline__ XsTile xs_tile(const int* __restrict__ col0, const Geo& g) {
-    XsTile t;
-    t.mode = g.mlo + blockIdx.x * kXsM + threadIdx.x;
-    t.in = t.mode < g.mhi;
-    t.r0 = blockIdx.y * kXsR;
-    t.r1 = min(t.r0 + kXsR, g.N) - 1;
-    t.jlo = col0[t.r0];
-    return t;
-}
-
-// the tile's stencil weights and the window of f (or of f + f2), split once
-__device__ __forceinline__ void xs_load(const double2* __restrict__ f, const double2* __restrict__ f2,
-                                        const double* __restrict__ w1, const int* __restrict__ col0,
-                                        float4* win, float2* sw, const XsTile& t, const Geo& g) {
-    const int tid = threadIdx.y * kXsM + threadIdx.x;
-    for (int i = tid; i < (t.r1 - t.r0 + 1) * kStencil; i += blockDim.x * blockDim.y)
-        sw[i] = xs::split_hl(w1[(size_t)t.r0 * kStencil + i]);
-    const int jhi = col0[t.r1] + kStencil - 1;
-    for (int j = t.jlo + threadIdx.y; j <= jhi; j += blockDim.y) {
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (t.in) {
-            double2 x = f[(size_t)j * g.nmode + t.mode];
-            if (f2) {
-                const double2 y = f2[(size_t)j * g.nmode + t.mode];
-                x.x += y.x;
-                x.y += y.y;
-            }
-            const float2 a = xs::split_hl(x.x), q = xs::split_hl(x.y);
-            v = make_float4(a.x, q.x, a.y, q.y);
-        }
-        win[(j - t.jlo) * kXsM + threadIdx.x] = v;
-    }
-    __syncthreads();
-}
-
-// D1 of the window's field at row r for this thread's mode
-__device__ __forceinline__ double2 xs_drow(const float4* win, const float2* sw, const int* __restrict__ col0,
-                                           const XsTile& t, int r) {
-    const int w0 = (col0[r] - t.jlo) * kXsM + threadIdx.x;
-    return xs_stencil(win + w0, kXsM, sw + (r - t.r0) * kStencil);
-}
-
-__global__ void __launch_bounds__(256) k_rhs_pressure_mx(const double2* __restrict__ u, const double2* __restrict__ up,
-                                                         const double2* __restrict__ Nc, const double2* __restrict__ Np,
-                                                         const double2* __restrict__ X, double2* __restrict__ b,
-                                                         const double* __restrict__ rn, const double* __restrict__ irn,
-                                                         const double* __restrict__ w1, const double* __restrict__ w2,
-                                                         const int* __restrict__ col0, Geo g) {
-    __shared__ float4 win[kXsWin * kXsM];
-    __shared__ float2 sw[kXsR * kStencil];
-    const XsTile t = xs_tile(col0, g);
-    xs_load(X, nullptr, w1, col0, win, sw, t, g);
-    if (!t.in) return;
-    const int mode = t.mode;
-    const int m = mode / g.nk;
-    const int k = mode - m * g.nk - g.K;
-    const bool mode00 = m == 0 && k == 0;
-    const double mm = g.mp * m, kk = g.kz * k;
-    for (int j = t.r0 + threadIdx.y; j <= t.r1; j += blockDim.y) {
-        if (j == 0 || j == g.N - 1) continue;   // k_rhs_pressure_walls
-        const size_t e = (size_t)j * g.nmode + mode;
-        const double ir = irn[j];
-        double2 out = make_double2(0.0, 0.0);
-        {
-            const double2 d = mode00 ? drow(X, w1, col0, j, g.nmode, mode) : xs_drow(win, sw, col0, t, j);
-            const double2 x = X[e];
-            const double2 n1 = Nc[e], n0 = Np[e], m1 = Nc[g.S + e], m0 = Np[g.S + e];
-            const double2 z1 = Nc[2 * g.S + e], z0 = Np[2 * g.S + e];
-            const double dpx = (2.0 * n1.x - n0.x) - (2.0 * m1.x - m0.x);
-            const double dpy = (2.0 * n1.y - n0.y) - (2.0 * m1.y - m0.y);
-            const double nzx = 2.0 * z1.x - z0.x, nzy = 2.0 * z1.y - z0.y;
-            out.x = -(d.x + x.x * ir + 0.5 * mm * ir * dpx - kk * nzy);
-            out.y = -(d.y + x.y * ir + 0.5 * mm * ir * dpy + kk * nzx);
-        }
-        b[e] = out;
-    }
-}
-
-__global__ void __launch_bounds__(256) k_rhs_velocity_mx(const double2* __restrict__ u, const double2* __restrict__ up,
-                                                         const double2* __restrict__ Nc, const double2* __restrict__ Np,
-                                                         const double2* __restrict__ ps, double2* __restrict__ rhs,
-                                                         double2* __restrict__ p_out, const double* __restrict__ irn,
-                                                         const double* __restrict__ w1, const int* __restrict__ col0,
-                                                         double Re_i, double Re_o, Geo g) {
-    __shared__ float4 win[kXsWin * kXsM];
-    __shared__ float2 sw[kXsR * kStencil];
-    const XsTile t = xs_tile(col0, g);
-    xs_load(ps, nullptr, w1, col0, win, sw, t, g);
-    if (!t.in) return;
-    const int mode = t.mode;
-    const int m = mode / g.nk;
-    const int k = mode - m * g.nk - g.K;
-    const bool mode00 = m == 0 && k == 0;
-    for (int j = t.r0 + threadIdx.y; j <= t.r1; j += blockDim.y) {
-        const size_t e = (size_t)j * g.nmode + mode;
-        const double2 pv = ps[e];
+// Step 3 right-hand sides, all three components together so that the radial stencil of p* is
+// applied once: (4u - u_prev)/(2dt) - (2N - N_prev) - grad_h p*; Dirichlet rows.
+// commit: p <- p* (p^{i+1} is completed in the update).
+__global__ void __launch_bounds__(128) k_rhs_velocity(const double2* __restrict__ u, const double2* __restrict__ up,
+                                                      const double2* __restrict__ Nc, const double2* __restrict__ Np,
+                                                      const double2* __restrict__ ps, double2* __restrict__ rhs,
+                                                      double2* __restrict__ p_out, const double* __restrict__ irn,
+                                                      double Re_i, double Re_o, Stencil s, Geo g) {
+    const Cols c = cols(g);
+    const double mm = g.mp * c.m, kk = g.kz * c.k;
+    tile_rows<false>(c, s, g, ps, nullptr, [&](int j, size_t e, double2 d) {
+        const double2 pv = __ldg(&ps[e]);
         if (p_out) p_out[e] = pv;
         if (j == 0 || j == g.N - 1) {
-            const double Re = (m == 0 && k == 0) ? (j == 0 ? Re_i : Re_o) : 0.0;
+            const double Re = (c.m == 0 && c.k == 0) ? (j == 0 ? Re_i : Re_o) : 0.0;
             rhs[e] = make_double2(0.0, Re);
             rhs[g.S + e] = make_double2(0.0, -Re);
             rhs[2 * g.S + e] = make_double2(0.0, 0.0);
-            continue;
+            return;
         }
-        const double2 d = mode00 ? drow(ps, w1, col0, j, g.nmode, mode) : xs_drow(win, sw, col0, t, j);
-        const double tt = g.mp * m * irn[j], kk = g.kz * k;
+        const double tt = mm * __ldg(&irn[j]);
         const double2 gp[3] = {make_double2(d.x - tt * pv.x, d.y - tt * pv.y),
                                make_double2(d.x + tt * pv.x, d.y + tt * pv.y),
                                make_double2(-kk * pv.y, kk * pv.x)};
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const size_t ec = (size_t)c * g.S + e;
-            const double2 a = u[ec], q = up[ec], n1 = Nc[ec], n0 = Np[ec];
-            rhs[ec] = make_double2((4.0 * a.x - q.x) * g.c1 - (2.0 * n1.x - n0.x) - gp[c].x,
-                                   (4.0 * a.y - q.y) * g.c1 - (2.0 * n1.y - n0.y) - gp[c].y);
+        for (int f = 0; f < 3; ++f) {
+            const size_t ec = f * g.S + e;
+            const double2 a = __ldg(&u[ec]), q = __ldg(&up[ec]), n1 = __ldg(&Nc[ec]), n0 = __ldg(&Np[ec]);
+            rhs[ec] = make_double2((4.0 * a.x - q.x) * g.c1 - (2.0 * n1.x - n0.x) - gp[f].x,
+                                   (4.0 * a.y - q.y) * g.c1 - (2.0 * n1.y - n0.y) - gp[f].y);
         }
-    }
+    });
 }
 
-__global__ void __launch_bounds__(256) k_rhs_div_mx(const double2* __restrict__ us, double2* __restrict__ b,
-                                                    const double* __restrict__ irn, const double* __restrict__ w1,
-                                                    const int* __restrict__ col0, Geo g) {
-    __shared__ float4 win[kXsWin * kXsM];
-    __shared__ float2 sw[kXsR * kStencil];
-    const XsTile t = xs_tile(col0, g);
-    xs_load(us, us + g.S, w1, col0, win, sw, t, g);   // the stencil of u*_+ + u*_-
-    if (!t.in) return;
-    const int mode = t.mode;
-    const int m = mode / g.nk;
-    const int k = mode - m * g.nk - g.K;
-    const bool mode00 = m == 0 && k == 0;
-    const double mm = g.mp * m, kk = g.kz * k;
-    for (int j = t.r0 + threadIdx.y; j <= t.r1; j += blockDim.y) {
-        const size_t e = (size_t)j * g.nmode + mode;
+// Step 4 right-hand side: div_h u* on interior rows, homogeneous Neumann / Dirichlet rows.
+__global__ void __launch_bounds__(128) k_rhs_div(const double2* __restrict__ us, double2* __restrict__ b,
+                                                 const double* __restrict__ irn, Stencil s, Geo g) {
+    const Cols c = cols(g);
+    const double mm = g.mp * c.m, kk = g.kz * c.k;
+    tile_rows<true>(c, s, g, us, us + g.S, [&](int j, size_t e, double2 d) {
         if (j == 0 || j == g.N - 1) {
             b[e] = make_double2(0.0, 0.0);
-            continue;
+            return;
         }
-        const double ir = irn[j];
-        double2 d;
-        if (mode00) {
-            const double2 dp = drow(us, w1, col0, j, g.nmode, mode), dm = drow(us + g.S, w1, col0, j, g.nmode, mode);
-            d = make_double2(dp.x + dm.x, dp.y + dm.y);
-        } else {
-            d = xs_drow(win, sw, col0, t, j);
-        }
-        const double2 vp = us[e], vm = us[g.S + e], vz = us[2 * g.S + e];
-        b[e] = make_double2(0.5 * d.x + 0.5 * (vp.x + vm.x) * ir + 0.5 * mm * ir * (vp.x - vm.x) - kk * vz.y,
-                            0.5 * d.y + 0.5 * (vp.y + vm.y) * ir + 0.5 * mm * ir * (vp.y - vm.y) + kk * vz.x);
-    }
+        const double hr = 0.5 * __ldg(&irn[j]), mr = mm * hr;
+        const double2 vp = __ldg(&us[e]), vm = __ldg(&us[g.S + e]), vz = __ldg(&us[2 * g.S + e]);
+        b[e] = make_double2(0.5 * d.x + (vp.x + vm.x) * hr + mr * (vp.x - vm.x) - kk * vz.y,
+                            0.5 * d.y + (vp.y + vm.y) * hr + mr * (vp.y - vm.y) + kk * vz.x);
+    });
 }
 
-__global__ void __launch_bounds__(256) k_update_mx(double2* u, double2* up, const double2* Nc, double2* Np, double2* p,
-                                                   const double2* __restrict__ us, const double2* __restrict__ phi,
-                                                   double2* __restrict__ u_out, const double* __restrict__ irn,
-                                                   const double* __restrict__ w1, const int* __restrict__ col0,
-                                                   int commit, int* __restrict__ nonfinite, Geo g) {
-    __shared__ float4 win[kXsWin * kXsM];
-    __shared__ float2 sw[kXsR * kStencil];
-    const XsTile t = xs_tile(col0, g);
-    xs_load(phi, nullptr, w1, col0, win, sw, t, g);
-    if (!t.in) return;
-    const int mode = t.mode;
-    const int m = mode / g.nk;
-    const int k = mode - m * g.nk - g.K;
-    const bool mode00 = m == 0 && k == 0;
+// Step 5, all components together: u^{i+1} = u* - grad_h phi; p^{i+1} = p* + 3 phi/(2dt).
+// commit: rotate the history in place (u_prev <- u^i, u <- u^{i+1}, N_prev <- N^i, p += 3 phi/(2dt));
+// otherwise write u^{i+1} to u_out only.
+__global__ void __launch_bounds__(128) k_update(double2* __restrict__ u, double2* __restrict__ up,
+                                                const double2* __restrict__ Nc, double2* __restrict__ Np,
+                                                double2* __restrict__ p, const double2* __restrict__ us,
+                                                const double2* __restrict__ phi, double2* __restrict__ u_out,
+                                                const double* __restrict__ irn, int commit,
+                                                int* __restrict__ nonfinite, Stencil s, Geo g) {
+    const Cols c = cols(g);
+    const double mm = g.mp * c.m, kk = g.kz * c.k, q = 3.0 * g.c1;
     bool bad = false;
-    for (int j = t.r0 + threadIdx.y; j <= t.r1; j += blockDim.y) {
-        const size_t e = (size_t)j * g.nmode + mode;
-        const double2 f = phi[e];
-        const double2 d = mode00 ? drow(phi, w1, col0, j, g.nmode, mode) : xs_drow(win, sw, col0, t, j);
-        const double tt = g.mp * m * irn[j], kk = g.kz * k;
+    tile_rows<false>(c, s, g, phi, nullptr, [&](int j, size_t e, double2 d) {
+        const double2 f = __ldg(&phi[e]);
+        const double tt = mm * __ldg(&irn[j]);
         const double2 gph[3] = {make_double2(d.x - tt * f.x, d.y - tt * f.y),
                                 make_double2(d.x + tt * f.x, d.y + tt * f.y),
                                 make_double2(-kk * f.y, kk * f.x)};
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const size_t ec = (size_t)c * g.S + e;
-            const double2 s = us[ec];
-            const double2 un = make_double2(s.x - gph[c].x, s.y - gph[c].y);
+        for (int i = 0; i < 3; ++i) {
+            const size_t ec = i * g.S + e;
+            const double2 v = __ldg(&us[ec]), un = make_double2(v.x - gph[i].x, v.y - gph[i].y);
             bad |= nonfinite2(un);
             if (commit) {
                 up[ec] = u[ec];
                 u[ec] = un;
-                Np[ec] = Nc[ec];
+                Np[ec] = __ldg(&Nc[ec]);
             } else {
                 u_out[ec] = un;
             }
         }
         if (commit) {
-            const double q = 3.0 * g.c1;
             const double2 a = p[e];
             p[e] = make_double2(a.x + q * f.x, a.y + q * f.y);
         }
-    }
+    });
     if (bad && nonfinite) *nonfinite = 1;
 }
 
@@ -1135,17 +958,11 @@ static tc_status launch_advance_split(tc_plan* p, const double2* u, double2* u_p
         const bool ring = (size_t)2 * nm * nf < (size_t)24 * 32 * p->num_sms;
         (ring ? k_band_solve_g<kGD> : k_band_solve_g<1>)<<<grid, 128, 0, s>>>(x, p->d_fac, p->d_piv, set, nf, g);
     };
-    // mixed form: the radial stencils in double-FP32 (the *_mx kernels), tiles of 32 x 32
-    const bool mx = p->precision == TC_MIXED;
-    const dim3 gx(blocks_for(nm, kXsM), blocks_for(g.N, kXsR)), bx(kXsM, 8);
+    const Stencil st{p->d_w1, p->d_col0, p->d_fx_w1, p->d_fx_ew};
+    const dim3 gt(blocks_for((size_t)2 * nm, 128), blocks_for(g.N, kTileRows));
     int slot = prof_begin(p, kKRhsPressure, s);
     k_nn_r<<<g1, 128, 0, s>>>(Ncur, N_prev, phi, g);
-    if (mx)
-        k_rhs_pressure_mx<<<gx, bx, 0, s>>>(u, u_prev, Ncur, N_prev, phi, ps, p->d_r, p->d_ir, p->d_w1, p->d_w2,
-                                            p->d_col0, g);
-    else
-        k_rhs_pressure<<<dim3(g.N - 2, blocks_for(nm, 128)), 128, 0, s>>>(u, u_prev, Ncur, N_prev, phi, ps, p->d_r,
-                                                                        p->d_ir, p->d_w1, p->d_w2, p->d_col0, g);
+    k_rhs_pressure<<<gt, 128, 0, s>>>(Ncur, N_prev, phi, ps, p->d_ir, st, g);
     k_rhs_pressure_walls<<<dim3(blocks_for(nm, 128), 2), 128, 0, s>>>(u, u_prev, phi, ps, p->d_r, p->d_w1, p->d_w2,
                                                                      p->d_col0, g);
     prof_end(p, slot, s);
@@ -1155,12 +972,8 @@ static tc_status launch_advance_split(tc_plan* p, const double2* u, double2* u_p
     prof_end(p, slot, s);
     TC_LAUNCHED(p, "k_band_solve_g");
     slot = prof_begin(p, kKRhsVelocity, s);
-    if (mx)
-        k_rhs_velocity_mx<<<gx, bx, 0, s>>>(u, u_prev, Ncur, N_prev, ps, us, commit ? p_out : nullptr, p->d_ir,
-                                            p->d_w1, p->d_col0, p->Re_i, p->Re_o, g);
-    else
-        k_rhs_velocity<<<g1, 128, 0, s>>>(u, u_prev, Ncur, N_prev, ps, us, commit ? p_out : nullptr, p->d_ir,
-                                          p->d_w1, p->d_col0, p->Re_i, p->Re_o, g);
+    k_rhs_velocity<<<gt, 128, 0, s>>>(u, u_prev, Ncur, N_prev, ps, us, commit ? p_out : nullptr, p->d_ir, p->Re_i,
+                                      p->Re_o, st, g);
     prof_end(p, slot, s);
     TC_LAUNCHED(p, "k_rhs_velocity");
     slot = prof_begin(p, kKSolveH, s);
@@ -1168,10 +981,7 @@ static tc_status launch_advance_split(tc_plan* p, const double2* u, double2* u_p
     prof_end(p, slot, s);
     TC_LAUNCHED(p, "k_band_solve_g");
     slot = prof_begin(p, kKRhsDiv, s);
-    if (mx)
-        k_rhs_div_mx<<<gx, bx, 0, s>>>(us, phi, p->d_ir, p->d_w1, p->d_col0, g);
-    else
-        k_rhs_div<<<g1, 128, 0, s>>>(us, phi, p->d_ir, p->d_w1, p->d_col0, g);
+    k_rhs_div<<<gt, 128, 0, s>>>(us, phi, p->d_ir, st, g);
     prof_end(p, slot, s);
     TC_LAUNCHED(p, "k_rhs_div");
     slot = prof_begin(p, kKSolveP, s);
@@ -1179,12 +989,8 @@ static tc_status launch_advance_split(tc_plan* p, const double2* u, double2* u_p
     prof_end(p, slot, s);
     TC_LAUNCHED(p, "k_band_solve_g");
     slot = prof_begin(p, kKUpdate, s);
-    if (mx)
-        k_update_mx<<<gx, bx, 0, s>>>(const_cast<double2*>(u), u_prev, Ncur, N_prev, p_out, us, phi, u_out, p->d_ir,
-                                      p->d_w1, p->d_col0, commit ? 1 : 0, p->d_nonfinite, g);
-    else
-        k_update<<<g1, 128, 0, s>>>(const_cast<double2*>(u), u_prev, Ncur, N_prev, p_out, us, phi, u_out, p->d_ir,
-                                    p->d_w1, p->d_col0, commit ? 1 : 0, p->d_nonfinite, g);
+    k_update<<<gt, 128, 0, s>>>(const_cast<double2*>(u), u_prev, Ncur, N_prev, p_out, us, phi, u_out, p->d_ir,
+                                commit ? 1 : 0, p->d_nonfinite, st, g);
     prof_end(p, slot, s);
     TC_LAUNCHED(p, "k_update");
     return TC_OK;
@@ -1205,7 +1011,8 @@ tc_status launch_advance(tc_plan* p, const double2* u, double2* u_prev, const do
     a.up_out = commit ? u_prev : nullptr;
     a.Np_out = commit ? N_prev : nullptr;
     a.p = commit ? p_out : nullptr;
-    a.rn = p->d_r; a.ir = p->d_ir; a.w1 = p->d_w1; a.w2 = p->d_w2; a.col0 = p->d_col0;
+    a.ir = p->d_ir; a.w1 = p->d_w1; a.w2 = p->d_w2; a.col0 = p->d_col0;
+    a.fw = p->d_fx_w1; a.few = p->d_fx_ew;
     a.fac = p->d_fac; a.piv = p->d_piv;
     a.fac2 = p->d_fac2; a.piv2 = p->d_piv2; a.spk = p->d_spk; a.rinv = p->d_rinv;
     a.nonfinite = p->d_nonfinite;
@@ -1213,12 +1020,7 @@ tc_status launch_advance(tc_plan* p, const double2* u, double2* u_prev, const do
     a.commit = commit ? 1 : 0;
     // two partitions while the 12 T substitution threads of the Helmholtz phase fit the block
     g.sh = (p->part_h > 0 && 12 * T <= (T <= 8 ? 128 : 256)) ? p->part_h : 0;
-    // mixed form: the split column and weights of the double-FP32 stencils after the rest
-    const bool mx = p->precision == TC_MIXED;
-    const size_t sm = (size_t)4 * p->N_r * T * sizeof(double2) + (size_t)3 * T * 16 * sizeof(double) +
-                      (mx ? (size_t)p->N_r * T * sizeof(float4) +
-                                (size_t)((p->N_r * kStencil + 1) & ~1) * sizeof(float2) +
-                                (size_t)p->N_r * sizeof(double2) : 0);
+    const size_t sm = (size_t)4 * p->N_r * T * sizeof(double2) + (size_t)3 * T * 16 * sizeof(double);
     // 128 threads up to 8 modes per block, 256 beyond (6T substitution threads plus helpers)
     const int slot = prof_begin(p, kKPC, s);
     auto run = [&](auto kern, int nth) -> tc_status {
@@ -1226,8 +1028,12 @@ tc_status launch_advance(tc_plan* p, const double2* u, double2* u_prev, const do
         kern<<<blocks_for(g.mhi - g.mlo, T), nth, sm, s>>>(a, g, T);
         return TC_OK;
     };
-    if (T <= 8) TC_TRY_STATUS(mx ? run(k_pc<128, true>, 128) : run(k_pc<128, false>, 128));
-    else TC_TRY_STATUS(mx ? run(k_pc<256, true>, 256) : run(k_pc<256, false>, 256));
+    // fixed-point stencils while enough warps share the FP64 pipe (14 per SM: 219 against 252 us,
+    // N_r = 64, M = 32, K = 64); with fewer than 8 per SM their conversions take longer than the
+    // FP64 FMAs (2 per SM: 90 against 61 us, N_r = 32, M = 8, K = 16)
+    const bool fxs = (size_t)blocks_for(g.mhi - g.mlo, T) * (T <= 8 ? 128 : 256) >= (size_t)256 * p->num_sms;
+    if (T <= 8) TC_TRY_STATUS(fxs ? run(k_pc<128, true>, 128) : run(k_pc<128, false>, 128));
+    else TC_TRY_STATUS(fxs ? run(k_pc<256, true>, 256) : run(k_pc<256, false>, 256));
     prof_end(p, slot, s);
     TC_LAUNCHED(p, "k_pc");
     return TC_OK;

@@ -164,6 +164,100 @@ __device__ __forceinline__ void smem_band_solve(double2* col, int T, int t, int 
     }
 }
 
+// The same substitution with the factors fetched in chunks, CF rows (forward) and CB rows
+// (backward) ahead in a second register buffer.  A ring that is refilled row by row leaves the
+// loads of several rows on one scoreboard, and waiting for a row then waits for the youngest of
+// them, a memory latency per row; a chunk's loads are waited for once, a chunk later.
+template <int CF, int CB>
+__device__ __forceinline__ void smem_band_solve_c(double2* col, int T, int t, int part, int N,
+                                                  const double* __restrict__ F, const uint8_t* __restrict__ P,
+                                                  int M1K1) {
+    double* x = reinterpret_cast<double*>(col) + 2 * t + part;   // x[j] at x[2 T j]
+    const int st = 2 * T;
+    const size_t rs = (size_t)kBands * M1K1;
+    double w0 = x[0], w1 = N > 1 ? x[st] : 0.0, w2 = N > 2 ? x[2 * st] : 0.0,
+           w3 = N > 3 ? x[3 * st] : 0.0, w4 = N > 4 ? x[4 * st] : 0.0;
+    {
+        double lr[2][CF][4];
+        int pr[2][CF];
+        auto load = [&](double (&l)[CF][4], int (&p)[CF], int c) {
+#pragma unroll
+            for (int d = 0; d < CF; ++d) {
+                const int j = min(c * CF + d, N - 1);
+                p[d] = __ldg(&P[(size_t)j * M1K1]);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) l[d][q] = __ldg(&F[(size_t)j * rs + (size_t)q * M1K1]);
+            }
+        };
+        load(lr[0], pr[0], 0);
+        const int nc = (N + CF - 1) / CF;
+        for (int c0 = 0; c0 < nc; c0 += 2) {
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+                if (c0 + b < nc) {
+                    load(lr[b ^ 1], pr[b ^ 1], c0 + b + 1);
+#pragma unroll
+                    for (int d = 0; d < CF; ++d) {
+                        const int j = (c0 + b) * CF + d;
+                        if (j < N) {
+                            const int pj = pr[b][d];
+                            if (pj == 1) { double q = w0; w0 = w1; w1 = q; }
+                            else if (pj == 2) { double q = w0; w0 = w2; w2 = q; }
+                            else if (pj == 3) { double q = w0; w0 = w3; w3 = q; }
+                            else if (pj == 4) { double q = w0; w0 = w4; w4 = q; }
+                            x[(size_t)j * st] = w0;
+                            w1 = fma(-lr[b][d][0], w0, w1);
+                            w2 = fma(-lr[b][d][1], w0, w2);
+                            w3 = fma(-lr[b][d][2], w0, w3);
+                            w4 = fma(-lr[b][d][3], w0, w4);
+                            w0 = w1; w1 = w2; w2 = w3; w3 = w4;
+                            w4 = (j + 5 < N) ? x[(size_t)(j + 5) * st] : 0.0;
+                        }
+                    }
+                }
+            }
+        }
+    }
+    double v1 = 0.0, v2 = 0.0, v3 = 0.0, v4 = 0.0, v5 = 0.0, v6 = 0.0, v7 = 0.0, v8 = 0.0;
+    double ur[2][CB][9];
+    auto load = [&](double (&u)[CB][9], int c) {
+#pragma unroll
+        for (int d = 0; d < CB; ++d) {
+            const int j = max(N - 1 - (c * CB + d), 0);
+#pragma unroll
+            for (int q = 0; q < 9; ++q) u[d][q] = __ldg(&F[(size_t)j * rs + (size_t)(4 + q) * M1K1]);
+        }
+    };
+    load(ur[0], 0);
+    const int nc = (N + CB - 1) / CB;
+    for (int c0 = 0; c0 < nc; c0 += 2) {
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            if (c0 + b < nc) {
+                load(ur[b ^ 1], c0 + b + 1);
+#pragma unroll
+                for (int d = 0; d < CB; ++d) {
+                    const int j = N - 1 - ((c0 + b) * CB + d);
+                    if (j >= 0) {
+                        double s = x[(size_t)j * st];
+                        s = fma(-ur[b][d][8], v8, s);
+                        s = fma(-ur[b][d][7], v7, s);
+                        s = fma(-ur[b][d][6], v6, s);
+                        s = fma(-ur[b][d][5], v5, s);
+                        s = fma(-ur[b][d][4], v4, s);
+                        s = fma(-ur[b][d][3], v3, s);
+                        s = fma(-ur[b][d][2], v2, s);
+                        s = fma(-ur[b][d][1], v1, s);
+                        const double xj = s * ur[b][d][0];
+                        x[(size_t)j * st] = xj;
+                        v8 = v7; v7 = v6; v6 = v5; v5 = v4; v4 = v3; v3 = v2; v2 = v1; v1 = xj;
+                    }
+                }
+            }
+        }
+    }
+}
+
 // D1 of column t of smem array C ([N][T]) at row j
 __device__ __forceinline__ double2 sdrow(const double2* C, const double* __restrict__ w1,
                                          const int* __restrict__ col0, int j, int T, int t) {
