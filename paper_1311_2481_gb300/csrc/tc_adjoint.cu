@@ -14,12 +14,11 @@ static int ablocks(size_t n, int bs) { return (int)((n + bs - 1) / bs); }
 // x <- A^{-T} x on one real part of column t of a [N][T] smem array, for A = P L U stored
 // as in smem_band_solve: first U^T y = x (forward), then for j = N-1..0 the transposed
 // elimination x_j -= sum_q l_q(j) x_{j+q} followed by the row interchange j <-> j + piv_j.
-// The factors of the next kPCDepth rows are kept in flight in a register ring (as in
-// smem_band_solve).
+// The factors come in chunks of CB (U) and CF (L) rows, as in smem_band_solve_c.
+template <int CF, int CB>
 __device__ __forceinline__ void smem_band_solve_T(double2* col, int T, int t, int part, int N,
                                                   const double* __restrict__ F,
                                                   const uint8_t* __restrict__ P, int M1K1) {
-    constexpr int D = kPCDepth;
     double* x = reinterpret_cast<double*>(col) + 2 * t + part;
     const int st = 2 * T;
     // U^T y = b: y_j = (b_j - sum_{q=1..8} U(j-q, j) y_{j-q}) / U_jj, column-oriented: p0..p7
@@ -31,72 +30,84 @@ __device__ __forceinline__ void smem_band_solve_T(double2* col, int T, int t, in
     double p3 = N > 3 ? x[(size_t)3 * st] : 0.0, p4 = N > 4 ? x[(size_t)4 * st] : 0.0;
     double p5 = N > 5 ? x[(size_t)5 * st] : 0.0, p6 = N > 6 ? x[(size_t)6 * st] : 0.0;
     double p7 = N > 7 ? x[(size_t)7 * st] : 0.0;
-    double ur[D][9];
+    {
+        double ur[2][CB][9];
+        auto load = [&](double (&u)[CB][9], int c) {
 #pragma unroll
-    for (int d = 0; d < D; ++d)
+            for (int d = 0; d < CB; ++d) {
+                const int j = min(c * CB + d, N - 1);
 #pragma unroll
-        for (int q = 0; q < 9; ++q) ur[d][q] = d < N ? __ldg(&F[(size_t)d * rs + (size_t)(4 + q) * M1K1]) : 0.0;
-    for (int j0 = 0; j0 < N; j0 += D) {
+                for (int q = 0; q < 9; ++q) u[d][q] = __ldg(&F[(size_t)j * rs + (size_t)(4 + q) * M1K1]);
+            }
+        };
+        load(ur[0], 0);
+        const int nc = (N + CB - 1) / CB;
+        for (int c0 = 0; c0 < nc; c0 += 2) {
 #pragma unroll
-        for (int d = 0; d < D; ++d) {
-            const int j = j0 + d;
-            if (j < N) {
-                double u[9];
+            for (int b = 0; b < 2; ++b) {
+                if (c0 + b < nc) {
+                    load(ur[b ^ 1], c0 + b + 1);
 #pragma unroll
-                for (int q = 0; q < 9; ++q) u[q] = ur[d][q];
-                if (j + D < N) {
-#pragma unroll
-                    for (int q = 0; q < 9; ++q) ur[d][q] = __ldg(&F[(size_t)(j + D) * rs + (size_t)(4 + q) * M1K1]);
+                    for (int d = 0; d < CB; ++d) {
+                        const int j = (c0 + b) * CB + d;
+                        if (j < N) {
+                            const double* u = ur[b][d];
+                            const double yj = p0 * u[0];
+                            x[(size_t)j * st] = yj;
+                            const double p8 = j + 8 < N ? x[(size_t)(j + 8) * st] : 0.0;
+                            p0 = fma(-u[1], yj, p1);
+                            p1 = fma(-u[2], yj, p2);
+                            p2 = fma(-u[3], yj, p3);
+                            p3 = fma(-u[4], yj, p4);
+                            p4 = fma(-u[5], yj, p5);
+                            p5 = fma(-u[6], yj, p6);
+                            p6 = fma(-u[7], yj, p7);
+                            p7 = fma(-u[8], yj, p8);
+                        }
+                    }
                 }
-                const double yj = p0 * u[0];
-                x[(size_t)j * st] = yj;
-                const double p8 = j + 8 < N ? x[(size_t)(j + 8) * st] : 0.0;
-                p0 = fma(-u[1], yj, p1);
-                p1 = fma(-u[2], yj, p2);
-                p2 = fma(-u[3], yj, p3);
-                p3 = fma(-u[4], yj, p4);
-                p4 = fma(-u[5], yj, p5);
-                p5 = fma(-u[6], yj, p6);
-                p6 = fma(-u[7], yj, p7);
-                p7 = fma(-u[8], yj, p8);
             }
         }
     }
     // transposed eliminations and interchanges, j = N-1 .. 0; w1..w4 hold x_{j+1..j+4}
     double w1 = 0.0, w2 = 0.0, w3 = 0.0, w4 = 0.0;
-    double lr[D][4];
-    int pr[D];
+    double lr[2][CF][4];
+    int pr[2][CF];
+    auto load = [&](double (&l)[CF][4], int (&p)[CF], int c) {
 #pragma unroll
-    for (int d = 0; d < D; ++d) {
-        const int j = N - 1 - d;
-        pr[d] = j >= 0 ? P[(size_t)j * M1K1] : 0;
+        for (int d = 0; d < CF; ++d) {
+            const int j = max(N - 1 - (c * CF + d), 0);
+            p[d] = __ldg(&P[(size_t)j * M1K1]);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) lr[d][q] = j >= 0 ? __ldg(&F[(size_t)j * rs + (size_t)q * M1K1]) : 0.0;
-    }
-    for (int j0 = N - 1; j0 >= 0; j0 -= D) {
+            for (int q = 0; q < 4; ++q) l[d][q] = __ldg(&F[(size_t)j * rs + (size_t)q * M1K1]);
+        }
+    };
+    load(lr[0], pr[0], 0);
+    const int nc = (N + CF - 1) / CF;
+    for (int c0 = 0; c0 < nc; c0 += 2) {
 #pragma unroll
-        for (int d = 0; d < D; ++d) {
-            const int j = j0 - d;
-            if (j >= 0) {
-                const double l1 = lr[d][0], l2 = lr[d][1], l3 = lr[d][2], l4 = lr[d][3];
-                const int pj = pr[d];
-                if (j - D >= 0) {
-                    pr[d] = P[(size_t)(j - D) * M1K1];
+        for (int b = 0; b < 2; ++b) {
+            if (c0 + b < nc) {
+                load(lr[b ^ 1], pr[b ^ 1], c0 + b + 1);
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) lr[d][q] = __ldg(&F[(size_t)(j - D) * rs + (size_t)q * M1K1]);
+                for (int d = 0; d < CF; ++d) {
+                    const int j = N - 1 - ((c0 + b) * CF + d);
+                    if (j >= 0) {
+                        const int pj = pr[b][d];
+                        double w0 = x[(size_t)j * st];
+                        // oldest values first: without an interchange at row j+1 only w1 is new
+                        w0 = fma(-lr[b][d][3], w4, w0);
+                        w0 = fma(-lr[b][d][2], w3, w0);
+                        w0 = fma(-lr[b][d][1], w2, w0);
+                        w0 = fma(-lr[b][d][0], w1, w0);
+                        if (pj == 1) { double q = w0; w0 = w1; w1 = q; }
+                        else if (pj == 2) { double q = w0; w0 = w2; w2 = q; }
+                        else if (pj == 3) { double q = w0; w0 = w3; w3 = q; }
+                        else if (pj == 4) { double q = w0; w0 = w4; w4 = q; }
+                        if (j + 4 < N) x[(size_t)(j + 4) * st] = w4;   // x_{j+4} is final
+                        w4 = w3; w3 = w2; w2 = w1; w1 = w0;
+                    }
                 }
-                double w0 = x[(size_t)j * st];
-                // oldest values first: without an interchange at row j+1 only w1 is new
-                w0 = fma(-l4, w4, w0);
-                w0 = fma(-l3, w3, w0);
-                w0 = fma(-l2, w2, w0);
-                w0 = fma(-l1, w1, w0);
-                if (pj == 1) { double q = w0; w0 = w1; w1 = q; }
-                else if (pj == 2) { double q = w0; w0 = w2; w2 = q; }
-                else if (pj == 3) { double q = w0; w0 = w3; w3 = q; }
-                else if (pj == 4) { double q = w0; w0 = w4; w4 = q; }
-                if (j + 4 < N) x[(size_t)(j + 4) * st] = w4;   // x_{j+4} is final
-                w4 = w3; w3 = w2; w2 = w1; w1 = w0;
             }
         }
     }
@@ -107,19 +118,7 @@ __device__ __forceinline__ void smem_band_solve_T(double2* col, int T, int t, in
     if (N > 3) x[(size_t)3 * st] = w4;
 }
 
-// (D1^T v)(c) for column t of smem array C ([N][T]): gather over the rows whose stencil
-// holds c, from the host-built table (row, weight) padded with zero weights.
-__device__ __forceinline__ double2 sdrowT(const double2* C, const int* __restrict__ trow,
-                                          const double* __restrict__ tw, int ntab, int c, int T, int t) {
-    double2 s = make_double2(0.0, 0.0);
-    for (int e = 0; e < ntab; ++e) {
-        const double w = __ldg(&tw[c * ntab + e]);
-        const double2 v = C[__ldg(&trow[c * ntab + e]) * T + t];
-        s.x = fma(w, v.x, s.x);
-        s.y = fma(w, v.y, s.y);
-    }
-    return s;
-}
+constexpr int kAdjChunkF = 4, kAdjChunkB = 2;
 
 struct PCAdjArgs {
     const double2* ubar_new;   // adjoint of u^{i+1}
@@ -142,7 +141,14 @@ struct PCAdjArgs {
 
 // Adjoint of k_pc (steps 2-5 of Sec. 3.2), phases in reverse order.  Shared memory as in
 // k_pc: C0 scalar column, C1..C3 vector columns, [N][T] each.
-__global__ void __launch_bounds__(256) k_pc_adj(PCAdjArgs a, Geo g, int T) {
+// Bound by latency and the FP64 pipe in turn (three substitutions of N rows, one DFMA per 64 cycles
+// and warp).  The element loops run over the real and imaginary parts, each thread staying with its
+// mode, divisions by dt are taken once, and ubar and u_prev's adjoint are written by the warps that
+// idle during the last substitution: 561 -> 419 us at N_r = 96, M = 32, K = 64.  The transposed
+// stencils stay FP64 sums in table order: the Poisson substitutions that follow magnify a rounding
+// of their input by up to 10^7, so fixed point (391 us) moves the wall rows of the result by 1e-9.
+template <int NTH>
+__global__ void __launch_bounds__(NTH, 512 / NTH) k_pc_adj(PCAdjArgs a, Geo g, int T) {
     extern __shared__ double2 sm[];
     const int N = g.N;
     const int items = N * T;
@@ -151,6 +157,7 @@ __global__ void __launch_bounds__(256) k_pc_adj(PCAdjArgs a, Geo g, int T) {
     double2* C2 = C1 + items;
     double2* C3 = C2 + items;
     double2* Cv[3] = {C1, C2, C3};
+    double *D0 = reinterpret_cast<double*>(C0), *D1 = D0 + 2 * items, *D2 = D1 + 2 * items, *D3 = D2 + 2 * items;
     const int mode0 = blockIdx.x * T;
     const int nT = min(T, g.nmode - mode0);
     const size_t per_set = (size_t)N * kBands * g.M1K1;
@@ -160,13 +167,22 @@ __global__ void __launch_bounds__(256) k_pc_adj(PCAdjArgs a, Geo g, int T) {
         m = mode / g.nk;
         k = mode - m * g.nk - g.K;
     };
+    // T divides the block size (k_pc): the modes of this thread in the element loops (tq) and in
+    // the stencil loops (ts, part)
+    const int tq = threadIdx.x % T, jstep = blockDim.x / T;
+    const bool in = tq < nT;
+    const int ts = threadIdx.x % (2 * T) >> 1, part = threadIdx.x & 1;
+    const bool ins = ts < nT;
+    int ms, ks;
+    minfo(ts, ms, ks);
+    const double mms = g.mp * ms, kks = (part ? 1 : -1) * (g.kz * ks);   // i k of the other part: kks times it
 
     // G': u*bar = ubar_new; phibar = -grad_h^T ubar_new
-    for (int idx = threadIdx.x; idx < items; idx += blockDim.x) {
-        const int j = idx / T, t = idx - (idx / T) * T;
+    for (int j = threadIdx.x / T; j < N; j += jstep) {
+        const int idx = j * T + tq;
         double2 v0 = make_double2(0.0, 0.0), v1 = v0, v2 = v0;
-        if (t < nT) {
-            const size_t e = (size_t)j * g.nmode + mode0 + t;
+        if (in) {
+            const size_t e = (size_t)j * g.nmode + mode0 + tq;
             v0 = a.ubar_new[e];
             v1 = a.ubar_new[g.S + e];
             v2 = a.ubar_new[2 * g.S + e];
@@ -176,28 +192,25 @@ __global__ void __launch_bounds__(256) k_pc_adj(PCAdjArgs a, Geo g, int T) {
         C3[idx] = v2;
     }
     __syncthreads();
-    // grad_h^T g = D1^T(g_+ + g_-) - m m_p (g_+ - g_-)/r - i k k_z g_z  (into C0, negated)
-    auto gradT = [&](int j, int t) {
-        int m, k;
-        minfo(t, m, k);
-        const double2 dp = sdrowT(C1, a.trow, a.tw, a.ntab, j, T, t);
-        const double2 dm = sdrowT(C2, a.trow, a.tw, a.ntab, j, T, t);
-        const double2 gp = C1[j * T + t], gm = C2[j * T + t], gz = C3[j * T + t];
-        const double mm = g.mp * m * a.ir[j], kk = g.kz * k;
-        double2 o;
-        o.x = dp.x + dm.x - mm * (gp.x - gm.x) + kk * gz.y;
-        o.y = dp.y + dm.y - mm * (gp.y - gm.y) - kk * gz.x;
+    // (D1^T f)(c) on the real or imaginary part i of this thread: gather over the rows whose stencil
+    // holds c, from the host-built table (row, weight) padded with zero weights
+    auto dT = [&](const double* f, int c) {
+        double o = 0.0;
+        for (int e = 0; e < a.ntab; ++e)
+            o = fma(__ldg(&a.tw[c * a.ntab + e]), f[__ldg(&a.trow[c * a.ntab + e]) * 2 * T], o);
         return o;
     };
-    for (int idx = threadIdx.x; idx < items; idx += blockDim.x) {
-        const int j = idx / T, t = idx - (idx / T) * T;
-        double2 o = make_double2(0.0, 0.0);
-        if (t < nT) {
-            const double2 q = gradT(j, t);
-            o = make_double2(-q.x, -q.y);
+    const int cs = threadIdx.x % (2 * T), sstep = blockDim.x / (2 * T);
+    // grad_h^T g = D1^T(g_+ + g_-) - m m_p (g_+ - g_-)/r - i k k_z g_z, negated, into C0
+    auto gradT = [&] {
+        for (int j = threadIdx.x / (2 * T); j < N; j += sstep) {
+            const int i = j * 2 * T + cs;
+            double o = 0.0;
+            if (ins) o = -(dT(D1 + cs, j) + dT(D2 + cs, j) - mms * __ldg(&a.ir[j]) * (D1[i] - D2[i]) - kks * D3[i ^ 1]);
+            D0[i] = o;
         }
-        C0[idx] = o;
-    }
+    };
+    gradT();
     __syncthreads();
     // F': bbar = P^{-T} phibar, wall rows carry no dependence
     if (threadIdx.x < 2 * nT) {
@@ -205,8 +218,8 @@ __global__ void __launch_bounds__(256) k_pc_adj(PCAdjArgs a, Geo g, int T) {
         int m, k;
         minfo(t, m, k);
         const size_t mk = (size_t)m * g.K1 + (k < 0 ? -k : k);
-        smem_band_solve_T(C0, T, t, part, N, a.fac + (size_t)kSetP * per_set + mk,
-                          a.piv + (size_t)kSetP * N * g.M1K1 + mk, g.M1K1);
+        smem_band_solve_T<kAdjChunkF, kAdjChunkB>(C0, T, t, part, N, a.fac + (size_t)kSetP * per_set + mk,
+                                                  a.piv + (size_t)kSetP * N * g.M1K1 + mk, g.M1K1);
     }
     __syncthreads();
     for (int t = threadIdx.x; t < T; t += blockDim.x) {
@@ -215,21 +228,14 @@ __global__ void __launch_bounds__(256) k_pc_adj(PCAdjArgs a, Geo g, int T) {
     }
     __syncthreads();
     // E': u*bar += div_h^T bbar:  t = D1^T b + b/r;  +: t/2 + m m_p b/(2r), -: t/2 - .., z: -i k k_z b
-    for (int idx = threadIdx.x; idx < items; idx += blockDim.x) {
-        const int j = idx / T, t = idx - (idx / T) * T;
-        if (t >= nT) continue;
-        int m, k;
-        minfo(t, m, k);
-        const double ir = a.ir[j];
-        const double2 d = sdrowT(C0, a.trow, a.tw, a.ntab, j, T, t);
-        const double2 b = C0[idx];
-        const double2 tt = make_double2(d.x + b.x * ir, d.y + b.y * ir);
-        const double mm = 0.5 * g.mp * m * ir, kk = g.kz * k;
-        double2 v;
-        v = C1[idx]; v.x += 0.5 * tt.x + mm * b.x; v.y += 0.5 * tt.y + mm * b.y; C1[idx] = v;
-        v = C2[idx]; v.x += 0.5 * tt.x - mm * b.x; v.y += 0.5 * tt.y - mm * b.y; C2[idx] = v;
-        v = C3[idx]; v.x += kk * b.y; v.y -= kk * b.x; C3[idx] = v;
-    }
+    if (ins)
+        for (int j = threadIdx.x / (2 * T); j < N; j += sstep) {
+            const int i = j * 2 * T + cs;
+            const double ir = __ldg(&a.ir[j]), b = D0[i], tt = dT(D0 + cs, j) + b * ir, mm = 0.5 * mms * ir;
+            D1[i] += 0.5 * tt + mm * b;
+            D2[i] += 0.5 * tt - mm * b;
+            D3[i] -= kks * D0[i ^ 1];
+        }
     __syncthreads();
     // D': rhsbar_c = H_c^{-T} u*bar_c; wall rows of rhs are constants
     if (threadIdx.x < 6 * nT) {
@@ -239,8 +245,8 @@ __global__ void __launch_bounds__(256) k_pc_adj(PCAdjArgs a, Geo g, int T) {
         minfo(t, m, k);
         const size_t mk = (size_t)m * g.K1 + (k < 0 ? -k : k);
         const int set = kSetHp + c;
-        smem_band_solve_T(Cv[c], T, t, part, N, a.fac + (size_t)set * per_set + mk,
-                          a.piv + (size_t)set * N * g.M1K1 + mk, g.M1K1);
+        smem_band_solve_T<kAdjChunkF, kAdjChunkB>(Cv[c], T, t, part, N, a.fac + (size_t)set * per_set + mk,
+                                                  a.piv + (size_t)set * N * g.M1K1 + mk, g.M1K1);
     }
     __syncthreads();
     for (int t = threadIdx.x; t < T; t += blockDim.x)
@@ -250,75 +256,58 @@ __global__ void __launch_bounds__(256) k_pc_adj(PCAdjArgs a, Geo g, int T) {
         }
     __syncthreads();
     // C': ubar += (4/(2dt)) rhsbar, up_bar = -rhsbar/(2dt); p*bar = -grad_h^T rhsbar (C0)
-    for (int idx = threadIdx.x; idx < items; idx += blockDim.x) {
-        const int j = idx / T, t = idx - (idx / T) * T;
-        double2 o = make_double2(0.0, 0.0);
-        if (t < nT) {
-            const size_t e = (size_t)j * g.nmode + mode0 + t;
-            for (int c = 0; c < 3; ++c) {
-                const size_t ec = (size_t)c * g.S + e;
-                const double2 rb = Cv[c][idx];
-                double2 ub = a.ubar_cur ? a.ubar_cur[ec] : make_double2(0.0, 0.0);
-                ub.x += 2.0 / dt * rb.x;
-                ub.y += 2.0 / dt * rb.y;
-                a.u_out[ec] = ub;
-                a.up_out[ec] = make_double2(-rb.x / (2.0 * dt), -rb.y / (2.0 * dt));
-            }
-            const double2 q = gradT(j, t);
-            o = make_double2(-q.x, -q.y);
-        }
-        C0[idx] = o;
-    }
+    gradT();
     __syncthreads();
-    // NNbar = -rhsbar (in place)
-    for (int idx = threadIdx.x; idx < 3 * items; idx += blockDim.x) {
-        double2* C = Cv[idx / items];
-        const int r = idx % items;
-        C[r] = make_double2(-C[r].x, -C[r].y);
-    }
-    __syncthreads();
-    // B': bpbar = P^{-T} p*bar
+    // B': bpbar = P^{-T} p*bar.  Meanwhile the warps without a substitution write ubar and up_bar.
+    const int helper0 = ((2 * nT + 31) / 32) * 32;
     if (threadIdx.x < 2 * nT) {
         const int t = threadIdx.x >> 1, part = threadIdx.x & 1;
         int m, k;
         minfo(t, m, k);
         const size_t mk = (size_t)m * g.K1 + (k < 0 ? -k : k);
-        smem_band_solve_T(C0, T, t, part, N, a.fac + (size_t)kSetP * per_set + mk,
-                          a.piv + (size_t)kSetP * N * g.M1K1 + mk, g.M1K1);
+        smem_band_solve_T<kAdjChunkF, kAdjChunkB>(C0, T, t, part, N, a.fac + (size_t)kSetP * per_set + mk,
+                                                  a.piv + (size_t)kSetP * N * g.M1K1 + mk, g.M1K1);
+    } else if (threadIdx.x >= helper0 && in) {   // helper0 < blockDim.x, and a multiple of T
+        const double c2 = 2.0 / dt, ch = 1.0 / (2.0 * dt);
+        for (int j = (threadIdx.x - helper0) / T; j < N; j += ((int)blockDim.x - helper0) / T) {
+            const size_t e = (size_t)j * g.nmode + mode0 + tq;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const size_t ec = (size_t)c * g.S + e;
+                const double2 rb = Cv[c][j * T + tq];
+                double2 ub = a.ubar_cur ? a.ubar_cur[ec] : make_double2(0.0, 0.0);
+                ub.x += c2 * rb.x;
+                ub.y += c2 * rb.y;
+                a.u_out[ec] = ub;
+                a.up_out[ec] = make_double2(-rb.x * ch, -rb.y * ch);
+            }
+        }
     }
     __syncthreads();
-    // A': interior rows b_p = div_h(-NN): NNbar += div_h^T(-bpbar_interior);
+    // A': interior rows b_p = div_h(-NN): NNbar = -rhsbar + div_h^T(-bpbar_interior);
     //     wall rows b_p = -NN_r + 2 Lap_r(u) - Lap_r(u_prev) (not the (0,0) row at r_o)
-    for (int idx = threadIdx.x; idx < items; idx += blockDim.x) {
-        const int j = idx / T, t = idx - (idx / T) * T;
-        if (t >= nT) continue;
-        int m, k;
-        minfo(t, m, k);
-        const double ir = a.ir[j];
-        // v = -bpbar on interior rows, 0 on wall rows
-        double2 d = make_double2(0.0, 0.0);
-        for (int e = 0; e < a.ntab; ++e) {
-            const int row = __ldg(&a.trow[j * a.ntab + e]);
-            if (row == 0 || row == N - 1) continue;
-            const double w = __ldg(&a.tw[j * a.ntab + e]);
-            const double2 b = C0[row * T + t];
-            d.x -= w * b.x;
-            d.y -= w * b.y;
+    if (ins)
+        for (int j = threadIdx.x / (2 * T); j < N; j += sstep) {
+            const int i = j * 2 * T + cs;
+            const bool wall = j == 0 || j == N - 1;
+            double d = 0.0;
+            for (int e = 0; e < a.ntab; ++e) {
+                const int row = __ldg(&a.trow[j * a.ntab + e]);
+                if (row == 0 || row == N - 1) continue;
+                d = fma(-__ldg(&a.tw[j * a.ntab + e]), D0[row * 2 * T + cs], d);
+            }
+            const double ir = __ldg(&a.ir[j]), b = D0[i], v = wall ? 0.0 : -b, o = wall ? 0.0 : D0[i ^ 1];
+            const double tt = d + v * ir, mm = 0.5 * mms * ir;
+            double p = 0.5 * tt + mm * v - D1[i], m = 0.5 * tt - mm * v - D2[i];
+            if (wall && !(j == N - 1 && ms == 0 && ks == 0)) {
+                p -= 0.5 * b;
+                m -= 0.5 * b;
+            }
+            D1[i] = p;
+            D2[i] = m;
+            D3[i] = kks * o - D3[i];
         }
-        double2 v = make_double2(0.0, 0.0);
-        if (j > 0 && j < N - 1) v = make_double2(-C0[idx].x, -C0[idx].y);
-        const double2 tt = make_double2(d.x + v.x * ir, d.y + v.y * ir);
-        const double mm = 0.5 * g.mp * m * ir, kk = g.kz * k;
-        double2 q;
-        q = C1[idx]; q.x += 0.5 * tt.x + mm * v.x; q.y += 0.5 * tt.y + mm * v.y;
-        if (j == 0 || (j == N - 1 && !(m == 0 && k == 0))) { q.x -= 0.5 * C0[idx].x; q.y -= 0.5 * C0[idx].y; }
-        C1[idx] = q;
-        q = C2[idx]; q.x += 0.5 * tt.x - mm * v.x; q.y += 0.5 * tt.y - mm * v.y;
-        if (j == 0 || (j == N - 1 && !(m == 0 && k == 0))) { q.x -= 0.5 * C0[idx].x; q.y -= 0.5 * C0[idx].y; }
-        C2[idx] = q;
-        q = C3[idx]; q.x += kk * v.y; q.y -= kk * v.x;
-        C3[idx] = q;
-    }
+    __syncthreads();
     // wall Laplacian transposes: column c of the wall stencils receives, for wall row jw with
     // value w: 1/2 (D2[jw][c] + D1[jw][c]/r_jw) w (+ 1/2 diag_pm w at c = jw), times 2 into
     // ubar and -1 into up_bar.  One thread per (column, mode) of the two wall stencils.
@@ -595,7 +584,7 @@ __global__ void k_band_solve_gT(double2* __restrict__ x, const double* __restric
     const size_t mk = (size_t)m * g.K1 + (k < 0 ? -k : k);
     const size_t per_set = (size_t)g.N * kBands * g.M1K1;
     const int set = set0 + fld;
-    smem_band_solve_T(x + (size_t)fld * g.S, g.nmode, mode, part, g.N, fac + (size_t)set * per_set + mk,
+    smem_band_solve_T<kAdjChunkF, kAdjChunkB>(x + (size_t)fld * g.S, g.nmode, mode, part, g.N, fac + (size_t)set * per_set + mk,
                       piv + (size_t)set * g.N * g.M1K1 + mk, g.M1K1);
 }
 
@@ -654,8 +643,7 @@ tc_status launch_adjoint_advance(tc_plan* p, const double2* ubar_new, const doub
         TC_LAUNCHED(p, "k_adjT");
         return TC_OK;
     }
-    int T = p->pc_modes > 0 ? p->pc_modes : 8;
-    while (T > 1 && (size_t)4 * p->N_r * T * sizeof(double2) > 96 * 1024) T /= 2;
+    const int T = pc_modes(p, g.nmode);
     PCAdjArgs a;
     a.ubar_new = ubar_new; a.ubar_cur = ubar_cur; a.Nbar_cur = Nbar_cur;
     a.u_out = u_out; a.up_out = up_out; a.N_out = N_out; a.Np_out = Np_out;
@@ -663,12 +651,13 @@ tc_status launch_adjoint_advance(tc_plan* p, const double2* ubar_new, const doub
     a.trow = p->d_d1t_row; a.tw = p->d_d1t_w; a.ntab = p->d1t_n;
     a.fac = p->d_fac; a.piv = p->d_piv;
     const size_t sm = (size_t)4 * p->N_r * T * sizeof(double2);
-    int threads = ((6 * T + 31) / 32) * 32;
-    if (threads < 128) threads = 128;
-    if (threads > 256) threads = 256;
-    TC_CUDA(p, cudaFuncSetAttribute(k_pc_adj, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     const int slot = prof_begin(p, kKPCAdj, s);
-    k_pc_adj<<<ablocks(g.nmode, T), threads, sm, s>>>(a, g, T);
+    auto run = [&](auto kern, int nth) -> tc_status {
+        TC_CUDA(p, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        kern<<<ablocks(g.nmode, T), nth, sm, s>>>(a, g, T);
+        return TC_OK;
+    };
+    TC_TRY_STATUS(T <= 8 ? run(k_pc_adj<128>, 128) : run(k_pc_adj<256>, 256));
     prof_end(p, slot, s);
     TC_LAUNCHED(p, "k_pc_adj");
     return TC_OK;

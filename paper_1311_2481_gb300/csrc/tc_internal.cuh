@@ -137,8 +137,8 @@ struct tc_plan {
     int2* d_fx_mm = nullptr;
     int fx_emm = 0;
     int4* d_fx_ir = nullptr;
-    int2* d_fx_w1 = nullptr;
-    int* d_fx_ew = nullptr;
+    int2* d_fx_w1 = nullptr;     // fixed-point weights of the radial stencil
+    int* d_fx_ew = nullptr;      // their exponents per row
     // non-finite flag: mapped pinned host memory that the update kernels set when they write
     // a NaN/Inf into the state; tc_step reports and clears it
     int* h_nonfinite = nullptr;
@@ -231,6 +231,7 @@ tc_status launch_nl_post32(tc_plan* p, const double2* u, double2* N, char* ws, c
 size_t mean00_part_doubles(const tc_plan* p);
 tc_status launch_mean00_part(tc_plan* p, const double2* u, char* ws, cudaStream_t s);
 tc_status launch_mean00_fin(tc_plan* p, double2* N, char* ws, cudaStream_t s);
+int pc_modes(const tc_plan* p, int nmode);                    // modes per block of the fused steps 2-5
 tc_status launch_solve(tc_plan* p, int set, const double2* rhs, double2* x, cudaStream_t s);
 tc_status launch_advance(tc_plan* p, const double2* u, double2* u_prev, const double2* Ncur,
                          double2* N_prev, double2* p_out, double2* u_out, char* ws,

@@ -16,7 +16,6 @@
 
 #include "tc_internal.cuh"
 #include "tc_solve_core.cuh"
-#include "tc_fx.cuh"
 
 namespace tc {
 
@@ -126,67 +125,6 @@ __device__ __forceinline__ double2 lap_pm(const double2* __restrict__ u, const P
     return make_double2(d2.x + ir * d1.x + diag * v.x, d2.y + ir * d1.y + diag * v.y);
 }
 
-// The element loops of k_pc with a radial stencil: body(j, i, d, pre(j)) for the real and imaginary
-// parts of all rows of the block's modes, i the index of the part's double in the [N][T] arrays
-// in shared memory, d the radial derivative at row j of F (of F + F2).  pre: the body's load from
-// device memory, issued ahead of the stencil.
-// FX: rows 4 .. N - 5 in tiles of kTileRows rows per thread in fixed point, the four next to each
-// wall in FP64 one per thread, by the other half of the block first.  Otherwise all in FP64.
-// The FP64 pipe takes 16 cycles of its SM per warp instruction, and k_pc issues 5900 of them per
-// 16 modes of 64 rows with FP64 stencils, 4400 without: 252 -> 219 us at N_r = 64, M = 32, K = 64
-// (8 rows per tile: 230 us, fewer threads with work and more rows left to FP64).
-constexpr int kTileRows = 4;   // rows per thread, here and in the split path
-template <bool FX, bool PAIR, class Pre, class Body>
-__device__ __forceinline__ void stencil_rows(const PCArgs& a, const double2* F, const double2* F2, int N, int T, Pre pre,
-                                             Body body) {
-    using namespace fx;
-    const int c = threadIdx.x % (2 * T), step = blockDim.x / (2 * T), st = 2 * T;
-    const double* f = reinterpret_cast<const double*>(F) + c;
-    const double* f2 = reinterpret_cast<const double*>(F2) + c;
-    auto fp64 = [&](int j, int c0) {
-        double o = 0.0;
-#pragma unroll
-        for (int q = 0; q < kStencil; ++q) {
-            const int n = (c0 + q) * st;
-            o = fma(__ldg(&a.w1[j * kStencil + q]), PAIR ? f[n] + f2[n] : f[n], o);
-        }
-        return o;
-    };
-    if (FX) {
-        for (int j0 = 4 + kTileRows * (threadIdx.x / st); j0 < N - 4; j0 += kTileRows * step) {
-            double d[kTileRows], g[kTileRows];
-#pragma unroll
-            for (int i = 0; i < kTileRows; ++i) g[i] = pre(min(j0 + i, N - 1));
-            {
-                Tile<kTileRows> X;
-                double v[kTileRows + 8], v2[kTileRows + 8];
-#pragma unroll
-                for (int i = 0; i < kTileRows + 8; ++i) {
-                    const int j = j0 - 4 + i;
-                    v[i] = j < N ? f[j * st] : 0.0;
-                    if (PAIR) v2[i] = j < N ? f2[j * st] : 0.0;
-                }
-                if (PAIR) X.load(v, v2);
-                else X.load(v);
-#pragma unroll
-                for (int i = 0; i < kTileRows; ++i) {
-                    const int j = min(j0 + i, N - 5);
-                    d[i] = X.far(i) ? fp64(j, j - 4) : X.row(i, a.fw + j * kStencil, __ldg(&a.few[j]));
-                }
-            }
-#pragma unroll
-            for (int i = 0; i < kTileRows; ++i)
-                if (j0 + i < N - 4) body(j0 + i, (j0 + i) * st + c, d[i], g[i]);
-        }
-    }
-    const int nw = FX ? min(N, 8) : N;   // FX: rows 0 .. 3 and N - 4 .. N - 1
-    for (int i = (threadIdx.x ^ (blockDim.x >> 1)) / st; i < nw; i += step) {
-        const int j = !FX || N < 8 || i < 4 ? i : N - 8 + i;
-        const double g = pre(j);
-        body(j, j * st + c, fp64(j, __ldg(&a.col0[j])), g);
-    }
-}
-
 // Steps 2-5 of Sec. 3.2 for the T modes of this block: pressure prediction (Eq. pressure
 // with the Neumann rows of Eq. ppBC), velocity prediction (Eq. vel), correction potential
 // (Eq. correction) and update (Eq. update).
@@ -246,7 +184,26 @@ __global__ void __launch_bounds__(NTH, 512 / NTH) k_pc(PCArgs a, Geo g, int T) {
     const double mms = g.mp * ms, kks = (part ? 1 : -1) * (g.kz * ks);   // i k of the other part: kks times it
     // A2: pressure right-hand side into C0
     auto ir = [&](int j) { return __ldg(&a.ir[j]); };
-    stencil_rows<FX, true>(a, C1, C2, N, T, ir, [&](int j, int i, double d, double irj) {
+    auto d1 = [&](const double* f, int j) {   // FP64 stencil at row j
+        const int c0 = __ldg(&a.col0[j]);
+        double o = 0.0;
+#pragma unroll
+        for (int q = 0; q < kStencil; ++q) o = fma(__ldg(&a.w1[j * kStencil + q]), f[(c0 + q) * 2 * T], o);
+        return o;
+    };
+    auto d1s = [&](const double* f, const double* f2, int j) {   // of f + f2
+        const int c0 = __ldg(&a.col0[j]);
+        double o = 0.0;
+#pragma unroll
+        for (int q = 0; q < kStencil; ++q) {
+            const int n = (c0 + q) * 2 * T;
+            o = fma(__ldg(&a.w1[j * kStencil + q]), f[n] + f2[n], o);
+        }
+        return o;
+    };
+    auto slow0 = [&](int j, int c) { return d1(D0 + c, j); };
+    auto slow12 = [&](int j, int c) { return d1s(D1 + c, D2 + c, j); };
+    stencil_rows<4, FX, true>(a.fw, a.few, C1, C2, N, T, slow12, ir, [&](int j, int i, double d, double irj) {
         double out = 0.0;
         const double n = D1[i], m = D2[i];
         if (j == 0 || j == N - 1) {
@@ -318,7 +275,7 @@ __global__ void __launch_bounds__(NTH, 512 / NTH) k_pc(PCArgs a, Geo g, int T) {
     __syncthreads();
     if (sp) spike_combine(a, g, C0, 1, kSetP, T, nT, mode0, Xr);
     // C: velocity right-hand sides: subtract grad_h p* on interior rows; p <- p* (commit)
-    stencil_rows<FX, false>(a, C0, nullptr, N, T, ir, [&](int j, int i, double d, double irj) {
+    stencil_rows<4, FX, false>(a.fw, a.few, C0, nullptr, N, T, slow0, ir, [&](int j, int i, double d, double irj) {
         if (!ins) return;
         const double pv = D0[i];
         if (a.commit) reinterpret_cast<double*>(a.p)[2 * ((size_t)j * g.nmode + modes) + part] = pv;
@@ -369,7 +326,7 @@ __global__ void __launch_bounds__(NTH, 512 / NTH) k_pc(PCArgs a, Geo g, int T) {
         }
     }
     // E: div_h u* into C0 (homogeneous Neumann / Dirichlet rows)
-    stencil_rows<FX, true>(a, C1, C2, N, T, ir, [&](int j, int i, double d, double irj) {
+    stencil_rows<4, FX, true>(a.fw, a.few, C1, C2, N, T, slow12, ir, [&](int j, int i, double d, double irj) {
         double out = 0.0;
         if (ins && j > 0 && j < N - 1) {
             const double hr = 0.5 * irj, vp = D1[i], vm = D2[i];
@@ -396,7 +353,7 @@ __global__ void __launch_bounds__(NTH, 512 / NTH) k_pc(PCArgs a, Geo g, int T) {
     bool bad = false;
     double* pw = a.commit && ins ? reinterpret_cast<double*>(a.p) + 2 * (size_t)modes + part : nullptr;
     auto p0 = [&](int j) { return pw ? pw[2 * (size_t)j * g.nmode] : 0.0; };
-    stencil_rows<FX, false>(a, C0, nullptr, N, T, p0, [&](int j, int i, double d, double p) {
+    stencil_rows<4, FX, false>(a.fw, a.few, C0, nullptr, N, T, slow0, p0, [&](int j, int i, double d, double p) {
         if (!ins) return;
         const size_t e = 2 * ((size_t)j * g.nmode + modes) + part;
         const double f = D0[i], tf = mms * __ldg(&a.ir[j]) * f;
@@ -900,7 +857,7 @@ size_t diag_red_doubles(const tc_plan* p) {
 // Modes per block of the fused kernel (a power of two): the most (up to 16) that still give every SM a block,
 // within 96 KB of shared memory for the four columns.  Each block's time is its substitution
 // chain, so more modes per block cost little while the blocks fit one wave.
-static int pc_modes(const tc_plan* p, int nmode) {
+int pc_modes(const tc_plan* p, int nmode) {
     int T = 16;
     if (p->pc_modes > 0)
         while (T > p->pc_modes) T /= 2;   // a power of two: it divides the block size
@@ -996,6 +953,13 @@ static tc_status launch_advance_split(tc_plan* p, const double2* u, double2* u_p
     return TC_OK;
 }
 
+// Fixed-point stencils in a launch of blocks of T modes, while enough warps share the FP64 pipe (14
+// per SM: 219 against 252 us for k_pc, N_r = 64, M = 32, K = 64); with fewer than 8 per SM their
+// conversions take longer than the FP64 FMAs (2 per SM: 90 against 61 us, N_r = 32, M = 8, K = 16).
+static bool fx_stencils(const tc_plan* p, int nmode, int T) {
+    return (size_t)blocks_for(nmode, T) * (T <= 8 ? 128 : 256) >= (size_t)256 * p->num_sms;
+}
+
 tc_status launch_advance(tc_plan* p, const double2* u, double2* u_prev, const double2* Ncur,
                          double2* N_prev, double2* p_out, double2* u_out, char* ws, bool commit,
                          cudaStream_t s, int ma, int mb) {
@@ -1028,10 +992,7 @@ tc_status launch_advance(tc_plan* p, const double2* u, double2* u_prev, const do
         kern<<<blocks_for(g.mhi - g.mlo, T), nth, sm, s>>>(a, g, T);
         return TC_OK;
     };
-    // fixed-point stencils while enough warps share the FP64 pipe (14 per SM: 219 against 252 us,
-    // N_r = 64, M = 32, K = 64); with fewer than 8 per SM their conversions take longer than the
-    // FP64 FMAs (2 per SM: 90 against 61 us, N_r = 32, M = 8, K = 16)
-    const bool fxs = (size_t)blocks_for(g.mhi - g.mlo, T) * (T <= 8 ? 128 : 256) >= (size_t)256 * p->num_sms;
+    const bool fxs = fx_stencils(p, g.mhi - g.mlo, T);
     if (T <= 8) TC_TRY_STATUS(fxs ? run(k_pc<128, true>, 128) : run(k_pc<128, false>, 128));
     else TC_TRY_STATUS(fxs ? run(k_pc<256, true>, 256) : run(k_pc<256, false>, 256));
     prof_end(p, slot, s);

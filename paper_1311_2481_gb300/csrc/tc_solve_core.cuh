@@ -4,6 +4,7 @@
 #pragma once
 
 #include "tc_internal.cuh"
+#include "tc_fx.cuh"
 
 namespace tc {
 
@@ -258,19 +259,57 @@ __device__ __forceinline__ void smem_band_solve_c(double2* col, int T, int t, in
     }
 }
 
-// D1 of column t of smem array C ([N][T]) at row j
-__device__ __forceinline__ double2 sdrow(const double2* C, const double* __restrict__ w1,
-                                         const int* __restrict__ col0, int j, int T, int t) {
-    const int c0 = col0[j];
-    double2 s = make_double2(0.0, 0.0);
+// The element loops of k_pc with a radial stencil: body(j, i, d, pre(j)) for the real
+// and imaginary parts of all rows of the block's modes, i the index of the part's double in the
+// [N][T] arrays in shared memory, d the stencil at row j of F (of F + F2).  pre: the body's load
+// from device memory, issued ahead of the stencil.  slow(j, c): the FP64 sum at row j of column c.
+// FX: all but the ZONE rows next to each wall in tiles of kTileRows rows per thread in fixed point
+// (weights fw, few), the others one per thread, by the other half of the block first.  Otherwise
+// all in FP64.
+// The FP64 pipe takes 16 cycles of its SM per warp instruction, and k_pc issues 5900 of them per
+// 16 modes of 64 rows with FP64 stencils, 4400 without: 252 -> 219 us at N_r = 64, M = 32, K = 64
+// (8 rows per tile: 230 us, fewer threads with work and more rows left to FP64).
+constexpr int kTileRows = 4;   // rows per thread, here and in the split path
+template <int ZONE, bool FX, bool PAIR, class Slow, class Pre, class Body>
+__device__ __forceinline__ void stencil_rows(const int2* __restrict__ fw, const int* __restrict__ few, const double2* F,
+                                             const double2* F2, int N, int T, Slow slow, Pre pre, Body body) {
+    using namespace fx;
+    const int c = threadIdx.x % (2 * T), step = blockDim.x / (2 * T), st = 2 * T;
+    if (FX) {
+        const double* f = reinterpret_cast<const double*>(F) + c;
+        const double* f2 = reinterpret_cast<const double*>(F2) + c;
+        for (int j0 = ZONE + kTileRows * (threadIdx.x / st); j0 < N - ZONE; j0 += kTileRows * step) {
+            double d[kTileRows], g[kTileRows];
 #pragma unroll
-    for (int q = 0; q < kStencil; ++q) {
-        const double wq = __ldg(&w1[j * kStencil + q]);
-        const double2 v = C[(c0 + q) * T + t];
-        s.x = fma(wq, v.x, s.x);
-        s.y = fma(wq, v.y, s.y);
+            for (int i = 0; i < kTileRows; ++i) g[i] = pre(min(j0 + i, N - 1));
+            {
+                Tile<kTileRows> X;
+                double v[kTileRows + 8], v2[kTileRows + 8];
+#pragma unroll
+                for (int i = 0; i < kTileRows + 8; ++i) {
+                    const int j = j0 - 4 + i;
+                    v[i] = j < N ? f[j * st] : 0.0;
+                    if (PAIR) v2[i] = j < N ? f2[j * st] : 0.0;
+                }
+                if (PAIR) X.load(v, v2);
+                else X.load(v);
+#pragma unroll
+                for (int i = 0; i < kTileRows; ++i) {
+                    const int j = min(j0 + i, N - ZONE - 1);
+                    d[i] = X.far(i) ? slow(j, c) : X.row(i, fw + j * kStencil, __ldg(&few[j]));
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < kTileRows; ++i)
+                if (j0 + i < N - ZONE) body(j0 + i, (j0 + i) * st + c, d[i], g[i]);
+        }
     }
-    return s;
+    const int nw = FX ? min(N, 2 * ZONE) : N;
+    for (int i = (threadIdx.x ^ (blockDim.x >> 1)) / st; i < nw; i += step) {
+        const int j = !FX || N < 2 * ZONE || i < ZONE ? i : N - 2 * ZONE + i;
+        const double g = pre(j);
+        body(j, j * st + c, slow(j, c), g);
+    }
 }
 
 }  // namespace tc

@@ -37,3 +37,28 @@ def test_steps_match_oracle(N_r, m_p, split, kind):
     for k in ("u", "p"):
         a, b = getattr(st, k).cpu().numpy(), getattr(ref, k)
         assert np.linalg.norm(a - b) <= 1e-10 * np.linalg.norm(b), k
+
+
+@pytest.mark.parametrize("N_r,m_p", [(9, 1), (18, 6), (19, 1), (20, 6), (25, 1), (32, 1)])
+def test_adjoint_step_matches_oracle(N_r, m_p):
+    """Blocks of 16 modes with idle warps beside the substitutions, node counts that end within the
+    chunks of factor rows.  The bound of the adjoint steps with fewer modes."""
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    from paper_1311_2481_gb300 import build, tc
+    build.build()
+    cfg = dict(N_r=N_r, M=18, K=64, m_p=m_p, eta=0.5, Re_i=50.0, Re_o=0.0, L_z=LZ, dt=1e-3)
+    ops = O.Operators(O.Params(**cfg))
+    u0 = I.initial_state(ops.r, 18, 64, m_p, LZ, 0.5, 50.0, 0.0, kind="broadband", amp=1e-2, seed=4)
+    st_o = O.step(ops, O.cold_state(u0))
+    y = [I.random_spectral((3,) + ops.prm.shape(), seed=s) for s in (21, 22, 23)]
+    ref = O.adjoint_step(ops, st_o, *y)
+    plan = tc.Plan(**cfg)
+    st = tc.State(plan, torch.from_numpy(st_o.u).cuda())
+    st.u_prev.copy_(torch.from_numpy(st_o.u_prev))
+    st.N_prev.copy_(torch.from_numpy(st_o.N_prev))
+    st.started = True
+    bar = tc.StateBar(*[torch.from_numpy(v).cuda() for v in y])
+    plan.adjoint_step(st, bar)
+    for got, want in zip((bar.u, bar.u_prev, bar.N_prev), ref):
+        assert np.linalg.norm(got.cpu().numpy() - want) <= 1e-11 * np.linalg.norm(want)
