@@ -47,9 +47,19 @@ struct PCArgs {
 
 constexpr int kChunkF = 4, kChunkB = 2;   // rows of factors per register chunk (3, 2: 2 % and 4, 3: 9 % slower k_pc)
 
+// CH: chunks; the row by row ring of kPCDepth rows reaches further ahead, which counts where a launch
+// has few warps and nothing else covers a load (N_r = 160, M = 8, K = 16: k_pc 223 against 239 us)
+template <bool CH>
+__device__ __forceinline__ void band_solve(double2* col, int T, int t, int part, int N, const double* __restrict__ F,
+                                           const uint8_t* __restrict__ P, int M1K1) {
+    if (CH) smem_band_solve_c<kChunkF, kChunkB>(col, T, t, part, N, F, P, M1K1);
+    else smem_band_solve<kPCDepth>(col, T, t, part, N, F, P, M1K1);
+}
+
 // Thread lt of the 4 nT threads of one system solves one half of it for one (mode, part):
 // threads [0, 2nT) rows [0, sh), threads [2nT, 4nT) rows [sh, N), each with the pivoted LU
 // factors of its diagonal block; the column then holds g = (A1^{-1} b1, A2^{-1} b2).
+template <bool CH>
 __device__ __forceinline__ void half_solve(const PCArgs& a, const Geo& g, double2* X, int set, int T, int nT,
                                            int mode0, int lt) {
     const int half = lt >= 2 * nT ? 1 : 0;
@@ -59,7 +69,7 @@ __device__ __forceinline__ void half_solve(const PCArgs& a, const Geo& g, double
     const size_t mk = (size_t)m * g.K1 + (k < 0 ? -k : k);
     const size_t per_set = (size_t)g.N * kBands * g.M1K1;
     const int r0 = half ? g.sh : 0, n = half ? g.N - g.sh : g.sh;
-    smem_band_solve_c<kChunkF, kChunkB>(X + (size_t)r0 * T, T, t, part, n,
+    band_solve<CH>(X + (size_t)r0 * T, T, t, part, n,
                               a.fac2 + (size_t)set * per_set + (size_t)r0 * kBands * g.M1K1 + mk,
                               a.piv2 + ((size_t)set * g.N + r0) * g.M1K1 + mk, g.M1K1);
 }
@@ -229,12 +239,12 @@ __global__ void __launch_bounds__(NTH, 512 / NTH) k_pc(PCArgs a, Geo g, int T) {
     const int helper0 = ((nsolve + 31) / 32) * 32;
     if (threadIdx.x < nsolve) {
         if (sp) {
-            half_solve(a, g, C0, kSetP, T, nT, mode0, threadIdx.x);
+            half_solve<FX>(a, g, C0, kSetP, T, nT, mode0, threadIdx.x);
         } else {
             const int t = threadIdx.x >> 1, part = threadIdx.x & 1;
             const int mode = mode0 + t, m = mode / g.nk, k = mode - m * g.nk - g.K;
             const size_t mk = (size_t)m * g.K1 + (k < 0 ? -k : k);
-            smem_band_solve_c<kChunkF, kChunkB>(C0, T, t, part, N, a.fac + (size_t)kSetP * per_set + mk,
+            band_solve<FX>(C0, T, t, part, N, a.fac + (size_t)kSetP * per_set + mk,
                             a.piv + (size_t)kSetP * N * g.M1K1 + mk, g.M1K1);
         }
     }
@@ -293,14 +303,14 @@ __global__ void __launch_bounds__(NTH, 512 / NTH) k_pc(PCArgs a, Geo g, int T) {
     if (threadIdx.x < nsolve1) {
         if (sp) {
             const int c = threadIdx.x / (4 * nT);
-            half_solve(a, g, C1 + (size_t)c * items, kSetHp + c, T, nT, mode0, threadIdx.x - c * 4 * nT);
+            half_solve<FX>(a, g, C1 + (size_t)c * items, kSetHp + c, T, nT, mode0, threadIdx.x - c * 4 * nT);
         } else {
             const int c = threadIdx.x / (2 * nT), rem = threadIdx.x - c * 2 * nT;
             const int t = rem >> 1, part = rem & 1;
             const int mode = mode0 + t, m = mode / g.nk, k = mode - m * g.nk - g.K;
             const size_t mk = (size_t)m * g.K1 + (k < 0 ? -k : k);
             const int set = kSetHp + c;
-            smem_band_solve_c<kChunkF, kChunkB>(C1 + (size_t)c * items, T, t, part, N, a.fac + (size_t)set * per_set + mk,
+            band_solve<FX>(C1 + (size_t)c * items, T, t, part, N, a.fac + (size_t)set * per_set + mk,
                             a.piv + (size_t)set * N * g.M1K1 + mk, g.M1K1);
         }
     } else if (a.commit && threadIdx.x >= helper1) {
@@ -338,12 +348,12 @@ __global__ void __launch_bounds__(NTH, 512 / NTH) k_pc(PCArgs a, Geo g, int T) {
     // F: phi = P^{-1} div_h u*
     if (threadIdx.x < nsolve) {
         if (sp) {
-            half_solve(a, g, C0, kSetP, T, nT, mode0, threadIdx.x);
+            half_solve<FX>(a, g, C0, kSetP, T, nT, mode0, threadIdx.x);
         } else {
             const int t = threadIdx.x >> 1, part = threadIdx.x & 1;
             const int mode = mode0 + t, m = mode / g.nk, k = mode - m * g.nk - g.K;
             const size_t mk = (size_t)m * g.K1 + (k < 0 ? -k : k);
-            smem_band_solve_c<kChunkF, kChunkB>(C0, T, t, part, N, a.fac + (size_t)kSetP * per_set + mk,
+            band_solve<FX>(C0, T, t, part, N, a.fac + (size_t)kSetP * per_set + mk,
                             a.piv + (size_t)kSetP * N * g.M1K1 + mk, g.M1K1);
         }
     }
@@ -722,7 +732,7 @@ __global__ void __launch_bounds__(128) k_band_solve_s2(const double2* rhs, doubl
     for (int j = threadIdx.x / T; j < N; j += blockDim.x / T)
         sm[j * T + t] = t < nT ? rhs[(size_t)j * g.nmode + mode0 + t] : make_double2(0.0, 0.0);
     __syncthreads();
-    if (threadIdx.x < 4 * nT) half_solve(a, g, sm, set, T, nT, mode0, threadIdx.x);
+    if (threadIdx.x < 4 * nT) half_solve<true>(a, g, sm, set, T, nT, mode0, threadIdx.x);
     __syncthreads();
     spike_combine(a, g, sm, 1, set, T, nT, mode0, reinterpret_cast<double*>(sm + (size_t)N * T));
     if (t < nT)
@@ -871,8 +881,10 @@ int pc_modes(const tc_plan* p, int nmode) {
 tc_status launch_solve(tc_plan* p, int set, const double2* rhs, double2* x, cudaStream_t s) {
     Geo g = geo(p);
     const int prof = set == kSetP ? kKSolveP : kKSolveH;
-    if (p->part_h > 0) {
-        // two partitions: half the chain of substitutions, which bounds this launch
+    if (p->part_h > 0 && g.nmode <= 64 * p->num_sms) {
+        // two partitions: half the chain of substitutions, which bounds a launch of few modes per SM
+        // (55: 103 against 127 us, N_r = 128); with many the coupling's work counts (110: 53 against
+        // 41 us, N_r = 32)
         g.sh = p->part_h;
         PCArgs a{};
         a.fac2 = p->d_fac2; a.piv2 = p->d_piv2; a.spk = p->d_spk; a.rinv = p->d_rinv;
@@ -955,9 +967,11 @@ static tc_status launch_advance_split(tc_plan* p, const double2* u, double2* u_p
 
 // Fixed-point stencils in a launch of blocks of T modes, while enough warps share the FP64 pipe (14
 // per SM: 219 against 252 us for k_pc, N_r = 64, M = 32, K = 64); with fewer than 8 per SM their
-// conversions take longer than the FP64 FMAs (2 per SM: 90 against 61 us, N_r = 32, M = 8, K = 16).
+// conversions take longer than the FP64 FMAs (2 per SM: 90 against 61 us, N_r = 32, M = 8, K = 16),
+// and so they do with few rows, a quarter of which are wall rows (575 against 528 us, N_r = 32,
+// M = 64, K = 128; 754 against 760 at N_r = 48).
 static bool fx_stencils(const tc_plan* p, int nmode, int T) {
-    return (size_t)blocks_for(nmode, T) * (T <= 8 ? 128 : 256) >= (size_t)256 * p->num_sms;
+    return p->N_r >= 48 && (size_t)blocks_for(nmode, T) * (T <= 8 ? 128 : 256) >= (size_t)256 * p->num_sms;
 }
 
 tc_status launch_advance(tc_plan* p, const double2* u, double2* u_prev, const double2* Ncur,

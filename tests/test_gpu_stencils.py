@@ -1,5 +1,5 @@
-"""The radial stencils of steps 2-5 in fixed point, fused (enough modes to share the FP64 pipe) and
-per stage, against the oracle: node counts at the edges of the tiles of rows and of the wall zones,
+"""The radial stencils of steps 2-5 in fixed point, fused (from 48 rows on, with enough modes to share
+the FP64 pipe) and per stage, against the oracle: node counts at the edges of the tiles of rows and of the wall zones,
 an azimuthal symmetry that makes columns fall off steeply, and a field that is zero but for the
 mean flow."""
 import math
@@ -18,7 +18,7 @@ LZ = 2 * math.pi / 3.16
 
 @pytest.mark.parametrize("kind", ["broadband", "zero"])
 @pytest.mark.parametrize("split", [-1, 1])
-@pytest.mark.parametrize("N_r,m_p", [(9, 1), (12, 1), (13, 6), (16, 1), (23, 6), (32, 1)])
+@pytest.mark.parametrize("N_r,m_p", [(9, 1), (12, 1), (13, 6), (16, 1), (23, 6), (32, 1), (49, 6)])
 def test_steps_match_oracle(N_r, m_p, split, kind):
     """Bound: the rounding of the wall Laplacian (weights of order N_r^4) in p, as between any two
     forms of these stages."""
