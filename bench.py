@@ -25,9 +25,9 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 if ROOT not in sys.path:
     sys.path.insert(0, ROOT)
 
-# DRAM bytes (read + write) of one FP64 theta-pass launch at the bench workload, from ncu
-# (58.44 MB read + 2.99 MB written; the H2 lines stay in L2)
-THETA_TRAFFIC = 61.43e6
+# DRAM bytes (read + write) of one theta-pass launch of the FP64 form at the bench workload: not
+# captured for the fixed-point kernel
+THETA_TRAFFIC = None
 CFG2 = dict(N_r=64, M=32, K=64, m_p=1, eta=0.5, Re_i=1000.0, Re_o=0.0, L_z=2 * math.pi / 3.16, dt=5e-4)
 # mid-size case for profiling (inputs larger than L2, a few GB on the device)
 CFG_MID = dict(N_r=128, M=128, K=256, m_p=1, eta=0.5, Re_i=1000.0, Re_o=0.0, L_z=2 * math.pi / 3.16, dt=5e-4)
@@ -158,8 +158,9 @@ FP64_PEAK = 152 * 2 * 2 * 2.07e9
 
 def kernel_rooflines(cfg, prof):
     """Every traced kernel at this workload: algorithmic bytes (inputs read once, outputs
-    written once) and, for the FP64 transforms, algorithmic flops; the fraction of the
-    measured HBM bandwidth and of the FP64 peak, and the roof that binds."""
+    written once) and, for the transforms of the FP64 form, algorithmic flops; the fraction of the
+    measured HBM bandwidth, the flops relative to the FP64 peak (the transforms run in 64-bit
+    fixed point on the integer pipes, so this is not bounded by 1), and the roof that binds."""
     N, M, K = cfg["N_r"], cfg["M"], cfg["K"]
     Pt, Pz = 3 * M, 3 * K
     S = N * (M + 1) * (2 * K + 1)
@@ -193,7 +194,7 @@ def kernel_rooflines(cfg, prof):
         out[name] = e
     return {"kernels": out, "hbm_peak_gbs": hbm, "hbm_peak_source": src,
             "fp64_peak_tflops": FP64_PEAK / 1e12,
-            "note": "k_pc: DP instructions ~380 per (row, mode) in its two-partition form (ncu: 103 M per launch at the bench size), bound by FP64 issue (16 cycles per warp instruction)"}
+            "note": "k_pc: 2.4 M FP64 warp instructions per launch at the bench size (ncu), 54 % of the FP64 pipe (16 cycles per warp instruction); the transforms' fp64_frac is their algorithmic flops over the FP64 peak, which their fixed-point arithmetic does not use"}
 
 
 def cufft_comparison(torch, cfg, dev, reps=20):
@@ -809,7 +810,8 @@ def run_ours(args):
 
     # per-kernel breakdown: a tracing pass over the same number of steps
     _, prof, _ = timed_steps(plan, st, K, profile=True)
-    launches = sum(n for n, _ in prof.values())
+    # one trace slot per kernel, but the inverse z pass launches its radial stencil kernel too
+    launches = sum(n for n, _ in prof.values()) + prof.get("k_zinv", (0, 0.0))[0] * (3 * cfg["K"] > 96)
     NL = ("k_zinv", "k_theta", "k_zfwd")
     nl_ms = sum(prof[k][1] for k in NL if k in prof) / K
     pc_ms = sum(v[1] for k, v in prof.items() if k not in NL) / K
@@ -831,7 +833,8 @@ def run_ours(args):
                 # this workload from one ncu --set full capture; None until the current kernel
                 # has been captured
                 "traffic": THETA_TRAFFIC if (top[0] == "k_theta" and main_is_bench) else None,
-                "peak_source": "152 SMs x 2 DFMA/clk/SM x 2 flop x 2.07 GHz (unit counts and max clock)",
+                "peak_source": "FP64: 152 SMs x 2 DFMA/clk/SM x 2 flop x 2.07 GHz (unit counts and max clock); "
+                               "the transforms run in fixed point, off that pipe",
                 "peak_measured": fp64_measured / 1e12,
                 "frac_of_measured": ach / fp64_measured,
                 "peak_measured_source": "tc_probe_fp64_fma: 8 independent FMA chains per thread, "

@@ -70,9 +70,9 @@ typedef struct {
     int P_z;          /* physical points in z;     0 -> 3K.  Must be 2^a 3^b >= 2K+1 */
     int precision;    /* tc_precision; TC_MIXED runs the transforms and products in FP32 */
     int host_only;    /* 1: build the host plan only (no device memory); for inspection */
-    int theta_zt;     /* launch tuning: z values per theta-pass block (0: automatic); in the
-                         mixed form a value > 0 also selects the generic theta kernel over the
-                         length-specialised one */
+    int theta_zt;     /* launch tuning: z values per theta-pass block (0: automatic); a value > 0
+                         also selects the kernels for any length over the length-specialised
+                         ones */
     int pc_modes;     /* launch tuning: modes per block of the steps-2-5 kernel, rounded down to
                          a power of two, at most 16 (0: automatic) */
     int no_adjoint;   /* 1: size the workspace without the adjoint regions (tc_adjoint_* then
@@ -92,8 +92,8 @@ typedef struct {
     int stage_rows;   /* radial rows per slab of the FP64 transform staging.  The transforms of
                          the nonlinear term (Sec. 3.2 step 1) and of its adjoint act on each
                          radial row independently, so they run slab by slab and the workspace
-                         holds the FP64 lines of one slab: 12 line sets of (M+1) P_z values per
-                         row for the FP64 forward term, 21 for the adjoint.  0: all rows while
+                         holds the lines of one slab (16 bytes per complex value): 12 line sets of
+                         (M+1) P_z values per row for the FP64 forward term, 21 for the adjoint.  0: all rows while
                          that staging stays within 4 GiB, else the most rows that do; the
                          mixed form's FP32 forward lines always cover all rows */
     int mean_fp32;    /* TC_MIXED only.  0 (default): the (m, k) = (0, 0) mode of N, the mean
@@ -264,14 +264,14 @@ tc_status tc_energy_gradient(tc_plan* plan, const void* u, void* g, void* stream
 /* Nonlinear term exactly as tc_nonlinear, for callers that cannot allocate device memory
  * (the paper has no counterpart: it is a packaging choice of this library).  Instead of a
  * caller workspace, the staging lines between the transform kernels live in one static
- * 80 MiB device array that every GPU loading the library keeps until the process exits.
- * The staging a plan needs is its workspace before N^i: for TC_FP64 plans 12 line sets of
- * stage_rows * (M+1) * P_z complex128 values (the transforms run slab by slab of stage_rows
- * radial rows); for TC_MIXED plans 12 line sets of N_r * (M+1) * P_z complex64 values and
+ * 80 MiB device array (and the exponents of its lines in another of 12 MiB) that every GPU
+ * loading the library keeps until the process exits.  The staging a plan needs is its workspace
+ * before the exponents and N^i: for TC_FP64 plans 12 line sets of stage_rows * (M+1) * P_z
+ * complex values of 16 bytes (the transforms run slab by slab of stage_rows radial rows); for TC_MIXED plans 12 line sets of N_r * (M+1) * P_z complex64 values and
  * 6 * N_r * (M+1) * (2K+1) complex64 values of the FP32 split of u and d_r u; each region
  * rounded up to 256 bytes.  Plans that need more than 80 MiB get TC_ERR_ARG before any
- * launch (a smaller stage_rows brings a TC_FP64 plan's need down).  Allocates nothing.  The first call on each device looks up the array's address
- * once (cudaGetSymbolAddress) and keeps it; make that call before any stream capture, and do
+ * launch (a smaller stage_rows brings a TC_FP64 plan's need down).  Allocates nothing.  The
+ * first call on each device looks up the array's address once (cudaGetSymbolAddress) and keeps it; make that call before any stream capture, and do
  * not call this entry point after a device reset (cudaDeviceReset or a primary-context reset
  * unloads the array and leaves the kept address stale).  All calls share the array: calls
  * whose GPU work overlaps (other streams, unordered plans) race on it. */

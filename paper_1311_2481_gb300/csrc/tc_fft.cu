@@ -1,23 +1,23 @@
 // Pseudospectral nonlinear term N(u) = u . grad u (Sec. 3.2 step 1, Eq. NS_cyl) on the
-// P_theta x P_z dealiased grid (Sec. 3.1).  Three kernels, one device-memory staging area
-// between each (the single-GPU counterpart of the paper's global transposes, Sec. 4):
+// P_theta x P_z dealiased grid (Sec. 3.1): the entry for both forms, and the theta pass of the
+// mixed form for lengths without a specialised kernel (tc_theta_s.cu).  Three passes, one
+// device-memory staging area between each (the single-GPU counterpart of the paper's global
+// transposes, Sec. 4):
 //
-//   k_zinv   per (r, m): radial FD derivative (Sec. 3.1 stencils) and d_z = i k k_z fused into
-//            the load; 9 zero-padded inverse transforms along z of the u_+, u_-, u_z lines and
-//            of their d_r and d_z lines.                                   -> H1[9][r][m][z]
-//   k_theta  per (r, z tile): the 12 real physical fields as 6 complex inverse transforms
-//            along theta (two real fields per complex line; d_theta = i m m_p applied here),
-//            the pointwise products with the curvature terms, and the forward transform
-//            of N_r + i N_theta (giving N_+ and N_- directly) and of N_z (two z per line).
-//                                                                          -> H2[3][r][m][z]
-//   k_zfwd   per (r, m): forward transforms along z, truncation to |k| <= K, 1/(P_theta P_z).
+//   inverse z  per (r, m): 9 zero-padded inverse transforms along z of the u_+, u_-, u_z lines
+//              and of their d_r and d_z lines                            -> H1[9][r][m][z]
+//   theta      per (r, z tile): the 12 real physical fields as 6 complex inverse transforms
+//              along theta (two real fields per complex line; d_theta = i m m_p applied here),
+//              the pointwise products with the curvature terms, and the forward transform of
+//              N_r + i N_theta (giving N_+ and N_- directly) and of N_z (two z per line).
+//                                                                        -> H2[3][r][m][z]
+//   forward z  per (r, m): forward transforms along z, truncation to |k| <= K, 1/(P_theta P_z).
 //
-// The mixed-precision form (tc_mixed.cu) shares k_theta with FP32 lines.
-// The transforms are mixed-radix (4, 2, 3) Stockham passes in shared memory with twiddles
-// from a long-double table.
+// FP64 form: 64-bit fixed-point lines (tc_fx_z.cu, tc_fx_theta.cu).  Mixed form: FP32 lines
+// (tc_mixed.cu); the transforms here are mixed-radix (4, 2, 3) Stockham passes in shared memory
+// with twiddles from a long-double table.
 #include "tc_internal.cuh"
 #include "tc_fft_core.cuh"
-#include "tc_fftc.cuh"
 
 namespace tc {
 
@@ -41,8 +41,8 @@ __global__ void __launch_bounds__(256) k_theta(const V* __restrict__ H1, V* __re
     const int z0 = (blockIdx.x % tiles) * zt;
     const size_t fstride = (size_t)nh * (M + 1) * Pz;
     const V* h = H1 + (size_t)r * (M + 1) * Pz + z0;
-    // FP32 lines: d_r u_z enters line 4 scaled by a power of two (1 for FP64 lines)
-    const T ds = sizeof(T) == 4 ? (T)dsc[r0 + r] : (T)1, ids = (T)1 / ds;
+    // d_r u_z enters line 4 scaled by a power of two
+    const T ds = (T)dsc[r0 + r], ids = (T)1 / ds;
 
     for (int idx = threadIdx.x; idx < nl * Pt; idx += blockDim.x) { a[idx].x = 0; a[idx].y = 0; }
     __syncthreads();

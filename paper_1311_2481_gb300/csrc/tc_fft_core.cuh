@@ -7,7 +7,6 @@
 namespace tc {
 
 template <typename V> struct Real;
-template <> struct Real<double2> { using type = double; };
 template <> struct Real<float2> { using type = float; };
 
 // small DFTs of the Stockham passes; inv selects exp(+2 pi i / R)

@@ -1,4 +1,4 @@
-// Transforms of compile-time length (FP32 or FP64 lines): radix plans, in-register DFT
+// Transforms of compile-time length (FP32 lines): radix plans, in-register DFT
 // codelets and Stockham passes over lines held in shared memory with one padding slot per
 // 32 entries, which keeps the strided accesses of every pass at the minimum number of
 // shared-memory wavefronts.  Used by the length-specialised theta and z passes.
@@ -45,7 +45,6 @@ template <int PT> __host__ __device__ constexpr int padded() { return PT + (PT +
 
 template <typename V> struct Elem;
 template <> struct Elem<float2> { using T = float; };
-template <> struct Elem<double2> { using T = double; };
 
 template <typename V> __device__ __forceinline__ V vmk(typename Elem<V>::T x, typename Elem<V>::T y) {
     V v;
@@ -228,23 +227,12 @@ __device__ __forceinline__ void pass_body(const V* in, V* out, const V* __restri
 }
 template <int PT, int R, int NS, int NL, int NT, bool INV, typename V, bool TWS = false>
 __device__ __forceinline__ void pass(const V* in, V* out, const V* __restrict__ tw, int zlo, int zhi) {
-    // A first radix-8 pass reads input q of butterfly j at j + q PT / 8.  When the zero band
-    // [zlo, zhi) holds [3 PT / 8, 5 PT / 8) (a dealiased spectrum, |m| <= PT / 3), inputs 3
-    // and 4 are zero in every butterfly.  Taken for FP64 lines only, where the FP64 pipe
-    // bounds the pass; FP32 lines, bound by latency, ran no faster with it.
-    if constexpr (NS == 1 && R == 8 && sizeof(V) == 16) {
-        constexpr int NB = PT / 8;
-        if (zlo <= 3 * NB && zhi >= 5 * NB) {
-            pass_body<PT, R, NS, NL, NT, INV, V, TWS, (1u << 3) | (1u << 4)>(in, out, tw, zlo, zhi);
-            return;
-        }
-    }
     pass_body<PT, R, NS, NL, NT, INV, V, TWS, 0u>(in, out, tw, zlo, zhi);
 }
 
 // all passes of the plan; returns the buffer that holds the result
 // zlo, zhi: zero band of the input (first pass only); zlo = zhi = PT for none
-template <int PT, int P, int NS, int NL, int NT, bool INV, typename V, bool R8 = sizeof(V) == 16, bool TWS = false>
+template <int PT, int P, int NS, int NL, int NT, bool INV, typename V, bool R8 = false, bool TWS = false>
 __device__ __forceinline__ V* passes(V* a, V* b, const V* __restrict__ tw, int zlo = PT, int zhi = PT) {
     if constexpr (P == Plan<PT, R8>::np) {
         return a;

@@ -43,7 +43,7 @@ struct FxPlan {
 // Every region is scratch of one library call; regions that no call uses at the same time
 // share memory (see tc_plan.cu).
 struct Workspace {
-    size_t H1;      // inverse z-pass output, 9 line sets [f][r][m][z]: FP64 lines of stage_rows
+    size_t H1;      // inverse z-pass output, 9 line sets [f][r][m][z]: 16-byte lines of stage_rows
                     // rows, or the mixed form's FP32 lines of all N_r rows
     size_t H2;      // theta-pass output: 3 line sets, rows and precision as H1
     size_t P32;     // mixed form: u', d_r u' in FP32, 6 x S float2
@@ -55,7 +55,7 @@ struct Workspace {
     size_t ustar;
     size_t phi;
     size_t red;     // diagnostics reduction buffer (diag_red_doubles doubles)
-    // adjoint regions (absent with tc_options.no_adjoint), FP64 lines of stage_rows rows
+    // adjoint regions (absent with tc_options.no_adjoint), 16-byte lines of stage_rows rows
     size_t H1a;     // recomputed forward lines of u: 9 line sets
     size_t Ha;      // adjoint lines of Nbar: 3 line sets
     size_t H3;      // adjoint theta-pass output: 9 line sets
@@ -84,16 +84,14 @@ struct tc_plan {
     int nmode_half;  // (M+1)(K+1)
     tc::Radices rad_z, rad_t;
     int fx_zt;                     // z values per fixed-point theta block
-    int zt, zt32;                  // z values per theta-pass block (FP64 / FP32 lines)
+    int zt32;                      // z values per theta-pass block (FP32 lines)
     int theta_zt_forced;           // tc_options.theta_zt (> 0: generic transform kernels)
     int theta_variant;             // tc_options.theta_variant (launch shape of the FP32 streamed theta pass)
     int pc_modes;                  // modes per block of the fused steps-2-5 kernel (0: auto)
     int num_sms = 152;             // multiprocessors of the plan's device
-    int thr_zinv, thr_theta, thr_zfwd;  // block sizes of the FP64 transform kernels
     bool pc_split;                      // steps 2-5 as separate kernels (large N_r)
     int part_h = 0;                     // fused kernel: systems cut into rows [0, h), [h, N_r) (0: uncut)
-    int zinv_lines, zinv_lines32;  // lines per inverse z-pass block (FP64 / FP32 lines)
-    int zfwd_lines, zfwd_lines32;  // lines per forward z-pass block (3 or 1)
+    int zinv_lines32, zfwd_lines32;  // lines per inverse and forward z-pass block of the mixed form
     tc::Workspace ws;
     // host plan
     std::vector<double> r, w1, w2;   // nodes; weights [N_r][9]
@@ -126,8 +124,6 @@ struct tc_plan {
     uint8_t* d_piv2 = nullptr;
     double* d_spk = nullptr;
     double* d_rinv = nullptr;
-    double2* d_tw_z = nullptr;
-    double2* d_tw_t = nullptr;
     float2* d_tw_z32 = nullptr;
     float2* d_tw_t32 = nullptr;
     // fixed-point constants: twiddles (two limbs of cos, two of sin), m m_p and 1/r_j (limbs and
@@ -223,7 +219,7 @@ int fx_zt(const tc_plan* p, int forced);
 const int* fx_static_radices(int n);   // radices of the compile-time plan of length n, nullptr if none
 tc_status launch_nonlinear(tc_plan* p, const double2* u, double2* N, char* ws, cudaStream_t s);
 tc_status launch_theta32(tc_plan* p, const float2* H1, float2* H2, cudaStream_t s);
-int theta_s_zt(const tc_plan* p, bool fp64);
+int theta_s_zt(const tc_plan* p);
 tc_status launch_theta_s(tc_plan* p, const float2* H1, float2* H2, cudaStream_t s);
 tc_status launch_nl_pre32(tc_plan* p, const double2* u, char* ws, cudaStream_t s, int ma, int mb);
 tc_status launch_nl_theta32(tc_plan* p, char* ws, cudaStream_t s);

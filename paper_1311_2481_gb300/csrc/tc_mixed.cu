@@ -553,7 +553,7 @@ tc_status launch_nl_pre32(tc_plan* p, const double2* u, char* ws, cudaStream_t s
 tc_status launch_nl_theta32(tc_plan* p, char* ws, cudaStream_t s) {
     const float2* H1 = reinterpret_cast<const float2*>(ws + p->ws.H1);
     float2* H2 = reinterpret_cast<float2*>(ws + p->ws.H2);
-    if (p->theta_zt_forced == 0 && theta_s_zt(p, false) > 0) return launch_theta_s(p, H1, H2, s);
+    if (p->theta_zt_forced == 0 && theta_s_zt(p) > 0) return launch_theta_s(p, H1, H2, s);
     return launch_theta32(p, H1, H2, s);
 }
 

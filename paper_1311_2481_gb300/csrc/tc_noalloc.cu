@@ -9,10 +9,11 @@
 // array of this library instead of a caller workspace.
 //
 // Costs and limits:
-//  - kStaticScratchBytes (80 MiB) of device memory is reserved on every GPU that loads this
-//    library, for as long as the process lives.  Plans whose staging needs more are rejected
-//    with TC_ERR_ARG before anything is launched.  The staging is everything the workspace
-//    holds before N^i: the z-pass lines H1 and H2 (12 line sets: complex128 lines of
+//  - 80 MiB of device memory for staging lines (kStaticScratchBytes), and 12 MiB for the
+//    exponents of fixed-point lines, are reserved on every GPU that loads this library, for as
+//    long as the process lives.  Plans whose staging needs more are rejected with TC_ERR_ARG
+//    before anything is launched.  The staging is everything the workspace holds before the
+//    exponents and N^i: the z-pass lines H1 and H2 (12 line sets: 16-byte complex lines of
 //    stage_rows radial rows for TC_FP64 plans, complex64 lines of all rows for TC_MIXED
 //    plans), and for TC_MIXED plans the FP32 split of u and d_r u, 6 * N_r * (M+1) * (2K+1)
 //    complex64 values, each region rounded up to 256 bytes.

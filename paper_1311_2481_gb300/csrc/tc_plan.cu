@@ -215,29 +215,6 @@ static std::vector<int4> fx_twiddles(const FxPlan& f) {
 
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// Block size for a kernel whose FP64 work is Stockham passes over `lines` transforms of
-// length rad.n (plus `lines2` of a second batch): the FP64 pipe is charged per warp
-// instruction, so pick the size that wastes the fewest lanes over all passes.
-static int choose_threads(const Radices& rad, int lines, int lines2) {
-    double best = -1.0;
-    int bestT = 256;
-    for (int T = 96; T <= 256; T += 32) {
-        double items = 0.0, slots = 0.0;
-        for (int batch = 0; batch < 2; ++batch) {
-            const int L = batch ? lines2 : lines;
-            if (L <= 0) continue;
-            for (int q = 0; q < rad.count; ++q) {
-                const double it = (double)L * rad.n / rad.r[q];
-                items += it;
-                slots += std::ceil(it / T) * T;
-            }
-        }
-        const double e = items / slots;
-        if (e > best + 1e-9 || (std::fabs(e - best) <= 1e-9 && T > bestT)) { best = e; bestT = T; }
-    }
-    return bestT;
-}
-
 // Banded LU with partial pivoting of one matrix given in row windows W[i][t] = A[i][i-kl+t],
 // t in [0, 2kl+ku] (kl = ku = 4).  On return W holds the multipliers of step j in
 // W[j+q][kl-q] (q = 1..kl, column j of L, LAPACK convention: not permuted by later steps)
@@ -519,8 +496,6 @@ static tc_status upload(tc_plan* p) {
         TC_CUDA(p, put((void**)&p->d_spk, p->spk.data(), p->spk.size() * sizeof(double)));
         TC_CUDA(p, put((void**)&p->d_rinv, p->rinv.data(), p->rinv.size() * sizeof(double)));
     }
-    TC_CUDA(p, put((void**)&p->d_tw_z, p->tw_z.data(), p->tw_z.size() * sizeof(double)));
-    TC_CUDA(p, put((void**)&p->d_tw_t, p->tw_t.data(), p->tw_t.size() * sizeof(double)));
     if (p->precision != TC_MIXED || p->adjoint) {   // constants of the fixed-point transforms
         // tables of the run-time plans, followed by those of the compile-time plans
         std::vector<int4> tz = fx_twiddles(p->fx_z), tt = fx_twiddles(p->fx_t);
@@ -625,7 +600,7 @@ static void free_device(tc_plan* p) {
         p->mean_stream = nullptr;
     }
     void* ptrs[] = {p->d_r, p->d_ir, p->d_w1, p->d_w1f, p->d_dsc, p->d_w2, p->d_col0, p->d_d1t_row, p->d_d1t_w, p->d_fac, p->d_piv,
-                    p->d_fac2, p->d_piv2, p->d_spk, p->d_rinv, p->d_tw_z, p->d_tw_t, p->d_tw_z32, p->d_tw_t32,
+                    p->d_fac2, p->d_piv2, p->d_spk, p->d_rinv, p->d_tw_z32, p->d_tw_t32,
                     p->d_fx_tw_z, p->d_fx_tw_t, p->d_fx_mm, p->d_fx_ir, p->d_fx_w1, p->d_fx_ew};
     for (void* q : ptrs)
         if (q) cudaFree(q);
@@ -767,11 +742,8 @@ tc_status tc_plan_create_ex(tc_plan** out, int N_r, int M, int K, int m_p, doubl
         while (zt > 1 && Pz % zt) zt /= 2;
         return zt;
     };
-    p->zinv_lines = lines_for(sizeof(double2), 9);
     p->zinv_lines32 = lines_for(sizeof(float2), 9);
-    p->zfwd_lines = lines_for(sizeof(double2), 3);
     p->zfwd_lines32 = lines_for(sizeof(float2), 3);
-    p->zt = zt_for(sizeof(double2), o.theta_zt > 0 ? o.theta_zt : 4, 200 * 1024);
     p->zt32 = zt_for(sizeof(float2), o.theta_zt > 0 ? o.theta_zt : 8, o.theta_zt > 0 ? 200 * 1024 : 76 * 1024);
     p->fx_z = fx_plan(Pz);
     p->fx_t = fx_plan(Pt);
@@ -779,9 +751,6 @@ tc_status tc_plan_create_ex(tc_plan** out, int N_r, int M, int K, int m_p, doubl
     p->pc_modes = o.pc_modes;
     p->theta_zt_forced = o.theta_zt;
     p->theta_variant = o.theta_variant;
-    p->thr_zinv = choose_threads(rz, p->zinv_lines, 0);
-    p->thr_theta = choose_threads(rt, 6 * p->zt, p->zt + (p->zt + 1) / 2);
-    p->thr_zfwd = choose_threads(rz, p->zfwd_lines, 0);
     if (o.theta_zt < 0 || o.theta_zt > 64 || o.pc_modes < 0 || o.pc_modes > 32 || o.pc_split < -1 || o.pc_split > 1 ||
         o.theta_variant < 0 || o.theta_variant > 4 || o.pc_partitions < 0 || o.pc_partitions > 2 ||
         o.stage_rows < 0 || o.mean_fp32 < 0 || o.mean_fp32 > 1) {
@@ -789,7 +758,7 @@ tc_status tc_plan_create_ex(tc_plan** out, int N_r, int M, int K, int m_p, doubl
         return TC_ERR_ARG;
     }
     {
-        // FP64 lines unless the plan is mixed without the (FP64) adjoint
+        // 16-byte lines unless the plan is mixed without the adjoint
         const size_t lb = (o.precision == TC_MIXED && o.no_adjoint) ? sizeof(float2) : cplx;
         if ((size_t)2 * 3 * Pz * lb > 220 * 1024 || (size_t)2 * 6 * Pt * lb > 220 * 1024) {
             delete p;
@@ -811,7 +780,7 @@ tc_status tc_plan_create_ex(tc_plan** out, int N_r, int M, int K, int m_p, doubl
         else if (per_row * (size_t)N_r > cap) rows = (int)std::max<size_t>(1, cap / std::max<size_t>(per_row, 1));
         p->stage_rows = rows;
     }
-    // forward transform staging: FP64 lines of stage_rows rows, or the mixed form's FP32
+    // forward transform staging: 16-byte lines of stage_rows rows, or the mixed form's FP32
     // lines of all rows and its FP32 u', d_r u'
     if (p->precision == TC_MIXED) {
         p->ws.H1 = take(9 * p->Hfield * sizeof(float2));

@@ -1,9 +1,8 @@
 // Length-specialised theta pass (Sec. 3.2 step 1, Eq. NS_cyl) for the common transform
-// lengths, FP32 or FP64 lines.  Same input (H1) and output (H2) as k_theta, organised
+// lengths, FP32 lines.  Same input (H1) and output (H2) as k_theta, organised
 // differently:
 //
-//  * the radices of each length are compile-time constants (e.g. 768 = 16 * 16 * 3 for FP32
-//    lines), so the Stockham index arithmetic folds and fewer passes are needed;
+//  * the radices of each length are compile-time constants (e.g. 768 = 16 * 16 * 3), so the Stockham index arithmetic folds and fewer passes are needed;
 //  * lines sit in shared memory with one padding slot per 32 entries, which makes the
 //    stride-R stores of the first pass and all later accesses bank-conflict free;
 //  * the products are streamed: u is transformed first and kept per physical point (in shared
@@ -60,9 +59,9 @@ __global__ void __launch_bounds__(NT, MINB) k_theta_s(const V* __restrict__ H1, 
     const V* h = H1 + (size_t)r * (M + 1) * Pz + z0;
     const T ir = (T)irn[r0 + r];   // 1 / r_j from the plan
     const T mpf = (T)mp;
-    // FP32 lines: d_r u_z enters the (u_z, d_r u_z) line scaled by a power of two, so that
-    // its rounding does not swamp u_z near the walls; FP64 lines are not scaled
-    const T ds = sizeof(V) == 8 ? (T)dsc[r0 + r] : (T)1, ids = (T)1 / ds;
+    // d_r u_z enters the (u_z, d_r u_z) line scaled by a power of two, so that
+    // its rounding does not swamp u_z near the walls
+    const T ds = (T)dsc[r0 + r], ids = (T)1 / ds;
     const int zi = threadIdx.x % ZT;        // z of this thread in the load and store loops
     const int mstep = NT / ZT;
     if constexpr (TWS) {
@@ -96,61 +95,23 @@ __global__ void __launch_bounds__(NT, MINB) k_theta_s(const V* __restrict__ H1, 
 #pragma unroll 1
     for (int phase = 0; phase < 3; ++phase) {
         // spectra of the two lines of each z (lines 2 zi and 2 zi + 1)
-        if constexpr (sizeof(V) == 16) {
-            // FP64 lines: the four fields of the phase for two m values per thread loaded
-            // before they are placed (measured faster; 2M+1 <= PT bounds the m values)
-            const int fa = phase == 0 ? 0 : phase == 1 ? 3 : 6;
-            const int fc = phase == 0 ? 2 : phase == 1 ? 0 : 2;
-            const int fd = phase == 0 ? 5 : phase == 1 ? 1 : 8;
-            constexpr int MI = (PT / 2 + 1 + NT / ZT - 1) / (NT / ZT);
-            constexpr int G = 2;
+        // one m value at a time (the extra registers of batched loads cost more than the
+        // latency they hide here)
+        for (int m = (int)threadIdx.x / ZT; m <= M; m += mstep) {
+            const size_t o = (size_t)m * Pz + zi;
+            const T mm = mpf * (T)m;
             V* L0 = A + (2 * zi) * LP;
             V* L1 = L0 + LP;
-#pragma unroll
-            for (int i0 = 0; i0 < MI; i0 += G) {
-                V va[G], vb[G], vc[G], vd[G];
-#pragma unroll
-                for (int i = 0; i < G; ++i) {
-                    const int m = (int)threadIdx.x / ZT + (i0 + i) * mstep;
-                    if (i0 + i < MI && m <= M) {
-                        const size_t o = (size_t)m * Pz + zi;
-                        va[i] = h[fa * fstride + o];
-                        vb[i] = h[(fa + 1) * fstride + o];
-                        vc[i] = h[fc * fstride + o];
-                        vd[i] = h[fd * fstride + o];
-                    }
-                }
-#pragma unroll
-                for (int i = 0; i < G; ++i) {
-                    const int m = (int)threadIdx.x / ZT + (i0 + i) * mstep;
-                    if (i0 + i < MI && m <= M) {
-                        const T mm = mpf * (T)m;
-                        put_pair(L0, PT, m, va[i], vb[i]);
-                        if (phase == 0) put_real2(L1, PT, m, vc[i], vd[i]);
-                        else if (phase == 1) put_pair(L1, PT, m, imul(vc[i], mm), imul(vd[i], mm));
-                        else put_real2(L1, PT, m, imul(vc[i], mm), vd[i]);
-                    }
-                }
-            }
-        } else {
-            // FP32 lines: one m value at a time (the extra registers of batched loads cost
-            // more than the latency they hide here)
-            for (int m = (int)threadIdx.x / ZT; m <= M; m += mstep) {
-                const size_t o = (size_t)m * Pz + zi;
-                const T mm = mpf * (T)m;
-                V* L0 = A + (2 * zi) * LP;
-                V* L1 = L0 + LP;
-                if (phase == 0) {
-                    put_pair(L0, PT, m, h[0 * fstride + o], h[1 * fstride + o]);
-                    const V drz = h[5 * fstride + o];
-                    put_real2(L1, PT, m, h[2 * fstride + o], vmk<V>(drz.x * ds, drz.y * ds));
-                } else if (phase == 1) {
-                    put_pair(L0, PT, m, h[3 * fstride + o], h[4 * fstride + o]);
-                    put_pair(L1, PT, m, imul(h[0 * fstride + o], mm), imul(h[1 * fstride + o], mm));
-                } else {
-                    put_pair(L0, PT, m, h[6 * fstride + o], h[7 * fstride + o]);
-                    put_real2(L1, PT, m, imul(h[2 * fstride + o], mm), h[8 * fstride + o]);
-                }
+            if (phase == 0) {
+                put_pair(L0, PT, m, h[0 * fstride + o], h[1 * fstride + o]);
+                const V drz = h[5 * fstride + o];
+                put_real2(L1, PT, m, h[2 * fstride + o], vmk<V>(drz.x * ds, drz.y * ds));
+            } else if (phase == 1) {
+                put_pair(L0, PT, m, h[3 * fstride + o], h[4 * fstride + o]);
+                put_pair(L1, PT, m, imul(h[0 * fstride + o], mm), imul(h[1 * fstride + o], mm));
+            } else {
+                put_pair(L0, PT, m, h[6 * fstride + o], h[7 * fstride + o]);
+                put_real2(L1, PT, m, imul(h[2 * fstride + o], mm), h[8 * fstride + o]);
             }
         }
         __syncthreads();
@@ -300,30 +261,21 @@ tc_status theta_s32(tc_plan* p, const float2* H1, float2* H2, cudaStream_t s) {
 
 }  // namespace
 
-// z values per block of the streamed theta pass for this plan and line type, 0 if none
-int theta_s_zt(const tc_plan* p, bool fp64) {
+// z values per block of the streamed theta pass for this plan, 0 if none
+int theta_s_zt(const tc_plan* p) {
     int zt = 0;
-    if (fp64) {
-        switch (p->P_t) {
-            case 96: zt = 4; break;
-            case 192: case 384: zt = 2; break;
-            case 768: case 1152: zt = 1; break;
-            default: return 0;
-        }
-    } else {
-        switch (p->P_t) {
-            case 48: case 96: zt = 8; break;
-            case 192: case 384: zt = 4; break;
-            case 768: case 1152: case 1536: zt = 2; break;
-            default: return 0;
-        }
+    switch (p->P_t) {
+        case 48: case 96: zt = 8; break;
+        case 192: case 384: zt = 4; break;
+        case 768: case 1152: case 1536: zt = 2; break;
+        default: return 0;
     }
     if (2 * p->M + 1 > p->P_t || p->P_z % zt) return 0;
     return zt;
 }
 
 tc_status launch_theta_s(tc_plan* p, const float2* H1, float2* H2, cudaStream_t s) {
-    if (theta_s_zt(p, false) == 0) return TC_ERR_ARG;
+    if (theta_s_zt(p) == 0) return TC_ERR_ARG;
     switch (p->P_t) {
         case 48: return theta_s32<48, 8, 128>(p, H1, H2, s);
         case 96: return theta_s32<96, 8, 256>(p, H1, H2, s);
