@@ -50,7 +50,8 @@ struct Sum {
 // values at that exponent, in units of 2^32, which bounds every sum of a theta line.  at(q, m)
 // gives (exponent, largest value) of field q < NF; bound calls f(kind, field, weighted by
 // m m_p) for each field of each kind; half: kinds that are one part of a pair of real fields
-// (m and -m both count).  The sum is taken in a fixed order: the exponents decide rounding.
+// (m and -m both count).  The sum is taken in a fixed order: the exponents decide rounding.  A
+// weighted kind has no m = 0 entry: er does not cover that one, whose 2^(v.x - er) may overflow.
 template <int NF, int NK, int NT, class AT, class BOUND>
 __device__ __forceinline__ void line_bounds(AT at, BOUND bound, unsigned half, int M, long long mp, int nt, int* s_E, float (*s_bound)[NK],
                                             int (&er)[NK], float (&sum)[NK]) {
@@ -85,6 +86,7 @@ __device__ __forceinline__ void line_bounds(AT at, BOUND bound, unsigned half, i
 #pragma unroll
         for (int q = 0; q < NF; ++q) v[q] = at(q, m);
         bound([&](int s, int q, bool mul) {
+            if (mul && m == 0) return;
             const int d = min(er[s] - v[q].x, 127);   // 2^-d, 0 below 2^-126
             const float x = (float)(unsigned)v[q].y * __int_as_float(max(127 - d, 0) << 23) * ((half >> s) & 1 ? 2.f : 1.f);
             sum[s] += mul ? x * mm : x;
