@@ -203,6 +203,7 @@ tc_status tc_diagnostics(tc_plan* plan, const void* u, tc_diag* out, void* ws, v
         double d = 0.0;
         for (int t = 0; t < kStencil; ++t) {
             int c = plan->col0[j] + t;
+            if (c < 0) continue;   // N_r < kStencil: weight 0
             double ut = 0.5 * (col[c].y - col[N + c].y);
             d += plan->w1[(size_t)j * kStencil + t] * ut / plan->r[c];
         }

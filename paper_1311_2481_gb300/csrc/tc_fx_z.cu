@@ -67,9 +67,9 @@ __global__ void __launch_bounds__(128) k_fx_dr(const double* __restrict__ u, dou
         double o = 0.0;
         if (j < 4 || j > N - 5 || x.far(i)) {
             const int c0 = __ldg(&col0[j]);
-            double v[kStencil];   // rows outside [0, N) (N < 9) have weight 0
+            double v[kStencil];
 #pragma unroll
-            for (int t = 0; t < kStencil; ++t) v[t] = (unsigned)(c0 + t) < (unsigned)N ? __ldg(&src[(ptrdiff_t)(c0 + t) * ncol]) : 0.0;
+            for (int t = 0; t < kStencil; ++t) v[t] = stencil_row(c0, t) ? __ldg(&src[(ptrdiff_t)(c0 + t) * ncol]) : 0.0;
 #pragma unroll
             for (int t = 0; t < kStencil; ++t) o = fma(__ldg(&w1[j * kStencil + t]), v[t], o);
         } else {
@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(kZThreads) k_fx_zinv(const double2* __restrict
         if (NL == 9 && d == 1 && !du) {   // d_r u here, in FP64
             const int j0 = __ldg(&col0[r0 + rl]);
             const double2* a = u + ((ptrdiff_t)c * N + j0) * nmode + (ptrdiff_t)m * nk;
-            double w[kStencil];   // rows outside [0, N) (N < 9) have weight 0
+            double w[kStencil];
 #pragma unroll
             for (int q = 0; q < kStencil; ++q) w[q] = __ldg(&w1[(r0 + rl) * kStencil + q]);
 #pragma unroll
@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(kZThreads) k_fx_zinv(const double2* __restrict
                     double2 y = make_double2(0.0, 0.0);   // two sums: half the chain of dependent FMAs
 #pragma unroll
                     for (int q = 0; q < kStencil; ++q) {
-                        const double2 v = (unsigned)(j0 + q) < (unsigned)N ? __ldg(&a[(ptrdiff_t)q * nmode + i0 + i * tl]) : make_double2(0.0, 0.0);
+                        const double2 v = stencil_row(j0, q) ? __ldg(&a[(ptrdiff_t)q * nmode + i0 + i * tl]) : make_double2(0.0, 0.0);
                         double2& o = q & 1 ? y : x[i];
                         o.x = fma(w[q], v.x, o.x);
                         o.y = fma(w[q], v.y, o.y);

@@ -175,6 +175,10 @@ __device__ __forceinline__ bool nonfinite2(double2 v) {
     return nonfinite1(v.x) | nonfinite1(v.y);
 }
 
+// Row c0 + t of a padded stencil may be read.  Plans of N_r < kStencil rows have c0 = N_r - kStencil < 0: the
+// rows below 0 have weight 0 and lie outside the field.
+__device__ __forceinline__ bool stencil_row(int c0, int t) { return c0 + t >= 0; }
+
 // ------------------------------------------------------------------ error helpers
 tc_status cuda_fail(tc_plan* p, cudaError_t e, const char* where);
 #define TC_CUDA(plan, call)                                            \

@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(256) k_prep32(const double2* __restrict__ u, f
     const double2* other = u + (size_t)(c == 1 ? 0 : 1) * S + (size_t)m * nk + kk;   // read only if c < 2
     for (int j = jlo + threadIdx.y; j <= jhi; j += blockDim.y) {
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (kin) {
+        if (kin && j >= 0) {   // rows below 0 (N_r < 9) have weight 0
             double2 x = base[(size_t)j * colstride];
             if (sub) x.y = 0.5 * (x.y + other[(size_t)j * colstride].y);
             const float2 a = split_hl(x.x), q = split_hl(x.y);
@@ -269,7 +269,7 @@ __device__ __forceinline__ void mean_flow_coeffs(const double2* __restrict__ u, 
     double dU = 0.0;
     const int c0 = col0[r];
     for (int t = 0; t < kStencil; ++t)
-        dU += w1[r * kStencil + t] * 0.5 * (up[(size_t)(c0 + t) * col].y - um[(size_t)(c0 + t) * col].y);
+        if (stencil_row(c0, t)) dU += w1[r * kStencil + t] * 0.5 * (up[(size_t)(c0 + t) * col].y - um[(size_t)(c0 + t) * col].y);
     const double U = 0.5 * (up[(size_t)r * col].y - um[(size_t)r * col].y);
     const double Ur = U / rnodes[r];
     const double q = 0.5 * (dU + Ur);
@@ -688,7 +688,7 @@ __global__ void __launch_bounds__(256) k_mean00(const double2* __restrict__ u, d
         const double2* base = u + (size_t)c * S + mode;
         for (int j = jlo + threadIdx.y; j <= jhi; j += blockDim.y) {
             float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (kin) {
+            if (kin && j >= 0) {   // rows below 0 (N_r < 9) have weight 0
                 const double2 x = base[(size_t)j * nmode];
                 const float2 a = split_hl(x.x), q = split_hl(x.y);
                 v = make_float4(a.x, q.x, a.y, q.y);

@@ -198,7 +198,8 @@ __global__ void __launch_bounds__(NTH, 512 / NTH) k_pc(PCArgs a, Geo g, int T) {
         const int c0 = __ldg(&a.col0[j]);
         double o = 0.0;
 #pragma unroll
-        for (int q = 0; q < kStencil; ++q) o = fma(__ldg(&a.w1[j * kStencil + q]), f[(c0 + q) * 2 * T], o);
+        for (int q = 0; q < kStencil; ++q)
+            if (stencil_row(c0, q)) o = fma(__ldg(&a.w1[j * kStencil + q]), f[(c0 + q) * 2 * T], o);
         return o;
     };
     auto d1s = [&](const double* f, const double* f2, int j) {   // of f + f2
@@ -206,6 +207,7 @@ __global__ void __launch_bounds__(NTH, 512 / NTH) k_pc(PCArgs a, Geo g, int T) {
         double o = 0.0;
 #pragma unroll
         for (int q = 0; q < kStencil; ++q) {
+            if (!stencil_row(c0, q)) continue;
             const int n = (c0 + q) * 2 * T;
             o = fma(__ldg(&a.w1[j * kStencil + q]), f[n] + f2[n], o);
         }
@@ -457,6 +459,7 @@ __device__ __forceinline__ void tile_rows(const Cols& c, const Stencil& s, const
                 const int c0 = __ldg(&s.col0[j]);
 #pragma unroll
                 for (int t = 0; t < kStencil; ++t) {
+                    if (!stencil_row(c0, t)) continue;
                     const size_t o = (size_t)(c0 + t) * st;
                     const double w = __ldg(&s.w1[j * kStencil + t]), x = __ldg(&f[o]);
                     d[i] = fma(w, PAIR ? x + __ldg(&f2[o]) : x, d[i]);
@@ -807,6 +810,7 @@ __global__ void k_diag(const double2* __restrict__ u, double* __restrict__ red,
             const int c0 = col0[j];
             double2 d = make_double2(0.0, 0.0);
             for (int t = 0; t < kStencil; ++t) {
+                if (!stencil_row(c0, t)) continue;
                 const double wt = w1[j * kStencil + t];
                 const size_t o = (size_t)(c0 + t) * g.nmode + mode;
                 const double2 p1 = u[o], p2 = u[g.S + o];

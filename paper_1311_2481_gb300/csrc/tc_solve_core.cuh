@@ -33,6 +33,7 @@ __device__ __forceinline__ double2 drow(const double2* __restrict__ f, const dou
     double2 s = make_double2(0.0, 0.0);
 #pragma unroll
     for (int t = 0; t < kStencil; ++t) {
+        if (!stencil_row(c0, t)) continue;
         const double wt = __ldg(&w[j * kStencil + t]);
         const double2 v = f[(size_t)(c0 + t) * nmode + mode];
         s.x += wt * v.x;
