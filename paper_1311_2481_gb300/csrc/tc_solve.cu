@@ -892,7 +892,8 @@ tc_status launch_solve(tc_plan* p, int set, const double2* rhs, double2* x, cuda
         g.sh = p->part_h;
         PCArgs a{};
         a.fac2 = p->d_fac2; a.piv2 = p->d_piv2; a.spk = p->d_spk; a.rinv = p->d_rinv;
-        const int T = 16;
+        int T = 16;   // a power of two: it divides the block size
+        while (T > 1 && (size_t)p->N_r * T * sizeof(double2) > 96 * 1024) T /= 2;
         const size_t sm = (size_t)p->N_r * T * sizeof(double2) + (size_t)T * 16 * sizeof(double);
         TC_CUDA(p, cudaFuncSetAttribute(k_band_solve_s2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
         const int slot = prof_begin(p, prof, s);
