@@ -178,6 +178,17 @@ __device__ __forceinline__ bool nonfinite2(double2 v) {
 // Row c0 + t of a padded stencil may be read.  Plans of N_r < kStencil rows have c0 = N_r - kStencil < 0: the
 // rows below 0 have weight 0 and lie outside the field.
 __device__ __forceinline__ bool stencil_row(int c0, int t) { return c0 + t >= 0; }
+// tap(t) for the rows c0 + t of a stencil that may be read.  A guard on each tap costs the sums in FP64 4 %
+// (k_pc, N_r = 160, M = 8, K = 16: 240 against 229 us); c0 has the same sign for every row of a plan.
+template <class Tap> __device__ __forceinline__ void stencil_taps(int c0, Tap tap) {
+    if (c0 >= 0) {
+#pragma unroll
+        for (int t = 0; t < kStencil; ++t) tap(t);
+    } else {
+#pragma unroll 1
+        for (int t = -c0; t < kStencil; ++t) tap(t);
+    }
+}
 
 // ------------------------------------------------------------------ error helpers
 tc_status cuda_fail(tc_plan* p, cudaError_t e, const char* where);

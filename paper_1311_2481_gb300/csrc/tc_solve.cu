@@ -128,8 +128,16 @@ __device__ __forceinline__ double2 lap_pm(const double2* __restrict__ u, const P
                                           double kk, const Geo& g) {
     const double2* f = u + (size_t)c * g.S;
     const double ir = a.ir[j], ir2 = ir * ir;
-    const double2 d1 = drow(f, a.w1, a.col0, j, g.nmode, mode);
-    const double2 d2 = drow(f, a.w2, a.col0, j, g.nmode, mode);
+    double2 d1 = make_double2(0.0, 0.0), d2 = d1;
+    const int c0 = a.col0[j];
+    stencil_taps(c0, [&](int t) {
+        const double2 x = f[(size_t)(c0 + t) * g.nmode + mode];
+        const double p = __ldg(&a.w1[j * kStencil + t]), q = __ldg(&a.w2[j * kStencil + t]);
+        d1.x += p * x.x;
+        d1.y += p * x.y;
+        d2.x += q * x.x;
+        d2.y += q * x.y;
+    });
     const double2 v = f[(size_t)j * g.nmode + mode];
     const double diag = -mm * mm * ir2 - kk * kk - ir2 + (c == 0 ? -2.0 : 2.0) * mm * ir2;
     return make_double2(d2.x + ir * d1.x + diag * v.x, d2.y + ir * d1.y + diag * v.y);
@@ -197,20 +205,16 @@ __global__ void __launch_bounds__(NTH, 512 / NTH) k_pc(PCArgs a, Geo g, int T) {
     auto d1 = [&](const double* f, int j) {   // FP64 stencil at row j
         const int c0 = __ldg(&a.col0[j]);
         double o = 0.0;
-#pragma unroll
-        for (int q = 0; q < kStencil; ++q)
-            if (stencil_row(c0, q)) o = fma(__ldg(&a.w1[j * kStencil + q]), f[(c0 + q) * 2 * T], o);
+        stencil_taps(c0, [&](int q) { o = fma(__ldg(&a.w1[j * kStencil + q]), f[(c0 + q) * 2 * T], o); });
         return o;
     };
     auto d1s = [&](const double* f, const double* f2, int j) {   // of f + f2
         const int c0 = __ldg(&a.col0[j]);
         double o = 0.0;
-#pragma unroll
-        for (int q = 0; q < kStencil; ++q) {
-            if (!stencil_row(c0, q)) continue;
+        stencil_taps(c0, [&](int q) {
             const int n = (c0 + q) * 2 * T;
             o = fma(__ldg(&a.w1[j * kStencil + q]), f[n] + f2[n], o);
-        }
+        });
         return o;
     };
     auto slow0 = [&](int j, int c) { return d1(D0 + c, j); };
@@ -457,13 +461,11 @@ __device__ __forceinline__ void tile_rows(const Cols& c, const Stencil& s, const
             if (!c.in || j >= N) continue;
             if (j < 4 || j > N - 5 || X.far(i)) {
                 const int c0 = __ldg(&s.col0[j]);
-#pragma unroll
-                for (int t = 0; t < kStencil; ++t) {
-                    if (!stencil_row(c0, t)) continue;
+                stencil_taps(c0, [&](int t) {
                     const size_t o = (size_t)(c0 + t) * st;
                     const double w = __ldg(&s.w1[j * kStencil + t]), x = __ldg(&f[o]);
                     d[i] = fma(w, PAIR ? x + __ldg(&f2[o]) : x, d[i]);
-                }
+                });
             } else {
                 d[i] = X.row(i, s.fw + j * kStencil, __ldg(&s.few[j]));
             }

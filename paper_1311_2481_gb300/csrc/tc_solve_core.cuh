@@ -31,14 +31,12 @@ __device__ __forceinline__ double2 drow(const double2* __restrict__ f, const dou
                                         const int* __restrict__ col0, int j, int nmode, int mode) {
     const int c0 = col0[j];
     double2 s = make_double2(0.0, 0.0);
-#pragma unroll
-    for (int t = 0; t < kStencil; ++t) {
-        if (!stencil_row(c0, t)) continue;
+    stencil_taps(c0, [&](int t) {
         const double wt = __ldg(&w[j * kStencil + t]);
         const double2 v = f[(size_t)(c0 + t) * nmode + mode];
         s.x += wt * v.x;
         s.y += wt * v.y;
-    }
+    });
     return s;
 }
 
