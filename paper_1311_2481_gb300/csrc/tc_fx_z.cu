@@ -341,16 +341,15 @@ __global__ void __launch_bounds__(kZThreads) k_fx_zfwd(const cx* __restrict__ H2
 Exps exps(tc_plan* p, char* ws) {
     Exps e;
     e.e1 = reinterpret_cast<int2*>(ws + p->ws.fxe);
-    e.e2max = reinterpret_cast<int*>(e.e1 + (size_t)9 * p->N_r * (p->M + 1));
-    e.e2 = e.e2max + 2 * p->N_r;
+    e.e2max = reinterpret_cast<int*>(e.e1 + (size_t)9 * p->stage_rows * (p->M + 1));
+    e.e2 = e.e2max + 2 * p->stage_rows;
     return e;
 }
 
 }  // namespace
 
-size_t fx_exp_bytes(const tc_plan* p) {
-    return (size_t)9 * p->N_r * (p->M + 1) * sizeof(int2) + (size_t)2 * p->N_r * sizeof(int) +
-           (size_t)2 * p->N_r * p->P_z * sizeof(int);
+size_t fx_exp_bytes(const tc_plan* p, int rows) {
+    return (size_t)rows * ((size_t)9 * (p->M + 1) * sizeof(int2) + 2 * sizeof(int) + (size_t)2 * p->P_z * sizeof(int));
 }
 
 namespace {

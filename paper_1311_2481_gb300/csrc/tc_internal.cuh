@@ -48,7 +48,8 @@ struct Workspace {
     size_t H2;      // theta-pass output: 3 line sets, rows and precision as H1
     size_t P32;     // mixed form: u', d_r u' in FP32, 6 x S float2
     size_t mean;    // mixed form: segment sums of the mean mode of N (mean00_part_doubles)
-    size_t fxe;     // FP64 plans: exponents of the fixed-point lines of all rows (tc_fx_nl.cu)
+    size_t fxe;     // FP64 plans and the adjoint: exponents of the fixed-point lines (tc_fx_z.cu), for N_r
+                    // rows, of which the first stage_rows are used
     size_t Ncur;    // N^i: vector field (everything before it is the forward staging)
     size_t uE;      // start-up Euler result: vector field
     size_t pstar;   // split path only: p* (scalar), u* (vector), phi (scalar)
@@ -225,7 +226,7 @@ void prof_end(tc_plan* p, int slot, cudaStream_t s);
 
 // ------------------------------------------------------------------ launchers
 tc_status launch_nonlinear_fx(tc_plan* p, const double2* u, double2* Nh, char* ws, cudaStream_t s);
-size_t fx_exp_bytes(const tc_plan* p);
+size_t fx_exp_bytes(const tc_plan* p, int rows);   // exponents of that many staged rows
 size_t fx_adj_exp_bytes(const tc_plan* p);
 int fx_zt_adj(const tc_plan* p, int forced);
 tc_status launch_adjoint_rows_fx(tc_plan* p, const double2* u, const double2* Nbar, double2* ubar, double2* Rh, char* ws,

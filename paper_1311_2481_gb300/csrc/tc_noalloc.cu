@@ -33,8 +33,9 @@
 namespace {
 
 constexpr size_t kStaticScratchBytes = (size_t)80 << 20;
-// behind the lines, the exponents of the FP64 form's fixed-point lines: at most 3/8 of a byte
-// per 8 bytes of lines (fx_exp_bytes against 12 line sets, P_z >= 3), and rounding
+// behind the lines, the exponents of the FP64 form's fixed-point lines (the staged rows'): a row has
+// 72 (M+1) + 8 + 8 P_z bytes of them (fx_exp_bytes) and 192 (M+1) P_z bytes of lines, M >= 1, P_z >= 3.
+// Where up to 2048 rows of lines fit 80 MiB, that is at most 10.1 MiB.
 constexpr size_t kStaticExpBytes = (size_t)12 << 20;
 constexpr int kMaxDevices = 64;
 
@@ -79,7 +80,7 @@ extern "C" tc_status tc_nonlinear_noalloc(tc_plan* plan, const void* u_hat, void
                  "holds %zu bytes (80 MiB); use tc_nonlinear with a workspace", need, kStaticScratchBytes);
         return TC_ERR_ARG;
     }
-    if (plan->ws.Ncur > kStaticScratchBytes + kStaticExpBytes) {
+    if (plan->precision != TC_MIXED && need + tc::fx_exp_bytes(plan, plan->stage_rows) > kStaticScratchBytes + kStaticExpBytes) {
         snprintf(plan->err, sizeof(plan->err), "tc_nonlinear_noalloc: the exponents of this plan do not fit the static scratch");
         return TC_ERR_ARG;
     }

@@ -795,7 +795,7 @@ tc_status tc_plan_create_ex(tc_plan** out, int N_r, int M, int K, int m_p, doubl
         p->ws.mean = take(0);
     }
     const size_t fwd_staging = off;
-    p->ws.fxe = take(p->precision == TC_MIXED && !p->adjoint ? 0 : fx_exp_bytes(p));
+    p->ws.fxe = take(p->precision == TC_MIXED && !p->adjoint ? 0 : fx_exp_bytes(p, N_r));
     p->ws.Ncur = take(3 * p->S * cplx);
     p->ws.uE = take(3 * p->S * cplx);
     // steps 2-5: fused kernel while 8 modes' four columns fit in 96 KB of shared memory,
