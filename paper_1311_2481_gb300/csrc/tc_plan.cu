@@ -643,6 +643,10 @@ tc_status tc_plan_create_ex(tc_plan** out, int N_r, int M, int K, int m_p, doubl
     if (!std::isfinite(Re_i) || !std::isfinite(Re_o) || !std::isfinite(L_z) || !std::isfinite(dt))
         return TC_ERR_ARG;
     if (o.precision != TC_FP64 && o.precision != TC_MIXED) return TC_ERR_ARG;
+    if (o.theta_zt < 0 || o.theta_zt > 64 || o.pc_modes < 0 || o.pc_modes > 32 || o.pc_split < -1 || o.pc_split > 1 ||
+        o.theta_variant < 0 || o.theta_variant > 4 || o.pc_partitions < 0 || o.pc_partitions > 2 ||
+        o.stage_rows < 0 || o.mean_fp32 < 0 || o.mean_fp32 > 1)
+        return TC_ERR_ARG;   // before they size anything
     double alpha = o.alpha == 0.0 ? 0.5 : (o.alpha < 0.0 ? 0.0 : o.alpha);
     if (alpha > 1.0) return TC_ERR_ARG;
     int Pt = o.P_theta ? o.P_theta : 3 * M;
@@ -751,12 +755,6 @@ tc_status tc_plan_create_ex(tc_plan** out, int N_r, int M, int K, int m_p, doubl
     p->pc_modes = o.pc_modes;
     p->theta_zt_forced = o.theta_zt;
     p->theta_variant = o.theta_variant;
-    if (o.theta_zt < 0 || o.theta_zt > 64 || o.pc_modes < 0 || o.pc_modes > 32 || o.pc_split < -1 || o.pc_split > 1 ||
-        o.theta_variant < 0 || o.theta_variant > 4 || o.pc_partitions < 0 || o.pc_partitions > 2 ||
-        o.stage_rows < 0 || o.mean_fp32 < 0 || o.mean_fp32 > 1) {
-        delete p;
-        return TC_ERR_ARG;
-    }
     {
         // 16-byte lines unless the plan is mixed without the adjoint
         const size_t lb = (o.precision == TC_MIXED && o.no_adjoint) ? sizeof(float2) : cplx;
