@@ -44,7 +44,7 @@ struct Exps {
 // start at multiples of kDrRows whatever r0, so that a row's result does not depend on the slab
 // it is staged in.
 __global__ void __launch_bounds__(128) k_fx_dr(const double* __restrict__ u, double* __restrict__ du,
-                                               const int2* __restrict__ w, const int* __restrict__ ew,
+                                               const int2* __restrict__ w, const int2* __restrict__ ew,
                                                const double* __restrict__ w1, const int* __restrict__ col0, int N,
                                                int ncol, int r0, int nh) {
     const int c = blockIdx.z, tile = (r0 / kDrRows + blockIdx.y) * kDrRows - r0, j0 = r0 + tile;
@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(128) k_fx_dr(const double* __restrict__ u, dou
         d[i] = j >= 0 && j < N ? __ldg(&src[(size_t)j * ncol]) : 0.0;
     }
     Tile<kDrRows> x;
-    x.load(d);
+    x.load(d, [&](int i) { return (unsigned)__ldg(&ew[min(max(j0 + i, 0), N - 1)].y); });
 #pragma unroll
     for (int i = 0; i < kDrRows; ++i) {
         const int j = j0 + i;
@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(128) k_fx_dr(const double* __restrict__ u, dou
 #pragma unroll
             for (int t = 0; t < kStencil; ++t) o = fma(__ldg(&w1[j * kStencil + t]), v[t], o);
         } else {
-            o = x.row(i, w + j * kStencil, __ldg(&ew[j]));
+            o = x.row(i, w + j * kStencil, __ldg(&ew[j].x));
         }
         du[((size_t)c * nh + tile + i) * ncol + col] = o;
     }

@@ -135,7 +135,7 @@ struct tc_plan {
     int fx_emm = 0;
     int4* d_fx_ir = nullptr;
     int2* d_fx_w1 = nullptr;     // fixed-point weights of the radial stencil
-    int* d_fx_ew = nullptr;      // their exponents per row
+    int2* d_fx_ew = nullptr;     // their exponent per row, and those of the four nearest weights (fx::Tile)
     // non-finite flag: mapped pinned host memory that the update kernels set when they write
     // a NaN/Inf into the state; tc_step reports and clears it
     int* h_nonfinite = nullptr;

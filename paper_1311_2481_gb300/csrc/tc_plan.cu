@@ -527,21 +527,26 @@ static tc_status upload(tc_plan* p) {
     }
     {   // fixed-point weights of the radial stencils
         std::vector<int2> w(p->w1.size(), make_int2(0, 0));
-        std::vector<int> ew(p->N_r);
+        std::vector<int2> ew(p->N_r);
         for (int j = 0; j < p->N_r; ++j) {
             long double sum = 0;
             for (int t = 0; t < kStencil; ++t) sum += std::fabs((long double)p->w1[(size_t)j * kStencil + t]);
-            std::frexp((double)sum * (1 + 1e-9), &ew[j]);
+            std::frexp((double)sum * (1 + 1e-9), &ew[j].x);
+            unsigned near = 0xffffffffu;   // of rows j - 2, j - 1, j + 1, j + 2: exponent of 2^ew / |w|, 255 for 0
             // the stencil of row j reaches rows j - 4 .. j + 4: entry t is row j - 4 + t
             for (int t = 0; t < kStencil; ++t) {
                 const int c = p->col0[j] + t - (j - 4);
                 const double v = p->w1[(size_t)j * kStencil + t];
-                if (v != 0.0 && c >= 0 && c < kStencil)
-                    fx_limbs(std::ldexp((long double)v, -ew[j]), w[(size_t)j * kStencil + c].x, w[(size_t)j * kStencil + c].y);
+                if (v == 0.0 || c < 0 || c >= kStencil) continue;
+                fx_limbs(std::ldexp((long double)v, -ew[j].x), w[(size_t)j * kStencil + c].x, w[(size_t)j * kStencil + c].y);
+                if (c < 2 || c > 6 || c == 4) continue;
+                const int at = 8 * (c < 4 ? c - 2 : c - 3), q = ew[j].x - std::ilogb(v);
+                near = (near & ~(255u << at)) | (unsigned)std::min(q, 255) << at;
             }
+            ew[j].y = (int)near;
         }
         TC_CUDA(p, put((void**)&p->d_fx_w1, w.data(), w.size() * sizeof(int2)));
-        TC_CUDA(p, put((void**)&p->d_fx_ew, ew.data(), ew.size() * sizeof(int)));
+        TC_CUDA(p, put((void**)&p->d_fx_ew, ew.data(), ew.size() * sizeof(int2)));
     }
     std::vector<float> f(p->tw_z.begin(), p->tw_z.end());
     TC_CUDA(p, put((void**)&p->d_tw_z32, f.data(), f.size() * sizeof(float)));

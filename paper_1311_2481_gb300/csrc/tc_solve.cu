@@ -32,8 +32,8 @@ struct PCArgs {
     const double* w1;
     const double* w2;
     const int* col0;
-    const int2* fw;       // fixed-point stencil weights and their exponents
-    const int* few;
+    const int2* fw;       // fixed-point stencil weights, their exponents and near ones (fx::Tile)
+    const int2* few;
     const double* fac;
     const uint8_t* piv;
     const double* fac2;   // two-partition form (g.sh > 0): factors of the diagonal blocks,
@@ -410,7 +410,7 @@ struct Stencil {
     const double* w1;
     const int* col0;
     const int2* fw;
-    const int* few;
+    const int2* few;
 };
 struct Cols {
     int mode, part, m, k, j0;
@@ -452,8 +452,9 @@ __device__ __forceinline__ void tile_rows(const Cols& c, const Stencil& s, const
             if (PAIR) v2[i] = on ? __ldg(&f2[(size_t)j * st]) : 0.0;
         }
         Tile<kTileRows> X;
-        if (PAIR) X.load(v, v2);
-        else X.load(v);
+        auto near = [&](int i) { return (unsigned)__ldg(&s.few[min(c.j0 + i, N - 1)].y); };
+        if (PAIR) X.load(v, v2, near);
+        else X.load(v, near);
 #pragma unroll
         for (int i = 0; i < kTileRows; ++i) {
             const int j = c.j0 + i;
@@ -467,7 +468,7 @@ __device__ __forceinline__ void tile_rows(const Cols& c, const Stencil& s, const
                     d[i] = fma(w, PAIR ? x + __ldg(&f2[o]) : x, d[i]);
                 });
             } else {
-                d[i] = X.row(i, s.fw + j * kStencil, __ldg(&s.few[j]));
+                d[i] = X.row(i, s.fw + j * kStencil, __ldg(&s.few[j].x));
             }
         }
     }

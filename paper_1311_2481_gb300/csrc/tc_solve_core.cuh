@@ -270,7 +270,7 @@ __device__ __forceinline__ void smem_band_solve_c(double2* col, int T, int t, in
 // (8 rows per tile: 230 us, fewer threads with work and more rows left to FP64).
 constexpr int kTileRows = 4;   // rows per thread, here and in the split path
 template <int ZONE, bool FX, bool PAIR, class Slow, class Pre, class Body>
-__device__ __forceinline__ void stencil_rows(const int2* __restrict__ fw, const int* __restrict__ few, const double2* F,
+__device__ __forceinline__ void stencil_rows(const int2* __restrict__ fw, const int2* __restrict__ few, const double2* F,
                                              const double2* F2, int N, int T, Slow slow, Pre pre, Body body) {
     using namespace fx;
     const int c = threadIdx.x % (2 * T), step = blockDim.x / (2 * T), st = 2 * T;
@@ -290,12 +290,13 @@ __device__ __forceinline__ void stencil_rows(const int2* __restrict__ fw, const 
                     v[i] = j < N ? f[j * st] : 0.0;
                     if (PAIR) v2[i] = j < N ? f2[j * st] : 0.0;
                 }
-                if (PAIR) X.load(v, v2);
-                else X.load(v);
+                auto near = [&](int i) { return (unsigned)__ldg(&few[min(j0 + i, N - ZONE - 1)].y); };
+                if (PAIR) X.load(v, v2, near);
+                else X.load(v, near);
 #pragma unroll
                 for (int i = 0; i < kTileRows; ++i) {
                     const int j = min(j0 + i, N - ZONE - 1);
-                    d[i] = X.far(i) ? slow(j, c) : X.row(i, fw + j * kStencil, __ldg(&few[j]));
+                    d[i] = X.far(i) ? slow(j, c) : X.row(i, fw + j * kStencil, __ldg(&few[j].x));
                 }
             }
 #pragma unroll
