@@ -479,9 +479,9 @@ template <int R> struct Tile {
         }
         return to_double(take(s + (m >> 32), m, 28), e + ew - 1084);
     }
-    // b: exponents of the window's entries; near(i): those of 2^ew / |w| of the entries i + 2, i + 3,
+    // b: exponents of the window's entries; limit: kFar, or more where less accuracy does; near(i): those of 2^ew / |w| of the entries i + 2, i + 3,
     // i + 5, i + 6 of row j0 + i, a byte each
-    template <class Near> __device__ __forceinline__ void exponents(const int (&b)[R + 8], Near near) {
+    template <class Near> __device__ __forceinline__ void exponents(const int (&b)[R + 8], int limit, Near near) {
         e = 0;
 #pragma unroll
         for (int i = 0; i < R + 8; ++i) e = max(e, b[i]);
@@ -491,24 +491,24 @@ template <int R> struct Tile {
             const unsigned q = near(i);
             const int c = min(min((int)(q & 255) - b[i + 2], (int)(q >> 8 & 255) - b[i + 3]),
                               min((int)(q >> 16 & 255) - b[i + 5], (int)(q >> 24) - b[i + 6]));
-            if (e + c > kFar) fp64 |= 1u << i;
+            if (e + c > limit) fp64 |= 1u << i;
         }
     }
-    template <class Near> __device__ __forceinline__ void load(const double (&d)[R + 8], Near near) {
+    template <class Near> __device__ __forceinline__ void load(const double (&d)[R + 8], int limit, Near near) {
         int b[R + 8];
 #pragma unroll
         for (int i = 0; i < R + 8; ++i) b[i] = bexp(d[i]);
-        exponents(b, near);
+        exponents(b, limit, near);
 #pragma unroll
         for (int i = 0; i < R + 8; ++i) x[i] = split(fix_tile(d[i], e + 2));
     }
     // the window of a + d, added after the conversion (one exponent more)
     template <class Near>
-    __device__ __forceinline__ void load(const double (&a)[R + 8], const double (&d)[R + 8], Near near) {
+    __device__ __forceinline__ void load(const double (&a)[R + 8], const double (&d)[R + 8], int limit, Near near) {
         int b[R + 8];
 #pragma unroll
         for (int i = 0; i < R + 8; ++i) b[i] = max(bexp(a[i]), bexp(d[i])) + 1;
-        exponents(b, near);
+        exponents(b, limit, near);
 #pragma unroll
         for (int i = 0; i < R + 8; ++i) x[i] = split(fix_tile(a[i], e + 2) + fix_tile(d[i], e + 2));
     }

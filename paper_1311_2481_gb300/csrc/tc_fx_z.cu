@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(128) k_fx_dr(const double* __restrict__ u, dou
         d[i] = j >= 0 && j < N ? __ldg(&src[(size_t)j * ncol]) : 0.0;
     }
     Tile<kDrRows> x;
-    x.load(d, [&](int i) { return (unsigned)__ldg(&ew[min(max(j0 + i, 0), N - 1)].y); });
+    x.load(d, kFar, [&](int i) { return (unsigned)__ldg(&ew[min(max(j0 + i, 0), N - 1)].y); });
 #pragma unroll
     for (int i = 0; i < kDrRows; ++i) {
         const int j = j0 + i;

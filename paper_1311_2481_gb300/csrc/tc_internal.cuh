@@ -181,8 +181,8 @@ __device__ __forceinline__ bool nonfinite2(double2 v) {
 __device__ __forceinline__ bool stencil_row(int c0, int t) { return c0 + t >= 0; }
 // tap(t) for the rows c0 + t of a stencil that may be read.  A guard on each tap costs the sums in FP64 4 %
 // (k_pc, N_r = 160, M = 8, K = 16: 240 against 229 us); c0 has the same sign for every row of a plan.
-template <class Tap> __device__ __forceinline__ void stencil_taps(int c0, Tap tap) {
-    if (c0 >= 0) {
+template <bool GUARD, class Tap> __device__ __forceinline__ void stencil_taps(int c0, Tap tap) {
+    if (!GUARD || c0 >= 0) {
 #pragma unroll
         for (int t = 0; t < kStencil; ++t) tap(t);
     } else {

@@ -43,35 +43,38 @@ struct PCArgs {
     int* nonfinite;       // set to 1 when a NaN/Inf is written into the state
     double Re_i, Re_o;
     int commit;
+    int far;              // rows left to FP64 sums by the fixed-point stencils (fx::Tile): limit
+    int sum;              // the block has a fifth column, for C1 + C2
 };
 
 constexpr int kChunkF = 4, kChunkB = 2;   // rows of factors per register chunk (3, 2: 2 % and 4, 3: 9 % slower k_pc)
 
 // CH: chunks; the row by row ring of kPCDepth rows reaches further ahead, which counts where a launch
-// has few warps and nothing else covers a load (N_r = 160, M = 8, K = 16: k_pc 223 against 239 us)
+// has few warps and nothing else covers a load (N_r = 160, M = 8, K = 16: k_pc 223 against 239 us).
 template <bool CH>
-__device__ __forceinline__ void band_solve(double2* col, int T, int t, int part, int N, const double* __restrict__ F,
+__device__ __forceinline__ void band_solve(double2* col, int off, int T, int N, const double* __restrict__ F,
                                            const uint8_t* __restrict__ P, int M1K1) {
-    if (CH) smem_band_solve_c<kChunkF, kChunkB>(col, T, t, part, N, F, P, M1K1);
-    else smem_band_solve<kPCDepth>(col, T, t, part, N, F, P, M1K1);
+    if (CH) smem_band_solve_c<kChunkF, kChunkB>(col, T, off, N, F, P, M1K1);
+    else smem_band_solve<kPCDepth>(col, T, off, N, F, P, M1K1);
 }
 
-// Thread lt of the 4 nT threads of one system solves one half of it for one (mode, part):
-// threads [0, 2nT) rows [0, sh), threads [2nT, 4nT) rows [sh, N), each with the pivoted LU
-// factors of its diagonal block; the column then holds g = (A1^{-1} b1, A2^{-1} b2).
+// Thread lt of the threads of one system (its column X in shared memory).  With two partitions
+// (g.sh > 0) 4 nT threads, each with one half of it for one (mode, part): threads [0, 2nT) rows [0, sh),
+// threads [2nT, 4nT) rows [sh, N), with the pivoted LU factors of the diagonal block; the column then
+// holds g = (A1^{-1} b1, A2^{-1} b2).  Otherwise 2 nT threads with the factors of the whole system.
 template <bool CH>
-__device__ __forceinline__ void half_solve(const PCArgs& a, const Geo& g, double2* X, int set, int T, int nT,
-                                           int mode0, int lt) {
+__device__ __forceinline__ void system_solve(const PCArgs& a, const Geo& g, double2* X, int set, int T, int nT, int mode0, int lt) {
+    const bool sp = g.sh > 0;
     const int half = lt >= 2 * nT ? 1 : 0;
     const int r = lt - half * 2 * nT;
     const int t = r >> 1, part = r & 1;
     const int mode = mode0 + t, m = mode / g.nk, k = mode - m * g.nk - g.K;
     const size_t mk = (size_t)m * g.K1 + (k < 0 ? -k : k);
     const size_t per_set = (size_t)g.N * kBands * g.M1K1;
-    const int r0 = half ? g.sh : 0, n = half ? g.N - g.sh : g.sh;
-    band_solve<CH>(X + (size_t)r0 * T, T, t, part, n,
-                              a.fac2 + (size_t)set * per_set + (size_t)r0 * kBands * g.M1K1 + mk,
-                              a.piv2 + ((size_t)set * g.N + r0) * g.M1K1 + mk, g.M1K1);
+    const int r0 = half ? g.sh : 0, n = half ? g.N - g.sh : sp ? g.sh : g.N;
+    band_solve<CH>(X + (size_t)r0 * T, 2 * t + part, T, n,
+                   (sp ? a.fac2 : a.fac) + (size_t)set * per_set + (size_t)r0 * kBands * g.M1K1 + mk,
+                   (sp ? a.piv2 : a.piv) + ((size_t)set * g.N + r0) * g.M1K1 + mk, g.M1K1);
 }
 
 // Couple the halves of nsys systems (columns X0 + s N T, factor sets set0 + s), block-wide:
@@ -130,7 +133,7 @@ __device__ __forceinline__ double2 lap_pm(const double2* __restrict__ u, const P
     const double ir = a.ir[j], ir2 = ir * ir;
     double2 d1 = make_double2(0.0, 0.0), d2 = d1;
     const int c0 = a.col0[j];
-    stencil_taps(c0, [&](int t) {
+    stencil_taps<true>(c0, [&](int t) {
         const double2 x = f[(size_t)(c0 + t) * g.nmode + mode];
         const double p = __ldg(&a.w1[j * kStencil + t]), q = __ldg(&a.w2[j * kStencil + t]);
         d1.x += p * x.x;
@@ -146,6 +149,11 @@ __device__ __forceinline__ double2 lap_pm(const double2* __restrict__ u, const P
 // Steps 2-5 of Sec. 3.2 for the T modes of this block: pressure prediction (Eq. pressure
 // with the Neumann rows of Eq. ppBC), velocity prediction (Eq. vel), correction potential
 // (Eq. correction) and update (Eq. update).
+// The stages run as iterations of a loop around one copy of the substitution, of its coupling and of
+// the work beside it.  Once a launch takes several waves its blocks are at different stages, and
+// with a copy per stage they waited for instructions (1.6 warps per issue, 0.7 in the loop's smaller
+// code): N_r = 64, M = 64, K = 128, fixed-point stencils: 969 -> 908 us; one wave, N_r = 64, M = 32,
+// K = 64: 224 -> 221.
 template <int NTH, bool FX>
 __global__ void __launch_bounds__(NTH, 512 / NTH) k_pc(PCArgs a, Geo g, int T) {
     extern __shared__ double2 sm[];
@@ -157,7 +165,6 @@ __global__ void __launch_bounds__(NTH, 512 / NTH) k_pc(PCArgs a, Geo g, int T) {
     double2* C3 = C2 + items;
     const int mode0 = g.mlo + blockIdx.x * T;
     const int nT = min(T, g.mhi - mode0);
-    const size_t per_set = (size_t)N * kBands * g.M1K1;
     const double c1 = g.c1;   // 1 / (2 dt)
     // T divides the block size, so every element a thread visits in the element loops below
     // belongs to the same mode t = threadIdx.x % T: its row index steps by blockDim / T, and
@@ -172,6 +179,7 @@ __global__ void __launch_bounds__(NTH, 512 / NTH) k_pc(PCArgs a, Geo g, int T) {
 
     const bool in = tq < nT;
     double2* Lw = C3 + items;   // scratch of the spikes, free until then: L_pm u at the walls
+    double2* C4 = Lw + 24 * T;   // a.sum: C1 + C2
 
     // A1: (2N - N_prev)_+, _-, _z into C1, C2, C3; the halves of the wall Laplacians of u and
     // u_prev, one (field, component, wall, mode) per thread
@@ -190,6 +198,7 @@ __global__ void __launch_bounds__(NTH, 512 / NTH) k_pc(PCArgs a, Geo g, int T) {
         C1[idx] = n[0];
         C2[idx] = n[1];
         C3[idx] = n[2];
+        if (!FX && a.sum) C4[idx] = make_double2(n[0].x + n[1].x, n[0].y + n[1].y);
     }
     for (int i = threadIdx.x / T; i < 8; i += jstep)
         if (in) Lw[i * T + tq] = lap_pm(i & 4 ? a.up : a.u, a, i & 1, i & 2 ? N - 1 : 0, modeq, mmq, kkq, g);
@@ -200,187 +209,161 @@ __global__ void __launch_bounds__(NTH, 512 / NTH) k_pc(PCArgs a, Geo g, int T) {
     const int ks = modes - ms * g.nk - g.K;
     const bool ins = ts < nT;
     const double mms = g.mp * ms, kks = (part ? 1 : -1) * (g.kz * ks);   // i k of the other part: kks times it
-    // A2: pressure right-hand side into C0
+    const bool sp = g.sh > 0;
+    double* Xr = reinterpret_cast<double*>(C3 + items);
+    const double c3 = 3.0 * c1;   // 3 / (2 dt)
+    double* pw = a.commit && ins ? reinterpret_cast<double*>(a.p) + 2 * (size_t)modes + part : nullptr;
+    bool bad = false;
+    int stage = 0;
+    const int far = modes == g.K ? fx::kFar : a.far;   // the mean mode (0, 0) rounds as in FP64
     auto ir = [&](int j) { return __ldg(&a.ir[j]); };
-    auto d1 = [&](const double* f, int j) {   // FP64 stencil at row j
+    auto p0 = [&](int j) { return pw ? pw[2 * (size_t)j * g.nmode] : 0.0; };
+    auto slow0 = [&](int j, int c, auto guard) {   // FP64 stencil at row j of C0
         const int c0 = __ldg(&a.col0[j]);
         double o = 0.0;
-        stencil_taps(c0, [&](int q) { o = fma(__ldg(&a.w1[j * kStencil + q]), f[(c0 + q) * 2 * T], o); });
+        stencil_taps<decltype(guard)::value>(c0, [&](int q) { o = fma(__ldg(&a.w1[j * kStencil + q]), D0[c + (c0 + q) * 2 * T], o); });
         return o;
     };
-    auto d1s = [&](const double* f, const double* f2, int j) {   // of f + f2
+    auto slow12 = [&](int j, int c, auto guard) {   // of C1 + C2
         const int c0 = __ldg(&a.col0[j]);
         double o = 0.0;
-        stencil_taps(c0, [&](int q) {
-            const int n = (c0 + q) * 2 * T;
-            o = fma(__ldg(&a.w1[j * kStencil + q]), f[n] + f2[n], o);
+        if (!FX && a.sum) {
+            const double* D4 = reinterpret_cast<const double*>(C4);
+            stencil_taps<decltype(guard)::value>(c0, [&](int q) { o = fma(__ldg(&a.w1[j * kStencil + q]), D4[c + (c0 + q) * 2 * T], o); });
+            return o;
+        }
+        stencil_taps<decltype(guard)::value>(c0, [&](int q) {
+            const int n = c + (c0 + q) * 2 * T;
+            o = fma(__ldg(&a.w1[j * kStencil + q]), D1[n] + D2[n], o);
         });
         return o;
     };
-    auto slow0 = [&](int j, int c) { return d1(D0 + c, j); };
-    auto slow12 = [&](int j, int c) { return d1s(D1 + c, D2 + c, j); };
-    stencil_rows<4, FX, true>(a.fw, a.few, C1, C2, N, T, slow12, ir, [&](int j, int i, double d, double irj) {
-        double out = 0.0;
-        const double n = D1[i], m = D2[i];
-        if (j == 0 || j == N - 1) {
-            if (ins && !(j == N - 1 && ms == 0 && ks == 0)) {
-                const double* L = reinterpret_cast<const double*>(Lw + (j == 0 ? 0 : 2 * T) + ts) + part;
-                out = -0.5 * (n + m) + (L[0] + L[2 * T]) - 0.5 * (L[8 * T] + L[10 * T]);
-            }
-        } else {
-            const double hr = 0.5 * irj;
-            out = -(fma(mms * hr, n - m, fma(n + m, hr, 0.5 * d)) + kks * D3[i ^ 1]);
-        }
-        D0[i] = out;
-    });
-    __syncthreads();
-    // B: p* = P^{-1} b_p (real and imaginary parts by separate threads).  Meanwhile the
-    // warps without a substitution precompute the part of the velocity right-hand sides that
-    // does not depend on p*, (4u - u_prev)/(2dt) - (2N - N_prev), in place of the latter, and the
-    // Dirichlet rows.
-    // With two partitions (g.sh > 0) 4 nT threads solve, two per (mode, part).
-    const bool sp = g.sh > 0;
-    double* Xr = reinterpret_cast<double*>(C3 + items);
-    const int nsolve = (sp ? 4 : 2) * nT;
-    const int helper0 = ((nsolve + 31) / 32) * 32;
-    if (threadIdx.x < nsolve) {
-        if (sp) {
-            half_solve<FX>(a, g, C0, kSetP, T, nT, mode0, threadIdx.x);
-        } else {
-            const int t = threadIdx.x >> 1, part = threadIdx.x & 1;
-            const int mode = mode0 + t, m = mode / g.nk, k = mode - m * g.nk - g.K;
-            const size_t mk = (size_t)m * g.K1 + (k < 0 ? -k : k);
-            band_solve<FX>(C0, T, t, part, N, a.fac + (size_t)kSetP * per_set + mk,
-                            a.piv + (size_t)kSetP * N * g.M1K1 + mk, g.M1K1);
-        }
-    }
-    // (with no spare warp the whole block does this after the substitution)
-    const bool spare0 = helper0 < (int)blockDim.x;
-    if (!spare0) __syncthreads();
-    if (spare0 ? threadIdx.x >= helper0 : true) {
-        const int first = spare0 ? helper0 : 0;   // a multiple of 32: (threadIdx.x - first) % T == tq
-        for (int j = (threadIdx.x - first) / T; j < N; j += ((int)blockDim.x - first) / T) {
-            const int idx = j * T + tq;
-            double2 o[3] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0), make_double2(0.0, 0.0)};
-            if (in) {
+    // div_h of (p, m, D3), given dr = 2 d_r v_r + 2 v_r / r of v_r = (p + m) / 2: one halving, which is
+    // exact, for three terms
+    auto div = [&](double p, double m, double dr, double irj, int i) {
+        return fma(kks, D3[i ^ 1], 0.5 * fma(mms * irj, p - m, dr));
+    };
+    auto stencils = [&] {
+        if (stage == 0) {         // A2: pressure right-hand side into C0
+            stencil_rows<4, FX, true>(a.fw, a.few, far, C1, C2, N, T, slow12, ir, [&](int j, int i, double d, double irj) {
+                double out = 0.0;
+                const double n = D1[i], m = D2[i];
                 if (j == 0 || j == N - 1) {
-                    if (mq == 0 && kq == 0) {
-                        const double Re = j == 0 ? a.Re_i : a.Re_o;
-                        o[0].y = Re;
-                        o[1].y = -Re;
+                    if (ins && !(j == N - 1 && ms == 0 && ks == 0)) {
+                        const double* L = reinterpret_cast<const double*>(Lw + (j == 0 ? 0 : 2 * T) + ts) + part;
+                        out = -0.5 * (n + m) + (L[0] + L[2 * T]) - 0.5 * (L[8 * T] + L[10 * T]);
                     }
                 } else {
-                    const size_t e = (size_t)j * g.nmode + modeq;
-                    o[0] = C1[idx];
-                    o[1] = C2[idx];
-                    o[2] = C3[idx];
+                    out = -div(n, m, fma(n + m, irj, d), irj, i);
+                }
+                D0[i] = out;
+            });
+        } else if (stage == 1) {  // C: velocity right-hand sides: subtract grad_h p* on interior rows; p <- p* (commit)
+            stencil_rows<4, FX, false>(a.fw, a.few, far, C0, nullptr, N, T, slow0, ir, [&](int j, int i, double d, double irj) {
+                if (!ins) return;
+                const double pv = D0[i];
+                if (pw) pw[2 * (size_t)j * g.nmode] = pv;
+                if (j == 0 || j == N - 1) return;
+                const double tp = mms * irj * pv;
+                D1[i] -= d - tp;
+                D2[i] -= d + tp;
+                D3[i] -= kks * D0[i ^ 1];
+            });
+        } else if (stage == 2) {  // E: div_h u* into C0 (homogeneous Neumann / Dirichlet rows)
+            if (!FX && a.sum) {
+                for (int i = threadIdx.x; i < items; i += blockDim.x) C4[i] = make_double2(C1[i].x + C2[i].x, C1[i].y + C2[i].y);
+                __syncthreads();
+            }
+            stencil_rows<4, FX, true>(a.fw, a.few, far, C1, C2, N, T, slow12, ir, [&](int j, int i, double d, double irj) {
+                double out = 0.0;
+                if (ins && j > 0 && j < N - 1) out = div(D1[i], D2[i], __dadd_rn(d, __dmul_rn(D1[i] + D2[i], irj)), irj, i);
+                D0[i] = out;
+            });
+        } else {                  // G: u^{i+1} = u* - grad_h phi, p^{i+1} = p* + 3 phi / (2 dt)
+            stencil_rows<4, FX, false>(a.fw, a.few, far, C0, nullptr, N, T, slow0, p0, [&](int j, int i, double d, double p) {
+                if (!ins) return;
+                const size_t e = 2 * ((size_t)j * g.nmode + modes) + part;
+                const double f = D0[i], tf = mms * __ldg(&a.ir[j]) * f;
+                const double un[3] = {D1[i] - (d - tf), D2[i] - (d + tf), D3[i] - kks * D0[i ^ 1]};
 #pragma unroll
-                    for (int c = 0; c < 3; ++c) {
-                        const size_t ec = (size_t)c * g.S + e;
-                        const double2 uu = a.u[ec], q = a.up[ec];
-                        o[c].x = (4.0 * uu.x - q.x) * c1 - o[c].x;
-                        o[c].y = (4.0 * uu.y - q.y) * c1 - o[c].y;
+                for (int c = 0; c < 3; ++c) {
+                    reinterpret_cast<double*>(a.u_out)[2 * c * g.S + e] = un[c];
+                    bad |= nonfinite1(un[c]);
+                }
+                if (pw) pw[2 * (size_t)j * g.nmode] = fma(c3, f, p);
+            });
+        }
+    };
+    // the warps without a substitution, from thread `first` (a multiple of T) on
+    auto beside = [&](int first) {
+        const int j0 = ((int)threadIdx.x - first) / T, dj = ((int)blockDim.x - first) / T;
+        if (stage == 0) {
+            // beside P: the part of the velocity right-hand sides that does not depend on p*,
+            // (4u - u_prev)/(2dt) - (2N - N_prev), in place of the latter, and the Dirichlet rows
+            for (int j = j0; j < N; j += dj) {
+                const int idx = j * T + tq;
+                double2 o[3] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0), make_double2(0.0, 0.0)};
+                if (in) {
+                    if (j == 0 || j == N - 1) {
+                        if (mq == 0 && kq == 0) {
+                            const double Re = j == 0 ? a.Re_i : a.Re_o;
+                            o[0].y = Re;
+                            o[1].y = -Re;
+                        }
+                    } else {
+                        const size_t e = (size_t)j * g.nmode + modeq;
+                        o[0] = C1[idx];
+                        o[1] = C2[idx];
+                        o[2] = C3[idx];
+#pragma unroll
+                        for (int c = 0; c < 3; ++c) {
+                            const size_t ec = (size_t)c * g.S + e;
+                            const double2 uu = a.u[ec], q = a.up[ec];
+                            o[c].x = (4.0 * uu.x - q.x) * c1 - o[c].x;
+                            o[c].y = (4.0 * uu.y - q.y) * c1 - o[c].y;
+                        }
                     }
                 }
+                C1[idx] = o[0];
+                C2[idx] = o[1];
+                C3[idx] = o[2];
             }
-            C1[idx] = o[0];
-            C2[idx] = o[1];
-            C3[idx] = o[2];
-        }
-    }
-    __syncthreads();
-    if (sp) spike_combine(a, g, C0, 1, kSetP, T, nT, mode0, Xr);
-    // C: velocity right-hand sides: subtract grad_h p* on interior rows; p <- p* (commit)
-    stencil_rows<4, FX, false>(a.fw, a.few, C0, nullptr, N, T, slow0, ir, [&](int j, int i, double d, double irj) {
-        if (!ins) return;
-        const double pv = D0[i];
-        if (a.commit) reinterpret_cast<double*>(a.p)[2 * ((size_t)j * g.nmode + modes) + part] = pv;
-        if (j == 0 || j == N - 1) return;
-        const double tp = mms * irj * pv;
-        D1[i] -= d - tp;
-        D2[i] -= d + tp;
-        D3[i] -= kks * D0[i ^ 1];
-    });
-    __syncthreads();
-    // D: the three Helmholtz solves.  Meanwhile the other warps rotate the history (nothing
-    // reads u_prev or N_prev after C): u_prev <- u^i, N_prev <- N^i (commit).
-    const int nsolve1 = (sp ? 12 : 6) * nT;
-    const int helper1 = ((nsolve1 + 31) / 32) * 32;
-    if (threadIdx.x < nsolve1) {
-        if (sp) {
-            const int c = threadIdx.x / (4 * nT);
-            half_solve<FX>(a, g, C1 + (size_t)c * items, kSetHp + c, T, nT, mode0, threadIdx.x - c * 4 * nT);
-        } else {
-            const int c = threadIdx.x / (2 * nT), rem = threadIdx.x - c * 2 * nT;
-            const int t = rem >> 1, part = rem & 1;
-            const int mode = mode0 + t, m = mode / g.nk, k = mode - m * g.nk - g.K;
-            const size_t mk = (size_t)m * g.K1 + (k < 0 ? -k : k);
-            const int set = kSetHp + c;
-            band_solve<FX>(C1 + (size_t)c * items, T, t, part, N, a.fac + (size_t)set * per_set + mk,
-                            a.piv + (size_t)set * N * g.M1K1 + mk, g.M1K1);
-        }
-    } else if (a.commit && threadIdx.x >= helper1) {
-        for (int idx = threadIdx.x - helper1; idx < 3 * items; idx += blockDim.x - helper1) {
-            const int c = idx / items, rem = idx - c * items;
-            const int j = rem / T, t = rem - (rem / T) * T;
-            if (t >= nT) continue;
-            const size_t ec = (size_t)c * g.S + (size_t)j * g.nmode + mode0 + t;
-            a.up_out[ec] = a.u[ec];
-            a.Np_out[ec] = a.Nc[ec];
-        }
-    }
-    __syncthreads();
-    if (sp) spike_combine(a, g, C1, 3, kSetHp, T, nT, mode0, Xr);
-    if (a.commit && helper1 >= (int)blockDim.x) {   // no spare warp: rotate here
-        for (int idx = threadIdx.x; idx < 3 * items; idx += blockDim.x) {
-            const int c = idx / items, rem = idx - c * items;
-            const int j = rem / T, t = rem - (rem / T) * T;
-            if (t >= nT) continue;
-            const size_t ec = (size_t)c * g.S + (size_t)j * g.nmode + mode0 + t;
-            a.up_out[ec] = a.u[ec];
-            a.Np_out[ec] = a.Nc[ec];
-        }
-    }
-    // E: div_h u* into C0 (homogeneous Neumann / Dirichlet rows)
-    stencil_rows<4, FX, true>(a.fw, a.few, C1, C2, N, T, slow12, ir, [&](int j, int i, double d, double irj) {
-        double out = 0.0;
-        if (ins && j > 0 && j < N - 1) {
-            const double hr = 0.5 * irj, vp = D1[i], vm = D2[i];
-            out = 0.5 * d + (vp + vm) * hr + mms * hr * (vp - vm) + kks * D3[i ^ 1];
-        }
-        D0[i] = out;
-    });
-    __syncthreads();
-    // F: phi = P^{-1} div_h u*
-    if (threadIdx.x < nsolve) {
-        if (sp) {
-            half_solve<FX>(a, g, C0, kSetP, T, nT, mode0, threadIdx.x);
-        } else {
-            const int t = threadIdx.x >> 1, part = threadIdx.x & 1;
-            const int mode = mode0 + t, m = mode / g.nk, k = mode - m * g.nk - g.K;
-            const size_t mk = (size_t)m * g.K1 + (k < 0 ? -k : k);
-            band_solve<FX>(C0, T, t, part, N, a.fac + (size_t)kSetP * per_set + mk,
-                            a.piv + (size_t)kSetP * N * g.M1K1 + mk, g.M1K1);
-        }
-    }
-    __syncthreads();
-    if (sp) spike_combine(a, g, C0, 1, kSetP, T, nT, mode0, Xr);
-    // G: u^{i+1} = u* - grad_h phi, p^{i+1} = p* + 3 phi / (2 dt), history rotation
-    bool bad = false;
-    double* pw = a.commit && ins ? reinterpret_cast<double*>(a.p) + 2 * (size_t)modes + part : nullptr;
-    auto p0 = [&](int j) { return pw ? pw[2 * (size_t)j * g.nmode] : 0.0; };
-    stencil_rows<4, FX, false>(a.fw, a.few, C0, nullptr, N, T, slow0, p0, [&](int j, int i, double d, double p) {
-        if (!ins) return;
-        const size_t e = 2 * ((size_t)j * g.nmode + modes) + part;
-        const double f = D0[i], tf = mms * __ldg(&a.ir[j]) * f;
-        const double un[3] = {D1[i] - (d - tf), D2[i] - (d + tf), D3[i] - kks * D0[i ^ 1]};
+        } else if (stage == 1 && a.commit && in) {
+            // beside H: rotate the history (nothing reads u_prev or N_prev any more):
+            // u_prev <- u^i, N_prev <- N^i
+            for (int j = j0; j < N; j += dj)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            reinterpret_cast<double*>(a.u_out)[2 * c * g.S + e] = un[c];
-            bad |= nonfinite1(un[c]);
+                for (int c = 0; c < 3; ++c) {
+                    const size_t ec = (size_t)c * g.S + (size_t)j * g.nmode + modeq;
+                    a.up_out[ec] = a.u[ec];
+                    a.Np_out[ec] = a.Nc[ec];
+                }
         }
-        if (pw) pw[2 * (size_t)j * g.nmode] = p + 3.0 * c1 * f;   // 3 / (2 dt)
-    });
+    };
+#pragma unroll 1
+    for (;; ++stage) {
+        stencils();
+        if (stage == 3) break;
+        __syncthreads();
+        // B: p* = P^{-1} b_p;  D: the three Helmholtz solves;  F: phi = P^{-1} div_h u* (real and
+        // imaginary parts by separate threads, two per (mode, part) with two partitions)
+        const int nsys = stage == 1 ? 3 : 1, set0 = stage == 1 ? kSetHp : kSetP, per = (sp ? 4 : 2) * nT;
+        const int helper = (nsys * per + 31) / 32 * 32;
+        const bool spare = helper < (int)blockDim.x;
+        double2* X0 = stage == 1 ? C1 : C0;
+        if ((int)threadIdx.x < nsys * per) {
+            const int c = nsys == 1 ? 0 : threadIdx.x / per;
+            system_solve<FX>(a, g, X0 + (size_t)c * items, set0 + c, T, nT, mode0, threadIdx.x - c * per);
+        } else if (spare && (int)threadIdx.x >= helper) {
+            beside(helper);
+        }
+        __syncthreads();
+        if (!spare) {   // with no spare warp the whole block does it
+            beside(0);
+            __syncthreads();
+        }
+        if (sp) spike_combine(a, g, X0, nsys, set0, T, nT, mode0, Xr);
+    }
     if (bad && a.nonfinite) *a.nonfinite = 1;
 }
 
@@ -411,6 +394,7 @@ struct Stencil {
     const int* col0;
     const int2* fw;
     const int2* few;
+    int far;   // limit of the rows left to FP64 sums
 };
 struct Cols {
     int mode, part, m, k, j0;
@@ -453,8 +437,9 @@ __device__ __forceinline__ void tile_rows(const Cols& c, const Stencil& s, const
         }
         Tile<kTileRows> X;
         auto near = [&](int i) { return (unsigned)__ldg(&s.few[min(c.j0 + i, N - 1)].y); };
-        if (PAIR) X.load(v, v2, near);
-        else X.load(v, near);
+        const int far = c.mode == g.K ? kFar : s.far;
+        if (PAIR) X.load(v, v2, far, near);
+        else X.load(v, far, near);
 #pragma unroll
         for (int i = 0; i < kTileRows; ++i) {
             const int j = c.j0 + i;
@@ -462,7 +447,7 @@ __device__ __forceinline__ void tile_rows(const Cols& c, const Stencil& s, const
             if (!c.in || j >= N) continue;
             if (j < 4 || j > N - 5 || X.far(i)) {
                 const int c0 = __ldg(&s.col0[j]);
-                stencil_taps(c0, [&](int t) {
+                stencil_taps<true>(c0, [&](int t) {
                     const size_t o = (size_t)(c0 + t) * st;
                     const double w = __ldg(&s.w1[j * kStencil + t]), x = __ldg(&f[o]);
                     d[i] = fma(w, PAIR ? x + __ldg(&f2[o]) : x, d[i]);
@@ -725,7 +710,7 @@ __global__ void k_band_solve_g(double2* __restrict__ x, const double* __restrict
     const double* F = fac + (size_t)set * per_set + mk;
     const uint8_t* P = piv + (size_t)set * g.N * g.M1K1 + mk;
     if (D > 1) gmem_band_solve<D>(reinterpret_cast<double*>(x + (size_t)fld * g.S + mode) + part, (size_t)2 * g.nmode, g.N, F, P, g.M1K1);
-    else smem_band_solve(x + (size_t)fld * g.S, g.nmode, mode, part, g.N, F, P, g.M1K1);
+    else smem_band_solve(x + (size_t)fld * g.S + mode, g.nmode, part, g.N, F, P, g.M1K1);
 }
 
 // Stand-alone solve of one system set for all modes (tc_helmholtz_solve): columns staged in
@@ -738,7 +723,7 @@ __global__ void __launch_bounds__(128) k_band_solve_s2(const double2* rhs, doubl
     for (int j = threadIdx.x / T; j < N; j += blockDim.x / T)
         sm[j * T + t] = t < nT ? rhs[(size_t)j * g.nmode + mode0 + t] : make_double2(0.0, 0.0);
     __syncthreads();
-    if (threadIdx.x < 4 * nT) half_solve<true>(a, g, sm, set, T, nT, mode0, threadIdx.x);
+    if (threadIdx.x < 4 * nT) system_solve<true>(a, g, sm, set, T, nT, mode0, threadIdx.x);
     __syncthreads();
     spike_combine(a, g, sm, 1, set, T, nT, mode0, reinterpret_cast<double*>(sm + (size_t)N * T));
     if (t < nT)
@@ -761,7 +746,7 @@ __global__ void __launch_bounds__(256) k_band_solve_s(const double2* rhs, double
         const int mode = mode0 + t, m = mode / g.nk, k = mode - m * g.nk - g.K;
         const size_t mk = (size_t)m * g.K1 + (k < 0 ? -k : k);
         const size_t per_set = (size_t)N * kBands * g.M1K1;
-        smem_band_solve<kPCDepth>(sm, T, t, part, N, fac + (size_t)set * per_set + mk, piv + (size_t)set * N * g.M1K1 + mk, g.M1K1);
+        smem_band_solve<kPCDepth>(sm, T, 2 * t + part, N, fac + (size_t)set * per_set + mk, piv + (size_t)set * N * g.M1K1 + mk, g.M1K1);
     }
     __syncthreads();
     for (int idx = threadIdx.x; idx < N * T; idx += blockDim.x) {
@@ -916,6 +901,12 @@ tc_status launch_solve(tc_plan* p, int set, const double2* rhs, double2* x, cuda
     return TC_OK;
 }
 
+// Limit of the rows that the fixed-point stencils of a mixed plan leave to FP64 sums: its transforms are in FP32, and
+// its stencils were double-FP32 dot products, good to 2^-46 of sum |w f|; this limit keeps them at 2^-47.
+// The mean mode keeps fx::kFar.  k_pc with fx::kFar throughout: 895 against 854 us (N_r = 64, M = 64,
+// K = 128).
+constexpr int kFarMixed = 12;
+
 static tc_status launch_advance_split(tc_plan* p, const double2* u, double2* u_prev, const double2* Ncur,
                                       double2* N_prev, double2* p_out, double2* u_out, char* ws, bool commit,
                                       cudaStream_t s, int ma, int mb) {
@@ -935,7 +926,7 @@ static tc_status launch_advance_split(tc_plan* p, const double2* u, double2* u_p
         const bool ring = (size_t)2 * nm * nf < (size_t)24 * 32 * p->num_sms;
         (ring ? k_band_solve_g<kGD> : k_band_solve_g<1>)<<<grid, 128, 0, s>>>(x, p->d_fac, p->d_piv, set, nf, g);
     };
-    const Stencil st{p->d_w1, p->d_col0, p->d_fx_w1, p->d_fx_ew};
+    const Stencil st{p->d_w1, p->d_col0, p->d_fx_w1, p->d_fx_ew, p->precision == TC_MIXED ? kFarMixed : fx::kFar};
     const dim3 gt(blocks_for((size_t)2 * nm, 128), blocks_for(g.N, kTileRows));
     int slot = prof_begin(p, kKRhsPressure, s);
     k_nn_r<<<g1, 128, 0, s>>>(Ncur, N_prev, phi, g);
@@ -973,13 +964,16 @@ static tc_status launch_advance_split(tc_plan* p, const double2* u, double2* u_p
     return TC_OK;
 }
 
-// Fixed-point stencils in a launch of blocks of T modes, while enough warps share the FP64 pipe (14
-// per SM: 219 against 252 us for k_pc, N_r = 64, M = 32, K = 64); with fewer than 8 per SM their
-// conversions take longer than the FP64 FMAs (2 per SM: 90 against 61 us, N_r = 32, M = 8, K = 16),
-// and so they do with few rows, a quarter of which are wall rows (575 against 528 us, N_r = 32,
-// M = 64, K = 128; 754 against 760 at N_r = 48).
+// Fixed-point stencils in a launch of blocks of T modes.  With fewer than 8 warps per SM their
+// conversions take longer than the FP64 FMAs (N_r = 160, M = 8, K = 16: 273 against 225 us).  With many
+// they are the faster form from some 76 rows on: below, two blocks with a fifth column for the sum of
+// u_+ and u_- (launch_advance) fit an SM, and the tiles of 4 rows do not spread evenly over the warps.
+// M = 64, K = 128, fixed point against FP64: N_r = 48 756 and 674 us, 64 909 and 890, 72 1017 and 1009;
+// M = K = 64: N_r = 80 556 and 563, 96 652 and 729.  In the mixed form, which leaves fewer rows to FP64
+// (kFarMixed), from 56 on: 48 696 and 674, 56 783 and 784, 64 874 and 890.
 static bool fx_stencils(const tc_plan* p, int nmode, int T) {
-    return p->N_r >= 48 && (size_t)blocks_for(nmode, T) * (T <= 8 ? 128 : 256) >= (size_t)256 * p->num_sms;
+    return p->N_r >= (p->precision == TC_MIXED ? 56 : 76) &&
+           (size_t)blocks_for(nmode, T) * (T <= 8 ? 128 : 256) >= (size_t)256 * p->num_sms;
 }
 
 tc_status launch_advance(tc_plan* p, const double2* u, double2* u_prev, const double2* Ncur,
@@ -1006,7 +1000,7 @@ tc_status launch_advance(tc_plan* p, const double2* u, double2* u_prev, const do
     a.commit = commit ? 1 : 0;
     // two partitions while the 12 T substitution threads of the Helmholtz phase fit the block
     g.sh = (p->part_h > 0 && 12 * T <= (T <= 8 ? 128 : 256)) ? p->part_h : 0;
-    const size_t sm = (size_t)4 * p->N_r * T * sizeof(double2) + (size_t)3 * T * 16 * sizeof(double);
+    size_t sm = (size_t)4 * p->N_r * T * sizeof(double2) + (size_t)3 * T * 16 * sizeof(double);
     // 128 threads up to 8 modes per block, 256 beyond (6T substitution threads plus helpers)
     const int slot = prof_begin(p, kKPC, s);
     auto run = [&](auto kern, int nth) -> tc_status {
@@ -1015,6 +1009,14 @@ tc_status launch_advance(tc_plan* p, const double2* u, double2* u_prev, const do
         return TC_OK;
     };
     const bool fxs = fx_stencils(p, g.mhi - g.mlo, T);
+    a.far = p->precision == TC_MIXED ? kFarMixed : fx::kFar;
+    // A fifth column for C1 + C2, whose FP64 stencils then take 9 operations less a row (N_r = 48, M = 64,
+    // K = 128: 716 -> 660 us), where it costs no block its place:
+    // per_sm blocks of an SM that the registers allow and the launch has.
+    const size_t col = (size_t)p->N_r * T * sizeof(double2);
+    const int per_sm = std::min(T <= 8 ? 4 : 2, (blocks_for(g.mhi - g.mlo, T) + p->num_sms - 1) / p->num_sms);
+    a.sum = !fxs && (sm + col + 1024) * per_sm <= (size_t)228 * 1024 ? 1 : 0;
+    if (a.sum) sm += col;
     if (T <= 8) TC_TRY_STATUS(fxs ? run(k_pc<128, true>, 128) : run(k_pc<128, false>, 128));
     else TC_TRY_STATUS(fxs ? run(k_pc<256, true>, 256) : run(k_pc<256, false>, 256));
     prof_end(p, slot, s);

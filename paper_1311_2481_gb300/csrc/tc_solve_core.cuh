@@ -31,7 +31,7 @@ __device__ __forceinline__ double2 drow(const double2* __restrict__ f, const dou
                                         const int* __restrict__ col0, int j, int nmode, int mode) {
     const int c0 = col0[j];
     double2 s = make_double2(0.0, 0.0);
-    stencil_taps(c0, [&](int t) {
+    stencil_taps<true>(c0, [&](int t) {
         const double wt = __ldg(&w[j * kStencil + t]);
         const double2 v = f[(size_t)(c0 + t) * nmode + mode];
         s.x += wt * v.x;
@@ -73,10 +73,10 @@ static __device__ double2 lap_r(const double2* __restrict__ u, const double* __r
 // a step streams more than L2 holds between two uses), and one row of arithmetic does not
 // cover that latency.
 template <int D = 1>
-__device__ __forceinline__ void smem_band_solve(double2* col, int T, int t, int part, int N,
+__device__ __forceinline__ void smem_band_solve(double2* col, int T, int off, int N,
                                                 const double* __restrict__ F, const uint8_t* __restrict__ P,
                                                 int M1K1) {
-    double* x = reinterpret_cast<double*>(col) + 2 * t + part;   // x[j] at x[2 T j]
+    double* x = reinterpret_cast<double*>(col) + off;   // x[j] at x[2 T j]
     const int st = 2 * T;
     const size_t rs = (size_t)kBands * M1K1;                      // one row of factors
     // forward: rows j .. j+4 live in w0..w4
@@ -169,17 +169,17 @@ __device__ __forceinline__ void smem_band_solve(double2* col, int T, int t, int 
 // loads of several rows on one scoreboard, and waiting for a row then waits for the youngest of
 // them, a memory latency per row; a chunk's loads are waited for once, a chunk later.
 template <int CF, int CB>
-__device__ __forceinline__ void smem_band_solve_c(double2* col, int T, int t, int part, int N,
+__device__ __forceinline__ void smem_band_solve_c(double2* col, int T, int off, int N,
                                                   const double* __restrict__ F, const uint8_t* __restrict__ P,
                                                   int M1K1) {
-    double* x = reinterpret_cast<double*>(col) + 2 * t + part;   // x[j] at x[2 T j]
+    double* x = reinterpret_cast<double*>(col) + off;   // x[j] at x[2 T j]
     const int st = 2 * T;
     const size_t rs = (size_t)kBands * M1K1;
     double w0 = x[0], w1 = N > 1 ? x[st] : 0.0, w2 = N > 2 ? x[2 * st] : 0.0,
            w3 = N > 3 ? x[3 * st] : 0.0, w4 = N > 4 ? x[4 * st] : 0.0;
     {
-        double lr[2][CF][4];
-        int pr[2][CF];
+        double lr[2][CF][4] = {};   // initialised: in k_pc's loop ptxas otherwise keeps them live around it and spills
+        int pr[2][CF] = {};
         auto load = [&](double (&l)[CF][4], int (&p)[CF], int c) {
 #pragma unroll
             for (int d = 0; d < CF; ++d) {
@@ -219,7 +219,7 @@ __device__ __forceinline__ void smem_band_solve_c(double2* col, int T, int t, in
         }
     }
     double v1 = 0.0, v2 = 0.0, v3 = 0.0, v4 = 0.0, v5 = 0.0, v6 = 0.0, v7 = 0.0, v8 = 0.0;
-    double ur[2][CB][9];
+    double ur[2][CB][9] = {};
     auto load = [&](double (&u)[CB][9], int c) {
 #pragma unroll
         for (int d = 0; d < CB; ++d) {
@@ -260,27 +260,31 @@ __device__ __forceinline__ void smem_band_solve_c(double2* col, int T, int t, in
 
 // The element loops of k_pc with a radial stencil: body(j, i, d, pre(j)) for the real
 // and imaginary parts of all rows of the block's modes, i the index of the part's double in the
-// [N][T] arrays in shared memory, d the stencil at row j of F (of F + F2).  pre: the body's load
-// from device memory, issued ahead of the stencil.  slow(j, c): the FP64 sum at row j of column c.
+// [N][T] arrays in shared memory, d the stencil at row j of F (of F + F2 with pair).  pre: the body's
+// load from device memory, issued ahead of the stencil.  slow(j, c): the FP64 sum at row j of column c.
+// slow's last argument: whether to guard the rows below 0 (N < kStencil).
 // FX: all but the ZONE rows next to each wall in tiles of kTileRows rows per thread in fixed point
-// (weights fw, few), the others one per thread, by the other half of the block first.  Otherwise
-// all in FP64.
-// The FP64 pipe takes 16 cycles of its SM per warp instruction, and k_pc issues 5900 of them per
-// 16 modes of 64 rows with FP64 stencils, 4400 without: 252 -> 219 us at N_r = 64, M = 32, K = 64
-// (8 rows per tile: 230 us, fewer threads with work and more rows left to FP64).
+// (weights fw, few; rows beyond the limit far in FP64, see fx::Tile), the others one per thread, by the
+// other half of the block first.  A tile's FP64 sums share one copy in a rolled loop: 9 to 18 instructions
+// a row unrolled four times are most of a stage's code, and they are rarely taken.
+// Otherwise all in FP64, two rows at a time: a warp may issue an FP64 instruction every 64 cycles, and one
+// chain of dependent FMAs does not fill that (N_r = 160, M = 8, K = 16: k_pc 229 -> 225 us; N_r = 64,
+// M = 64, K = 128: 903 -> 873 us).
 constexpr int kTileRows = 4;   // rows per thread, here and in the split path
 template <int ZONE, bool FX, bool PAIR, class Slow, class Pre, class Body>
-__device__ __forceinline__ void stencil_rows(const int2* __restrict__ fw, const int2* __restrict__ few, const double2* F,
+__device__ __forceinline__ void stencil_rows(const int2* __restrict__ fw, const int2* __restrict__ few, int far, const double2* F,
                                              const double2* F2, int N, int T, Slow slow, Pre pre, Body body) {
     using namespace fx;
     const int c = threadIdx.x % (2 * T), step = blockDim.x / (2 * T), st = 2 * T;
     if (FX) {
         const double* f = reinterpret_cast<const double*>(F) + c;
         const double* f2 = reinterpret_cast<const double*>(F2) + c;
+#pragma unroll 1
         for (int j0 = ZONE + kTileRows * (threadIdx.x / st); j0 < N - ZONE; j0 += kTileRows * step) {
             double d[kTileRows], g[kTileRows];
 #pragma unroll
             for (int i = 0; i < kTileRows; ++i) g[i] = pre(min(j0 + i, N - 1));
+            unsigned fp64;
             {
                 Tile<kTileRows> X;
                 double v[kTileRows + 8], v2[kTileRows + 8];
@@ -291,24 +295,49 @@ __device__ __forceinline__ void stencil_rows(const int2* __restrict__ fw, const 
                     if (PAIR) v2[i] = j < N ? f2[j * st] : 0.0;
                 }
                 auto near = [&](int i) { return (unsigned)__ldg(&few[min(j0 + i, N - ZONE - 1)].y); };
-                if (PAIR) X.load(v, v2, near);
-                else X.load(v, near);
+                if (PAIR) X.load(v, v2, far, near);
+                else X.load(v, far, near);
+                fp64 = X.fp64;
 #pragma unroll
                 for (int i = 0; i < kTileRows; ++i) {
                     const int j = min(j0 + i, N - ZONE - 1);
-                    d[i] = X.far(i) ? slow(j, c) : X.row(i, fw + j * kStencil, __ldg(&few[j].x));
+                    d[i] = X.row(i, fw + j * kStencil, __ldg(&few[j].x));
                 }
+            }
+            if (fp64) {
+#pragma unroll 1
+                for (int i = 0; i < kTileRows; ++i)
+                    if ((fp64 >> i) & 1) {
+                        const double o = slow(min(j0 + i, N - ZONE - 1), c, std::false_type{});
+#pragma unroll
+                        for (int q = 0; q < kTileRows; ++q) d[q] = i == q ? o : d[q];
+                    }
             }
 #pragma unroll
             for (int i = 0; i < kTileRows; ++i)
                 if (j0 + i < N - ZONE) body(j0 + i, (j0 + i) * st + c, d[i], g[i]);
         }
     }
-    const int nw = FX ? min(N, 2 * ZONE) : N;
-    for (int i = (threadIdx.x ^ (blockDim.x >> 1)) / st; i < nw; i += step) {
-        const int j = !FX || N < 2 * ZONE || i < ZONE ? i : N - 2 * ZONE + i;
+    if (FX) {
+        for (int i = (threadIdx.x ^ (blockDim.x >> 1)) / st; i < min(N, 2 * ZONE); i += step) {
+            const int j = N < 2 * ZONE || i < ZONE ? i : N - 2 * ZONE + i;
+            const double g = pre(j);
+            body(j, j * st + c, slow(j, c, std::false_type{}), g);
+        }
+        return;
+    }
+    int j = threadIdx.x / st;
+    if (N >= kStencil) {
+        for (; j + step < N; j += 2 * step) {
+            const double g = pre(j), g2 = pre(j + step);
+            const double o = slow(j, c, std::false_type{}), o2 = slow(j + step, c, std::false_type{});
+            body(j, j * st + c, o, g);
+            body(j + step, (j + step) * st + c, o2, g2);
+        }
+    }
+    for (; j < N; j += step) {
         const double g = pre(j);
-        body(j, j * st + c, slow(j, c), g);
+        body(j, j * st + c, slow(j, c, std::true_type{}), g);
     }
 }
 
