@@ -964,8 +964,9 @@ static tc_status launch_advance_split(tc_plan* p, const double2* u, double2* u_p
     return TC_OK;
 }
 
-// Fixed-point stencils in a launch of blocks of T modes.  With fewer than 8 warps per SM their
-// conversions take longer than the FP64 FMAs (N_r = 160, M = 8, K = 16: 273 against 225 us).  With many
+// Fixed-point stencils in a launch of blocks of T modes.  With up to 8 warps per SM, one block of 256
+// threads, their conversions take longer than the FP64 FMAs (N_r = 160, M = 8, K = 16: 273 against 225 us;
+// N_r = 64, M = 24, K = 48, 152 blocks: 184 against 160 in the mixed form).  With more
 // they are the faster form from some 76 rows on: below, two blocks with a fifth column for the sum of
 // u_+ and u_- (launch_advance) fit an SM, and the tiles of 4 rows do not spread evenly over the warps.
 // M = 64, K = 128, fixed point against FP64: N_r = 48 756 and 674 us, 64 909 and 890, 72 1017 and 1009;
@@ -973,7 +974,7 @@ static tc_status launch_advance_split(tc_plan* p, const double2* u, double2* u_p
 // (kFarMixed), from 56 on: 48 696 and 674, 56 783 and 784, 64 874 and 890.
 static bool fx_stencils(const tc_plan* p, int nmode, int T) {
     return p->N_r >= (p->precision == TC_MIXED ? 56 : 76) &&
-           (size_t)blocks_for(nmode, T) * (T <= 8 ? 128 : 256) >= (size_t)256 * p->num_sms;
+           (size_t)blocks_for(nmode, T) * (T <= 8 ? 128 : 256) > (size_t)256 * p->num_sms;
 }
 
 tc_status launch_advance(tc_plan* p, const double2* u, double2* u_prev, const double2* Ncur,
