@@ -453,7 +453,8 @@ __device__ __forceinline__ double nan64() { return __longlong_as_double(0x7ff800
 // against rationals over columns that are smooth, wavy, vanish at the walls or go as r^+-32, r^+-192
 // (N_r = 48 to 256): at most 0.9 in a row, 2.3 with FP64 sums; columns in norm as good or
 // better.  The four rows next to each wall, whose stencils are shorter, and rows near a NaN, an Inf
-// or the smallest numbers are FP64 sums too.
+// or the smallest numbers are FP64 sums too, but windows of zeros (modes that a flow does not have)
+// are not.
 constexpr int kFar = 6, kLowExp = 70;
 // fix() for emax > kLowExp, where zeros and subnormals are shifted out like all that is small
 __device__ __forceinline__ long long fix_tile(double d, int emax) {
@@ -481,11 +482,18 @@ template <int R> struct Tile {
     }
     // b: exponents of the window's entries; limit: kFar, or more where less accuracy does; near(i): those of 2^ew / |w| of the entries i + 2, i + 3,
     // i + 5, i + 6 of row j0 + i, a byte each
-    template <class Near> __device__ __forceinline__ void exponents(const int (&b)[R + 8], int limit, Near near) {
+    // zero: all entries are zero (not merely small): the rows are then 0 without an FP64 sum.  Returns the
+    // exponent to convert the window to.
+    template <class Near, class Zero>
+    __device__ __forceinline__ int exponents(const int (&b)[R + 8], int limit, Near near, Zero zero) {
         e = 0;
 #pragma unroll
         for (int i = 0; i < R + 8; ++i) e = max(e, b[i]);
         fp64 = e >= 2047 || e <= kLowExp ? ~0u : 0u;
+        if (e <= 1 && zero()) {
+            fp64 = 0;
+            return 4096;   // shifts all out
+        }
 #pragma unroll
         for (int i = 0; i < R; ++i) {
             const unsigned q = near(i);
@@ -493,14 +501,21 @@ template <int R> struct Tile {
                               min((int)(q >> 16 & 255) - b[i + 5], (int)(q >> 24) - b[i + 6]));
             if (e + c > limit) fp64 |= 1u << i;
         }
+        return e + 2;
+    }
+    static __device__ __forceinline__ bool zeros(const double (&d)[R + 8]) {
+        unsigned any = 0;
+#pragma unroll
+        for (int i = 0; i < R + 8; ++i) any |= (unsigned)__double2hiint(d[i]) << 1 | (unsigned)__double2loint(d[i]);
+        return any == 0;
     }
     template <class Near> __device__ __forceinline__ void load(const double (&d)[R + 8], int limit, Near near) {
         int b[R + 8];
 #pragma unroll
         for (int i = 0; i < R + 8; ++i) b[i] = bexp(d[i]);
-        exponents(b, limit, near);
+        const int to = exponents(b, limit, near, [&] { return zeros(d); });
 #pragma unroll
-        for (int i = 0; i < R + 8; ++i) x[i] = split(fix_tile(d[i], e + 2));
+        for (int i = 0; i < R + 8; ++i) x[i] = split(fix_tile(d[i], to));
     }
     // the window of a + d, added after the conversion (one exponent more)
     template <class Near>
@@ -508,9 +523,9 @@ template <int R> struct Tile {
         int b[R + 8];
 #pragma unroll
         for (int i = 0; i < R + 8; ++i) b[i] = max(bexp(a[i]), bexp(d[i])) + 1;
-        exponents(b, limit, near);
+        const int to = exponents(b, limit, near, [&] { return zeros(a) && zeros(d); });
 #pragma unroll
-        for (int i = 0; i < R + 8; ++i) x[i] = split(fix_tile(a[i], e + 2) + fix_tile(d[i], e + 2));
+        for (int i = 0; i < R + 8; ++i) x[i] = split(fix_tile(a[i], to) + fix_tile(d[i], to));
     }
 };
 }  // namespace fx
