@@ -13,8 +13,7 @@ namespace {
 //   phase 0: (u_r, u_t) and (u_z, d_r u_z);  1: (d_r u_r, d_r u_t) and (d_t u_r, d_t u_t);
 //   phase 2: (d_z u_r, d_z u_t) and (d_t u_z, d_z u_z).
 // Per physical point Ua = (u_r, u_t / r), Ub = (u_z, N_z), Nn = (N_r, N_t) stay in shared
-// memory.  The last pass of a phase keeps its outputs in registers; the threads of L0 and
-// then those of L1 add their products.
+// memory.  After the last pass of a phase the products of its lines are added, a point per thread.
 
 template <class PL, int ZT, int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB) k_fx_theta(ThetaArgs a, FxPlan f) {

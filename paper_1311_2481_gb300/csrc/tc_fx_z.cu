@@ -403,7 +403,7 @@ tc_status z_pass(tc_plan* p, const ZPass& a, const int4* tw, cudaStream_t s) {
 
 tc_status run_z(tc_plan* p, const ZPass& a, cudaStream_t s);
 
-// lengths with a compile-time plan, and the z values of their theta blocks (0: none)
+// lengths with a compile-time plan
 bool static_z(int P) {
     switch (P) {
         case 12: case 24: case 36: case 48: case 72: case 96: case 144: case 192: case 288: case 384: case 576: case 768: case 1152:

@@ -51,10 +51,10 @@ constexpr int kChunkF = 4, kChunkB = 2;   // rows of factors per register chunk 
 
 // CH: chunks; the row by row ring of kPCDepth rows reaches further ahead, which counts where a launch
 // has few warps and nothing else covers a load (N_r = 160, M = 8, K = 16: k_pc 223 against 239 us).
-template <bool CH>
+template <bool CH, bool LOOP>
 __device__ __forceinline__ void band_solve(double2* col, int off, int T, int N, const double* __restrict__ F,
                                            const uint8_t* __restrict__ P, int M1K1) {
-    if (CH) smem_band_solve_c<kChunkF, kChunkB>(col, T, off, N, F, P, M1K1);
+    if (CH) smem_band_solve_c<kChunkF, kChunkB, LOOP>(col, T, off, N, F, P, M1K1);
     else smem_band_solve<kPCDepth>(col, T, off, N, F, P, M1K1);
 }
 
@@ -62,7 +62,7 @@ __device__ __forceinline__ void band_solve(double2* col, int off, int T, int N, 
 // (g.sh > 0) 4 nT threads, each with one half of it for one (mode, part): threads [0, 2nT) rows [0, sh),
 // threads [2nT, 4nT) rows [sh, N), with the pivoted LU factors of the diagonal block; the column then
 // holds g = (A1^{-1} b1, A2^{-1} b2).  Otherwise 2 nT threads with the factors of the whole system.
-template <bool CH>
+template <bool CH, bool LOOP>
 __device__ __forceinline__ void system_solve(const PCArgs& a, const Geo& g, double2* X, int set, int T, int nT, int mode0, int lt) {
     const bool sp = g.sh > 0;
     const int half = lt >= 2 * nT ? 1 : 0;
@@ -72,7 +72,7 @@ __device__ __forceinline__ void system_solve(const PCArgs& a, const Geo& g, doub
     const size_t mk = (size_t)m * g.K1 + (k < 0 ? -k : k);
     const size_t per_set = (size_t)g.N * kBands * g.M1K1;
     const int r0 = half ? g.sh : 0, n = half ? g.N - g.sh : sp ? g.sh : g.N;
-    band_solve<CH>(X + (size_t)r0 * T, 2 * t + part, T, n,
+    band_solve<CH, LOOP>(X + (size_t)r0 * T, 2 * t + part, T, n,
                    (sp ? a.fac2 : a.fac) + (size_t)set * per_set + (size_t)r0 * kBands * g.M1K1 + mk,
                    (sp ? a.piv2 : a.piv) + ((size_t)set * g.N + r0) * g.M1K1 + mk, g.M1K1);
 }
@@ -353,7 +353,7 @@ __global__ void __launch_bounds__(NTH, 512 / NTH) k_pc(PCArgs a, Geo g, int T) {
         double2* X0 = stage == 1 ? C1 : C0;
         if ((int)threadIdx.x < nsys * per) {
             const int c = nsys == 1 ? 0 : threadIdx.x / per;
-            system_solve<FX>(a, g, X0 + (size_t)c * items, set0 + c, T, nT, mode0, threadIdx.x - c * per);
+            system_solve<FX, true>(a, g, X0 + (size_t)c * items, set0 + c, T, nT, mode0, threadIdx.x - c * per);
         } else if (spare && (int)threadIdx.x >= helper) {
             beside(helper);
         }
@@ -606,11 +606,9 @@ __global__ void __launch_bounds__(128) k_update(double2* __restrict__ u, double2
     if (bad && nonfinite) *nonfinite = 1;
 }
 
-// x <- A^{-1} x for every mode of nfields consecutive fields (system sets set0, set0+1, ...):
-// thread (field, mode, part) runs the register-window substitution down its global column.
 // smem_band_solve on a column in global memory, in the same arithmetic: the right-hand side's
 // rows come in through the ring with the factors, D rows ahead.  Used while a launch has few
-// warps (launch_split_solve): there each row waited one memory latency.
+// warps (launch_advance_split): there each row waited one memory latency.
 constexpr int kGD = 6;   // ring depth (2, 3, 4, 5, 6, 8: 325, 325, 290, 275, 267, 267 us for a Poisson solve, N_r = 256, M = 64, K = 128)
 template <int D>
 __device__ __forceinline__ void gmem_band_solve(double* __restrict__ x, size_t st, int N, const double* __restrict__ F,
@@ -694,6 +692,8 @@ __device__ __forceinline__ void gmem_band_solve(double* __restrict__ x, size_t s
     }
 }
 
+// x <- A^{-1} x for every mode of nfields consecutive fields (system sets set0, set0+1, ...):
+// thread (field, mode, part) runs the register-window substitution down its global column.
 template <int D>
 __global__ void k_band_solve_g(double2* __restrict__ x, const double* __restrict__ fac,
                                const uint8_t* __restrict__ piv, int set0, int nfields, Geo g) {
@@ -713,23 +713,24 @@ __global__ void k_band_solve_g(double2* __restrict__ x, const double* __restrict
     else smem_band_solve(x + (size_t)fld * g.S + mode, g.nmode, part, g.N, F, P, g.M1K1);
 }
 
-// Stand-alone solve of one system set for all modes (tc_helmholtz_solve): columns staged in
-// shared memory, real and imaginary parts by separate threads.
-// One system for every mode in two partitions, T modes per block (as in k_pc's solve phases).
-// rhs may be x: a block reads its columns before it writes them.
+// Stand-alone solves of one system set for all modes (tc_helmholtz_solve): columns staged in shared
+// memory, real and imaginary parts by separate threads.  rhs may be x: a block reads its columns
+// before it writes them.
+// In two partitions, T modes per block (as in k_pc's solve phases):
 __global__ void __launch_bounds__(128) k_band_solve_s2(const double2* rhs, double2* x, PCArgs a, int set, Geo g, int T) {
     extern __shared__ double2 sm[];
     const int N = g.N, mode0 = blockIdx.x * T, nT = min(T, g.nmode - mode0), t = threadIdx.x % T;
     for (int j = threadIdx.x / T; j < N; j += blockDim.x / T)
         sm[j * T + t] = t < nT ? rhs[(size_t)j * g.nmode + mode0 + t] : make_double2(0.0, 0.0);
     __syncthreads();
-    if (threadIdx.x < 4 * nT) system_solve<true>(a, g, sm, set, T, nT, mode0, threadIdx.x);
+    if (threadIdx.x < 4 * nT) system_solve<true, false>(a, g, sm, set, T, nT, mode0, threadIdx.x);
     __syncthreads();
     spike_combine(a, g, sm, 1, set, T, nT, mode0, reinterpret_cast<double*>(sm + (size_t)N * T));
     if (t < nT)
         for (int j = threadIdx.x / T; j < N; j += blockDim.x / T) x[(size_t)j * g.nmode + mode0 + t] = sm[j * T + t];
 }
 
+// In one:
 __global__ void __launch_bounds__(256) k_band_solve_s(const double2* rhs, double2* x, const double* __restrict__ fac,
                                                       const uint8_t* __restrict__ piv, int set, Geo g, int T) {
     extern __shared__ double2 sm[];
@@ -855,7 +856,6 @@ size_t diag_red_doubles(const tc_plan* p) {
     return kDiagPartials + (size_t)blocks_for((size_t)p->nmode, 256) * p->N_r;
 }
 
-// modes per block of the fused kernel: four complex columns of N_r rows in shared memory
 // Modes per block of the fused kernel (a power of two): the most (up to 16) that still give every SM a block,
 // within 96 KB of shared memory for the four columns.  Each block's time is its substitution
 // chain, so more modes per block cost little while the blocks fit one wave.

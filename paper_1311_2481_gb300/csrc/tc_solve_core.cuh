@@ -168,7 +168,8 @@ __device__ __forceinline__ void smem_band_solve(double2* col, int T, int off, in
 // (backward) ahead in a second register buffer.  A ring that is refilled row by row leaves the
 // loads of several rows on one scoreboard, and waiting for a row then waits for the youngest of
 // them, a memory latency per row; a chunk's loads are waited for once, a chunk later.
-template <int CF, int CB>
+// INIT: set the buffers first, for a call within a loop, around which ptxas otherwise keeps them live and spills.
+template <int CF, int CB, bool INIT>
 __device__ __forceinline__ void smem_band_solve_c(double2* col, int T, int off, int N,
                                                   const double* __restrict__ F, const uint8_t* __restrict__ P,
                                                   int M1K1) {
@@ -178,8 +179,16 @@ __device__ __forceinline__ void smem_band_solve_c(double2* col, int T, int off, 
     double w0 = x[0], w1 = N > 1 ? x[st] : 0.0, w2 = N > 2 ? x[2 * st] : 0.0,
            w3 = N > 3 ? x[3 * st] : 0.0, w4 = N > 4 ? x[4 * st] : 0.0;
     {
-        double lr[2][CF][4] = {};   // initialised: in k_pc's loop ptxas otherwise keeps them live around it and spills
-        int pr[2][CF] = {};
+        double lr[2][CF][4];
+        int pr[2][CF];
+        if (INIT) {
+#pragma unroll
+            for (int i = 0; i < 2 * CF; ++i) {
+                pr[i / CF][i % CF] = 0;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) lr[i / CF][i % CF][q] = 0.0;
+            }
+        }
         auto load = [&](double (&l)[CF][4], int (&p)[CF], int c) {
 #pragma unroll
             for (int d = 0; d < CF; ++d) {
@@ -219,7 +228,13 @@ __device__ __forceinline__ void smem_band_solve_c(double2* col, int T, int off, 
         }
     }
     double v1 = 0.0, v2 = 0.0, v3 = 0.0, v4 = 0.0, v5 = 0.0, v6 = 0.0, v7 = 0.0, v8 = 0.0;
-    double ur[2][CB][9] = {};
+    double ur[2][CB][9];
+    if (INIT) {
+#pragma unroll
+        for (int i = 0; i < 2 * CB; ++i)
+#pragma unroll
+            for (int q = 0; q < 9; ++q) ur[i / CB][i % CB][q] = 0.0;
+    }
     auto load = [&](double (&u)[CB][9], int c) {
 #pragma unroll
         for (int d = 0; d < CB; ++d) {
