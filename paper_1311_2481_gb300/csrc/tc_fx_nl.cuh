@@ -18,6 +18,7 @@ struct ThetaArgs {
     const int2* e1;
     int* e2;
     int* e2max;
+    double* s2;        // sum of N_t over the points of each block [nh][tiles]
     const int4* ir;    // 1 / r_j: limbs, exponent
     const int2* mm;    // m m_p: limbs of m m_p 2^(62 - emm)
     const int4* tw;

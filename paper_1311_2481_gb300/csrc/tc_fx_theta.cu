@@ -14,6 +14,8 @@ namespace {
 //   phase 2: (d_z u_r, d_z u_t) and (d_t u_z, d_z u_z).
 // Per physical point Ua = (u_r, u_t / r), Ub = (u_z, N_z), Nn = (N_r, N_t) stay in shared
 // memory.  After the last pass of a phase the products of its lines are added, a point per thread.
+// The sum of N_t over the block goes out beside the lines: its mean drives the mean flow and is
+// far smaller than N_r, with which it shares the exponent of a line from there on.
 
 template <class PL, int ZT, int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB) k_fx_theta(ThetaArgs a, FxPlan f) {
@@ -22,6 +24,7 @@ __global__ void __launch_bounds__(NT, MINB) k_fx_theta(ThetaArgs a, FxPlan f) {
     __shared__ float s_bound[NT / 32][8];
     __shared__ unsigned s_mx[3][4];   // largest parts of phase, {L0.x, L0.y, L1.x, L1.y}
     __shared__ unsigned long long s_sum[2][NT / 32];
+    __shared__ long long s_t[2][NT / 32];   // sum of N_t over a warp, in units of 2^52 and of 1
     const PL pl(f);
     const int P = pl.size(), M = a.M, Pz = a.Pz, zt = ZT ? ZT : a.zt, lp = line_pitch(P), nl = 2 * zt;
     auto divz = [&](int i) { return ZT ? i / (ZT ? ZT : 1) : udiv(i, a.mzt); };
@@ -54,6 +57,7 @@ __global__ void __launch_bounds__(NT, MINB) k_fx_theta(ThetaArgs a, FxPlan f) {
             a.e2[(r * tiles + tile) * 2 + threadIdx.x] = kExpNaN;
             atomicMax(&a.e2max[r * 2 + threadIdx.x], kExpNaN);
         }
+        if (threadIdx.x == 0) a.s2[r * tiles + tile] = nan64();
         return;
     }
     const int4 irv = a.ir[a.r0 + r];
@@ -104,6 +108,7 @@ __global__ void __launch_bounds__(NT, MINB) k_fx_theta(ThetaArgs a, FxPlan f) {
             sz.set(ENz, Eut + eu, Euz + ev);
         }
         unsigned long long th = 0, tz = 0;
+        long long yh = 0, yl = 0;   // the sum of N_t, exactly: high and low words
         const int EN = max(ENr, ENt), dr = min(EN - ENr, 63), dt = min(EN - ENt, 63);
 #pragma unroll 2
         for (int pt = threadIdx.x; pt < zt * P; pt += nt) {
@@ -131,6 +136,8 @@ __global__ void __launch_bounds__(NT, MINB) k_fx_theta(ThetaArgs a, FxPlan f) {
                 Ub[pt].y = nz;
                 th += (((unsigned long long)llabs(s.x) >> 12) >> dr) + (((unsigned long long)llabs(s.y) >> 12) >> dt) + 2;
                 tz += ((unsigned long long)llabs(nz) >> 12) + 1;
+                yh += s.y >> 32;
+                yl += (unsigned)s.y;
             }
         }
         if (PH == 2) {   // sums of the moduli of N over the block
@@ -139,9 +146,16 @@ __global__ void __launch_bounds__(NT, MINB) k_fx_theta(ThetaArgs a, FxPlan f) {
                 th += __shfl_xor_sync(0xffffffffu, th, o);
                 tz += __shfl_xor_sync(0xffffffffu, tz, o);
             }
+            // over the warp in three chunks of 26 bits
+            const unsigned lo = 0x3ffffffu;
+            const long long hi = (yh << 6) + (yl >> 26);
+            const unsigned c0 = __reduce_add_sync(0xffffffffu, (unsigned)yl & lo), c1 = __reduce_add_sync(0xffffffffu, (unsigned)hi & lo);
+            const int c2 = (int)__reduce_add_sync(0xffffffffu, (unsigned)(hi >> 26));
             if (lane == 0) {
                 s_sum[0][wid] = th;
                 s_sum[1][wid] = tz;
+                s_t[0][wid] = c2;
+                s_t[1][wid] = ((long long)c1 << 26) + c0;
             }
         }
     };
@@ -150,9 +164,12 @@ __global__ void __launch_bounds__(NT, MINB) k_fx_theta(ThetaArgs a, FxPlan f) {
     // stays below 2^62
     auto fill_forward = [&]() {
         unsigned long long th = 0, tz = 0;
+        long long yh = 0, yl = 0;
         for (int w = 0; w < nw; ++w) {
             th += s_sum[0][w];
             tz += s_sum[1][w];
+            yh += s_t[0][w];
+            yl += s_t[1][w];
         }
         const int EN = max(ENr, ENt), fh = bits64(th) - 50, fz = bits64(tz) - 50;   // right shift (left if negative)
         const int fr = min(fh + EN - ENr, 62), ft = min(fh + EN - ENt, 62);
@@ -161,6 +178,7 @@ __global__ void __launch_bounds__(NT, MINB) k_fx_theta(ThetaArgs a, FxPlan f) {
             a.e2[(r * tiles + tile) * 2 + threadIdx.x] = E;
             atomicMax(&a.e2max[r * 2 + threadIdx.x], E);
         }
+        if (threadIdx.x == 2) a.s2[r * tiles + tile] = to_double(yh, ENt - 10) + to_double(yl, ENt - 62);
         const long long hr = half_of(fr), ht = half_of(ft), hz = half_of(fz);
         auto sft = [](long long x, int s, long long h) { return s >= 0 ? (x + h) >> s : x << -s; };
 #pragma unroll 2

@@ -32,11 +32,12 @@ constexpr int kDrRows = 8;      // rows per thread of k_fx_dr
 constexpr int kZThreads = 512;  // most threads of a transform block (128 registers each)
 
 // exponent arrays of nh staged rows, in the fxe region: e1[9][nh][M+1] (exponent, largest
-// |re| + |im| in units of 2^32), e2[nh][tiles][2], e2max[nh][2]
+// |re| + |im| in units of 2^32), e2max[nh][2], e2[nh][tiles][2]; behind them s2[nh][tiles], the sums of N_t
 struct Exps {
     int2* e1;
     int* e2;
     int* e2max;
+    double* s2;
 };
 
 // ---------------------------------------------------------------- radial derivative
@@ -217,10 +218,11 @@ __global__ void __launch_bounds__(kZThreads) k_fx_zinv(const double2* __restrict
     if (on) {
         // sum of moduli < s_l1 2^43: shifted to below 2^62
         const int s = max(0, bits(s_l1[line]) - 19);
+        const long long h = half_of(s);
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int k = i0 + i * tl - K;
-            if (k <= K) buf[line * lp + (k >= 0 ? k : k + P)] = mk(v[i].x >> s, v[i].y >> s);
+            if (k <= K) buf[line * lp + (k >= 0 ? k : k + P)] = mk((v[i].x + h) >> s, (v[i].y + h) >> s);
         }
     }
     __syncthreads();
@@ -250,6 +252,7 @@ __global__ void __launch_bounds__(kZThreads) k_fx_zinv(const double2* __restrict
 struct ZfwdOut {
     double2* out;    // N, or ubar
     double2* Rh;     // Rhat of the staged rows
+    const double* s2;   // of N: sums of N_t over the theta blocks
     double scale;    // of N
     double kz;
     int l0;
@@ -261,6 +264,7 @@ __global__ void __launch_bounds__(kZThreads) k_fx_zfwd(const cx* __restrict__ H2
                                                        unsigned mzt, FxPlan f, const int4* __restrict__ tw, int tl, unsigned mtl) {
     extern __shared__ cx buf[];
     __shared__ unsigned s_l1[NL];
+    __shared__ double s_mean;
     const PL pl(f);
     constexpr int NE = ADJ ? 6 : 2;
     const int P = pl.size(), lp = line_pitch(P), nk = 2 * K + 1, nmode = (M + 1) * nk;
@@ -270,12 +274,22 @@ __global__ void __launch_bounds__(kZThreads) k_fx_zfwd(const cx* __restrict__ H2
     t /= NB;
     const int m = t % (M + 1), rl = t / (M + 1);
     if (threadIdx.x < NL) s_l1[threadIdx.x] = 0;
+    if (!ADJ && m == 0 && threadIdx.x < 32) {
+        // (0, 0): N_t from the sums over the theta blocks, which have an exponent of their own
+        double y = 0.0;
+        for (int i = threadIdx.x; i < P / zt; i += 32) y += __ldg(&w.s2[rl * (P / zt) + i]);
+#pragma unroll
+        for (int o = 16; o; o >>= 1) y += __shfl_xor_sync(0xffffffffu, y, o);
+        if (threadIdx.x == 0) s_mean = y;
+    }
     __syncthreads();
     const int line = NL == 1 ? 0 : udiv(threadIdx.x, mtl), i0 = threadIdx.x - line * tl;
     const bool on = line < NL;
     // component and kind (A, R, Z) of this thread's line, its field and exponent
     const int c = ADJ ? b : b * NL + line, l = ADJ ? (NL == 1 ? w.l0 : line) : 0;
-    const int field = 3 * l + c, ie = 2 * l + (c == 2);
+    // N_- of m = 0 is the mirrored conjugate of N_+: taken from the same line, so that it is that exactly
+    const bool mirror = !ADJ && m == 0 && c == 1;
+    const int field = mirror ? 0 : 3 * l + c, ie = 2 * l + (c == 2);
     const int E = on ? e2max[rl * NE + ie] : 0;
     cx v[8];
     unsigned l1 = 0;
@@ -310,11 +324,21 @@ __global__ void __launch_bounds__(kZThreads) k_fx_zfwd(const cx* __restrict__ H2
     };
     const size_t e0 = ((size_t)c * N + r0 + rl) * nmode + (size_t)m * nk, h0 = ((size_t)c * nh + rl) * nmode + (size_t)m * nk;
     if (!ADJ) {
-        if (on)
+        if (!on) return;
+        if (m == 0) {   // of a real field: k < 0 is the conjugate of k > 0
             for (int kk = i0; kk < nk; kk += tl) {
-                const double2 o = value(line, kk, E);
+                const bool flip = c == 1 || (c == 2 && kk < K);
+                double2 o = value(line, flip ? 2 * K - kk : kk, E);
+                if (flip) o.y = -o.y;
+                if (c < 2 && kk == K) o.y = c == 0 ? s_mean : -s_mean;
                 w.out[e0 + kk] = make_double2(o.x * w.scale, o.y * w.scale);
             }
+            return;
+        }
+        for (int kk = i0; kk < nk; kk += tl) {
+            const double2 o = value(line, kk, E);
+            w.out[e0 + kk] = make_double2(o.x * w.scale, o.y * w.scale);
+        }
         return;
     }
     const int* em = e2max + rl * NE + (c == 2);
@@ -343,13 +367,14 @@ Exps exps(tc_plan* p, char* ws) {
     e.e1 = reinterpret_cast<int2*>(ws + p->ws.fxe);
     e.e2max = reinterpret_cast<int*>(e.e1 + (size_t)9 * p->stage_rows * (p->M + 1));
     e.e2 = e.e2max + 2 * p->stage_rows;
+    e.s2 = reinterpret_cast<double*>(e.e2 + (size_t)2 * p->stage_rows * p->P_z);
     return e;
 }
 
 }  // namespace
 
 size_t fx_exp_bytes(const tc_plan* p, int rows) {
-    return (size_t)rows * ((size_t)9 * (p->M + 1) * sizeof(int2) + 2 * sizeof(int) + (size_t)2 * p->P_z * sizeof(int));
+    return (size_t)rows * ((size_t)9 * (p->M + 1) * sizeof(int2) + 2 * sizeof(int) + (size_t)p->P_z * (2 * sizeof(int) + sizeof(double)));
 }
 
 namespace {
@@ -465,12 +490,12 @@ tc_status fx_rows(tc_plan* p, const double2* u, double2* Nh, char* ws, cudaStrea
     const Exps e = exps(p, ws);
     TC_TRY_STATUS(zinv_u(p, u, reinterpret_cast<double2*>(H2), H1, e, s, r0, nh));
     int slot = prof_begin(p, kKTheta, s);
-    ThetaArgs a{H1, H2, e.e1, e.e2, e.e2max, p->d_fx_ir, p->d_fx_mm, p->d_fx_tw_t, r0, nh, p->M, p->P_z, p->fx_zt, p->fx_emm,
+    ThetaArgs a{H1, H2, e.e1, e.e2, e.e2max, e.s2, p->d_fx_ir, p->d_fx_mm, p->d_fx_tw_t, r0, nh, p->M, p->P_z, p->fx_zt, p->fx_emm,
                 magic(p->fx_zt), magic(p->P_t), (long long)p->m_p};
     TC_TRY_STATUS(launch_fx_theta(p, a, s));
     prof_end(p, slot, s);
     slot = prof_begin(p, kKZfwd, s);
-    TC_TRY_STATUS(run_z(p, ZPass{false, false, nullptr, nullptr, H2, nullptr, e.e2max, e.e2, {Nh, nullptr, 0, 0, 0}, r0, nh, p->fx_zt}, s));
+    TC_TRY_STATUS(run_z(p, ZPass{false, false, nullptr, nullptr, H2, nullptr, e.e2max, e.e2, {Nh, nullptr, e.s2, 0, 0, 0}, r0, nh, p->fx_zt}, s));
     prof_end(p, slot, s);
     return TC_OK;
 }
@@ -504,7 +529,7 @@ tc_status launch_adjoint_rows_fx(tc_plan* p, const double2* u, const double2* Nb
     TC_TRY_STATUS(launch_fx_theta_adj(p, a, s));
     prof_end(p, slot, s);
     slot = prof_begin(p, kKZfwdAdj, s);
-    TC_TRY_STATUS(run_z(p, ZPass{false, true, nullptr, nullptr, H3, nullptr, e2max, e2, {ubar, Rh, 0, 0, 0}, r0, nh, zt}, s));
+    TC_TRY_STATUS(run_z(p, ZPass{false, true, nullptr, nullptr, H3, nullptr, e2max, e2, {ubar, Rh, nullptr, 0, 0, 0}, r0, nh, zt}, s));
     prof_end(p, slot, s);
     return TC_OK;
 }
