@@ -18,7 +18,7 @@ struct ThetaArgs {
     const int2* e1;
     int* e2;
     int* e2max;
-    double* s2;        // sum of N_t over the points of each block [nh][tiles]
+    longlong2* s2;     // sum of N_t over the points of each block [nh][tiles] (see block_sum)
     const int4* ir;    // 1 / r_j: limbs, exponent
     const int2* mm;    // m m_p: limbs of m m_p 2^(62 - emm)
     const int4* tw;
@@ -156,6 +156,12 @@ struct ThetaAdjArgs {
     unsigned mzt, mP;
     long long mp;
 };
+
+// The sum of a block's N_t, h 2^52 + l in units of 2^(E - 62), is stored as (l, h and E)
+__device__ __forceinline__ double block_sum(longlong2 v) {
+    const int E = (int)(unsigned)v.y;
+    return E > kExpNaN / 2 ? nan64() : to_double(v.y >> 32, E - 10) + to_double(v.x, E - 62);
+}
 
 tc_status launch_fx_theta_adj(tc_plan* p, ThetaAdjArgs a, cudaStream_t s);
 tc_status launch_fx_theta(tc_plan* p, ThetaArgs a, cudaStream_t s);

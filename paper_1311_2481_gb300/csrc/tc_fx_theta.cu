@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(NT, MINB) k_fx_theta(ThetaArgs a, FxPlan f) {
             a.e2[(r * tiles + tile) * 2 + threadIdx.x] = kExpNaN;
             atomicMax(&a.e2max[r * 2 + threadIdx.x], kExpNaN);
         }
-        if (threadIdx.x == 0) a.s2[r * tiles + tile] = nan64();
+        if (threadIdx.x == 0) a.s2[r * tiles + tile] = make_longlong2(0, kExpNaN);
         return;
     }
     const int4 irv = a.ir[a.r0 + r];
@@ -178,7 +178,7 @@ __global__ void __launch_bounds__(NT, MINB) k_fx_theta(ThetaArgs a, FxPlan f) {
             a.e2[(r * tiles + tile) * 2 + threadIdx.x] = E;
             atomicMax(&a.e2max[r * 2 + threadIdx.x], E);
         }
-        if (threadIdx.x == 2) a.s2[r * tiles + tile] = to_double(yh, ENt - 10) + to_double(yl, ENt - 62);
+        if (threadIdx.x == 2) a.s2[r * tiles + tile] = make_longlong2(yl, (yh << 32) | (unsigned)ENt);
         const long long hr = half_of(fr), ht = half_of(ft), hz = half_of(fz);
         auto sft = [](long long x, int s, long long h) { return s >= 0 ? (x + h) >> s : x << -s; };
 #pragma unroll 2

@@ -37,7 +37,7 @@ struct Exps {
     int2* e1;
     int* e2;
     int* e2max;
-    double* s2;
+    longlong2* s2;
 };
 
 // ---------------------------------------------------------------- radial derivative
@@ -252,7 +252,7 @@ __global__ void __launch_bounds__(kZThreads) k_fx_zinv(const double2* __restrict
 struct ZfwdOut {
     double2* out;    // N, or ubar
     double2* Rh;     // Rhat of the staged rows
-    const double* s2;   // of N: sums of N_t over the theta blocks
+    const longlong2* s2;   // of N: sums of N_t over the theta blocks
     double scale;    // of N
     double kz;
     int l0;
@@ -274,30 +274,33 @@ __global__ void __launch_bounds__(kZThreads) k_fx_zfwd(const cx* __restrict__ H2
     t /= NB;
     const int m = t % (M + 1), rl = t / (M + 1);
     if (threadIdx.x < NL) s_l1[threadIdx.x] = 0;
-    if (!ADJ && m == 0 && threadIdx.x < 32) {
-        // (0, 0): N_t from the sums over the theta blocks, which have an exponent of their own
-        double y = 0.0;
-        for (int i = threadIdx.x; i < P / zt; i += 32) y += __ldg(&w.s2[rl * (P / zt) + i]);
-#pragma unroll
-        for (int o = 16; o; o >>= 1) y += __shfl_xor_sync(0xffffffffu, y, o);
-        if (threadIdx.x == 0) s_mean = y;
-    }
     __syncthreads();
     const int line = NL == 1 ? 0 : udiv(threadIdx.x, mtl), i0 = threadIdx.x - line * tl;
     const bool on = line < NL;
     // component and kind (A, R, Z) of this thread's line, its field and exponent
     const int c = ADJ ? b : b * NL + line, l = ADJ ? (NL == 1 ? w.l0 : line) : 0;
-    // N_- of m = 0 is the mirrored conjugate of N_+: taken from the same line, so that it is that exactly
-    const bool mirror = !ADJ && m == 0 && c == 1;
-    const int field = mirror ? 0 : 3 * l + c, ie = 2 * l + (c == 2);
+    // the - component of m = 0 is the mirrored conjugate of the + one: taken from the same line, so that
+    // it is that exactly
+    const bool mirror = m == 0 && c == 1;
+    const int field = 3 * l + (mirror ? 0 : c), ie = 2 * l + (c == 2);
     const int E = on ? e2max[rl * NE + ie] : 0;
     cx v[8];
     unsigned l1 = 0;
     if (on) {
         const cx* h = H2 + (((size_t)field * nh + rl) * (M + 1) + m) * P;
-        const int* er = e2 + (size_t)rl * (P / zt) * NE + ie;
 #pragma unroll
         for (int i = 0; i < 8; ++i) v[i] = i0 + i * tl < P ? h[i0 + i * tl] : mk(0, 0);
+    }
+    if (!ADJ && m == 0 && threadIdx.x < 32) {
+        // (0, 0): N_t from the sums over the theta blocks, while the line comes in
+        double y = 0.0;
+        for (int i = threadIdx.x; i < P / zt; i += 32) y += block_sum(__ldg(&w.s2[rl * (P / zt) + i]));
+        for (int o = 16; o; o >>= 1)
+            if (o < P / zt) y += __shfl_xor_sync(0xffffffffu, y, o);
+        if (threadIdx.x == 0) s_mean = y;
+    }
+    if (on) {
+        const int* er = e2 + (size_t)rl * (P / zt) * NE + ie;
 #pragma unroll
         for (int i = 0; i < 8; ++i)
             if (i0 + i * tl < P) {
@@ -342,24 +345,35 @@ __global__ void __launch_bounds__(kZThreads) k_fx_zfwd(const cx* __restrict__ H2
         return;
     }
     const int* em = e2max + rl * NE + (c == 2);
+    auto coeff = [&](int q, int kk, int Eq) {   // with m = 0 of real fields as above (c is the block's)
+        const bool flip = m == 0 && (c == 1 || (c == 2 && kk < K));
+        double2 o = value(q, flip ? 2 * K - kk : kk, Eq);
+        if (flip) o.y = -o.y;
+        return o;
+    };
     for (int kk = threadIdx.x; kk < nk; kk += blockDim.x) {
         const double kzk = w.kz * (kk - K);
         if (NL == 3 || w.l0 != 1) {
             double2 u = w.out[e0 + kk];
             if (NL == 3 || w.l0 == 0) {
-                const double2 A = value(0, kk, em[0]);
+                const double2 A = coeff(0, kk, em[0]);
                 u.x += A.x;
                 u.y += A.y;
             }
             if (NL == 3 || w.l0 == 2) {
-                const double2 Z = value(NL == 3 ? 2 : 0, kk, em[4]);
+                const double2 Z = coeff(NL == 3 ? 2 : 0, kk, em[4]);
                 u.x += kzk * Z.y;
                 u.y -= kzk * Z.x;
             }
             w.out[e0 + kk] = u;
         }
-        if (NL == 3 || w.l0 == 1) w.Rh[h0 + kk] = value(NL == 3 ? 1 : 0, kk, em[2]);
+        if (NL == 3 || w.l0 == 1) w.Rh[h0 + kk] = coeff(NL == 3 ? 1 : 0, kk, em[2]);
     }
+}
+
+// bytes of e1, e2max and e2 of so many rows, up to the 16-byte boundary of s2
+size_t fx_s2_offset(const tc_plan* p, int rows) {
+    return ((size_t)rows * ((size_t)9 * (p->M + 1) * sizeof(int2) + 2 * sizeof(int) + (size_t)2 * p->P_z * sizeof(int)) + 15) & ~(size_t)15;
 }
 
 Exps exps(tc_plan* p, char* ws) {
@@ -367,14 +381,14 @@ Exps exps(tc_plan* p, char* ws) {
     e.e1 = reinterpret_cast<int2*>(ws + p->ws.fxe);
     e.e2max = reinterpret_cast<int*>(e.e1 + (size_t)9 * p->stage_rows * (p->M + 1));
     e.e2 = e.e2max + 2 * p->stage_rows;
-    e.s2 = reinterpret_cast<double*>(e.e2 + (size_t)2 * p->stage_rows * p->P_z);
+    e.s2 = reinterpret_cast<longlong2*>(reinterpret_cast<char*>(e.e1) + fx_s2_offset(p, p->stage_rows));
     return e;
 }
 
 }  // namespace
 
 size_t fx_exp_bytes(const tc_plan* p, int rows) {
-    return (size_t)rows * ((size_t)9 * (p->M + 1) * sizeof(int2) + 2 * sizeof(int) + (size_t)p->P_z * (2 * sizeof(int) + sizeof(double)));
+    return fx_s2_offset(p, rows) + (size_t)rows * p->P_z * sizeof(longlong2);
 }
 
 namespace {

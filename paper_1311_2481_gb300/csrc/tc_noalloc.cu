@@ -34,8 +34,8 @@ namespace {
 
 constexpr size_t kStaticScratchBytes = (size_t)80 << 20;
 // behind the lines, the exponents of the FP64 form's fixed-point lines (the staged rows'): a row has
-// 72 (M+1) + 8 + 16 P_z bytes of them (fx_exp_bytes) and 192 (M+1) P_z bytes of lines, M >= 1, P_z >= 3.
-// Where up to 2048 rows of lines fit 80 MiB, that is at most 10.1 MiB.
+// 72 (M+1) + 8 + 24 P_z bytes of them (fx_exp_bytes) and 192 (M+1) P_z bytes of lines, M >= 1, P_z >= 3.
+// Where up to 2048 rows of lines fit 80 MiB, that is at most 10.2 MiB.
 constexpr size_t kStaticExpBytes = (size_t)12 << 20;
 constexpr int kMaxDevices = 64;
 

@@ -63,3 +63,30 @@ def test_azimuthal_mean(N_r, M, K, kw, amp):
     bound = 8 * 2.0 ** -61 * 4 * U * np.abs((d[:, 0, K] + ut[:, 0, K] / r).real) + 2.0 ** -50 * np.abs(terms).sum((1, 2))
     err = np.abs(got - want)
     assert (err <= bound)[1:-1].all(), (err / bound).max()
+
+
+@pytest.mark.parametrize("N_r,M,K,kw", [(12, 4, 8, {}), (33, 8, 16, {}), (20, 25, 50, dict(P_theta=81, P_z=162)),
+                                        (10, 2, 384, dict(P_z=1152)), (24, 32, 64, dict(stage_rows=7))])
+def test_adjoint_keeps_m0_lines_of_real_fields(N_r, M, K, kw):
+    """Of adjoint fields whose m = 0 lines are those of real fields: + and - stay mirrored conjugates (the
+    transforms' part exactly, the solves' as x and its conjugate take the same operations), and with
+    them D1^T (g_+ + g_-) of the mean mode has no imaginary part for P^{-T} to magnify."""
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    from paper_1311_2481_gb300 import build, tc
+    build.build()
+    plan = tc.Plan(N_r, M, K, 1, 0.5, 1000.0, 0.0, LZ, 1e-6, **kw)
+    u = I.initial_state(plan.nodes(), M, K, 1, LZ, 0.5, 1000.0, 0.0, kind="broadband", amp=1e-2, seed=5)
+    st = tc.State(plan, torch.from_numpy(u).cuda())
+    st.started = True
+    y = []
+    for s in (1, 2, 3):
+        v = I.random_spectral((3,) + u.shape[1:], seed=s, hermitian_K=K)
+        v[1, :, 0] = np.conj(v[0, :, 0, ::-1])
+        v[:2, :, 0, K] = 1j * v[:1, :, 0, K].imag * np.array([1, -1])[:, None]   # the mean mode has no radial part
+        y.append(torch.from_numpy(v).cuda())
+    bar = tc.StateBar(*y)
+    for _ in range(2):
+        plan.adjoint_step(st, bar)
+        for f in (bar.u, bar.u_prev, bar.N_prev):
+            assert torch.equal(f[1, :, 0], f[0, :, 0].flip(-1).conj())
