@@ -25,9 +25,8 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 if ROOT not in sys.path:
     sys.path.insert(0, ROOT)
 
-# DRAM bytes (read + write) of one theta-pass launch of the FP64 form at the bench workload: not
-# captured for the fixed-point kernel
-THETA_TRAFFIC = None
+# DRAM bytes (read + write) of one launch in the FP64 step at the bench workload, from ncu
+TRAFFIC = {"k_pc": 113.6e6, "k_theta": 60.7e6}
 CFG2 = dict(N_r=64, M=32, K=64, m_p=1, eta=0.5, Re_i=1000.0, Re_o=0.0, L_z=2 * math.pi / 3.16, dt=5e-4)
 # mid-size case for profiling (inputs larger than L2, a few GB on the device)
 CFG_MID = dict(N_r=128, M=128, K=256, m_p=1, eta=0.5, Re_i=1000.0, Re_o=0.0, L_z=2 * math.pi / 3.16, dt=5e-4)
@@ -194,7 +193,7 @@ def kernel_rooflines(cfg, prof):
         out[name] = e
     return {"kernels": out, "hbm_peak_gbs": hbm, "hbm_peak_source": src,
             "fp64_peak_tflops": FP64_PEAK / 1e12,
-            "note": "k_pc: 2.4 M FP64 warp instructions per launch at the bench size (ncu), 54 % of the FP64 pipe (16 cycles per warp instruction); the transforms' fp64_frac is their algorithmic flops over the FP64 peak, which their fixed-point arithmetic does not use"}
+            "note": "k_pc: FP64 pipe 75 % busy at the bench size (ncu; a warp instruction takes it 16 cycles); the transforms' fp64_frac is their algorithmic flops over the FP64 peak, which their fixed-point arithmetic does not use"}
 
 
 def cufft_comparison(torch, cfg, dev, reps=20):
@@ -818,7 +817,9 @@ def run_ours(args):
     top = max(prof.items(), key=lambda kv: kv[1][1])
     Pt, Pz = 3 * cfg["M"], 3 * cfg["K"]
     flops = {"k_theta": theta_flops(cfg, Pt, Pz), "k_zinv": zpass_flops(cfg, Pz, 9),
-             "k_zfwd": zpass_flops(cfg, Pz, 3)}
+             "k_zfwd": zpass_flops(cfg, Pz, 3),
+             # five substitutions, four radial stencils and 60 more per complex value
+             "k_pc": cfg["N_r"] * (cfg["M"] + 1) * (2 * cfg["K"] + 1) * (5 * 52 + 4 * 36 + 60.0)}
     fp64_peak = FP64_PEAK
     # the FP64 FMA rate measured on this device by libtc's probe (8 independent FMA chains per
     # thread, 8 blocks of 256 threads per SM): the achievable counterpart of the unit-count peak
@@ -829,17 +830,17 @@ def run_ours(args):
         ach = flops[top[0]] / avg_s
         roof = {"kernel": top[0], "bound": "alu", "achieved": ach / 1e12, "peak": fp64_peak / 1e12,
                 "unit": "TFLOP/s", "frac": ach / fp64_peak,
-                # dram__bytes_read.sum + dram__bytes_write.sum of the FP64 theta pass per launch at
-                # this workload from one ncu --set full capture; None until the current kernel
-                # has been captured
-                "traffic": THETA_TRAFFIC if (top[0] == "k_theta" and main_is_bench) else None,
+                # dram__bytes_read.sum + dram__bytes_write.sum per launch at this workload
+                "traffic": TRAFFIC.get(top[0]) if main_is_bench else None,
                 "peak_source": "FP64: 152 SMs x 2 DFMA/clk/SM x 2 flop x 2.07 GHz (unit counts and max clock); "
                                "the transforms run in fixed point, off that pipe",
                 "peak_measured": fp64_measured / 1e12,
                 "frac_of_measured": ach / fp64_measured,
                 "peak_measured_source": "tc_probe_fp64_fma: 8 independent FMA chains per thread, "
                                         "8 x 256 threads per SM, best of 5 launches (CUDA events)",
-                "algorithmic": "7.5 complex FFTs of P_theta at 5 n log2 n + 25 flop/point per (r, z)"}
+                "algorithmic": "5 substitutions at 52 flop, 4 stencils at 36 and 60 more per complex value"
+                               if top[0] == "k_pc" else
+                               "7.5 complex FFTs of P_theta at 5 n log2 n + 25 flop/point per (r, z)"}
     else:
         roof = {"kernel": top[0], "bound": "alu", "achieved": None, "peak": fp64_peak / 1e12,
                 "unit": "TFLOP/s", "frac": None, "traffic": None, "peak_measured": fp64_measured / 1e12}

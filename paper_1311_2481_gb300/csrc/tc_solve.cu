@@ -387,8 +387,8 @@ __global__ void k_nn_r(const double2* __restrict__ Nc, const double2* __restrict
 // part of one mode per thread in fixed point (fx::Tile; FP64 next to the walls); the two threads of
 // a mode then trade halves, and each has both parts of half the rows for the rest, in FP64.  With
 // FP64 stencils the FP64 pipe bounded these kernels; now memory and what FP64 is left do.  N_r = 256,
-// M = 64, K = 128, before and after: right-hand sides of step 2 478 -> 257 us, of step 3 443 -> 309,
-// of step 4 438 -> 168, update 301 -> 277 (8 rows per tile: 263, 313, 185, 328).
+// M = 64, K = 128, before and after: right-hand sides of step 2 478 -> 270 us, of step 3 443 -> 312,
+// of step 4 438 -> 178, update 301 -> 277.
 struct Stencil {
     const double* w1;
     const int* col0;
